@@ -127,12 +127,12 @@ typedef struct {
  *               bit. A batch numbers its nodes from node_word0 on.
  *   zero_map    0: automatic (the autotuner's choice for the node set, else
  *               on; always on with a control variate); 1 on; 2 off. With it
- *               on, the path kernel of a context
- *               reads one shared all-zero drift record wherever the drift
- *               records of a stretch of cells are all zero (w constant
- *               there): the same values, so the same results bit for bit,
- *               with fewer L1 wavefronts and a few more instructions per
- *               sub-step. Batches ignore it. */
+ *               on, the path kernel of a context skips the drift where the
+ *               records of a tile's cells are all zero (w constant there): the
+ *               same values, so the same results bit for bit, with fewer
+ *               gathers and a few more instructions per sub-step. The kernel
+ *               leaves the map aside when nearly every tile has drift. Batches
+ *               and grids of more than 2^23 cells ignore it. */
 typedef struct {
     double dt;
     double Dt;

@@ -114,9 +114,7 @@ struct sdd_ctx {
     DevBuf<double> faces64;
     DevBuf<float> faces32;
     DevBuf<float4> bcoef, fcoef;  // bcoef holds one more record, all zero, after the cells'
-    DevBuf<uint32_t> zmap;        // zero map of the drift records (see PathArgs)
-    uint32_t zshift = 0;
-    int zwords = 0;
+    DevBuf<uint8_t> zmap;         // zero map of the drift records (kZmapBytes)
     DevBuf<uint4> cvcoef;      // control-variate table (per slice and cell, half-precision corners)
     int cv_slices = 0;
     int cv_mode = 0;           // 0 off, 1 the table as set, 2 the model re-tabulated per estimate, 3 field gradient
@@ -268,13 +266,12 @@ std::vector<int> block_edges(int n, int parts)
 }
 
 
-// The zero map of a single instance's drift records (map null: launches without it).
+// A single instance's tables for the path kernels: its zero map (map null: launches without it)
+// and the index of its all-zero drift record.
 struct ZmapRef {
     bool single = false;   // one instance: its tables go to the kernel as parameters
     InstDev inst{};        // the instance's tables (host copy of inst[0])
-    const uint32_t* map = nullptr;   // null: no zero map
-    int words = 0;
-    uint32_t shift = 0;
+    const uint8_t* map = nullptr;    // null: no zero map
     uint32_t cell = 0;
 };
 
@@ -289,8 +286,6 @@ InstDev inst_host(const sdd_ctx* c)
     I.ny = c->ny;
     I.sx = (float)(c->nx - 1);
     I.sy = (float)(c->ny - 1);
-    I.gxmax = std::nextafter((float)(c->nx - 1), 0.0f);
-    I.gymax = std::nextafter((float)(c->ny - 1), 0.0f);
     I.cell_bias = 0x4B000000u * (uint32_t)c->nx;
     I.cv_slices = c->cv_slices;
     I.cvcoef = c->cvcoef.p;
@@ -301,13 +296,12 @@ InstDev inst_host(const sdd_ctx* c)
 ZmapRef ctx_zmap(const sdd_ctx* c, bool use_map = true)
 {
     ZmapRef z;
+    const long long cells = (long long)(c->nx - 1) * (c->ny - 1);
+    if (cells > kOneMaxCells) return z;   // larger grids run the batch kernels, whose cell index is an integer's
     z.single = true;
     z.inst = inst_host(c);
-    if (!use_map) return z;
-    z.map = c->zmap.p;
-    z.words = c->zwords;
-    z.shift = c->zshift;
-    z.cell = (uint32_t)((size_t)(c->nx - 1) * (c->ny - 1));
+    z.cell = (uint32_t)cells;
+    if (use_map) z.map = c->zmap.p;
     return z;
 }
 
@@ -332,8 +326,7 @@ sdd_status prepare_parts(sdd_ctx* c, cudaStream_t s, bool w_part, bool f_part)
     }
     if (dw || df) {
         CU(c, launch_prep_cells(c->w.p, c->fld[c->cur][0].p, c->fld[c->cur][1].p, c->nx, c->ny,
-                                dw ? c->bcoef.p : nullptr, df ? c->fcoef.p : nullptr, c->d_status.p, s, c->zmap.p,
-                                c->zshift));
+                                dw ? c->bcoef.p : nullptr, df ? c->fcoef.p : nullptr, c->d_status.p, s, c->zmap.p));
     }
     if (w_part) c->dirty_w = false;
     if (f_part) c->dirty_fields = false;
@@ -348,7 +341,7 @@ sdd_status prepare(sdd_ctx* c, cudaStream_t s)
             CU(c, launch_winslow_faces(c->w.p, c->nx, c->ny, c->faces64.p, c->faces32.p, s));
         }
         CU(c, launch_prep_cells(c->w.p, c->fld[c->cur][0].p, c->fld[c->cur][1].p, c->nx, c->ny, c->bcoef.p,
-                                c->fcoef.p, c->d_status.p, s, c->zmap.p, c->zshift));
+                                c->fcoef.p, c->d_status.p, s, c->zmap.p));
         c->dirty_w = c->dirty_fields = false;
         return SDD_OK;
     }
@@ -504,8 +497,8 @@ sdd_status build_plan_segs(std::string* err, int sm_count, Plan& P, const std::v
         NodeDev& nd = P.nodes[k];
         nd.x = x[k];
         nd.y = y[k];
-        nd.xf = (float)x[k];
-        nd.yf = (float)y[k];
+        nd.xf = start_coord(x[k]);
+        nd.yf = start_coord(y[k]);
         nd.inst = inst_of[k];
         nd.ctr = ctr_of[k];
         nd.n_paths = (int32_t)np[k];
@@ -695,12 +688,8 @@ sdd_status run_plan_on(std::string* err, Plan& P, const InstDev* inst, const Out
         if (zm.single) {
             a.single = 1;
             a.one = zm.inst;
-            if (zm.map && zm.words > 0 && zm.words <= kZmapMaxWords) {
-                a.zmap = zm.map;
-                a.zwords = zm.words;
-                a.zshift = zm.shift;
-                a.zcell = zm.cell;
-            }
+            a.zmap = zm.map;
+            a.zcell = zm.cell;
         }
         const bool cv = cv_slices > 0;
         const int cvm = !cv ? 0 : cv_cell ? 2 : 1;
@@ -714,11 +703,12 @@ sdd_status run_plan_on(std::string* err, Plan& P, const InstDev* inst, const Out
         const int block = std::min(P.block, path_kernel_max_block(exit_mode, cvm, a.single != 0));
         const int64_t per_block = block / 32;
         int grid_max = P.grid;
-        if (block != P.block || cv || a.single) {
+        if (block != P.block || cv || a.single || surv) {
             int dev = 0, sms = 0;
             cudaGetDevice(&dev);
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-            grid_max = sms * path_kernel_blocks_per_sm(exit_mode, rec != nullptr, block, cvm, a.zwords, a.single != 0);
+            grid_max = sms * path_kernel_blocks_per_sm(exit_mode, rec != nullptr, block, cvm, a.zmap != nullptr, a.single != 0,
+                                                       surv != nullptr);
         }
         const int grid = (int)std::min<int64_t>(grid_max, std::max<int64_t>(1, (P.ntasks + per_block - 1) / per_block));
         if (ev_a) CU(err, cudaEventRecordWithFlags(ev_a, s, cudaEventRecordExternal));
@@ -1450,9 +1440,7 @@ sdd_status sdd_init(sdd_ctx** out, const sdd_grid* g, const float* w, const doub
     INIT_CU(c->faces32.alloc(faces_len(c)));
     INIT_CU(c->bcoef.alloc(2 * (cells + 1)));
     INIT_CU(cudaMemset(c->bcoef.p + 2 * cells, 0, 2 * sizeof(float4)));   // the all-zero record
-    c->zshift = zmap_shift((long long)cells);
-    c->zwords = zmap_words((long long)cells, c->zshift);
-    INIT_CU(c->zmap.alloc(c->zwords));
+    INIT_CU(c->zmap.alloc(kZmapBytes));
     INIT_CU(c->fcoef.alloc(2 * cells));
     INIT_CU(c->d_status.alloc(1));
     INIT_CU(c->d_step.alloc(1));
@@ -2045,8 +2033,8 @@ static sdd_status capture_step(sdd_ctx* c, const sdd_step_params* p, int K, int 
     }
     if (st == SDD_OK && c->pipe) {
         // the drift records; the face data come from the third branch forked above
-        cu(launch_prep_cells(c->w.p, nullptr, nullptr, c->nx, c->ny, c->bcoef.p, nullptr, c->d_status.p, s, c->zmap.p,
-                             c->zshift));
+        cu(launch_prep_cells(c->w.p, nullptr, nullptr, c->nx, c->ny, c->bcoef.p, nullptr, c->d_status.p, s,
+                             c->zmap.p));
         if (!c->user_faces && p->exit_mode != 0) cu(cudaStreamWaitEvent(s, c->fev[1], 0));
         c->dirty_w = false;
     } else if (st == SDD_OK) {

@@ -32,7 +32,6 @@ struct InstDev {
     const double* faces64; // face data, double precision
     int32_t nx, ny;
     float sx, sy;          // nx - 1, ny - 1 (inverse spacings)
-    float gxmax, gymax;    // largest floats below nx - 1, ny - 1
     uint32_t cell_bias;    // 0x4B000000 * nx (mod 2^32): cell index from the float bits of 2^23 + floor(g)
     int32_t cv_slices;     // slices of the control-variate table (0: none)
     const uint4* cvcoef;   // per slice and cell 2 uint4: corner values (half precision) of the xi model's gradient, then the eta model's
@@ -104,27 +103,29 @@ struct PathArgs {
     RecDev rec;
     const uint8_t* node_mask; // if non-null, only nodes with a nonzero entry run their paths
     void* surv;               // if non-null, survivors and plain exits leave records here, scored later (rec0 + path)
-    // zero map of the drift records (single-instance launches; zwords = 0: none): bit k of word k / 32
-    // set when a drift record of cells [k 2^zshift, (k + 1) 2^zshift) is nonzero; record zcell is all zero
-    const uint32_t* zmap;
-    int32_t zwords;
-    uint32_t zshift;
-    uint32_t zcell;
+    const uint8_t* zmap;      // zero map of the drift records (single-instance launches; null: none)
+    uint32_t zcell;           // index of a record that lanes without a cell read: the all-zero one (batches: 0)
     InstDev one;              // single: the one instance's tables (inst[0]), read as parameters
     int32_t single;           // 1: every task is of instance 0 and `one` holds its tables
 };
 
-// The zero map's size: at most kZmapMaxWords words (16 KB of shared memory per block of the path kernel).
-constexpr int kZmapMaxWords = 4096;
-inline uint32_t zmap_shift(long long cells)
+// Zero map of the drift records: one byte per tile of a 47 x 47 division of the unit square, 1 when a
+// drift record of a cell that reaches into the tile (or within 0.01 cells of it) is nonzero. Padded to 16 bytes.
+// 47 tiles: rows of 11.75 words fall on different banks, so a warp's 32 lookups take 2.6 shared-memory
+// wavefronts (with 127 tiles, rows a multiple of four words less one byte, about 10: a moving-front step
+// at 257^2 took 2.0 ms of paths against 1.83), and 2.2 KB per block leave L1 to the records.
+constexpr int kZmapTiles = 47;
+constexpr int kZmapBytes = (kZmapTiles * kZmapTiles + 15) / 16 * 16;
+
+// Largest grid of the single-instance path kernels: cell indices that single precision adds to 2^23 exactly.
+constexpr long long kOneMaxCells = 1LL << 23;
+
+// Start coordinate of a node's paths: the node's in single precision, inside the square when the node is.
+inline float start_coord(double v)
 {
-    uint32_t s = 0;
-    while (((cells + (1LL << s) - 1) >> s) > 32LL * kZmapMaxWords) ++s;
-    return s;
+    const float below_one = 0.99999994039535522461f;   // 1 - 2^-24
+    return v < 1.0 && (float)v > below_one ? below_one : (float)v;
 }
-inline int zmap_words(long long cells, uint32_t shift) { return (int)((((cells + (1LL << shift) - 1) >> shift) + 31) / 32); }
-// Shared memory for a map of `words` words: whole groups of 32, as the kernel's slots permute each group.
-inline size_t zmap_smem_bytes(int words) { return sizeof(uint32_t) * (size_t)((words + 31) / 32 * 32); }
 
 struct FinalArgs {
     const InstDev* inst;
@@ -160,17 +161,16 @@ cudaError_t launch_paths(const PathArgs& a, int exit_mode, bool record, int grid
 // exit_mode 0 with an even number of sub-steps has its own kernel (no odd last pair)
 cudaError_t launch_finalize(const FinalArgs& a, cudaStream_t s);
 cudaError_t launch_score_surv(const ScoreArgs& a, bool cv, cudaStream_t s);
-int path_kernel_blocks_per_sm(int exit_mode, bool record, int block, int cvm = 0, int zwords = 0,
-                              bool single = false);
+int path_kernel_blocks_per_sm(int exit_mode, bool record, int block, int cvm = 0, bool map = false,
+                              bool single = false, bool defer = false);
 // the largest block the path kernel of this exit mode is compiled for (single: one instance)
 int path_kernel_max_block(int exit_mode, int cvm = 0, bool single = false);
 
 // Cell records of the drift (from w; bcoef null: skipped) and of the fields
 // (from xi, eta; fcoef null: skipped); with the drift records, if zmap is
-// non-null, their zero map (zmap_words(cells, zshift) words, see PathArgs).
+// non-null, their zero map (kZmapBytes bytes).
 cudaError_t launch_prep_cells(const float* w, const double* xi, const double* eta, int nx, int ny, float4* bcoef,
-                              float4* fcoef, int* status, cudaStream_t s, uint32_t* zmap = nullptr,
-                              uint32_t zshift = 0);
+                              float4* fcoef, int* status, cudaStream_t s, uint8_t* zmap = nullptr);
 // The paper's boundary data from w (faces64) and, if faces32 is non-null, its single-precision copy.
 cudaError_t launch_winslow_faces(const float* w, int nx, int ny, double* faces64, float* faces32, cudaStream_t s);
 cudaError_t launch_cv_cells(const double* grad, int slices, int nx, int ny, uint4* cvcoef, cudaStream_t s);

@@ -65,13 +65,15 @@ __global__ void __launch_bounds__(PREP_TX * PREP_TY) k_prep_cells(const float* _
                                                                   const double* __restrict__ xi,
                                                                   const double* __restrict__ eta, int nx, int ny,
                                                                   float4* __restrict__ bcoef,
-                                                                  float4* __restrict__ fcoef, int* status)
+                                                                  float4* __restrict__ fcoef, int* status,
+                                                                  uint8_t* __restrict__ zmap)
 {
     __shared__ double2 bn[PREP_TY + 1][PREP_TX + 1];
     const int ix0 = blockIdx.x * PREP_TX, iy0 = blockIdx.y * PREP_TY;
     const int ix = ix0 + threadIdx.x, iy = iy0 + threadIdx.y;
     const bool cell_in = ix < nx - 1 && iy < ny - 1;
     if (bcoef) {
+        bool nonzero = false;
         const double rx = 0.5 * (double)(nx - 1), ry = 0.5 * (double)(ny - 1);
         const int tid = threadIdx.y * PREP_TX + threadIdx.x;
         for (int k = tid; k < (PREP_TX + 1) * (PREP_TY + 1); k += PREP_TX * PREP_TY) {
@@ -91,8 +93,26 @@ __global__ void __launch_bounds__(PREP_TX * PREP_TY) k_prep_cells(const float* _
             const int tx = threadIdx.x, ty = threadIdx.y;
             const double2 b00 = bn[ty][tx], b10 = bn[ty][tx + 1], b01 = bn[ty + 1][tx], b11 = bn[ty + 1][tx + 1];
             const long long cell = (long long)iy * (nx - 1) + ix;
-            bilinear_coefs2(b00.x, b10.x, b01.x, b11.x, b00.y, b10.y, b01.y, b11.y, bcoef[2 * cell + 0],
-                            bcoef[2 * cell + 1]);
+            float4 lo, hi;
+            bilinear_coefs2(b00.x, b10.x, b01.x, b11.x, b00.y, b10.y, b01.y, b11.y, lo, hi);
+            bcoef[2 * cell + 0] = lo;
+            bcoef[2 * cell + 1] = hi;
+            nonzero = lo.x != 0.f || lo.y != 0.f || lo.z != 0.f || lo.w != 0.f || hi.x != 0.f || hi.y != 0.f ||
+                      hi.z != 0.f || hi.w != 0.f;
+        }
+        if (zmap) {
+            // mark the tiles that the cell reaches, once per run of cells of a warp's row in the same tiles
+            const float fx = (float)kZmapTiles / (float)(nx - 1), fy = (float)kZmapTiles / (float)(ny - 1);
+            const int x0 = max(0, (int)floorf(((float)ix - 0.01f) * fx));
+            const int x1 = min(kZmapTiles - 1, (int)floorf(((float)ix + 1.01f) * fx));
+            const int run = nonzero ? x0 * kZmapTiles + x1 : -1;
+            const int before = __shfl_up_sync(0xffffffffu, run, 1);
+            if (nonzero && (threadIdx.x == 0 || run != before)) {
+                const int y0 = max(0, (int)floorf(((float)iy - 0.01f) * fy));
+                const int y1 = min(kZmapTiles - 1, (int)floorf(((float)iy + 1.01f) * fy));
+                for (int ty = y0; ty <= y1; ++ty)
+                    for (int tx = x0; tx <= x1; ++tx) zmap[ty * kZmapTiles + tx] = 1;
+            }
         }
     }
     if (fcoef && cell_in) {
@@ -196,44 +216,18 @@ __global__ void k_faces32(const double* __restrict__ f64, float* __restrict__ f3
     if (k < n) f32[k] = (float)f64[k];
 }
 
-// Zero map of the drift records: one block per map word (32 segments of 2^zshift consecutive cells in
-// row-major order); bit k set when a record of segment k has a nonzero coefficient. The last word's bits
-// past the last cell stay clear (no path reaches those cells).
-__global__ void __launch_bounds__(256) k_drift_zmap(const float4* __restrict__ bcoef, long long cells,
-                                                    uint32_t zshift, uint32_t* __restrict__ zmap)
-{
-    __shared__ int nz[32];
-    if (threadIdx.x < 32) nz[threadIdx.x] = 0;
-    __syncthreads();
-    const long long c0 = (long long)blockIdx.x << (zshift + 5);
-    const long long span = 32LL << zshift;
-    for (long long k = threadIdx.x; k < span; k += blockDim.x) {
-        const long long c = c0 + k;
-        if (c >= cells) break;
-        const float4 lo = bcoef[2 * c], hi = bcoef[2 * c + 1];
-        if (lo.x != 0.f || lo.y != 0.f || lo.z != 0.f || lo.w != 0.f || hi.x != 0.f || hi.y != 0.f ||
-            hi.z != 0.f || hi.w != 0.f)
-            nz[k >> zshift] = 1;
-    }
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        const unsigned word = __ballot_sync(0xffffffffu, nz[threadIdx.x] != 0);
-        if (threadIdx.x == 0) zmap[blockIdx.x] = word;
-    }
-}
-
 }  // namespace
 
 cudaError_t launch_prep_cells(const float* w, const double* xi, const double* eta, int nx, int ny, float4* bcoef,
-                              float4* fcoef, int* status, cudaStream_t s, uint32_t* zmap, uint32_t zshift)
+                              float4* fcoef, int* status, cudaStream_t s, uint8_t* zmap)
 {
     const dim3 block(PREP_TX, PREP_TY);
     const dim3 grid((nx - 1 + PREP_TX - 1) / PREP_TX, (ny - 1 + PREP_TY - 1) / PREP_TY);
-    k_prep_cells<<<grid, block, 0, s>>>(w, xi, eta, nx, ny, bcoef, fcoef, status);
     if (bcoef && zmap) {
-        const long long cells = (long long)(nx - 1) * (ny - 1);
-        k_drift_zmap<<<zmap_words(cells, zshift), 256, 0, s>>>(bcoef, cells, zshift, zmap);
+        const cudaError_t e = cudaMemsetAsync(zmap, 0, kZmapBytes, s);
+        if (e != cudaSuccess) return e;
     }
+    k_prep_cells<<<grid, block, 0, s>>>(w, xi, eta, nx, ny, bcoef, fcoef, status, zmap);
     return cudaGetLastError();
 }
 

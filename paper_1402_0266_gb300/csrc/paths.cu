@@ -10,10 +10,10 @@
 //
 // Execution: a persistent grid; each warp repeatedly takes a task (one node,
 // a contiguous range of its paths) from a counter, on its own. Each lane runs one path at
-// a time and, when its path ends, takes the task's next unstarted path, so
-// lanes stay busy when paths leave early. In the paper's (plain) exit mode one
-// Philox block supplies the normals of two consecutive sub-steps, so paths are
-// only started at even sub-step boundaries. Scores are summed per lane with
+// a time; idle lanes take the task's next unstarted paths when some path of the
+// warp reaches the end of the step or enough lanes are idle. In the paper's
+// (plain) exit mode one Philox block supplies the normals of two consecutive
+// sub-steps, so a warp advances its paths by sub-step pairs. Scores are summed per lane with
 // compensation (single precision, shifted by the node's start coordinates),
 // then per warp in double precision; the per-node reduction over tasks runs in
 // a fixed order, so results do not depend on scheduling.
@@ -46,54 +46,45 @@ __device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b
 
 struct Cell {
     float2 st;        // local coordinates (s, t) in [0, 1)
-    uint32_t idx;     // row-major cell index
+    uint32_t idx;     // row-major cell index (plus kCellBits in single-instance kernels)
 };
 
-// Cell of pos and local coordinates. floor() through a directed add of 2^23:
+// Cell of pos, strictly inside the unit square, and local coordinates. g = pos (n - 1) stays below n - 1: the
+// largest single-precision pos below 1 is 1 - 2^-24, and (n - 1)(1 - 2^-24) lies more than half an ulp below
+// n - 1 (or is the float below it, for a power of two). floor() through a directed add of 2^23:
 // for 0 <= g < 2^23, (g + 2^23) rounded down is 2^23 + floor(g) exactly, and
-// its bits are 0x4B000000 + floor(g); cell_bias removes that offset from the
+// its bits are 0x4B000000 + floor(g). ONE (at most kOneMaxCells cells): the cell index by one exact
+// multiply-add in single precision, 2^23 + j (nx - 1) + i, left in its float bits; the table
+// pointers take the offset of those bits (rec2). Otherwise cell_bias removes the offset from the
 // row-major cell index in 32-bit wrap-around arithmetic.
+constexpr uint32_t kCellBits = 0x4B000000u;
+
+template <bool ONE>
 __device__ __forceinline__ Cell locate(const InstDev& I, float2 pos)
 {
-    float2 g = __fmul2_rn(pos, f2(I.sx, I.sy));
-    g.x = fminf(g.x, I.gxmax);
-    g.y = fminf(g.y, I.gymax);
+    const float2 g = __fmul2_rn(pos, f2(I.sx, I.sy));
     const float2 t = __fadd2_rd(g, f2(8388608.0f, 8388608.0f));
-    const uint32_t cell = __float_as_uint(t.y) * (uint32_t)(I.nx - 1) + __float_as_uint(t.x) - I.cell_bias;
     const float2 fl = __fadd2_rn(t, f2(-8388608.0f, -8388608.0f));    // floor(g), exact
     Cell c;
     c.st = __ffma2_rn(fl, f2(-1.0f, -1.0f), g);                        // g - floor(g), exact
-    c.idx = cell;
+    c.idx = ONE ? __float_as_uint(__fmaf_rn(fl.y, I.sx, t.x))
+                : __float_as_uint(t.y) * (uint32_t)(I.nx - 1) + __float_as_uint(t.x) - I.cell_bias;
     return c;
 }
 
-// The two coefficient records of cell idx in a table of cell records.
-__device__ __forceinline__ const float4* rec2(const float4* base, uint32_t idx) { return base + 2 * (size_t)idx; }
-
-// The drift records of a cell. With the zero map (ZM), a cell of a segment
-// whose drift records are all zero (w constant around it: b = -grad w / w = 0
-// exactly) reads the all-zero record at index zcell instead: the same values,
-// so the same arithmetic and results, but every lane of a warp that is in such
-// a segment reads the same 32 bytes, one L1 wavefront for all of them, where
-// each lane's own cell would cost one wavefront per lane. zsm: the map in
-// shared memory, bit k of word k / 32 set when a record of cells
-// [k 2^zshift, (k + 1) 2^zshift) is nonzero; word w sits at zmap_slot(w).
-// Shared-memory slot of map word w: the word's bank (its low five bits) xored
-// with the next five bits. A warp's lanes sit in nearby rows of cells, whose
-// words lie a multiple of 32 apart where rows are 32 words long or a divisor
-// of that: unswizzled they would share a bank and serialise the load.
-__device__ __forceinline__ uint32_t zmap_slot(uint32_t w) { return w ^ ((w >> 5) & 31u); }
-
-template <bool ZM>
-__device__ __forceinline__ const float4* drift_rec(const InstDev& I, const Cell& c, const uint32_t* zsm,
-                                                   const PathArgs& a)
+// The record of cell idx in a table of records.
+template <bool ONE, typename T>
+__device__ __forceinline__ const T* record(const T* base, uint32_t idx, int per_cell)
 {
-    uint32_t idx = c.idx;
-    if (ZM) {
-        const uint32_t seg = idx >> a.zshift;
-        if (!((zsm[zmap_slot(seg >> 5)] >> (seg & 31u)) & 1u)) idx = a.zcell;
-    }
-    return rec2(I.bcoef, idx);
+    const long long bytes = (long long)sizeof(T) * per_cell;
+    return reinterpret_cast<const T*>(reinterpret_cast<const char*>(base) - (ONE ? bytes * (long long)kCellBits : 0) +
+                                      bytes * (long long)idx);
+}
+
+template <bool ONE>
+__device__ __forceinline__ const float4* rec2(const float4* base, uint32_t idx)
+{
+    return record<ONE>(base, idx, 2);
 }
 
 // A cell's two records in one 256-bit read-only load (records are 32-byte
@@ -122,13 +113,12 @@ __device__ __forceinline__ float2 em(const float4& lo, const float4& hi, float2 
     return __fadd2_rn(__ffma2_rn(eval2(lo, hi, st), dt2, pos), z);
 }
 
-// Strictly inside the unit square: x - x^2 > 0 and y - y^2 > 0. Each is one
-// rounding of the exact value, whose sign it keeps (barring underflow below
-// 2^-126, which no position of a path reaches).
+// Strictly inside the unit square: x^2 < x and y^2 < y. Rounding keeps the order
+// (x^2 and x are at least an ulp of x apart, or x^2 underflows below x). False for a NaN.
 __device__ __forceinline__ bool inside2(float2 p)
 {
-    const float2 q = __ffma2_rn(f2(-p.x, -p.y), p, p);
-    return fminf(q.x, q.y) > 0.0f;
+    const float2 q = __fmul2_rn(p, p);
+    return q.x < p.x && q.y < p.y;
 }
 
 // Face `face` at tangential coordinate s: the offset of its table (field 0;
@@ -242,9 +232,10 @@ __device__ __forceinline__ float2 corners2(const uint4& r, float2 ss, float2 oms
 
 // Control variate: the model gradients of xi and eta at the cell's point
 // (slice q), gxi = (d/dx, d/dy) of the xi model, geta of the eta model.
+template <bool ONE>
 __device__ __forceinline__ void cv_eval(const InstDev& I, const Cell& c, int q, float2& gxi, float2& geta)
 {
-    const uint4* r = I.cvcoef + 2 * ((size_t)q * (size_t)(I.nx - 1) * (size_t)(I.ny - 1) + c.idx);
+    const uint4* r = record<ONE>(I.cvcoef + 2 * ((size_t)q * (size_t)(I.nx - 1) * (size_t)(I.ny - 1)), c.idx, 2);
     uint4 gx, ge;
     load_words(r, gx, ge);
     const float2 ss = f2(c.st.x, c.st.x), tt = f2(c.st.y, c.st.y);
@@ -255,9 +246,10 @@ __device__ __forceinline__ void cv_eval(const InstDev& I, const Cell& c, int q, 
 
 // Control variate of one value per cell: (d/dx, d/dy) of xi, then of eta, on
 // the cell holding the point, in one 128-bit read-only load.
+template <bool ONE>
 __device__ __forceinline__ void cv_cell(const InstDev& I, const Cell& c, float2& gxi, float2& geta)
 {
-    const float4 g = __ldg(I.cvcell + c.idx);
+    const float4 g = __ldg(record<ONE>(I.cvcell, c.idx, 1));
     gxi = f2(g.x, g.y);
     geta = f2(g.z, g.w);
 }
@@ -270,6 +262,7 @@ __device__ __forceinline__ void cv_acc(float2 gxi, float2 geta, float2 z, float2
     acc_eta = __ffma2_rn(geta, z, acc_eta);
 }
 
+// Compensated sums of a lane's scores and their squares.
 struct Acc {
     float s, cs, q, cq;
     __device__ __forceinline__ void add(float v)
@@ -328,232 +321,301 @@ __device__ __forceinline__ float2 exit_record(float x, float y, float xn, float 
     return f2(-1.0f - (float)face, t);
 }
 
-// Lanes refilled together below this count spend a loop pass drawing their
-// first normals instead of a divergent Philox block (front257: 2.7% faster).
-constexpr int WARM_MIN = 8;
+// Idle lanes that call for a refill. A lane whose path left the domain stays
+// idle until this many do, or until some path of the warp reaches the end of
+// the step: a refill costs its warp about one pass's worth of bookkeeping.
+constexpr int REFILL_MIN = 8;
+
+// The draws of one path: Philox block d of path p, its first two rounds reduced
+// to what changes with d. With counter (p, node, d, step), round 1 multiplies p
+// and d, round 2 multiplies a word of d and the node and one of p and the step:
+// of the two rounds' four products only the two of d are formed per draw.
+struct PathWords {
+    uint32_t u, v, w;
+};
+
+__device__ __forceinline__ PathWords path_words(uint32_t path, uint32_t step, const PhiloxKeys& K)
+{
+    const unsigned long long p0 = (unsigned long long)0xD2511F53u * path;
+    const uint32_t z1 = (uint32_t)(p0 >> 32) ^ step ^ K.rk[1];
+    const unsigned long long p1 = (unsigned long long)0xCD9E8D57u * z1;
+    return PathWords{(uint32_t)(p1 >> 32) ^ K.rk[2], (uint32_t)p1, (uint32_t)p0 ^ K.rk[3]};
+}
+
+// Rounds 1 and 2 of block d: nodek is the node word xor round 1's first key.
+__device__ __forceinline__ uint4 draw_begin(const PathWords& q, uint32_t nodek, uint32_t d)
+{
+    const unsigned long long p1 = (unsigned long long)0xCD9E8D57u * d;
+    const unsigned long long p0 = (unsigned long long)0xD2511F53u * ((uint32_t)(p1 >> 32) ^ nodek);
+    return make_uint4(q.u ^ (uint32_t)p1, q.v, (uint32_t)(p0 >> 32) ^ q.w, (uint32_t)p0);
+}
+
+// Tile of the zero map that holds p (shared-memory offset): floor(T p) per axis,
+// T = kZmapTiles, by one fused multiply-add rounded down at 2, whose unit is
+// 2^-22: the float bits are 0x40000000 + tile, and with the pitch T = 4 q - 1 the
+// two offsets cancel (0x40000000 * 4 q = 0 mod 2^32). Positions outside the
+// square land on any byte of the map: their lanes' results are not used.
+__device__ __forceinline__ uint32_t zmap_offset(float2 p)
+{
+    static_assert(kZmapTiles % 4 == 3, "the pitch cancels the offset of the float bits");
+    constexpr float scale = kZmapTiles * (1.0f / 4194304.0f);
+    const float2 t = __ffma2_rd(p, f2(scale, scale), f2(2.0f, 2.0f));
+    return min(__float_as_uint(t.y) * (uint32_t)kZmapTiles + __float_as_uint(t.x), (uint32_t)kZmapBytes - 1u);
+}
 
 // MODE 0: the paper's test, sub-step pairs; MODE 1: with the bridge test;
 // MODE 2: as MODE 0 when K is even (every pair has both sub-steps).
 // CVM: 0 no control variate; otherwise subtract sum_j G(s_j, X_j) . sqrt(2) dW_j
 // from both scores, G from node values interpolated bilinearly in time slices
 // (1, cv_eval) or one value per cell (2, cv_cell).
-// Kernel variants by where the tables come from: VAR_MULTI, each task's
-// instance from the instance table (batches); VAR_ONE, a single instance whose
-// tables are kernel parameters (no registers held for them); VAR_ZM, VAR_ONE
-// with the zero map of the drift records. Launch shapes: a single instance's
-// kernel fits 40 registers (48 warps per SM; 64 with the control variate of
-// node values, 48 with that of cell values), the batch kernel 64 (32 warps;
-// 80 with a control variate).
-constexpr int VAR_MULTI = 0, VAR_ONE = 1, VAR_ZM = 2;
-constexpr int kCvCellBlocks = 5;   // cell-valued control variate, single instance: 48 registers, 40 warps per SM
+// VAR_MULTI: each task's instance from the instance table (batches); VAR_ONE: a
+// single instance whose tables are kernel parameters, with its zero map if it has one.
+// DEFER: survivors and plain exits leave records for k_score_surv.
+constexpr int VAR_MULTI = 0, VAR_ONE = 1;
 constexpr int kOneMaxBlock = 256;
 constexpr int paths_max_block(int cvm, int var) { return cvm ? kCvMaxBlock : var != VAR_MULTI ? kOneMaxBlock : 512; }
-constexpr int paths_min_blocks(int cvm, int var)
+constexpr int paths_min_blocks(int cvm, int var, bool defer)
 {
-    return cvm == 2 ? (var != VAR_MULTI ? kCvCellBlocks : 3) : cvm ? (var != VAR_MULTI ? 4 : 3)
-                                                                    : (var != VAR_MULTI ? 6 : 2);
+    return cvm ? (var != VAR_MULTI ? 4 : 3) : var != VAR_MULTI ? 5 : 2;
 }
 
-template <int MODE, bool RECORD, int CVM, int VAR>
-__global__ void __launch_bounds__(paths_max_block(CVM, VAR), paths_min_blocks(CVM, VAR))
-    k_paths(const PathArgs a)
+// A lane's sums over a task, in shared memory: they change once per path, and the
+// registers they would hold through every sub-step are worth more there.
+// Word k of thread i at [k][i]: no bank conflicts.
+template <int BLOCK, bool SCORES>
+struct LaneSums {
+    int exits[BLOCK], steps[BLOCK];
+    float acc[SCORES ? 8 : 1][SCORES ? BLOCK : 1];
+
+    __device__ __forceinline__ void clear()
+    {
+        exits[threadIdx.x] = steps[threadIdx.x] = 0;
+        if (SCORES)
+#pragma unroll
+            for (int k = 0; k < 8; ++k) acc[k][threadIdx.x] = 0.f;
+    }
+    __device__ __forceinline__ Acc get(int f) const
+    {
+        return Acc{acc[4 * f][threadIdx.x], acc[4 * f + 1][threadIdx.x], acc[4 * f + 2][threadIdx.x],
+                   acc[4 * f + 3][threadIdx.x]};
+    }
+    __device__ __forceinline__ void add(int f, float v)
+    {
+        Acc x = get(f);
+        x.add(v);
+        acc[4 * f][threadIdx.x] = x.s;
+        acc[4 * f + 1][threadIdx.x] = x.cs;
+        acc[4 * f + 2][threadIdx.x] = x.q;
+        acc[4 * f + 3][threadIdx.x] = x.cq;
+    }
+};
+
+// Node data read again where a path starts or ends rather than held in registers
+// (volatile: the compiler would otherwise keep the first read).
+__device__ __forceinline__ float2 node_start(const NodeDev* nd)
 {
-    constexpr bool ZM = VAR == VAR_ZM;
+    float2 v;
+    asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(&nd->xf));
+    return v;
+}
+
+__device__ __forceinline__ long long node_records(const NodeDev* nd)
+{
+    long long v;
+    asm volatile("ld.global.nc.s64 %0, [%1];" : "=l"(v) : "l"(&nd->rec0));
+    return v;
+}
+
+__device__ __forceinline__ unsigned lanes_below()
+{
+    unsigned m;
+    asm volatile("mov.u32 %0, %%lanemask_lt;" : "=r"(m));
+    return m;
+}
+
+// The tasks of one warp. MAP: the drift is read through the zero map zsm: a lane in
+// an unmarked tile has zero drift (it reads the all-zero record when other lanes of
+// its warp need theirs), and a warp without a lane in a marked tile only adds the increment.
+//
+// What bounds it (GB300, two sub-steps of a warp's 32 paths = one pass): a gather of 32 records that
+// miss L1 takes 34 cycles of the SM whatever its width (32 bytes per cycle from L2), so a pass with
+// drift everywhere costs 64 or more (2.7e11 path-steps/s at 2049^2, L1 data pipe 87 % busy); a pass
+// without drift is 119 instructions, 45 cycles, bound by issue slots and the FMA pipe's wide
+// multiplies (4.5e11). Hence the branch around the gather, the draws' shared first rounds, the sums
+// in shared memory and 48 registers (40 warps per SM; 32 and 48 warps are within 2 %), a draw made
+// where it is used rather than a pass ahead (fewer registers and moves; the other warps cover the
+// gathers), and bookkeeping only when a path ends. On a 2049^2 ring (28,609 nodes x 2e4 paths x 100
+// sub-steps): 145 ms per launch against 179 ms for the kernel that tested every path in every pass
+// and redirected gathers without skipping them, 92 instructions per path-step.
+template <int MODE, bool RECORD, int CVM, int VAR, bool DEFER, bool MAP>
+__device__ __forceinline__ void walk_tasks(const PathArgs& a, const uint8_t* zsm,
+                                           LaneSums<paths_max_block(CVM, VAR), !DEFER || MODE == 1>& sums)
+{
     constexpr bool CV = CVM != 0;
     constexpr bool CVT = CVM == 1;   // node values in time slices
-    extern __shared__ uint32_t zsm[];   // the zero map of the drift records (ZM)
-    if (ZM) {
-        for (int k = threadIdx.x; k < a.zwords; k += blockDim.x) zsm[zmap_slot((uint32_t)k)] = a.zmap[k];
-        __syncthreads();
-    }
-    const int lane = threadIdx.x & 31;
-    const unsigned below = (1u << lane) - 1u;
+    constexpr bool ONE = VAR != VAR_MULTI;
+    constexpr bool PAIRS = MODE != 1;
+    constexpr bool ACC = !DEFER || MODE == 1;   // some scores are summed here
     const uint32_t step = a.step_ptr ? *a.step_ptr : a.step_index;
     const int K = a.K;
-    const float dt = a.dt;
-    constexpr bool PAIRS = MODE != 1;
+    const int P = PAIRS ? (K + 1) >> 1 : K;   // passes of a path: sub-step pairs, or sub-steps
+    const float2 dt2 = f2(a.dt, a.dt);
+    // records that lanes without a cell read: the all-zero one (batches: any), the first cell's
+    const uint32_t zcell = (ONE ? kCellBits : 0u) + a.zcell, cell0 = ONE ? kCellBits : 0u;
 
     // Each warp takes the next task as soon as its last one is done (no wait
     // for the block's other warps); tasks go node by node, so warps started
     // together share the node's neighbourhood in L1.
     for (;;) {
         int tq = 0;
-        if (lane == 0) tq = atomicAdd(a.queue, 1);
+        if (lanes_below() == 0) tq = atomicAdd(a.queue, 1);
         const int t = __shfl_sync(FULL, tq, 0);
         if (t >= a.ntasks) return;
 
         const Task task = a.tasks[t];
         if (a.node_mask && !a.node_mask[task.node]) continue;   // not a key point this step
-        const NodeDev& nd = a.nodes[task.node];
+        const NodeDev* const nd = a.nodes + task.node;
         // a single instance's tables come from the kernel parameters (no registers held for them)
         InstDev Iloc;
-        if (VAR == VAR_MULTI) Iloc = a.inst[nd.inst];
+        if (VAR == VAR_MULTI) Iloc = a.inst[nd->inst];
         const InstDev& I = VAR != VAR_MULTI ? a.one : Iloc;
-        const float x0 = nd.xf, y0 = nd.yf;
-        const uint32_t nctr = nd.ctr;
-        const int end = task.path0 + task.npaths;
-        int next = task.path0 + 32;
-        int path = task.path0 + lane;
-        bool alive = path < end;
-        float2 pos = f2(x0, y0);
-        int m = 0;  // draw index: the sub-step pair (plain mode) or the sub-step (bridge mode)
-        // normals of draw m, already scaled by sqrt(2 dt): zA for the first
-        // sub-step, zB for the second (plain mode); ub the bridge uniform
-        float2 zA = f2(0.f, 0.f), zB = f2(0.f, 0.f);
-        float ub = 1.f;
+        const uint32_t nodek = nd->ctr ^ a.keys.rk[0];
+        const uint32_t end = (uint32_t)task.path0 + (uint32_t)task.npaths;
+        uint32_t next = (uint32_t)task.path0, path = 0;
+        bool alive = false;
+        PathWords pw{};
+        float2 pos = f2(0.5f, 0.5f);
+        int m = 0;        // the path's pass: its draw
         float2 cvx = f2(0.f, 0.f), cve = f2(0.f, 0.f);  // control-variate sums of the path
         int cvq = 0, cvn = CVT ? a.cv_bound[1] : 0;      // slice of the current sub-step, start of the next
-        const float2 dt2 = f2(dt, dt);
-        auto first_draw = [&]() {
-            uint4 r = make_uint4((uint32_t)path, nctr, 0u, step);
-            philox_rounds_rk<0, 10>(r, a.keys);
-            if (PAIRS) {
-                box_muller2(r, a.bm_scale, zA, zB);
-            } else {
-                box_muller(r.x, r.y, a.bm_scale, zA.x, zA.y);
-                ub = uniform_pos(r.z);
-            }
-        };
-        if (alive) first_draw();
-        Acc ax{0.f, 0.f, 0.f, 0.f}, ae{0.f, 0.f, 0.f, 0.f};
-        int exits = 0, steps = 0;
+        sums.clear();
 
-        while (__any_sync(FULL, alive)) {
-            if (alive) {
-                bool done = false;
-                int code = -1, taken = 0;
-                float yxi = 0.f, yeta = 0.f, xe = 0.f, ye = 0.f;
-                const bool warm = m < 0;   // draw -1: the pass draws the path's first normals
-                float2 seg = f2(REC_SKIP, 0.f);   // a plain exit's crossing, scored later
-                // sub-step A: gather, then the next draw's first rounds while the gather is in flight
-                const Cell cA = locate(I, pos);
-                float4 gA0, gA1;
-                load_cell(drift_rec<ZM>(I, cA, zsm, a), gA0, gA1);
+        // One sub-step from p with increment z, for lanes with ok (the others' results are not used,
+        // and their p may lie anywhere): p + b(p) dt + z.
+        auto advance = [&](float2 p, float2 z, bool ok, bool count, int j) -> float2 {
+            bool g = ok;
+            if (MAP) g = zsm[zmap_offset(p)] != 0 && ok;
+            float2 q = __fadd2_rn(p, z);
+            if (CV || !MAP || __any_sync(FULL, g)) {
+                Cell c = locate<ONE>(I, p);
+                if (CV) c.idx = ok ? c.idx : cell0;
+                float4 lo, hi;
+                load_cell(rec2<ONE>(I.bcoef, g ? c.idx : zcell), lo, hi);
                 if (CV) {
-                    float2 gxA, geA;   // the model at X_j
+                    // the model at X_j; the sub-step counts only when the path takes it
+                    const float2 zt = count ? z : f2(0.f, 0.f);
+                    float2 gx, ge;
                     if (CVT) {
-                        const int j = PAIRS ? 2 * m : m;
-                        if (j >= cvn) cvn = a.cv_bound[++cvq + 1];
-                        cv_eval(I, cA, cvq, gxA, geA);
+                        if (count && j >= cvn) cvn = a.cv_bound[++cvq + 1];
+                        cv_eval<ONE>(I, c, cvq, gx, ge);
                     } else {
-                        cv_cell(I, cA, gxA, geA);
+                        cv_cell<ONE>(I, c, gx, ge);
                     }
-                    cv_acc(gxA, geA, zA, cvx, cve);
+                    cv_acc(gx, ge, zt, cvx, cve);
                 }
-                uint4 r = make_uint4((uint32_t)path, nctr, (uint32_t)(m + 1), step);
-                philox_rounds_rk<0, 5>(r, a.keys);
-                const float2 pa = em(gA0, gA1, cA.st, pos, dt2, zA);
-                const bool outA = !inside2(pa);
-                if (PAIRS) {
-                    // sub-step B from the point A reached (or from X_j when A left: harmless, in bounds)
-                    const float2 pq = outA ? pos : pa;
-                    const Cell cB = locate(I, pq);
-                    float4 gB0, gB1;
-                    load_cell(drift_rec<ZM>(I, cB, zsm, a), gB0, gB1);
-                    philox_rounds_rk<5, 10>(r, a.keys);
-                    float2 nA, nB;
-                    box_muller2(r, a.bm_scale, nA, nB);
-                    const float2 pb = em(gB0, gB1, cB.st, pq, dt2, zB);
-                    const bool haveB = (MODE == 2) || 2 * m + 1 < K;
-                    const bool outB = haveB && !outA && !inside2(pb);
-                    if (CV) {
-                        // the second sub-step counts only when the path takes it
-                        const float2 zt = (haveB && !outA) ? zB : f2(0.f, 0.f);
-                        float2 gxB, geB;
+                q = em(lo, hi, c.st, p, dt2, z);
+            }
+            return q;
+        };
+
+        int k = 0;   // passes until a path of the warp ends with the step
+        for (;;) {
+            if (k == 0) {
+                // the lanes without a path take the task's next ones, in lane order
+                const unsigned idle = __ballot_sync(FULL, !alive);
+                if (next < end) {
+                    const uint32_t cand = next + __popc(idle & lanes_below());
+                    next += __popc(idle);
+                    if (!alive && cand < end) {
+                        alive = true;
+                        path = cand;
+                        pw = path_words(path, step, a.keys);
+                        pos = node_start(nd);
+                        m = 0;
+                        if (CV) cvx = cve = f2(0.f, 0.f);
                         if (CVT) {
-                            if (haveB && 2 * m + 1 >= cvn) cvn = a.cv_bound[++cvq + 1];
-                            cv_eval(I, cB, cvq, gxB, geB);
-                        } else {
-                            cv_cell(I, cB, gxB, geB);
-                        }
-                        cv_acc(gxB, geB, zt, cvx, cve);
-                    }
-                    if (warm) {
-                        // a path taken up mid-task: this pass only drew its first normals
-                    } else if (outA) {
-                        if (a.surv) seg = exit_record(pos.x, pos.y, pa.x, pa.y), code = 0;
-                        else plain_exit(I, pos.x, pos.y, pa.x, pa.y, code, yxi, yeta, xe, ye);
-                        done = true;
-                        taken = 2 * m + 1;
-                    } else if (outB) {
-                        if (a.surv) seg = exit_record(pa.x, pa.y, pb.x, pb.y), code = 0;
-                        else plain_exit(I, pa.x, pa.y, pb.x, pb.y, code, yxi, yeta, xe, ye);
-                        done = true;
-                        taken = 2 * m + 2;
-                    } else {
-                        pos = haveB ? pb : pa;
-                    }
-                    zA = nA;
-                    zB = nB;
-                    ++m;
-                    if (!warm && !done && 2 * m >= K) {
-                        done = true;
-                        taken = K;
-                    }
-                } else {
-                    philox_rounds_rk<5, 10>(r, a.keys);
-                    float2 nA;
-                    box_muller(r.x, r.y, a.bm_scale, nA.x, nA.y);
-                    const float nub = uniform_pos(r.z);
-                    if (warm) {
-                        // a path taken up mid-task: this pass only drew its first normals
-                    } else if (outA) {
-                        if (a.surv) seg = exit_record(pos.x, pos.y, pa.x, pa.y), code = 0;
-                        else plain_exit(I, pos.x, pos.y, pa.x, pa.y, code, yxi, yeta, xe, ye);
-                        done = true;
-                    } else {
-                        const float dm0 = fminf(fminf(pos.x, 1.0f - pos.x), fminf(pos.y, 1.0f - pos.y));
-                        const float dm1 = fminf(fminf(pa.x, 1.0f - pa.x), fminf(pa.y, 1.0f - pa.y));
-                        if (dm0 * dm1 < a.bridge_cut &&
-                            bridge_exit(I, pos.x, pos.y, pa.x, pa.y, dt, ub, code, yxi, yeta, xe, ye)) {
-                            code += 4;
-                            done = true;
-                        } else {
-                            pos = pa;
+                            cvq = 0;
+                            cvn = a.cv_bound[1];
                         }
                     }
-                    zA = nA;
-                    ub = nub;
-                    ++m;
-                    taken = m;
-                    if (!warm && !done && m >= K) done = true;
+                } else if (idle == FULL) {
+                    break;
                 }
-                if (done) {
-                    bool later = false;   // scored by k_score_surv once the fields are final
-                    if (code < 0) {
-                        if (a.surv) {
-                            later = true;
-                            put_record<CV>(a.surv, nd.rec0 + path, pos, cvx.x + cvx.y, cve.x + cve.y);
+                k = __reduce_min_sync(FULL, alive ? P - m : 0x7fffffff);
+            }
+            // one pass: the sub-step pair (bridge mode: the sub-step) of draw m
+            uint4 r = draw_begin(pw, nodek, (uint32_t)m);
+            philox_rounds_rk<2, 10>(r, a.keys);
+            float2 zA, zB = f2(0.f, 0.f);
+            if (PAIRS) box_muller2(r, a.bm_scale, zA, zB);
+            else box_muller(r.x, r.y, a.bm_scale, zA.x, zA.y);
+            const float2 pa = advance(pos, zA, alive, alive, PAIRS ? 2 * m : m);
+            const bool inA = inside2(pa);
+            float2 pn = pa;   // where the pass ends
+            bool out;
+            int code = 0;
+            float yxi = 0.f, yeta = 0.f, xe = 0.f, ye = 0.f;
+            if (PAIRS) {
+                // an odd K: the last pair has no sub-step B
+                const bool haveB = MODE == 2 || 2 * m + 1 < K;
+                const float2 pb = advance(pa, zB, alive && inA, alive && inA && haveB, 2 * m + 1);
+                if (haveB) pn = pb;
+                out = alive && !(inA && (!haveB || inside2(pb)));
+            } else {
+                out = alive && !inA;
+                const float dm0 = fminf(fminf(pos.x, 1.0f - pos.x), fminf(pos.y, 1.0f - pos.y));
+                const float dm1 = fminf(fminf(pa.x, 1.0f - pa.x), fminf(pa.y, 1.0f - pa.y));
+                if (alive && inA && dm0 * dm1 < a.bridge_cut &&
+                    bridge_exit(I, pos.x, pos.y, pa.x, pa.y, a.dt, uniform_pos(r.z), code, yxi, yeta, xe, ye)) {
+                    code += 4;
+                    out = true;
+                }
+            }
+            --k;
+            if (k == 0 || __any_sync(FULL, out)) {
+                if (out || (alive && m == P - 1)) {
+                    const long long ri = DEFER || RECORD ? node_records(nd) + (long long)path : 0;
+                    int taken = K;
+                    bool later = DEFER;   // scored by k_score_surv once the fields are final
+                    if (out) {
+                        ++sums.exits[threadIdx.x];
+                        taken = !PAIRS ? m + 1 : inA ? 2 * m + 2 : 2 * m + 1;
+                        const float2 p0 = PAIRS && inA ? pa : pos, p1 = PAIRS && inA ? pn : pa;
+                        if (MODE == 1 && code >= 4) {
+                            // a bridge exit is scored here; its record holds the skip mark
+                            later = false;
+                            if (DEFER) put_record<CV>(a.surv, ri, f2(REC_SKIP, 0.f), cvx.x + cvx.y, cve.x + cve.y);
+                        } else if (DEFER) {
+                            put_record<CV>(a.surv, ri, exit_record(p0.x, p0.y, p1.x, p1.y), cvx.x + cvx.y,
+                                           cve.x + cve.y);
                         } else {
-                            // survived the mesh step: xi, eta of its start at the end point
-                            const Cell c = locate(I, pos);
-                            float4 f0, f1;
-                            load_cell(rec2(I.fcoef, c.idx), f0, f1);
-                            const float2 v = eval2(f0, f1, c.st);
-                            yxi = v.x;
-                            yeta = v.y;
-                            xe = pos.x;
-                            ye = pos.y;
+                            plain_exit(I, p0.x, p0.y, p1.x, p1.y, code, yxi, yeta, xe, ye);
                         }
+                    } else if (DEFER) {
+                        put_record<CV>(a.surv, ri, pn, cvx.x + cvx.y, cve.x + cve.y);
                     } else {
-                        ++exits;
-                        if (a.surv) {
-                            // a plain exit leaves its sub-step, a bridge exit (scored here) the skip mark
-                            later = seg.x != REC_SKIP;
-                            put_record<CV>(a.surv, nd.rec0 + path, seg, cvx.x + cvx.y, cve.x + cve.y);
-                        }
+                        // survived the mesh step: xi, eta of its start at the end point
+                        const Cell c = locate<ONE>(I, pn);
+                        float4 f0, f1;
+                        load_cell(rec2<ONE>(I.fcoef, c.idx), f0, f1);
+                        const float2 v = eval2(f0, f1, c.st);
+                        yxi = v.x;
+                        yeta = v.y;
+                        xe = pn.x;
+                        ye = pn.y;
+                        code = -1;
                     }
-                    if (!later) {
+                    sums.steps[threadIdx.x] += taken;
+                    if (ACC && !later) {
                         if (CV) {
                             yxi -= cvx.x + cvx.y;
                             yeta -= cve.x + cve.y;
                         }
-                        ax.add(yxi - x0);
-                        ae.add(yeta - y0);
+                        const float2 c = node_start(nd);
+                        sums.add(0, yxi - c.x);
+                        sums.add(1, yeta - c.y);
                     }
-                    steps += taken;
                     if (RECORD) {
-                        const long long ri = nd.rec0 + path;
                         if (a.rec.steps) a.rec.steps[ri] = taken;
                         if (a.rec.code) a.rec.code[ri] = code;
                         if (a.rec.score_xi) a.rec.score_xi[ri] = yxi;
@@ -563,49 +625,53 @@ __global__ void __launch_bounds__(paths_max_block(CVM, VAR), paths_min_blocks(CV
                     }
                     alive = false;
                 }
+                // take new paths now if enough lanes are idle, or all
+                const int idle = 32 - __popc(__ballot_sync(FULL, alive));
+                if (idle == 32 || (idle >= REFILL_MIN && next < end)) k = 0;
             }
-            // lanes whose path ended take the task's next paths, in lane order
-            const unsigned need = __ballot_sync(FULL, !alive);
-            if (need != 0u && next < end) {
-                const int cand = next + __popc(need & below);
-                if (!alive && cand < end) {
-                    path = cand;
-                    alive = true;
-                    pos = f2(x0, y0);
-                    m = 0;
-                    if (CV) cvx = cve = f2(0.f, 0.f);
-                    if (CVT) {
-                        cvq = 0;
-                        cvn = a.cv_bound[1];
-                    }
-                    if (__popc(need) >= WARM_MIN) {
-                        first_draw();
-                    } else {
-                        // few lanes refill: rather than run the first draw's Philox block
-                        // with the others idle, the lane spends the next pass drawing it
-                        m = -1;
-                        zA = zB = f2(0.f, 0.f);
-                        ub = 1.f;
-                    }
-                }
-                next += __popc(need);
-            }
+            pos = pn;
+            ++m;
         }
 
-        const double sx = warp_sum(ax.sum()), qx = warp_sum(ax.sumsq());
-        const double se = warp_sum(ae.sum()), qe = warp_sum(ae.sumsq());
-        const long long ex = warp_sum_ll(exits), st = warp_sum_ll(steps);
-        if (lane == 0) {
-            Partial p;
-            p.s_xi = sx;
-            p.q_xi = qx;
-            p.s_eta = se;
-            p.q_eta = qe;
-            p.exits = ex;
-            p.steps = st;
-            a.partials[t] = p;
+        Partial p{};
+        if (ACC) {
+            const Acc ax = sums.get(0), ae = sums.get(1);
+            p.s_xi = warp_sum(ax.sum());
+            p.q_xi = warp_sum(ax.sumsq());
+            p.s_eta = warp_sum(ae.sum());
+            p.q_eta = warp_sum(ae.sumsq());
+        }
+        p.exits = warp_sum_ll(sums.exits[threadIdx.x]);
+        p.steps = warp_sum_ll(sums.steps[threadIdx.x]);
+        if (lanes_below() == 0) a.partials[t] = p;
+    }
+}
+
+template <int MODE, bool RECORD, int CVM, int VAR, bool DEFER>
+__global__ void __launch_bounds__(paths_max_block(CVM, VAR), paths_min_blocks(CVM, VAR, DEFER))
+    k_paths(const PathArgs a)
+{
+    __shared__ LaneSums<paths_max_block(CVM, VAR), !DEFER || MODE == 1> sums;
+    if (VAR == VAR_ONE && a.zmap) {
+        // stage the zero map, and leave it unused where nearly every tile is marked
+        extern __shared__ __align__(16) uint8_t zsm[];
+        __shared__ int marked;
+        if (threadIdx.x == 0) marked = 0;
+        __syncthreads();
+        int mine = 0;
+        for (int k = threadIdx.x; k < kZmapBytes / 16; k += blockDim.x) {
+            const uint4 v = reinterpret_cast<const uint4*>(a.zmap)[k];
+            reinterpret_cast<uint4*>(zsm)[k] = v;
+            mine += __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);   // marks are ones
+        }
+        atomicAdd(&marked, mine);
+        __syncthreads();
+        if (marked < kZmapTiles * kZmapTiles * 7 / 8) {
+            walk_tasks<MODE, RECORD, CVM, VAR, DEFER, true>(a, zsm, sums);
+            return;
         }
     }
+    walk_tasks<MODE, RECORD, CVM, VAR, DEFER, false>(a, nullptr, sums);
 }
 
 // Exponential time-stepping (exit_mode 2), the alternative integrator Sec. 4
@@ -626,7 +692,7 @@ __global__ void __launch_bounds__(512, 2) k_paths_exp(const PathArgs a)
     const float ln2dt = a.dt * 0.69314718055994530942f;
     for (;;) {
         int tq = 0;
-        if (lane == 0) tq = atomicAdd(a.queue, 1);
+        if (lanes_below() == 0) tq = atomicAdd(a.queue, 1);
         const int t = __shfl_sync(FULL, tq, 0);
         if (t >= a.ntasks) return;
         const Task task = a.tasks[t];
@@ -658,9 +724,9 @@ __global__ void __launch_bounds__(512, 2) k_paths_exp(const PathArgs a)
                 float2 z;
                 box_muller(r.x, r.y, -2.77258872223978123767f * tau, z.x, z.y);   // -4 ln 2 tau: sqrt(2 tau) N(0,1)
                 const float ub = uniform_pos(r.z);
-                const Cell c = locate(I, pos);
+                const Cell c = locate<false>(I, pos);
                 float4 g0, g1;
-                load_cell(rec2(I.bcoef, c.idx), g0, g1);
+                load_cell(rec2<false>(I.bcoef, c.idx), g0, g1);
                 const float2 pn = em(g0, g1, c.st, pos, f2(tau, tau), z);
                 bool done = false;
                 int code = -1;
@@ -690,9 +756,9 @@ __global__ void __launch_bounds__(512, 2) k_paths_exp(const PathArgs a)
                             later = true;
                             put_record<false>(a.surv, nd.rec0 + path, pos, 0.f, 0.f);
                         } else {
-                            const Cell cf = locate(I, pos);
+                            const Cell cf = locate<false>(I, pos);
                             float4 f0, f1;
-                            load_cell(rec2(I.fcoef, cf.idx), f0, f1);
+                            load_cell(rec2<false>(I.fcoef, cf.idx), f0, f1);
                             const float2 v = eval2(f0, f1, cf.st);
                             yxi = v.x;
                             yeta = v.y;
@@ -812,8 +878,8 @@ __global__ void __launch_bounds__(SCORE_THREADS, 1024 / SCORE_THREADS) k_score_s
 #pragma unroll
         for (int u = 0; u < SCORE_BATCH; ++u) {
             if (r[u].x >= 0.f) {
-                const Cell c = locate(I, r[u]);
-                load_cell(rec2(I.fcoef, c.idx), f0[u], f1[u]);
+                const Cell c = locate<false>(I, r[u]);
+                load_cell(rec2<false>(I.fcoef, c.idx), f0[u], f1[u]);
                 st[u] = c.st;
             } else if (r[u].x != REC_SKIP) {
                 int k;
@@ -1002,178 +1068,67 @@ __global__ void k_rng_draw(uint64_t seed, const uint32_t* __restrict__ ctrs, lon
     }
 }
 
-template <int MODE, bool RECORD, int CVM, int VAR>
-const void* kernel_ptr()
+template <int MODE, int CVM, int VAR>
+const void* pick_out(bool record, bool defer)
 {
-    return (const void*)k_paths<MODE, RECORD, CVM, VAR>;
+    if (defer) return (const void*)k_paths<MODE, false, CVM, VAR, true>;
+    return record ? (const void*)k_paths<MODE, true, CVM, VAR, false> : (const void*)k_paths<MODE, false, CVM, VAR, false>;
 }
 
 template <int CVM, int VAR>
-const void* pick_cv(int mode, bool record)
+const void* pick_mode(int mode, bool record, bool defer)
 {
-    if (mode == 3) return record ? (const void*)k_paths_exp<true> : (const void*)k_paths_exp<false>;
-    if (mode == 0) return record ? kernel_ptr<0, true, CVM, VAR>() : kernel_ptr<0, false, CVM, VAR>();
-    if (mode == 2) return record ? kernel_ptr<2, true, CVM, VAR>() : kernel_ptr<2, false, CVM, VAR>();
-    return record ? kernel_ptr<1, true, CVM, VAR>() : kernel_ptr<1, false, CVM, VAR>();
+    if (mode == 0) return pick_out<0, CVM, VAR>(record, defer);
+    if (mode == 2) return pick_out<2, CVM, VAR>(record, defer);
+    return pick_out<1, CVM, VAR>(record, defer);
 }
 
 template <int VAR>
-const void* pick_var(int mode, bool record, int cvm)
+const void* pick_var(int mode, bool record, int cvm, bool defer)
 {
-    if (cvm == 2) return pick_cv<2, VAR>(mode, record);
-    return cvm ? pick_cv<1, VAR>(mode, record) : pick_cv<0, VAR>(mode, record);
+    if (cvm == 2) return pick_mode<2, VAR>(mode, record, defer);
+    return cvm ? pick_mode<1, VAR>(mode, record, defer) : pick_mode<0, VAR>(mode, record, defer);
 }
 
 // cvm: 0 no control variate, 1 node values in time slices, 2 one value per cell
-const void* pick(int mode, bool record, int cvm, int var)
+const void* pick(int mode, bool record, int cvm, bool single, bool defer)
 {
-    if (var == VAR_ZM) return pick_var<VAR_ZM>(mode, record, cvm);
-    if (var == VAR_ONE) return pick_var<VAR_ONE>(mode, record, cvm);
-    return pick_var<VAR_MULTI>(mode, record, cvm);
+    if (mode == 3) return record ? (const void*)k_paths_exp<true> : (const void*)k_paths_exp<false>;
+    return single ? pick_var<VAR_ONE>(mode, record, cvm, defer) : pick_var<VAR_MULTI>(mode, record, cvm, defer);
 }
 
-// The variant of a launch: the zero map where the arguments carry one, else the single instance's
-// tables as parameters where the launch has one instance.
-int path_var(const PathArgs& a)
+int kernel_mode(int exit_mode, int K)
 {
-    if (a.zwords > 0 && a.zmap != nullptr) return VAR_ZM;
-    return a.single ? VAR_ONE : VAR_MULTI;
+    if (exit_mode == 2) return 3;   // exponential time-stepping
+    return exit_mode == 1 ? 1 : ((K & 1) == 0 ? 2 : 0);
 }
 
 }  // namespace
-
-static void prefer_l1();
 
 int path_kernel_max_block(int exit_mode, int cvm, bool single)
 {
     return exit_mode == 2 ? 512 : paths_max_block(cvm, single ? VAR_ONE : VAR_MULTI);
 }
 
-int path_kernel_blocks_per_sm(int exit_mode, bool record, int block, int cvm, int zwords, bool single)
+int path_kernel_blocks_per_sm(int exit_mode, bool record, int block, int cvm, bool map, bool single, bool defer)
 {
-    prefer_l1();
     int n = 0;
     // the even-K kernel has the same footprint class; size the grid for the larger of the two
     const int mode = exit_mode == 2 ? 3 : exit_mode == 1 ? 1 : 0;
-    const int var = zwords > 0 ? VAR_ZM : single ? VAR_ONE : VAR_MULTI;
-    const size_t smem = var == VAR_ZM && mode != 3 ? zmap_smem_bytes(zwords) : 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, pick(mode, record, cvm, var), block, smem) !=
+    const size_t smem = map && mode != 3 ? kZmapBytes : 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, pick(mode, record, cvm, single, defer), block, smem) !=
         cudaSuccess)
         return 1;
     return n > 0 ? n : 1;
 }
 
-// The shared-memory carveout (percent of the SM's largest) that holds `blocks` blocks of `smem`
-// dynamic bytes each, so that the zero map costs the launch no occupancy and L1 keeps the rest.
-static unsigned carveout_pct(int blocks, size_t smem)
-{
-    int dev = 0, most = 0, resv = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-    cudaDeviceGetAttribute(&resv, cudaDevAttrReservedSharedMemoryPerBlock, dev);
-    if (most <= 0) return 100;
-    const double need = (double)blocks * (double)(smem + (size_t)resv);
-    const int pct = (int)std::ceil(100.0 * need / (double)most);
-    return (unsigned)std::min(100, std::max(0, pct));
-}
-
-static int kernel_mode(int exit_mode, int K)
-{
-    if (exit_mode == 2) return 3;   // exponential time-stepping
-    return exit_mode == 1 ? 1 : ((K & 1) == 0 ? 2 : 0);
-}
-
-// Without the zero map the path kernel keeps no data in shared memory: give L1 the whole carveout.
-// The kernels with the map prefer the largest carveout (so that occupancy queries see the blocks the
-// registers allow); each launch then asks, by a launch attribute, for the carveout its blocks need.
-static void prefer_l1()
-{
-    static bool done = false;
-    if (done) return;
-    done = true;
-    for (int mode : {0, 1, 2, 3})
-        for (bool rec : {false, true})
-            for (int cvm : {0, 1, 2})
-                for (int var : {VAR_MULTI, VAR_ONE, VAR_ZM})
-                    cudaFuncSetAttribute(pick(mode, rec, cvm, var), cudaFuncAttributePreferredSharedMemoryCarveout,
-                                         var == VAR_ZM && mode != 3 ? 100 : 0);
-    cudaGetLastError();
-}
-
-// A launch of a kernel with the zero map: dynamic shared memory for the map, and the carveout that the
-// blocks the registers allow need (with less, the CUDA runtime may fit fewer blocks; with more, L1 shrinks).
-// The preference is the function's, set before each launch (launches of one function inside a step
-// graph share one shape, so they need the same value).
-static void launch_zm(const void* fn, const PathArgs& a, int grid, int block, size_t smem, cudaStream_t s)
-{
-    struct Pref {
-        const void* fn;
-        int block;
-        size_t smem;
-        int pct;
-    };
-    static Pref cache[64];
-    static int ncache = 0;
-    int pct = -1;
-    for (int k = 0; k < ncache; ++k)
-        if (cache[k].fn == fn && cache[k].block == block && cache[k].smem == smem) pct = cache[k].pct;
-    if (pct < 0) {
-        int n = 1;
-        cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, block, smem) != cudaSuccess || n < 1) n = 1;
-        pct = (int)carveout_pct(n, smem);
-        if (ncache < 64) cache[ncache++] = Pref{fn, block, smem, pct};
-    }
-    cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
-    void* args[] = {(void*)&a};
-    cudaLaunchKernel(fn, dim3((unsigned)grid), dim3((unsigned)block), args, smem, s);
-}
-
-template <int CVM, int VAR>
-static void launch_mode(const PathArgs& a, int mode, bool record, int grid, int block, size_t smem, cudaStream_t s)
-{
-    if (VAR == VAR_ZM && mode != 3) {
-        launch_zm(pick(mode, record, CVM, VAR_ZM), a, grid, block, smem, s);
-        return;
-    }
-    switch (mode) {
-    case 3:
-        if (record) k_paths_exp<true><<<grid, block, 0, s>>>(a);
-        else k_paths_exp<false><<<grid, block, 0, s>>>(a);
-        break;
-    case 0:
-        if (record) k_paths<0, true, CVM, VAR><<<grid, block, smem, s>>>(a);
-        else k_paths<0, false, CVM, VAR><<<grid, block, smem, s>>>(a);
-        break;
-    case 2:
-        if (record) k_paths<2, true, CVM, VAR><<<grid, block, smem, s>>>(a);
-        else k_paths<2, false, CVM, VAR><<<grid, block, smem, s>>>(a);
-        break;
-    default:
-        if (record) k_paths<1, true, CVM, VAR><<<grid, block, smem, s>>>(a);
-        else k_paths<1, false, CVM, VAR><<<grid, block, smem, s>>>(a);
-    }
-}
-
-
 cudaError_t launch_paths(const PathArgs& a, int exit_mode, bool record, int grid, int block, cudaStream_t s, int cvm)
 {
-    prefer_l1();
     const int mode = kernel_mode(exit_mode, a.K);
-    const int var = path_var(a);
-    const size_t smem = var == VAR_ZM && mode != 3 ? zmap_smem_bytes(a.zwords) : 0;
-    switch (var * 3 + cvm) {
-    case VAR_ZM * 3 + 0: launch_mode<0, VAR_ZM>(a, mode, record, grid, block, smem, s); break;
-    case VAR_ZM * 3 + 1: launch_mode<1, VAR_ZM>(a, mode, record, grid, block, smem, s); break;
-    case VAR_ZM * 3 + 2: launch_mode<2, VAR_ZM>(a, mode, record, grid, block, smem, s); break;
-    case VAR_ONE * 3 + 0: launch_mode<0, VAR_ONE>(a, mode, record, grid, block, 0, s); break;
-    case VAR_ONE * 3 + 1: launch_mode<1, VAR_ONE>(a, mode, record, grid, block, 0, s); break;
-    case VAR_ONE * 3 + 2: launch_mode<2, VAR_ONE>(a, mode, record, grid, block, 0, s); break;
-    case VAR_MULTI * 3 + 0: launch_mode<0, VAR_MULTI>(a, mode, record, grid, block, 0, s); break;
-    case VAR_MULTI * 3 + 1: launch_mode<1, VAR_MULTI>(a, mode, record, grid, block, 0, s); break;
-    default: launch_mode<2, VAR_MULTI>(a, mode, record, grid, block, 0, s);
-    }
-    return cudaGetLastError();
+    const size_t smem = a.zmap && mode != 3 ? kZmapBytes : 0;
+    void* args[] = {(void*)&a};
+    return cudaLaunchKernel(pick(mode, record, cvm, a.single != 0, a.surv != nullptr), dim3((unsigned)grid),
+                            dim3((unsigned)block), args, smem, s);
 }
 
 cudaError_t launch_score_surv(const ScoreArgs& a, bool cv, cudaStream_t s)

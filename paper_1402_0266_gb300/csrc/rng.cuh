@@ -77,6 +77,21 @@ __device__ __forceinline__ float sqrt_approx(float v)
     return r;
 }
 
+// The special functions with subnormals flushed: their arguments here are never
+// subnormal, and the flag saves the scaling that subnormal arguments would need.
+__device__ __forceinline__ float lg2_approx(float v)
+{
+    float r;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+    return r;
+}
+
+__device__ __forceinline__ void sincos_approx(float v, float& s, float& c)
+{
+    asm("sin.approx.ftz.f32 %0, %1;" : "=f"(s) : "f"(v));
+    asm("cos.approx.ftz.f32 %0, %1;" : "=f"(c) : "f"(v));
+}
+
 // Box--Muller pair scaled by sigma: (sigma R cos 2 pi u2, sigma R sin 2 pi u2),
 // R = sqrt(-2 ln u1). `scale` = -2 sigma^2 ln 2, so that
 // sigma R = sqrt(scale * log2(u1)). The angle is taken as 2 pi (u2 - 1/2),
@@ -86,9 +101,9 @@ __device__ __forceinline__ void box_muller(uint32_t a, uint32_t b, float scale, 
 {
     const float u1 = 2.0f - __uint_as_float(0x3F800000u | (a & 0x7FFFFFu));
     const float v = __uint_as_float(0x3F800000u | (b & 0x7FFFFFu)) - 1.5f;
-    const float r = sqrt_approx(scale * __log2f(u1));
+    const float r = sqrt_approx(scale * lg2_approx(u1));
     float s, c;
-    __sincosf(6.28318530717958647692f * v, &s, &c);
+    sincos_approx(6.28318530717958647692f * v, s, c);
     z0 = -r * c;
     z1 = -r * s;
 }
@@ -104,14 +119,14 @@ __device__ __forceinline__ void box_muller2(uint4 r, float scale, float2& zA, fl
                                   __uint_as_float(0x3F800000u | (r.w & 0x7FFFFFu)));
     const float2 u1 = __ffma2_rn(f1, make_float2(-1.0f, -1.0f), make_float2(2.0f, 2.0f));   // exact
     const float2 v = __fadd2_rn(f2, make_float2(-1.5f, -1.5f));                            // exact
-    const float2 l = __fmul2_rn(make_float2(__log2f(u1.x), __log2f(u1.y)), make_float2(scale, scale));
+    const float2 l = __fmul2_rn(make_float2(lg2_approx(u1.x), lg2_approx(u1.y)), make_float2(scale, scale));
     const float ra = sqrt_approx(l.x), rb = sqrt_approx(l.y);
     const float2 ang = __fmul2_rn(v, make_float2(6.28318530717958647692f, 6.28318530717958647692f));
     float sa, ca, sb, cb;
-    __sincosf(ang.x, &sa, &ca);
-    __sincosf(ang.y, &sb, &cb);
-    zA = __fmul2_rn(make_float2(-ra, -ra), make_float2(ca, sa));
-    zB = __fmul2_rn(make_float2(-rb, -rb), make_float2(cb, sb));
+    sincos_approx(ang.x, sa, ca);
+    sincos_approx(ang.y, sb, cb);
+    zA = make_float2(-ra * ca, -ra * sa);
+    zB = make_float2(-rb * cb, -rb * sb);
 }
 
 __device__ __forceinline__ float uniform_pos(uint32_t w)

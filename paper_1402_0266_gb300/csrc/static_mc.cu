@@ -173,8 +173,8 @@ sdd_status sdd_interface_mc_static(const sdd_fields* f, const sdd_nodes* nodes, 
         std::memset(&nd, 0, sizeof nd);
         nd.x = nodes->x[k];
         nd.y = nodes->y[k];
-        nd.xf = (float)nd.x;
-        nd.yf = (float)nd.y;
+        nd.xf = start_coord(nd.x);
+        nd.yf = start_coord(nd.y);
         nd.inst = 0;
         nd.ctr = p->node_word0 + (uint32_t)k;
         nd.n_paths = (int32_t)nodes->n_paths[k];
@@ -203,8 +203,6 @@ sdd_status sdd_interface_mc_static(const sdd_fields* f, const sdd_nodes* nodes, 
     g_inst_host.ny = ny;
     g_inst_host.sx = (float)(nx - 1);
     g_inst_host.sy = (float)(ny - 1);
-    g_inst_host.gxmax = std::nextafter((float)(nx - 1), 0.0f);
-    g_inst_host.gymax = std::nextafter((float)(ny - 1), 0.0f);
     g_inst_host.cell_bias = 0x4B000000u * (uint32_t)nx;
 
 #define STATIC_CU(expr)                             \
