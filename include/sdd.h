@@ -477,7 +477,9 @@ sdd_status sdd_keypoint_fill(sdd_ctx* ctx, const uint8_t* mask, double* values_x
  *                      fields keep their previous values); slower than
  *                      Jacobi-PCG on these sizes, so never chosen automatically;
  *   SDD_SOLVER_JACOBI  Jacobi preconditioner; one thread-block cluster per
- *                      subdomain, register-resident when the subdomain fits;
+ *                      subdomain; when the subdomain fits its registers,
+ *                      Chebyshev iterations first (at most max_iter of
+ *                      them) and conjugate gradients for what they leave;
  *   SDD_SOLVER_MG      a geometric multigrid V-cycle as preconditioner
  *                      (available when every subdomain has the same odd
  *                      sizes that halve, (m - 1) / 2, down to a box of at

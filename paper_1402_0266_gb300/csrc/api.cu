@@ -791,7 +791,7 @@ sdd_status setup_solver(sdd_ctx* c)
     const std::vector<int> xs = block_edges(c->nx, c->sub_x), ys = block_edges(c->ny, c->sub_y);
     // subdomains (both fields solved together by the register-resident kernel)
     std::vector<SolveSys> subs;
-    int min_rows = 1 << 30;
+    int min_rows = 1 << 30, most_mx = 0, most_my = 0;
     for (int b = 0; b < c->sub_y; ++b)
         for (int a = 0; a < c->sub_x; ++a) {
             SolveSys S{};
@@ -803,11 +803,13 @@ sdd_status setup_solver(sdd_ctx* c)
             if (S.i1 > S.i0 && S.j1 > S.j0) {
                 subs.push_back(S);
                 min_rows = std::min(min_rows, S.j1 - S.j0);
+                most_mx = std::max(most_mx, S.i1 - S.i0);
+                most_my = std::max(most_my, S.j1 - S.j0);
             }
         }
     c->solve_upt = 0;
     if (!subs.empty()) {
-        const int C = solve_cluster_size((int)subs.size(), min_rows, c->sm_count);
+        const int C = solve_cluster_size((int)subs.size(), min_rows, most_mx, most_my);
         int band_max = 0, rows_max = 0, mx_max = 0;
         for (const SolveSys& S : subs) {
             const int my = S.j1 - S.j0, mx = S.i1 - S.i0;
@@ -836,13 +838,13 @@ sdd_status setup_solver(sdd_ctx* c)
                 S.field = field;
                 c->systems.push_back(S);
             }
-        c->solve_cluster = c->systems.empty() ? 1 : solve_cluster_size((int)c->systems.size(), min_rows, c->sm_count);
+        c->solve_cluster = c->systems.empty() ? 1 : solve_cluster_size((int)c->systems.size(), min_rows, most_mx, most_my);
     }
     CU(c, c->d_systems.alloc(std::max<size_t>(c->systems.size(), 1)));
     if (!c->systems.empty())
         CU(c, cudaMemcpy(c->d_systems.p, c->systems.data(), c->systems.size() * sizeof(SolveSys),
                          cudaMemcpyHostToDevice));
-    CU(c, c->d_iters.alloc(std::max<size_t>(std::max(c->systems.size(), subs.size()), 1)));
+    CU(c, c->d_iters.alloc(2 * std::max<size_t>(std::max(c->systems.size(), subs.size()), 1)));
 
     // multigrid: every subdomain the same odd sizes, coarsening down to a small box
     c->mg_ok = false;

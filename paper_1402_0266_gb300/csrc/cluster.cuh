@@ -42,7 +42,7 @@ __device__ __forceinline__ void cluster_sum2(cg::cluster_group& cl, ClusterSlots
     __syncthreads();
     if (threadIdx.x == 0) {
         T t0 = 0, t1 = 0;
-        for (int q = 0; q < SOLVE_WARPS; ++q) {
+        for (int q = 0; q < (int)(blockDim.x >> 5); ++q) {
             t0 += S.warp_part[0][q];
             t1 += S.warp_part[1][q];
         }
@@ -98,7 +98,7 @@ __device__ __forceinline__ void cluster_sum4(cg::cluster_group& cl, ClusterSlots
     __syncthreads();
     if (threadIdx.x < 4) {
         T t = 0;
-        for (int q = 0; q < SOLVE_WARPS; ++q) t += S.warp_part[threadIdx.x][q];
+        for (int q = 0; q < (int)(blockDim.x >> 5); ++q) t += S.warp_part[threadIdx.x][q];
         S.block_part[threadIdx.x] = t;
     }
     cl.sync();

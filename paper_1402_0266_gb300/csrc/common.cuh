@@ -249,7 +249,7 @@ struct SolveArgs {
     int32_t max_outer;       // refinement sweeps allowed
     double rtol;             // on the double-precision residual, relative to ||b||
     float inner_tol;         // inner reduction of ||r|| per refinement sweep
-    int32_t* iters;          // per system: total inner iterations (max_iter + 1 when not converged)
+    int32_t* iters;          // per system: total inner iterations (max_iter + 1 when not converged); then, per system, 1 when the first kernel solved it
     int* status;
 };
 
@@ -316,7 +316,7 @@ cudaError_t launch_mgc(const MgArgs& a, int upt, int C, int rows_max, size_t sme
 cudaError_t launch_solve_setup(const float* w, const double* prev_xi, const double* prev_eta, int nx, int ny,
                                double Dt, double* cx, double* cy, double* dg, double* rhs0, float* cxf, float* cyf,
                                float* dgf, float* dinvf, cudaStream_t s);
-int solve_cluster_size(int nsys, int min_rows, int sm_count);
+int solve_cluster_size(int nsys, int min_rows, int max_mx, int max_my);
 cudaError_t launch_dirichlet(const double* faces64, const double* prev_xi, const double* prev_eta,
                              const double* iface_xi, const double* iface_eta, const int32_t* iface_idx,
                              int n_iface, int nx, int ny, double* xi_out, double* eta_out, cudaStream_t s);

@@ -8,12 +8,12 @@
 //   xi_ij / (w_ij Dt) + sum_nb c_nb (xi_ij - xi_nb) = xi^{n-1}_ij / (w_ij Dt),
 //   c_nb = 1 / (wbar h^2),  wbar = (w_ij + w_nb) / 2,
 //
-// a symmetric positive definite M-matrix, solved per subdomain and field by
-// Jacobi-preconditioned conjugate gradients.
+// a symmetric positive definite M-matrix, solved per subdomain by Chebyshev
+// iterations and conjugate gradients, both with the diagonal as preconditioner.
 //
 // Precision: the solution and its residual are double precision; the
-// conjugate-gradient sweeps run on the residual equation A d = r in single
-// precision (iterative refinement): each sweep reduces ||r|| by inner_tol,
+// sweeps run on the residual equation A d = r in single precision (iterative
+// refinement): each sweep reduces ||r|| by inner_tol or more,
 // then x += d and r = b - A x are formed again in double precision, until
 // ||r|| <= rtol ||b||. On GB300 double-precision arithmetic runs at a small
 // fraction of the single-precision rate; only the residuals use it.
@@ -24,6 +24,9 @@
 // every block takes the same branch. All loops are bounded by max_iter and
 // max_outer; non-convergence sets a status bit.
 #include <cooperative_groups.h>
+
+#include <algorithm>
+#include <cstdlib>
 
 #include "cluster.cuh"
 #include "common.cuh"
@@ -104,6 +107,7 @@ __global__ void __launch_bounds__(SOLVE_THREADS) k_pcg_cluster(const SolveArgs a
     cg::cluster_group cl = cg::this_cluster();
     const int C = (int)cl.num_blocks();
     const int rank = (int)cl.block_rank();
+    if (a.iters[a.nsys + blockIdx.x / C]) return;   // solved by k_cheb
     const SolveSys S = a.sys[blockIdx.x / C];
     const int nx = a.nx;
     const int mx = S.i1 - S.i0, my = S.j1 - S.j0;
@@ -215,7 +219,196 @@ __global__ void __launch_bounds__(SOLVE_THREADS) k_pcg_cluster(const SolveArgs a
     cl.sync();  // no block leaves while others may still read its shared memory
 }
 
-// Register-resident variant for subdomains whose band fits in the block:
+// Chebyshev iterations for subdomains whose bands fit the blocks of a cluster, both fields together. Solves with
+// their set-up, before and after: 4 x 19^2 unknowns 157 -> 71 us, 4 x 63^2 520 -> 156, 9 x 65^2 1358 -> 288,
+// 9 x 119^2 2918 -> 875, 16 x 95^2 2548 -> 1272. The method:
+// A d = r with the diagonal as preconditioner over the interval [lo, 1 + rho] of the eigenvalues of
+// D^-1 A, in single precision, inside the double-precision refinement of the other kernels.
+// rho is Gershgorin's bound, the largest row sum of D^-1 (D - A) (below 1: the mass term), so the upper
+// end holds; lo adds to 1 - rho most of what the Dirichlet frame contributes with uniform coefficients.
+// Where that is too much, the modes below lo fall more slowly than the rest, never grow, and k_pcg_cg2,
+// which closes every solve, takes them over.
+//
+// Why not conjugate gradients alone: an iteration of theirs is a product, two barriers and a reduction of
+// six sums, a latency chain of about 2.3 us whatever the cluster size; here it is one barrier (one block:
+// a block barrier) and a product whose operands are in registers and shared memory, with no scalar to wait
+// for. The iteration count is the same to 1.4 times theirs in this range of mass terms.
+//
+// Layout: each thread keeps UPT unknowns (scaled coefficients and, per field, scaled residual z, step d,
+// correction e) in registers; the steps d live in shared memory as pairs (both fields), a zero frame around
+// the band and halo rows that the neighbouring blocks store into before the barrier. Planes alternate with the
+// iteration's parity: a plane is rewritten only after the next iteration's barrier, which every reader has passed.
+template <int UPT, bool ONE>
+__global__ void __launch_bounds__(SOLVE_THREADS) k_cheb(const SolveArgs a, int rows_max)
+{
+    extern __shared__ float2 planes[];   // [parity]: (rows_max + 2) x (mx + 2)
+    __shared__ ClusterSlots<double> red64[2];
+    __shared__ float warp_max[SOLVE_WARPS], block_max;
+    cg::cluster_group cl = cg::this_cluster();
+    const int C = ONE ? 1 : (int)cl.num_blocks();
+    const int rank = ONE ? 0 : (int)cl.block_rank();
+    const int T = (int)blockDim.x;
+    const SolveSys S = a.sys[blockIdx.x / C];
+    const int nx = a.nx;
+    const int mx = S.i1 - S.i0, my = S.j1 - S.j0;
+    const int row0 = S.j0 + (my * rank) / C, rows = S.j0 + (my * (rank + 1)) / C - row0;
+    const int m = rows * mx, W = mx + 2, plane = (rows_max + 2) * W;
+    const int rows_below = rank > 0 ? ((my * rank) / C) - ((my * (rank - 1)) / C) : 0;
+    double* __restrict__ x0 = a.x[0];
+    double* __restrict__ x1 = a.x[1];
+    const double* __restrict__ rhs0 = a.rhs0;
+    const double* __restrict__ rhs1 = a.rhs0 + (long long)nx * a.ny;
+    int seq = 0;
+    auto sync = [&]() {
+        if (ONE) __syncthreads();
+        else cl.sync();
+    };
+
+    for (int k = threadIdx.x; k < 2 * plane; k += T) planes[k] = make_float2(0.f, 0.f);
+    float2* nb_lo = (C > 1 && rank > 0) ? cl.map_shared_rank(planes, rank - 1) : nullptr;     // block below
+    float2* nb_hi = (C > 1 && rank < C - 1) ? cl.map_shared_rank(planes, rank + 1) : nullptr; // block above
+
+    int n_[UPT], sidx[UPT];   // grid index (-1: no unknown), place in a plane
+    float cw[UPT], ce[UPT], cs[UPT], cn[UPT];   // couplings to unknowns over the diagonal (0 to Dirichlet nodes)
+    float z[2][UPT], d[2][UPT], e[2][UPT];
+    float rho = 0.f;
+    double bb[2] = {0.0, 0.0};
+#pragma unroll
+    for (int k = 0; k < UPT; ++k) {
+        const int u = threadIdx.x + k * T;
+        n_[k] = -1;
+        sidx[k] = 0;
+        cw[k] = ce[k] = cs[k] = cn[k] = 0.f;
+#pragma unroll
+        for (int f = 0; f < 2; ++f) z[f][k] = d[f][k] = e[f][k] = 0.f;
+        if (u >= m) continue;
+        const int lr = u / mx, lc = u - lr * mx;
+        const int i = S.i0 + lc, j = row0 + lr, n = j * nx + i;
+        n_[k] = n;
+        sidx[k] = (lr + 1) * W + lc + 1;
+        const float di = a.dinvf[n];
+        double b0 = rhs0[n], b1 = rhs1[n];
+        if (i > S.i0) cw[k] = a.cxf[n - 1] * di;
+        else b0 += a.cx[n - 1] * x0[n - 1], b1 += a.cx[n - 1] * x1[n - 1];
+        if (i < S.i1 - 1) ce[k] = a.cxf[n] * di;
+        else b0 += a.cx[n] * x0[n + 1], b1 += a.cx[n] * x1[n + 1];
+        if (j > S.j0) cs[k] = a.cyf[n - nx] * di;
+        else b0 += a.cy[n - nx] * x0[n - nx], b1 += a.cy[n - nx] * x1[n - nx];
+        if (j < S.j1 - 1) cn[k] = a.cyf[n] * di;
+        else b0 += a.cy[n] * x0[n + nx], b1 += a.cy[n] * x1[n + nx];
+        rho = fmaxf(rho, cw[k] + ce[k] + cs[k] + cn[k]);
+        bb[0] += b0 * b0;
+        bb[1] += b1 * b1;
+    }
+    // the largest row sum over the cluster
+    rho = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(rho)));   // nonnegative: ordered as integers
+    if ((threadIdx.x & 31) == 0) warp_max[threadIdx.x >> 5] = rho;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int q = 1; q < T / 32; ++q) rho = fmaxf(rho, warp_max[q]);
+        block_max = rho;
+    }
+    cluster_sum2(cl, red64, seq, bb[0], bb[1]);   // its barrier publishes block_max
+    for (int q = 0; q < C; ++q) rho = fmaxf(rho, ONE ? block_max : *cl.map_shared_rank(&block_max, q));
+    rho = fminf(fmaxf(rho, 1e-3f), 0.9999999f);
+    const double stop2[2] = {a.rtol * a.rtol * bb[0], a.rtol * a.rtol * bb[1]};
+
+    // the interval, and the factor per iteration
+    const float ix = (float)(nx - 1), iy = (float)(a.ny - 1), px = ix * ix, py = iy * iy;
+    const float frame = (px * (1.f - cospif(1.f / (float)(mx + 1))) + py * (1.f - cospif(1.f / (float)(my + 1)))) / (px + py);
+    const float hi = 1.f + rho, lo = fminf((1.f - rho) + 0.7f * rho * frame, 0.5f * hi);
+    const float theta = 0.5f * (hi + lo), delta = 0.5f * (hi - lo), sigma = theta / delta;
+    const float per_iter = logf(sigma + sqrtf((sigma - 1.f) * (sigma + 1.f)));
+
+    int total = 0, b = 0;
+    bool converged = false;
+    for (int sweep = 0; sweep < 6; ++sweep) {
+        // the residual, double precision
+        double rr[2] = {0.0, 0.0};
+#pragma unroll
+        for (int k = 0; k < UPT; ++k) {
+            const int n = n_[k];
+            if (n < 0) continue;
+            const float di = a.dinvf[n];
+            const double g = a.dg[n], w = a.cx[n - 1], o = a.cx[n], s = a.cy[n - nx], t = a.cy[n];
+#pragma unroll
+            for (int f = 0; f < 2; ++f) {
+                const double* x = f ? x1 : x0;
+                const double r = (f ? rhs1[n] : rhs0[n]) -
+                                 (g * x[n] - w * x[n - 1] - o * x[n + 1] - s * x[n - nx] - t * x[n + nx]);
+                rr[f] += r * r;
+                z[f][k] = (float)r * di;
+                e[f][k] = 0.f;
+            }
+        }
+        cluster_sum2(cl, red64, seq, rr[0], rr[1]);
+        // iterations for what is left of the reduction, at most 1e-5 per sweep
+        float left = 0.f;
+        bool active[2];
+#pragma unroll
+        for (int f = 0; f < 2; ++f) {
+            active[f] = rr[f] > stop2[f];
+            if (active[f]) left = fmaxf(left, stop2[f] > 0.0 ? 0.5f * (float)log(rr[f] / stop2[f]) : 100.f);
+            else
+#pragma unroll
+                for (int k = 0; k < UPT; ++k) z[f][k] = 0.f;
+        }
+        converged = !active[0] && !active[1];
+        if (converged) break;
+        int its = (int)ceilf((fminf(left, 11.5f) + 2.f) / per_iter);
+        its = max(1, min(its, min(a.max_iter, 4000) - total));
+        if (total >= min(a.max_iter, 4000)) break;
+        total += its;
+        float r_old = 1.f / sigma, ca = 0.f, cb = 1.f / theta;
+        for (int it = 0; it < its; ++it, b ^= 1) {
+            float2* mine = planes + b * plane;
+#pragma unroll
+            for (int k = 0; k < UPT; ++k) {
+                if (n_[k] < 0) continue;
+#pragma unroll
+                for (int f = 0; f < 2; ++f) {
+                    d[f][k] = ca * d[f][k] + cb * z[f][k];
+                    e[f][k] += d[f][k];
+                }
+                const float2 v = make_float2(d[0][k], d[1][k]);
+                mine[sidx[k]] = v;
+                if (!ONE) {
+                    const int lr = sidx[k] / W - 1;
+                    if (lr == 0 && nb_lo) nb_lo[b * plane + sidx[k] + rows_below * W] = v;
+                    if (lr == rows - 1 && nb_hi) nb_hi[b * plane + sidx[k] - rows * W] = v;
+                }
+            }
+            const float r_new = 1.f / (2.f * sigma - r_old);
+            ca = r_new * r_old;
+            cb = 2.f * r_new / delta;
+            r_old = r_new;
+            sync();
+#pragma unroll
+            for (int k = 0; k < UPT; ++k) {
+                const float2* v = mine + sidx[k];
+                if (n_[k] < 0) continue;
+                const float2 vw = v[-1], ve = v[1], vs = v[-W], vn = v[W];
+                z[0][k] += cw[k] * vw.x + ce[k] * ve.x + cs[k] * vs.x + cn[k] * vn.x - d[0][k];
+                z[1][k] += cw[k] * vw.y + ce[k] * ve.y + cs[k] * vs.y + cn[k] * vn.y - d[1][k];
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < UPT; ++k)
+            if (n_[k] >= 0) {
+                x0[n_[k]] += (double)e[0][k];
+                x1[n_[k]] += (double)e[1][k];
+            }
+        sync();   // the next residual reads the neighbours' x
+    }
+    if (threadIdx.x == 0 && rank == 0) {
+        a.iters[blockIdx.x / C] = total;
+        a.iters[a.nsys + blockIdx.x / C] = converged ? 1 : 0;
+    }
+    if (!ONE) cl.sync();   // no block leaves while others may still write into its shared memory
+}
+
+// Register-resident conjugate gradients for subdomains whose band fits in the block, run after k_cheb on
+// the systems that it left short of rtol (little mass, strong contrasts: the modes below its interval):
 // one cluster solves both fields of a subdomain (same matrix, two right-hand
 // sides), so the cluster barriers are shared by the two solves. Each thread
 // keeps UPT unknowns (coefficients and, per field, the CG vectors) in
@@ -230,15 +423,21 @@ __global__ void __launch_bounds__(SOLVE_THREADS) k_pcg_cluster(const SolveArgs a
 // double-buffered by the iteration's parity; a buffer is rewritten only two
 // barriers after it was read. A field that has converged stops changing
 // while the other one finishes.
-template <int UPT>
+template <int UPT, bool ONE>
 __global__ void __launch_bounds__(SOLVE_THREADS) k_pcg_cg2(const SolveArgs a, int rows_max)
 {
     extern __shared__ float m_s[];  // u: [parity][field] planes of (rows_max + 2) x (mx + 2), zero frame
-    __shared__ float4 slots[2][16][2];  // [parity][block]: (gamma, delta, rr) of field 0, then field 1
-    __shared__ float warp_part[6][SOLVE_WARPS];
+    __shared__ float slots[2][16][8];   // [parity][block]: (gamma, delta, rr) of field 0, then field 1
+    __shared__ float warp_part[2][SOLVE_WARPS][8];
     cg::cluster_group cl = cg::this_cluster();
-    const int C = (int)cl.num_blocks();
-    const int rank = (int)cl.block_rank();
+    const int C = ONE ? 1 : (int)cl.num_blocks();
+    const int rank = ONE ? 0 : (int)cl.block_rank();
+    const int T = (int)blockDim.x;      // a multiple of 32, at most SOLVE_THREADS
+    auto sync = [&]() {
+        if (ONE) __syncthreads();
+        else cl.sync();
+    };
+    if (a.iters[a.nsys + blockIdx.x / C]) return;   // solved by k_cheb
     const SolveSys S = a.sys[blockIdx.x / C];
     const int nx = a.nx;
     const int mx = S.i1 - S.i0, my = S.j1 - S.j0;
@@ -257,7 +456,7 @@ __global__ void __launch_bounds__(SOLVE_THREADS) k_pcg_cg2(const SolveArgs a, in
     __shared__ ClusterSlots<double> red64[2];
     int seq = 0;
 
-    for (int k = threadIdx.x; k < 4 * plane; k += SOLVE_THREADS) m_s[k] = 0.0f;
+    for (int k = threadIdx.x; k < 4 * plane; k += T) m_s[k] = 0.0f;
     float* nb_lo = (C > 1 && rank > 0) ? cl.map_shared_rank(m_s, rank - 1) : nullptr;     // block below
     float* nb_hi = (C > 1 && rank < C - 1) ? cl.map_shared_rank(m_s, rank + 1) : nullptr; // block above
 
@@ -270,7 +469,7 @@ __global__ void __launch_bounds__(SOLVE_THREADS) k_pcg_cg2(const SolveArgs a, in
     float r[2][UPT], u[2][UPT], w[2][UPT], s[2][UPT], p[2][UPT], d[2][UPT];
 #pragma unroll
     for (int k = 0; k < UPT; ++k) {
-        const int uu0 = threadIdx.x + k * SOLVE_THREADS;
+        const int uu0 = threadIdx.x + k * T;
         own[k] = uu0 < m;
         const int uu = own[k] ? uu0 : 0;
         const int lr = uu / mx;
@@ -313,43 +512,43 @@ __global__ void __launch_bounds__(SOLVE_THREADS) k_pcg_cg2(const SolveArgs a, in
         const int c0 = sidx[k];
         return dgv[k] * v[c0] - cw[k] * v[c0 - 1] - ce[k] * v[c0 + 1] - cs[k] * v[c0 - W] - cn[k] * v[c0 + W];
     };
-    // block partials of six sums, pushed to every block's slot [b][rank]; the barrier follows
-    auto push6 = [&](int b, float (&v)[6]) {
+    // Six sums over the cluster, in two halves around a barrier. A warp's six values go through a
+    // butterfly that halves the values with each of its first three steps (7 exchanges, then 2 more):
+    // lane q & 7 ends with value q's warp sum. (Six full butterflies are 30 exchanges: with them and
+    // their like after the barrier, the SM's one exchange a cycle took most of an iteration, 2.3 us.)
+    auto push6 = [&](int b, const float (&v)[6]) {
+        const bool h4 = lane & 4, h2 = lane & 2, h1 = lane & 1;
+        const float in[8] = {v[0], v[1], v[2], v[3], v[4], v[5], 0.f, 0.f};
+        float q4[4], q2[2], t;
 #pragma unroll
-        for (int q = 0; q < 6; ++q) {
+        for (int k = 0; k < 4; ++k)
+            q4[k] = (h4 ? in[k + 4] : in[k]) + __shfl_xor_sync(0xffffffffu, h4 ? in[k] : in[k + 4], 4);
 #pragma unroll
-            for (int off = 16; off > 0; off >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], off);
-            if (lane == 0) warp_part[q][warp] = v[q];
-        }
+        for (int k = 0; k < 2; ++k)
+            q2[k] = (h2 ? q4[k + 2] : q4[k]) + __shfl_xor_sync(0xffffffffu, h2 ? q4[k] : q4[k + 2], 2);
+        t = (h1 ? q2[1] : q2[0]) + __shfl_xor_sync(0xffffffffu, h1 ? q2[0] : q2[1], 1);
+        t += __shfl_xor_sync(0xffffffffu, t, 8);
+        t += __shfl_xor_sync(0xffffffffu, t, 16);
+        if (lane < 8) warp_part[b][warp][lane] = t;
+        if (ONE) return;
         __syncthreads();
         if (warp == 0) {
-            float t[6];
-#pragma unroll
-            for (int q = 0; q < 6; ++q) {
-                t[q] = lane < SOLVE_WARPS ? warp_part[q][lane] : 0.f;
-#pragma unroll
-                for (int off = 16; off > 0; off >>= 1) t[q] += __shfl_xor_sync(0xffffffffu, t[q], off);
-            }
-            if (lane < C) {
-                float4* dst = cl.map_shared_rank(&slots[b][rank][0], lane);
-                dst[0] = make_float4(t[0], t[1], t[2], 0.f);
-                dst[1] = make_float4(t[3], t[4], t[5], 0.f);
-            }
+            // value lane & 7 of the block, stored into every block's slot
+            t = 0.f;
+            for (int q = lane >> 3; q < (T >> 5); q += 4) t += warp_part[b][q][lane & 7];
+            t += __shfl_xor_sync(0xffffffffu, t, 8);
+            t += __shfl_xor_sync(0xffffffffu, t, 16);
+            for (int q = lane >> 3; q < C; q += 4) cl.map_shared_rank(&slots[b][rank][0], q)[lane & 7] = t;
         }
     };
-    // after the barrier, in every warp: lane q takes block q's partials, then a fixed butterfly
+    // after the barrier, in every warp: the partials of the blocks (of the warps, for one block), in a fixed order
     auto read6 = [&](int b, float (&v)[6]) {
-        float4 a0 = make_float4(0.f, 0.f, 0.f, 0.f), a1 = a0;
-        if (lane < C) {
-            a0 = slots[b][lane][0];
-            a1 = slots[b][lane][1];
-        }
-        v[0] = a0.x; v[1] = a0.y; v[2] = a0.z; v[3] = a1.x; v[4] = a1.y; v[5] = a1.z;
+        float t = 0.f;
+        for (int q = lane >> 3; q < (ONE ? T >> 5 : C); q += 4) t += ONE ? warp_part[b][q][lane & 7] : slots[b][q][lane & 7];
+        t += __shfl_xor_sync(0xffffffffu, t, 8);
+        t += __shfl_xor_sync(0xffffffffu, t, 16);
 #pragma unroll
-        for (int q = 0; q < 6; ++q) {
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], off);
-        }
+        for (int q = 0; q < 6; ++q) v[q] = __shfl_sync(0xffffffffu, t, q);
     };
 
     // ||b||^2 of both fields
@@ -426,7 +625,7 @@ __global__ void __launch_bounds__(SOLVE_THREADS) k_pcg_cg2(const SolveArgs a, in
             const int b = it & 1;
             ++it;
             publish(b);
-            cl.sync();
+            sync();
             float v[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll
             for (int f = 0; f < 2; ++f) {
@@ -439,7 +638,7 @@ __global__ void __launch_bounds__(SOLVE_THREADS) k_pcg_cg2(const SolveArgs a, in
                 }
             }
             push6(b, v);
-            cl.sync();
+            sync();
             read6(b, v);
 #pragma unroll
             for (int f = 0; f < 2; ++f) {
@@ -475,13 +674,13 @@ __global__ void __launch_bounds__(SOLVE_THREADS) k_pcg_cg2(const SolveArgs a, in
                 x0[n_[k]] += (double)d[0][k];
                 x1[n_[k]] += (double)d[1][k];
             }
-        cl.sync();
+        sync();
     }
     if (threadIdx.x == 0 && rank == 0) {
-        a.iters[blockIdx.x / C] = converged ? total : a.max_iter + 1;
+        a.iters[blockIdx.x / C] = converged ? total + a.iters[blockIdx.x / C] : a.max_iter + 1;
         if (!converged) atomicOr(a.status, STATUS_NOCONV);
     }
-    cl.sync();  // no block leaves while others may still write into its shared memory
+    if (!ONE) cl.sync();  // no block leaves while others may still write into its shared memory
 }
 
 __global__ void k_bump_step(uint32_t* step)
@@ -531,32 +730,52 @@ cudaError_t launch_scatter_iface(const double* iface_xi, const double* iface_eta
     return cudaGetLastError();
 }
 
-// Blocks per system: a power of two up to 16, no more than the SMs allow for
-// all systems at once and no more than the smallest system's rows.
-int solve_cluster_size(int nsys, int min_rows, int sm_count)
+// Clusters of 2^k blocks that run at once, a block per SM (nine clusters of 16 do not, although 144 SMs
+// would hold them: clusters stay inside the GPU's groups of SMs).
+static int clusters_at_once(int k)
 {
-    static int max_c = -1;
-    if (max_c < 0) {
-        max_c = 8;
-        if (cudaFuncSetAttribute(k_pcg_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3(16);
-            cfg.blockDim = dim3(SOLVE_THREADS);
-            cudaLaunchAttribute at[1];
-            at[0].id = cudaLaunchAttributeClusterDimension;
-            at[0].val.clusterDim.x = 16;
-            at[0].val.clusterDim.y = 1;
-            at[0].val.clusterDim.z = 1;
-            cfg.attrs = at;
-            cfg.numAttrs = 1;
-            int n = 0;
-            if (cudaOccupancyMaxActiveClusters(&n, k_pcg_cluster, &cfg) == cudaSuccess && n > 0) max_c = 16;
-        }
+    static int at_once[5] = {-1, -1, -1, -1, -1};
+    if (at_once[k] < 0) {
+        const auto fn = k_cheb<4, false>;
+        cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(1u << k);
+        cfg.blockDim = dim3(SOLVE_THREADS);
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = 1u << k;
+        at[0].val.clusterDim.y = 1;
+        at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        int n = 0;
+        at_once[k] = cudaOccupancyMaxActiveClusters(&n, fn, &cfg) == cudaSuccess ? n : 0;
         cudaGetLastError();
     }
-    int c = 1;
-    while (c * 2 <= max_c && (long long)c * 2 * nsys <= sm_count && c * 2 <= min_rows) c *= 2;
-    return c;
+    return at_once[k];
+}
+
+// Blocks per system (a power of two up to 16, no more than the smallest system's rows) for systems of at
+// most max_mx columns and max_my rows: the least time by what k_cheb measured, rounds of clusters that run
+// at once x (0.4 us + 0.25 us per unknown of a thread) an iteration. One block (no cluster barrier) pays for
+// up to 256 unknowns; above, its SM's few double-precision units make the residuals longer than the barrier.
+// Bands that need more than 4 unknowns per thread leave the register-resident kernels and are the last choice.
+int solve_cluster_size(int nsys, int min_rows, int max_mx, int max_my)
+{
+    if (max_mx * max_my <= 256) return 1;
+    int best = 1;
+    double least = 1e30;
+    for (int k = 0; k < 5 && (1 << k) <= min_rows; ++k) {
+        const int n = clusters_at_once(k), band = (max_my + (1 << k) - 1) / (1 << k) * max_mx;
+        if (n < 1) continue;
+        const double upt = std::max(0.25, (double)band / SOLVE_THREADS);
+        const double t = (double)((nsys + n - 1) / n) * (0.4 + 0.25 * upt) * (solve_reg_upt(band) ? 1.0 : 100.0);
+        if (t < least) {
+            least = t;
+            best = 1 << k;
+        }
+    }
+    return best;
 }
 
 static cudaLaunchConfig_t cluster_config(const SolveArgs& a, size_t smem, cudaStream_t s, cudaLaunchAttribute* at)
@@ -579,14 +798,35 @@ template <int UPT>
 static cudaError_t launch_reg(const SolveArgs& a, int rows_max, int max_mx, cudaStream_t s)
 {
     const size_t smem = 4 * (size_t)(rows_max + 2) * (size_t)(max_mx + 2) * sizeof(float);
-    if (a.cluster > 8) cudaFuncSetAttribute(k_pcg_cg2<UPT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    const auto fn = a.cluster == 1 ? k_pcg_cg2<UPT, true> : k_pcg_cg2<UPT, false>;
+    if (a.cluster > 8) cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_pcg_cg2<UPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
     cudaLaunchAttribute at[1];
     cudaLaunchConfig_t cfg = cluster_config(a, smem, s, at);
-    return cudaLaunchKernelEx(&cfg, k_pcg_cg2<UPT>, a, rows_max);
+    // no more warps than the largest band needs (their sums cost exchanges)
+    const int band = rows_max * max_mx;
+    cfg.blockDim = dim3((unsigned)std::min(SOLVE_THREADS, ((band + UPT - 1) / UPT + 31) / 32 * 32));
+    return cudaLaunchKernelEx(&cfg, fn, a, rows_max);
+}
+
+template <int UPT>
+static cudaError_t launch_cheb(const SolveArgs& a, int rows_max, int max_mx, cudaStream_t s)
+{
+    const size_t smem = 2 * (size_t)(rows_max + 2) * (size_t)(max_mx + 2) * sizeof(float2);
+    const auto fn = a.cluster == 1 ? k_cheb<UPT, true> : k_cheb<UPT, false>;
+    if (a.cluster > 8) cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (smem > 48 * 1024) {
+        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    cudaLaunchAttribute at[1];
+    cudaLaunchConfig_t cfg = cluster_config(a, smem, s, at);
+    const int band = rows_max * max_mx;
+    cfg.blockDim = dim3((unsigned)std::min(SOLVE_THREADS, ((band + UPT - 1) / UPT + 31) / 32 * 32));
+    return cudaLaunchKernelEx(&cfg, fn, a, rows_max);
 }
 
 // Unknowns per thread of the register-resident kernel for these systems
@@ -603,11 +843,13 @@ int solve_reg_upt(int max_band_unknowns)
 cudaError_t launch_pcg(const SolveArgs& a, int upt, int rows_max, int max_mx, cudaStream_t s)
 {
     if (a.nsys <= 0) return cudaSuccess;
+    cudaError_t e;
     switch (upt) {
-    case 1: return launch_reg<1>(a, rows_max, max_mx, s);
-    case 2: return launch_reg<2>(a, rows_max, max_mx, s);
-    case 4: return launch_reg<4>(a, rows_max, max_mx, s);
+    case 1: return (e = launch_cheb<1>(a, rows_max, max_mx, s)) != cudaSuccess ? e : launch_reg<1>(a, rows_max, max_mx, s);
+    case 2: return (e = launch_cheb<2>(a, rows_max, max_mx, s)) != cudaSuccess ? e : launch_reg<2>(a, rows_max, max_mx, s);
+    case 4: return (e = launch_cheb<4>(a, rows_max, max_mx, s)) != cudaSuccess ? e : launch_reg<4>(a, rows_max, max_mx, s);
     default: {
+        if (a.cluster > 8) cudaFuncSetAttribute(k_pcg_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         cudaLaunchAttribute at[1];
         cudaLaunchConfig_t cfg = cluster_config(a, 0, s, at);
         return cudaLaunchKernelEx(&cfg, k_pcg_cluster, a);
