@@ -281,18 +281,46 @@ struct Acc {
     __device__ __forceinline__ double sumsq() const { return (double)q - (double)cq; }
 };
 
-__device__ __forceinline__ double warp_sum(double v)
+// Sums of four values over the warp, value lane & 3 in each lane: the first two
+// steps halve the values held, so a lane makes 6 double-precision additions where
+// four butterflies make 20. A warp's addition takes 16 cycles of its SM's two
+// double-precision lanes: with 32-path tasks the sums were a sixth of an estimate.
+__device__ __forceinline__ double warp_sum4(double v0, double v1, double v2, double v3)
 {
+    const bool h2 = threadIdx.x & 2, h1 = threadIdx.x & 1;
+    const double a = (h2 ? v2 : v0) + __shfl_xor_sync(FULL, h2 ? v0 : v2, 2);
+    const double b = (h2 ? v3 : v1) + __shfl_xor_sync(FULL, h2 ? v1 : v3, 2);
+    double t = (h1 ? b : a) + __shfl_xor_sync(FULL, h1 ? a : b, 1);
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(FULL, v, off);
-    return v;
+    for (int off = 4; off < 32; off <<= 1) t += __shfl_xor_sync(FULL, t, off);
+    return t;
 }
 
+// Sum of nonnegative 64-bit integers below 2^58 over the warp.
 __device__ __forceinline__ long long warp_sum_ll(long long v)
 {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(FULL, v, off);
-    return v;
+    const unsigned lo = __reduce_add_sync(FULL, (unsigned)(v & 0xffff));
+    const unsigned mid = __reduce_add_sync(FULL, (unsigned)((v >> 16) & 0xffff));
+    const unsigned hi = __reduce_add_sync(FULL, (unsigned)(v >> 32));
+    return (long long)lo + ((long long)mid << 16) + ((long long)hi << 32);
+}
+
+// A lane's counts over a task (each nonnegative, below 2^31).
+__device__ __forceinline__ long long warp_sum_int(int v)
+{
+    return (long long)__reduce_add_sync(FULL, (unsigned)v & 0xffffu) +
+           ((long long)__reduce_add_sync(FULL, (unsigned)v >> 16) << 16);
+}
+
+// The sums of a task: lanes 0 to 3 hold the sums of Partial's order.
+__device__ __forceinline__ void put_partial(Partial* p, double sum, long long exits, long long steps)
+{
+    const int lane = threadIdx.x & 31;
+    if (lane < 4) reinterpret_cast<double*>(p)[lane] = sum;
+    if (lane == 0) {
+        p->exits = exits;
+        p->steps = steps;
+    }
 }
 
 // Deferred scoring: a path's record in the survivor buffer, one float2 (two
@@ -633,17 +661,12 @@ __device__ __forceinline__ void walk_tasks(const PathArgs& a, const uint8_t* zsm
             ++m;
         }
 
-        Partial p{};
+        double tot = 0.0;
         if (ACC) {
             const Acc ax = sums.get(0), ae = sums.get(1);
-            p.s_xi = warp_sum(ax.sum());
-            p.q_xi = warp_sum(ax.sumsq());
-            p.s_eta = warp_sum(ae.sum());
-            p.q_eta = warp_sum(ae.sumsq());
+            tot = warp_sum4(ax.sum(), ax.sumsq(), ae.sum(), ae.sumsq());
         }
-        p.exits = warp_sum_ll(sums.exits[threadIdx.x]);
-        p.steps = warp_sum_ll(sums.steps[threadIdx.x]);
-        if (lanes_below() == 0) a.partials[t] = p;
+        put_partial(a.partials + t, tot, warp_sum_int(sums.exits[threadIdx.x]), warp_sum_int(sums.steps[threadIdx.x]));
     }
 }
 
@@ -802,19 +825,8 @@ __global__ void __launch_bounds__(512, 2) k_paths_exp(const PathArgs a)
                 next += __popc(need);
             }
         }
-        const double sx = warp_sum(ax.sum()), qx = warp_sum(ax.sumsq());
-        const double se = warp_sum(ae.sum()), qe = warp_sum(ae.sumsq());
-        const long long ex = warp_sum_ll(exits), st = warp_sum_ll(steps);
-        if (lane == 0) {
-            Partial p;
-            p.s_xi = sx;
-            p.q_xi = qx;
-            p.s_eta = se;
-            p.q_eta = qe;
-            p.exits = ex;
-            p.steps = st;
-            a.partials[t] = p;
-        }
+        const double tot = warp_sum4(ax.sum(), ax.sumsq(), ae.sum(), ae.sumsq());
+        put_partial(a.partials + t, tot, warp_sum_int(exits), warp_sum_int(steps));
     }
 }
 
@@ -833,7 +845,7 @@ __global__ void __launch_bounds__(512, 2) k_paths_exp(const PathArgs a)
 // more nodes than SMs, T = 1024 gives each node's paths four times the threads.
 constexpr int SCORE_BATCH = 2;
 
-__device__ void finalize_node(const FinalArgs& a, int node, int lane, const double* add0);
+__device__ void finalize_node(const FinalArgs& a, int node, int lane, double more);
 
 template <bool CV, int SCORE_THREADS>
 __global__ void __launch_bounds__(SCORE_THREADS, 1024 / SCORE_THREADS) k_score_surv(const ScoreArgs a)
@@ -844,7 +856,7 @@ __global__ void __launch_bounds__(SCORE_THREADS, 1024 / SCORE_THREADS) k_score_s
     const NodeDev& nd = a.nodes[node];
     if (nd.ntasks == 0 || (a.fin.node_mask && !a.fin.node_mask[node])) {
         // a boundary node or one left to the interface fill: no paths to score
-        if (warp == 0) finalize_node(a.fin, node, lane, nullptr);
+        if (warp == 0) finalize_node(a.fin, node, lane, 0.0);
         return;   // uniform over the block
     }
     const InstDev I = a.inst[nd.inst];
@@ -920,14 +932,15 @@ __global__ void __launch_bounds__(SCORE_THREADS, 1024 / SCORE_THREADS) k_score_s
             cvs[u] = cn[u];
         }
     }
-    const double v[4] = {warp_sum(ax.sum()), warp_sum(ax.sumsq()), warp_sum(ae.sum()), warp_sum(ae.sumsq())};
-    if (lane == 0)
-        for (int q = 0; q < 4; ++q) red[warp][q] = v[q];
+    const double v = warp_sum4(ax.sum(), ax.sumsq(), ae.sum(), ae.sumsq());
+    if (lane < 4) red[warp][lane] = v;
     __syncthreads();
     if (warp == 0) {
-        double tot[4] = {0.0, 0.0, 0.0, 0.0};
-        for (int g = 0; g < SCORE_THREADS / 32; ++g)
-            for (int q = 0; q < 4; ++q) tot[q] += red[g][q];
+        // sum lane & 3 over the block's warps, in a fixed order
+        double tot = 0.0;
+        for (int g = lane >> 2; g < SCORE_THREADS / 32; g += 8) tot += red[g][lane & 3];
+#pragma unroll
+        for (int off = 4; off < 32; off <<= 1) tot += __shfl_xor_sync(FULL, tot, off);
         finalize_node(a.fin, node, lane, tot);   // the node's mean and standard error
     }
 }
@@ -948,10 +961,11 @@ __device__ __forceinline__ double face_value64(const InstDev& I, int field, int 
 }
 
 // One warp per node: compensated sums of the node's task partials (each lane a
-// fixed stride of tasks; add0, if non-null, added to the first task's), a
-// fixed butterfly across the warp, then the mean and the standard error
-// s / sqrt(N), s^2 = (Q - S^2 / N) / (N - 1) of the shifted scores.
-__device__ void finalize_node(const FinalArgs& a, int node, int lane, const double* add0)
+// fixed stride of tasks), a fixed butterfly across the warp that leaves sum
+// lane & 3 in each lane (`more` joins it there), then the mean and the standard error
+// s / sqrt(N), s^2 = (Q - S^2 / N) / (N - 1) of the shifted scores: lane 0 for
+// xi, lane 2 for eta.
+__device__ void finalize_node(const FinalArgs& a, int node, int lane, double more)
 {
     const NodeDev nd = a.nodes[node];
     const OutDev o = a.out_table ? a.out_table[nd.inst] : a.out0;
@@ -1001,12 +1015,14 @@ __device__ void finalize_node(const FinalArgs& a, int node, int lane, const doub
     long long ex = 0, st = 0;
     for (int t = nd.task0 + lane; t < nd.task0 + nd.ntasks; t += 32) {
         const Partial p = a.partials[t];
-        double in[4] = {p.s_xi, p.q_xi, p.s_eta, p.q_eta};
-        if (add0 && t == nd.task0)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) in[q] += add0[q];
+        const double in[4] = {p.s_xi, p.q_xi, p.s_eta, p.q_eta};
+        const bool first = t < nd.task0 + 32;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
+            if (first) {
+                v[q] = in[q];
+                continue;
+            }
             const double y = in[q] - c[q];
             const double tt = v[q] + y;
             c[q] = (tt - v[q]) - y;
@@ -1015,23 +1031,20 @@ __device__ void finalize_node(const FinalArgs& a, int node, int lane, const doub
         ex += p.exits;
         st += p.steps;
     }
-    double tot[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) tot[q] = warp_sum(v[q] - c[q]);
+    const double tot = warp_sum4(v[0] - c[0], v[1] - c[1], v[2] - c[2], v[3] - c[3]) + more;
+    const double sq = __shfl_down_sync(FULL, tot, 1);   // lane 0: Q of xi, lane 2: Q of eta
     ex = warp_sum_ll(ex);
     st = warp_sum_ll(st);
-    if (lane == 0) {
+    if (lane == 0 || lane == 2) {
         const double N = (double)nd.n_paths;
-        const double mx = tot[0] / N, me = tot[2] / N;
-        double vx = 0.0, ve = 0.0;
-        if (nd.n_paths > 1) {
-            vx = fmax(0.0, (tot[1] - tot[0] * mx) / (N - 1.0));
-            ve = fmax(0.0, (tot[3] - tot[2] * me) / (N - 1.0));
-        }
-        if (o.mean_xi) o.mean_xi[k] = (double)nd.xf + mx;
-        if (o.mean_eta) o.mean_eta[k] = (double)nd.yf + me;
-        if (o.se_xi) o.se_xi[k] = sqrt(vx / N);
-        if (o.se_eta) o.se_eta[k] = sqrt(ve / N);
+        const double m = tot / N;
+        const double var = nd.n_paths > 1 ? fmax(0.0, (sq - tot * m) / (N - 1.0)) : 0.0;
+        double* const mean = lane ? o.mean_eta : o.mean_xi;
+        double* const se = lane ? o.se_eta : o.se_xi;
+        if (mean) mean[k] = (double)(lane ? nd.yf : nd.xf) + m;
+        if (se) se[k] = sqrt(var / N);
+    }
+    if (lane == 0) {
         if (o.n_exit) o.n_exit[k] = ex;
         if (o.path_steps) o.path_steps[k] = st;
     }
@@ -1042,7 +1055,7 @@ __global__ void k_finalize(const FinalArgs a)
     const int node = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5);
     const int lane = threadIdx.x & 31;
     if (node >= a.nnodes) return;
-    finalize_node(a, node, lane, nullptr);
+    finalize_node(a, node, lane, 0.0);
 }
 
 __global__ void k_rng_draw(uint64_t seed, const uint32_t* __restrict__ ctrs, long long count,
@@ -1149,7 +1162,7 @@ cudaError_t launch_score_surv(const ScoreArgs& a, bool cv, cudaStream_t s)
 
 cudaError_t launch_finalize(const FinalArgs& a, cudaStream_t s)
 {
-    const int block = 256;
+    const int block = 64;   // few nodes per block: their double-precision sums spread over the SMs
     const long long threads = (long long)a.nnodes * 32;
     const int grid = (int)((threads + block - 1) / block);
     if (grid > 0) k_finalize<<<grid, block, 0, s>>>(a);
