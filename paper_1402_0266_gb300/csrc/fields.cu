@@ -20,6 +20,15 @@ namespace sdd {
 
 namespace {
 
+// 1 / v to about an ulp for a positive v that single precision holds: a single-precision reciprocal and two
+// Newton steps, four operations of the SM's two double-precision lanes where a division takes about ten.
+__device__ __forceinline__ double reciprocal(double v)
+{
+    double r = (double)__frcp_rn((float)v);
+    r = fma(r, fma(-v, r, 1.0), r);
+    return fma(r, fma(-v, r, 1.0), r);
+}
+
 __device__ __forceinline__ double2 node_drift(const float* __restrict__ w, int nx, int ny, int i, int j,
                                               double rx, double ry)
 {
@@ -40,8 +49,8 @@ __device__ __forceinline__ double2 node_drift(const float* __restrict__ w, int n
               (double)col[(long long)(ny - 3) * nx]) * ry;
     else
         wy = ((double)col[(long long)(j + 1) * nx] - (double)col[(long long)(j - 1) * nx]) * ry;
-    const double wc = (double)row[i];
-    return make_double2(-wx / wc, -wy / wc);
+    const double r = -reciprocal((double)row[i]);
+    return make_double2(wx * r, wy * r);
 }
 
 // Bilinear coefficients of two fields u, v on one cell, interleaved so that one
@@ -57,10 +66,12 @@ __device__ __forceinline__ void bilinear_coefs2(double u00, double u10, double u
 
 __device__ __forceinline__ bool bad_w(float v) { return !(v > 0.0f) || !isfinite(v); }
 
-// One block per 32 x 8 cells: the drift at the tile's 33 x 9 nodes once (in
-// shared memory, double precision), then each cell's records.
-constexpr int PREP_TX = 32, PREP_TY = 8;
+// One block per 32 x TY cells: the drift at the tile's 33 x (TY + 1) nodes once (in
+// shared memory, double precision), then each cell's records. TY is 8, or 2 where blocks of 8 rows
+// would not give every SM four of them: the kernel is bound by the double-precision lanes of the SMs in use.
+constexpr int PREP_TX = 32;
 
+template <int PREP_TY>
 __global__ void __launch_bounds__(PREP_TX * PREP_TY) k_prep_cells(const float* __restrict__ w,
                                                                   const double* __restrict__ xi,
                                                                   const double* __restrict__ eta, int nx, int ny,
@@ -151,16 +162,18 @@ __global__ void k_cv_cells(const double* __restrict__ g, int slices, int nx, int
     cv[2 * cell + 1] = make_uint4(w[4], w[5], w[6], w[7]);
 }
 
-// Cumulative trapezoid of one line of w, normalised by its total, by one warp:
-// each lane sums a contiguous run of intervals, the run totals are scanned
-// across the warp, then each lane writes its run.
-__device__ void warp_cumtrapz(const float* __restrict__ v, long long stride, int n, double* __restrict__ out)
+// Face data of one line of w: the cumulative trapezoid over its total, by one block: each thread sums a
+// contiguous run of intervals, the run totals are scanned over the block, then each thread writes its run.
+// (By one warp per line a 2049^2 grid's faces took 280 us, 64 dependent loads a thread.)
+constexpr int FACE_THREADS = 256;
+
+__device__ void block_cumtrapz(const float* __restrict__ v, long long stride, int n, double* __restrict__ out,
+                               float* __restrict__ out32)
 {
-    const int lane = threadIdx.x & 31;
-    const int intervals = n - 1;
-    const int run = (intervals + 31) / 32;
-    const int k0 = 1 + lane * run;
-    const int k1 = min(k0 + run, n);
+    __shared__ double part[FACE_THREADS / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int run = (n - 1 + FACE_THREADS - 1) / FACE_THREADS;
+    const int k0 = min(1 + (int)threadIdx.x * run, n), k1 = min(k0 + run, n);
     double mine = 0.0;
     for (int k = k0; k < k1; ++k) mine += 0.5 * ((double)v[(k - 1) * stride] + (double)v[k * stride]);
     double incl = mine;
@@ -169,44 +182,48 @@ __device__ void warp_cumtrapz(const float* __restrict__ v, long long stride, int
         const double o = __shfl_up_sync(0xffffffffu, incl, off);
         if (lane >= off) incl += o;
     }
-    const double total = __shfl_sync(0xffffffffu, incl, 31);
-    double acc = incl - mine;
-    if (lane == 0) out[0] = 0.0;
+    if (lane == 31) part[warp] = incl;
+    __syncthreads();
+    double acc = incl - mine, total = 0.0;
+    for (int q = 0; q < FACE_THREADS / 32; ++q) {
+        if (q < warp) acc += part[q];
+        total += part[q];
+    }
+    if (threadIdx.x == 0) {
+        out[0] = 0.0;
+        if (out32) out32[0] = 0.f;
+    }
     for (int k = k0; k < k1; ++k) {
         acc += 0.5 * ((double)v[(k - 1) * stride] + (double)v[k * stride]);
-        out[k] = acc / total;
+        const double f = acc / total;
+        out[k] = f;
+        if (out32) out32[k] = (float)f;
     }
 }
 
-__global__ void k_winslow_faces(const float* __restrict__ w, int nx, int ny, double* __restrict__ faces,
-                                float* __restrict__ faces32)
+// Block 0, 1: xi on y = 0, 1; 2, 3: eta on x = 0, 1; 4: xi on x = 0, 1 and eta on y = 0, 1 (0 and 1).
+__global__ void __launch_bounds__(FACE_THREADS) k_winslow_faces(const float* __restrict__ w, int nx, int ny,
+                                                                double* __restrict__ faces,
+                                                                float* __restrict__ faces32)
 {
     const long long per_field = 2LL * ny + 2LL * nx;
-    double* xl = faces;
-    double* xr = faces + ny;
-    double* xb = faces + 2LL * ny;
-    double* xt = faces + 2LL * ny + nx;
-    double* el = faces + per_field;
-    double* er = faces + per_field + ny;
-    double* eb = faces + per_field + 2LL * ny;
-    double* et = faces + per_field + 2LL * ny + nx;
-    const int warp = threadIdx.x >> 5;
-    if (warp == 0) warp_cumtrapz(w, 1, nx, xb);                                   // xi on y = 0
-    if (warp == 1) warp_cumtrapz(w + (long long)(ny - 1) * nx, 1, nx, xt);        // xi on y = 1
-    if (warp == 2) warp_cumtrapz(w, nx, ny, el);                                  // eta on x = 0
-    if (warp == 3) warp_cumtrapz(w + (nx - 1), nx, ny, er);                       // eta on x = 1
-    for (int k = threadIdx.x; k < ny; k += blockDim.x) {
-        xl[k] = 0.0;
-        xr[k] = 1.0;
+    // line q of a field: left, right (ny), bottom, top (nx)
+    auto line = [&](int field, int q) { return field * per_field + (q < 2 ? q * (long long)ny : 2LL * ny + (q - 2) * (long long)nx); };
+    const int b = blockIdx.x;
+    if (b < 4) {
+        const long long at = b < 2 ? line(0, 2 + b) : line(1, b - 2);
+        const float* v = b == 0 ? w : b == 1 ? w + (long long)(ny - 1) * nx : b == 2 ? w : w + (nx - 1);
+        block_cumtrapz(v, b < 2 ? 1 : nx, b < 2 ? nx : ny, faces + at, faces32 ? faces32 + at : nullptr);
+        return;
     }
-    for (int k = threadIdx.x; k < nx; k += blockDim.x) {
-        eb[k] = 0.0;
-        et[k] = 1.0;
-    }
-    if (faces32) {
-        // the single-precision copy the path kernel scores exits with
-        __syncthreads();
-        for (long long k = threadIdx.x; k < 2 * per_field; k += blockDim.x) faces32[k] = (float)faces[k];
+    for (int q = 0; q < 4; ++q) {
+        const long long at = q < 2 ? line(0, q) : line(1, q);
+        const int n = q < 2 ? ny : nx;
+        const double f = q & 1 ? 1.0 : 0.0;
+        for (int k = threadIdx.x; k < n; k += blockDim.x) {
+            faces[at + k] = f;
+            if (faces32) faces32[at + k] = (float)f;
+        }
     }
 }
 
@@ -221,13 +238,15 @@ __global__ void k_faces32(const double* __restrict__ f64, float* __restrict__ f3
 cudaError_t launch_prep_cells(const float* w, const double* xi, const double* eta, int nx, int ny, float4* bcoef,
                               float4* fcoef, int* status, cudaStream_t s, uint8_t* zmap)
 {
-    const dim3 block(PREP_TX, PREP_TY);
-    const dim3 grid((nx - 1 + PREP_TX - 1) / PREP_TX, (ny - 1 + PREP_TY - 1) / PREP_TY);
+    const unsigned tiles = (unsigned)(nx - 1 + PREP_TX - 1) / PREP_TX;
     if (bcoef && zmap) {
         const cudaError_t e = cudaMemsetAsync(zmap, 0, kZmapBytes, s);
         if (e != cudaSuccess) return e;
     }
-    k_prep_cells<<<grid, block, 0, s>>>(w, xi, eta, nx, ny, bcoef, fcoef, status, zmap);
+    if ((long long)tiles * ((ny - 1 + 7) / 8) >= 4 * 152)
+        k_prep_cells<8><<<dim3(tiles, (ny - 1 + 7) / 8), dim3(PREP_TX, 8), 0, s>>>(w, xi, eta, nx, ny, bcoef, fcoef, status, zmap);
+    else
+        k_prep_cells<2><<<dim3(tiles, (ny - 1 + 1) / 2), dim3(PREP_TX, 2), 0, s>>>(w, xi, eta, nx, ny, bcoef, fcoef, status, zmap);
     return cudaGetLastError();
 }
 
@@ -241,7 +260,7 @@ cudaError_t launch_cv_cells(const double* grad, int slices, int nx, int ny, uint
 
 cudaError_t launch_winslow_faces(const float* w, int nx, int ny, double* faces64, float* faces32, cudaStream_t s)
 {
-    k_winslow_faces<<<1, 128, 0, s>>>(w, nx, ny, faces64, faces32);
+    k_winslow_faces<<<5, FACE_THREADS, 0, s>>>(w, nx, ny, faces64, faces32);
     return cudaGetLastError();
 }
 
