@@ -1241,7 +1241,7 @@ sdd_status train_loop(sdd_ctx* c, float* theta, const float* norm, const float* 
     if (nb < 1) return fail(c, SDD_EINVAL, "fewer rows than one batch");
     int64_t total = (int64_t)p->epochs * nb;
     const int64_t run = p->max_steps > 0 ? std::min<int64_t>(p->max_steps, total) : total;
-    const int nblk = p->batch / tile;
+    const int nblk = mlp_grad_blocks(p->batch);
     CU(c, c->cv_m.alloc(2 * (size_t)kMlpStride));
     CU(c, c->cv_v.alloc(2 * (size_t)kMlpStride));
     CU(c, c->cv_part.alloc(2 * (size_t)nblk * kMlpStride));
@@ -1770,7 +1770,7 @@ sdd_status sdd_mlp_grad(sdd_ctx* c, const float* theta, const float* norm, const
     const int tile = mlp_tile_rows();
     if (rows < tile || rows % tile != 0 || rows > (1LL << 28))
         return fail(c, SDD_EINVAL, "rows must be a positive multiple of %d", tile);
-    const int nblk = (int)(rows / tile);
+    const int nblk = mlp_grad_blocks(rows);
     CU(c, c->cv_grad_part.alloc(2 * (size_t)nblk * kMlpStride));
     const float inv = (float)(1.0 / (double)rows);
     CU(c, launch_mlp_grad(theta, norm, feats, targets, 0, rows, inv, c->cv_grad_part.p, c->stream));

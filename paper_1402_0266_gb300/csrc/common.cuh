@@ -207,7 +207,8 @@ cudaError_t launch_cv_scatter(const double* xs, const double* ys, const double* 
                               cudaStream_t s);
 size_t mlp_norm_scratch_doubles();
 cudaError_t launch_mlp_norm(const float* feats, long long n, double* scratch, float* norm, cudaStream_t s);
-int mlp_tile_rows();
+int mlp_tile_rows();                      // batches are multiples of this
+int mlp_grad_blocks(long long rows);      // partial gradients per network that a batch of `rows` writes
 cudaError_t launch_mlp_grad(const float* theta, const float* norm, const float* feats, const float* targets,
                             long long row0, long long rows, float inv_batch, float* part, cudaStream_t s);
 cudaError_t launch_mlp_reduce(const float* part, int nblk, float inv_rows, float* grad, float* loss, cudaStream_t s);

@@ -13,8 +13,8 @@
 //                               finite differences of the drift (FP64);
 //   k_cv_scatter                training rows from single-path estimates;
 //   k_moments / k_norm          feature standardisation (two-pass, FP64);
-//   k_mlp_grad                  forward and backward pass over a tile of 64
-//                               rows in shared memory, FP32 SIMT; per-tile
+//   k_mlp_grad                  forward and backward pass over tiles of 64
+//                               rows in shared memory, FP32 SIMT; per-block
 //                               partial gradients, reduced in a fixed order;
 //   k_mlp_reduce / k_mlp_adam   the batch gradient; Adam (Kingma & Ba 2015);
 //   k_cv_tabulate               the table G at every node and time slice by
@@ -36,8 +36,9 @@ constexpr int D = kMlpInputs;
 constexpr int OW1 = 0, OB1 = H * D, OW2 = OB1 + H, OB2 = OW2 + H * H, OW3 = OB2 + H, OB3 = OW3 + H;
 static_assert(OB3 + 1 == kMlpParams, "parameter layout");
 
-constexpr int TILE = 64;     // rows per block of the training kernel
+constexpr int TILE = 64;     // rows of a tile of the training kernel
 constexpr int LD = 68;       // row stride of the activation tiles (16-byte rows, conflict-free float4 reads)
+constexpr int ZS = 8;        // row stride of the inputs (five, the fifth in the second float4)
 constexpr int GRAD_THREADS = 256;
 
 // ---------------------------------------------------------------- node fields
@@ -260,199 +261,285 @@ __global__ void k_norm(const double* __restrict__ part, int nblk, long long n, d
 struct GradSmem {
     float th[kMlpStride];      // the network's parameters
     float w2t[H * H];          // W2 transposed: [k][j]
-    float z[TILE * D];
-    float y[TILE];
-    float d[TILE];
     float h1[TILE * LD];       // tanh(a1), later dL/da1
     float h2[TILE * LD];       // tanh(a2), later dL/da2
+    float z[TILE * ZS];
+    float y[TILE];
+    float d[TILE];
+    float quarter[4][H];       // sums over a quarter of the tile's rows
     float red[GRAD_THREADS / 32];
 };
 
-// One 64-row tile of one network (blockIdx.y): forward, backward, and the
-// tile's share of the gradient of the batch loss (1 / batch) sum (g - y)^2,
-// written to part[(f nblk + tile) stride + p]; part[.. + kMlpParams] = the
-// tile's sum of squared errors.
-__global__ void __launch_bounds__(GRAD_THREADS) k_mlp_grad(const float* __restrict__ theta,
-                                                           const float* __restrict__ norm,
-                                                           const float* __restrict__ feats,
-                                                           const float* __restrict__ targets, long long row0,
-                                                           float inv_batch, float* __restrict__ part)
+// A sum over tiles: value and rounding error (Knuth's two-sum), so that a block's tiles lose nothing that
+// one tile's sum does not.
+struct TileSum {
+    float s = 0.f, c = 0.f;
+    __device__ __forceinline__ void add(float v)
+    {
+        const float t = s + v;
+        const float b = t - s;
+        c += (s - (t - b)) + (v - b);
+        s = t;
+    }
+    __device__ __forceinline__ float value() const { return s + c; }
+};
+
+// dst[r][c] += sum_q a[row(r)][q] b[q][4 tx + c] over q < 64: a row-major with stride LD, read four q at a
+// time (a warp reads two rows of a and 64 columns of b), b with stride H.
+template <int RPT>
+__device__ __forceinline__ void tile_product(float (&acc)[RPT][4], const float* a, const float* b, int tx, int ty)
 {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    GradSmem& S = *reinterpret_cast<GradSmem*>(smem_raw);
-    const int f = blockIdx.y, tile = blockIdx.x, nblk = gridDim.x, t = threadIdx.x;
-    const float* th = theta + (long long)f * kMlpStride;
-    for (int p = t; p < kMlpParams; p += GRAD_THREADS) S.th[p] = th[p];
-    for (int p = t; p < H * H; p += GRAD_THREADS) {
-        const int j = p >> 6, k = p & 63;
-        S.w2t[k * H + j] = th[OW2 + p];
-    }
-    const long long r0 = row0 + (long long)tile * TILE;
-    for (int p = t; p < TILE * D; p += GRAD_THREADS) {
-        const int c = p % D;
-        S.z[p] = (feats[r0 * D + p] - norm[c]) * norm[D + c];
-    }
-    for (int i = t; i < TILE; i += GRAD_THREADS) S.y[i] = targets[2 * (r0 + i) + f];
-    __syncthreads();
-
-    // layer 1: thread owns unit j and rows (t >> 6) + 4 m
-    {
-        const int j = t & 63;
-        float wj[D];
-#pragma unroll
-        for (int c = 0; c < D; ++c) wj[c] = S.th[OW1 + j * D + c];
-        const float bj = S.th[OB1 + j];
 #pragma unroll 4
-        for (int i = t >> 6; i < TILE; i += 4) {
-            float a = bj;
+    for (int q = 0; q < H; q += 4) {
+        float4 bv[4];
 #pragma unroll
-            for (int c = 0; c < D; ++c) a = fmaf(wj[c], S.z[i * D + c], a);
-            S.h1[i * LD + j] = tanhf(a);
-        }
-    }
-    __syncthreads();
-
-    const int tx = t & 15, ty = t >> 4;   // 4 x 4 blocks of the 64 x 64 tiles
-    // layer 2: a2[i][j] = b2[j] + sum_k h1[i][k] W2[j][k], rows 4 ty.., units 4 tx..
-    {
-        float acc[4][4];
+        for (int e = 0; e < 4; ++e) bv[e] = *reinterpret_cast<const float4*>(&b[(q + e) * H + 4 * tx]);
 #pragma unroll
-        for (int r = 0; r < 4; ++r)
+        for (int r = 0; r < RPT; ++r) {
+            const float4 av = *reinterpret_cast<const float4*>(&a[(ty + 16 * r) * LD + q]);
+            const float ae[4] = {av.x, av.y, av.z, av.w};
 #pragma unroll
-            for (int c = 0; c < 4; ++c) acc[r][c] = S.th[OB2 + 4 * tx + c];
-#pragma unroll 8
-        for (int k = 0; k < H; ++k) {
-            const float4 wv = *reinterpret_cast<const float4*>(&S.w2t[k * H + 4 * tx]);
-#pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                const float h = S.h1[(4 * ty + r) * LD + k];
-                acc[r][0] = fmaf(h, wv.x, acc[r][0]);
-                acc[r][1] = fmaf(h, wv.y, acc[r][1]);
-                acc[r][2] = fmaf(h, wv.z, acc[r][2]);
-                acc[r][3] = fmaf(h, wv.w, acc[r][3]);
+            for (int e = 0; e < 4; ++e) {
+                acc[r][0] = fmaf(ae[e], bv[e].x, acc[r][0]);
+                acc[r][1] = fmaf(ae[e], bv[e].y, acc[r][1]);
+                acc[r][2] = fmaf(ae[e], bv[e].z, acc[r][2]);
+                acc[r][3] = fmaf(ae[e], bv[e].w, acc[r][3]);
             }
-        }
-#pragma unroll
-        for (int r = 0; r < 4; ++r)
-#pragma unroll
-            for (int c = 0; c < 4; ++c) S.h2[(4 * ty + r) * LD + 4 * tx + c] = tanhf(acc[r][c]);
-    }
-    __syncthreads();
-
-    // output and dL/dg: one warp per 8 rows, lanes split the 64 units
-    const int lane = t & 31, wid = t >> 5;
-    {
-        float sq = 0.f;
-        for (int i = wid * 8; i < wid * 8 + 8; ++i) {
-            float v = S.th[OW3 + lane] * S.h2[i * LD + lane] + S.th[OW3 + lane + 32] * S.h2[i * LD + lane + 32];
-            for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            const float e = v + S.th[OB3] - S.y[i];
-            if (lane == 0) S.d[i] = 2.f * e * inv_batch;
-            sq = fmaf(e, e, sq);
-        }
-        if (lane == 0) S.red[wid] = sq;
-    }
-    __syncthreads();
-    float* out = part + ((long long)f * nblk + tile) * kMlpStride;
-    // dL/dw3[j] = sum_i d_i h2[i][j], dL/db3 = sum_i d_i, loss
-    if (t < H) {
-        float a = 0.f;
-        for (int i = 0; i < TILE; ++i) a = fmaf(S.d[i], S.h2[i * LD + t], a);
-        out[OW3 + t] = a;
-    } else if (t == H) {
-        float a = 0.f;
-        for (int i = 0; i < TILE; ++i) a += S.d[i];
-        out[OB3] = a;
-    } else if (t == H + 1) {
-        float a = 0.f;
-        for (int q = 0; q < GRAD_THREADS / 32; ++q) a += S.red[q];
-        out[kMlpParams] = a;
-    }
-    __syncthreads();
-    // dL/da2 = d_i w3_j (1 - h2^2), in place
-    {
-        const int j = t & 63;
-        const float w3 = S.th[OW3 + j];
-        for (int i = t >> 6; i < TILE; i += 4) {
-            const float h = S.h2[i * LD + j];
-            S.h2[i * LD + j] = S.d[i] * w3 * (1.f - h * h);
-        }
-    }
-    __syncthreads();
-    // dL/dW2[j][k] = sum_i g2[i][j] h1[i][k] (units 4 ty.., inputs 4 tx..), dL/db2
-    {
-        float acc[4][4] = {};
-        float db[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 4
-        for (int i = 0; i < TILE; ++i) {
-            const float4 g = *reinterpret_cast<const float4*>(&S.h2[i * LD + 4 * ty]);
-            const float4 h = *reinterpret_cast<const float4*>(&S.h1[i * LD + 4 * tx]);
-            const float gv[4] = {g.x, g.y, g.z, g.w};
-#pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                acc[r][0] = fmaf(gv[r], h.x, acc[r][0]);
-                acc[r][1] = fmaf(gv[r], h.y, acc[r][1]);
-                acc[r][2] = fmaf(gv[r], h.z, acc[r][2]);
-                acc[r][3] = fmaf(gv[r], h.w, acc[r][3]);
-                db[r] += gv[r];
-            }
-        }
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            *reinterpret_cast<float4*>(&out[OW2 + (4 * ty + r) * H + 4 * tx]) =
-                make_float4(acc[r][0], acc[r][1], acc[r][2], acc[r][3]);
-            if (tx == 0) out[OB2 + 4 * ty + r] = db[r];
-        }
-    }
-    // dL/da1[i][k] = (sum_j g2[i][j] W2[j][k]) (1 - h1[i][k]^2), rows 4 ty.., inputs 4 tx..;
-    // each thread overwrites only its own h1 entries, which no other thread reads in this phase
-    __syncthreads();
-    {
-        float acc[4][4] = {};
-#pragma unroll 8
-        for (int j = 0; j < H; ++j) {
-            const float4 wv = *reinterpret_cast<const float4*>(&S.th[OW2 + j * H + 4 * tx]);
-#pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                const float g = S.h2[(4 * ty + r) * LD + j];
-                acc[r][0] = fmaf(g, wv.x, acc[r][0]);
-                acc[r][1] = fmaf(g, wv.y, acc[r][1]);
-                acc[r][2] = fmaf(g, wv.z, acc[r][2]);
-                acc[r][3] = fmaf(g, wv.w, acc[r][3]);
-            }
-        }
-#pragma unroll
-        for (int r = 0; r < 4; ++r)
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                float& h = S.h1[(4 * ty + r) * LD + 4 * tx + c];
-                h = acc[r][c] * (1.f - h * h);
-            }
-    }
-    __syncthreads();
-    // dL/dW1[j][c] = sum_i g1[i][j] z[i][c], dL/db1[j] = sum_i g1[i][j]
-    for (int o = t; o < H * (D + 1); o += GRAD_THREADS) {
-        const int j = o & 63, c = o >> 6;
-        float a = 0.f;
-        if (c < D) {
-            for (int i = 0; i < TILE; ++i) a = fmaf(S.h1[i * LD + j], S.z[i * D + c], a);
-            out[OW1 + j * D + c] = a;
-        } else {
-            for (int i = 0; i < TILE; ++i) a += S.h1[i * LD + j];
-            out[OB1 + j] = a;
         }
     }
 }
 
-// Sum of the tiles' partials in tile order (FP64): the batch gradient and mean loss.
-__global__ void k_mlp_reduce(const float* __restrict__ part, int nblk, float inv_rows, float* __restrict__ grad,
-                             float* __restrict__ loss)
+// Forward and backward over the block's tiles of one network (blockIdx.y): its share of the
+// gradient of the batch loss (1 / batch) sum (g - y)^2, written to part[(f nblk + block) stride + p];
+// part[.. + kMlpParams] = its sum of squared errors.
+//
+// Three 64 x 64 products and 128 tanhf per row: 4-by-4 register tiles, operands read four deep (12
+// shared-memory wavefronts per 64 FMAs a thread; read one by one they were 6 per 16), W2's gradient kept in
+// registers over the tiles. A tile's partial gradient is 18 KB, so blocks take several tiles and write one.
+// 65,536 rows: 126 us (147 us for a block and a partial per tile, whose sum took 163 us more; now 9), issue slots
+// 60 % busy, the shared-memory loads the next bound; tiles of 128 rows were within 3 %.
+__global__ void __launch_bounds__(GRAD_THREADS, 2) k_mlp_grad(const float* __restrict__ theta,
+                                                              const float* __restrict__ norm,
+                                                              const float* __restrict__ feats,
+                                                              const float* __restrict__ targets, long long row0,
+                                                              long long rows, float inv_batch,
+                                                              float* __restrict__ part)
+{
+    constexpr int ROWS = TILE, RPT = ROWS / 16, QROWS = ROWS / 4;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    GradSmem& S = *reinterpret_cast<GradSmem*>(smem_raw);
+    const int f = blockIdx.y, t = threadIdx.x;
+    const int lane = t & 31, wid = t >> 5, tx = t & 15, ty = t >> 4;
+    const int j = t & 63, quarter = t >> 6;
+    const float* th = theta + (long long)f * kMlpStride;
+    for (int p = t; p < kMlpParams; p += GRAD_THREADS) S.th[p] = th[p];
+    for (int p = t; p < H * H; p += GRAD_THREADS) S.w2t[(p & 63) * H + (p >> 6)] = th[OW2 + p];
+
+    TileSum gw2[4][4], gb2[4], small[2], loss;   // small: thread t's outputs of W1, b1 (t, t + 256) or w3 (loss: b3 too)
+    TileSum gw3, gb3;
+    const int ntiles = (int)((rows + ROWS - 1) / ROWS);
+    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+        const long long r0 = row0 + (long long)tile * ROWS;
+        const int have = (int)min((long long)ROWS, row0 + rows - r0);
+        __syncthreads();   // the tile before is done (and the parameters are in place)
+        for (int p = t; p < ROWS * D; p += GRAD_THREADS) {
+            const int c = p % D;
+            S.z[p / D * ZS + c] = p < have * D ? (feats[r0 * D + p] - norm[c]) * norm[D + c] : 0.f;
+        }
+        for (int i = t; i < ROWS; i += GRAD_THREADS) S.y[i] = i < have ? targets[2 * (r0 + i) + f] : 0.f;
+        __syncthreads();
+
+        // layer 1: thread owns unit j and rows quarter + 4 m
+        {
+            float wj[D];
+#pragma unroll
+            for (int c = 0; c < D; ++c) wj[c] = S.th[OW1 + j * D + c];
+            const float bj = S.th[OB1 + j];
+#pragma unroll 4
+            for (int i = quarter; i < ROWS; i += 4) {
+                const float4 z = *reinterpret_cast<const float4*>(&S.z[i * ZS]);
+                float a = fmaf(wj[0], z.x, bj);
+                a = fmaf(wj[1], z.y, a);
+                a = fmaf(wj[2], z.z, a);
+                a = fmaf(wj[3], z.w, a);
+                a = fmaf(wj[4], S.z[i * ZS + 4], a);
+                S.h1[i * LD + j] = tanhf(a);
+            }
+        }
+        __syncthreads();
+
+        // layer 2: a2[i][j] = b2[j] + sum_k h1[i][k] W2[j][k], rows ty + 16 r, units 4 tx..
+        {
+            float acc[RPT][4];
+#pragma unroll
+            for (int r = 0; r < RPT; ++r)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) acc[r][c] = S.th[OB2 + 4 * tx + c];
+            tile_product<RPT>(acc, S.h1, S.w2t, tx, ty);
+#pragma unroll
+            for (int r = 0; r < RPT; ++r)
+                *reinterpret_cast<float4*>(&S.h2[(ty + 16 * r) * LD + 4 * tx]) =
+                    make_float4(tanhf(acc[r][0]), tanhf(acc[r][1]), tanhf(acc[r][2]), tanhf(acc[r][3]));
+        }
+        __syncthreads();
+
+        // output and dL/dg: 256 / ROWS neighbouring threads per row, each with its share of the units
+        {
+            constexpr int SPLIT = GRAD_THREADS / ROWS, UNITS = H / SPLIT;
+            const int i = t / SPLIT, part0 = (t % SPLIT) * UNITS;
+            float v = 0.f;
+#pragma unroll
+            for (int u = 0; u < UNITS; u += 4) {
+                const float4 h = *reinterpret_cast<const float4*>(&S.h2[i * LD + part0 + u]);
+                const float4 w = *reinterpret_cast<const float4*>(&S.th[OW3 + part0 + u]);
+                v += (w.x * h.x + w.y * h.y) + (w.z * h.z + w.w * h.w);
+            }
+#pragma unroll
+            for (int o = SPLIT / 2; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            const float e = i < have ? v + S.th[OB3] - S.y[i] : 0.f;
+            float sq = t % SPLIT == 0 ? e * e : 0.f;
+            if (t % SPLIT == 0) S.d[i] = 2.f * e * inv_batch;
+            for (int o = 16; o; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+            if (lane == 0) S.red[wid] = sq;
+        }
+        __syncthreads();
+        // dL/dw3[j] = sum_i d_i h2[i][j] by quarters of the rows, dL/db3 = sum_i d_i, the loss;
+        // then dL/da2 = d_i w3_j (1 - h2^2) in place, rows by the same threads
+        {
+            const float w3 = S.th[OW3 + j];
+            float a = 0.f;
+#pragma unroll 8
+            for (int i = quarter * QROWS; i < (quarter + 1) * QROWS; ++i) {
+                const float h = S.h2[i * LD + j], d = S.d[i];
+                a = fmaf(d, h, a);
+                S.h2[i * LD + j] = d * w3 * (1.f - h * h);
+            }
+            S.quarter[quarter][j] = a;
+        }
+        __syncthreads();
+        if (t < H) {
+            gw3.add((S.quarter[0][t] + S.quarter[1][t]) + (S.quarter[2][t] + S.quarter[3][t]));
+        } else if (wid == 2) {
+            float a = 0.f;
+            for (int i = lane; i < ROWS; i += 32) a += S.d[i];
+            for (int o = 16; o; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+            gb3.add(a);
+        } else if (t == 96) {
+            float a = 0.f;
+            for (int q = 0; q < GRAD_THREADS / 32; ++q) a += S.red[q];
+            loss.add(a);
+        }
+        // dL/dW2[j][k] = sum_i g2[i][j] h1[i][k] (units 4 ty.., inputs 4 tx..), dL/db2
+        {
+            float acc[4][4] = {};
+            float db[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+            for (int i = 0; i < ROWS; ++i) {
+                const float4 g = *reinterpret_cast<const float4*>(&S.h2[i * LD + 4 * ty]);
+                const float4 h = *reinterpret_cast<const float4*>(&S.h1[i * LD + 4 * tx]);
+                const float gv[4] = {g.x, g.y, g.z, g.w};
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    acc[r][0] = fmaf(gv[r], h.x, acc[r][0]);
+                    acc[r][1] = fmaf(gv[r], h.y, acc[r][1]);
+                    acc[r][2] = fmaf(gv[r], h.z, acc[r][2]);
+                    acc[r][3] = fmaf(gv[r], h.w, acc[r][3]);
+                    db[r] += gv[r];
+                }
+            }
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+#pragma unroll
+                for (int c = 0; c < 4; ++c) gw2[r][c].add(acc[r][c]);
+                gb2[r].add(db[r]);
+            }
+        }
+        __syncthreads();   // h1 is overwritten next
+        // dL/da1[i][k] = (sum_j g2[i][j] W2[j][k]) (1 - h1[i][k]^2), rows ty + 16 r, inputs 4 tx..;
+        // each thread overwrites only its own h1 entries, which no other thread reads in this phase
+        {
+            float acc[RPT][4] = {};
+            tile_product<RPT>(acc, S.h2, S.th + OW2, tx, ty);
+#pragma unroll
+            for (int r = 0; r < RPT; ++r) {
+                float4* const h = reinterpret_cast<float4*>(&S.h1[(ty + 16 * r) * LD + 4 * tx]);
+                const float4 v = *h;
+                *h = make_float4(acc[r][0] * (1.f - v.x * v.x), acc[r][1] * (1.f - v.y * v.y),
+                                 acc[r][2] * (1.f - v.z * v.z), acc[r][3] * (1.f - v.w * v.w));
+            }
+        }
+        __syncthreads();
+        // dL/dW1[j][c] = sum_i g1[i][j] z[i][c], dL/db1[j] = sum_i g1[i][j], by quarters of the rows
+        {
+            float a[D + 1] = {};
+#pragma unroll 4
+            for (int i = quarter * QROWS; i < (quarter + 1) * QROWS; ++i) {
+                const float g = S.h1[i * LD + j];
+                const float4 z = *reinterpret_cast<const float4*>(&S.z[i * ZS]);
+                a[0] = fmaf(g, z.x, a[0]);
+                a[1] = fmaf(g, z.y, a[1]);
+                a[2] = fmaf(g, z.z, a[2]);
+                a[3] = fmaf(g, z.w, a[3]);
+                a[4] = fmaf(g, S.z[i * ZS + 4], a[4]);
+                a[D] += g;
+            }
+            // dL/da2 is no longer needed: its place takes the quarters' sums
+#pragma unroll
+            for (int c = 0; c <= D; ++c) S.h2[(quarter * (D + 1) + c) * H + j] = a[c];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int o = t + q * GRAD_THREADS;
+            constexpr int Q = H * (D + 1);
+            if (o < Q) small[q].add((S.h2[o] + S.h2[Q + o]) + (S.h2[2 * Q + o] + S.h2[3 * Q + o]));
+        }
+    }
+
+    float* out = part + ((long long)f * gridDim.x + blockIdx.x) * kMlpStride;
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const int o = t + q * GRAD_THREADS;
+        if (o < H * D) out[OW1 + (o & 63) * D + (o >> 6)] = small[q].value();
+        else if (o < H * (D + 1)) out[OB1 + (o & 63)] = small[q].value();
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        *reinterpret_cast<float4*>(&out[OW2 + (4 * ty + r) * H + 4 * tx]) =
+            make_float4(gw2[r][0].value(), gw2[r][1].value(), gw2[r][2].value(), gw2[r][3].value());
+        if (tx == 0) out[OB2 + 4 * ty + r] = gb2[r].value();
+    }
+    if (t < H) out[OW3 + t] = gw3.value();
+    else if (t == 64) out[OB3] = gb3.value();
+    else if (t == 96) out[kMlpParams] = loss.value();
+}
+
+// Sum over the blocks' partials of parameter p (kMlpParams: the loss) in double precision: SUM_SPLIT threads
+// (threadIdx.y) each take every SUM_SPLIT-th block, thread y = 0 gets the total. (One thread per parameter
+// and 1,024 partials took 163 us, a chain of loads and additions on 36 SMs.)
+constexpr int SUM_SPLIT = 16;
+
+__device__ __forceinline__ double part_sum(const float* __restrict__ part, int nblk, int f, int p)
+{
+    __shared__ double red[SUM_SPLIT][32];
+    double a = 0.0;
+    if (p <= kMlpParams)
+        for (int b = threadIdx.y; b < nblk; b += SUM_SPLIT) a += (double)part[((long long)f * nblk + b) * kMlpStride + p];
+    red[threadIdx.y][threadIdx.x] = a;
+    __syncthreads();
+    if (threadIdx.y == 0)
+        for (int q = 1; q < SUM_SPLIT; ++q) a += red[q][threadIdx.x];
+    return a;
+}
+
+// The batch gradient and mean loss from the blocks' partials.
+__global__ void __launch_bounds__(32 * SUM_SPLIT) k_mlp_reduce(const float* __restrict__ part, int nblk, float inv_rows,
+                                                               float* __restrict__ grad, float* __restrict__ loss)
 {
     const int f = blockIdx.y;
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p > kMlpParams) return;
-    double a = 0.0;
-    for (int b = 0; b < nblk; ++b) a += (double)part[((long long)f * nblk + b) * kMlpStride + p];
+    const int p = blockIdx.x * 32 + threadIdx.x;
+    const double a = part_sum(part, nblk, f, p);
+    if (threadIdx.y != 0 || p > kMlpParams) return;
     if (p < kMlpParams) {
         grad[(long long)f * kMlpStride + p] = (float)a;
     } else if (loss) {
@@ -470,15 +557,14 @@ struct AdamArgs {
 };
 
 // Adam (Kingma & Ba 2015, Algorithm 1) on the batch gradient, reduced from
-// the tiles' partials in tile order.
-__global__ void k_mlp_adam(float* __restrict__ theta, float* __restrict__ m, float* __restrict__ v,
+// the blocks' partials.
+__global__ void __launch_bounds__(32 * SUM_SPLIT) k_mlp_adam(float* __restrict__ theta, float* __restrict__ m, float* __restrict__ v,
                            const float* __restrict__ part, AdamArgs a, float* __restrict__ losses, long long steps)
 {
     const int f = blockIdx.y;
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p > kMlpParams) return;
-    double s = 0.0;
-    for (int b = 0; b < a.nblk; ++b) s += (double)part[((long long)f * a.nblk + b) * kMlpStride + p];
+    const int p = blockIdx.x * 32 + threadIdx.x;
+    const double s = part_sum(part, a.nblk, f, p);
+    if (threadIdx.y != 0 || p > kMlpParams) return;
     if (p == kMlpParams) {
         if (losses) losses[(long long)f * steps + a.step] = (float)(s * a.inv_rows);
         return;
@@ -843,21 +929,24 @@ cudaError_t launch_mlp_norm(const float* feats, long long n, double* scratch, fl
 
 int mlp_tile_rows() { return TILE; }
 
+// Two blocks per SM, one for each network (three, at 80 registers, took as long).
+int mlp_grad_blocks(long long rows) { return (int)std::min<long long>(152, (rows + TILE - 1) / TILE); }
+
 cudaError_t launch_mlp_grad(const float* theta, const float* norm, const float* feats, const float* targets,
                             long long row0, long long rows, float inv_batch, float* part, cudaStream_t s)
 {
     const size_t smem = sizeof(GradSmem);
     cudaError_t e = cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    const dim3 grid((unsigned)(rows / TILE), 2);
-    k_mlp_grad<<<grid, GRAD_THREADS, smem, s>>>(theta, norm, feats, targets, row0, inv_batch, part);
+    const dim3 grid((unsigned)mlp_grad_blocks(rows), 2);
+    k_mlp_grad<<<grid, GRAD_THREADS, smem, s>>>(theta, norm, feats, targets, row0, rows, inv_batch, part);
     return cudaGetLastError();
 }
 
 cudaError_t launch_mlp_reduce(const float* part, int nblk, float inv_rows, float* grad, float* loss, cudaStream_t s)
 {
-    const dim3 grid((kMlpParams + 1 + 255) / 256, 2);
-    k_mlp_reduce<<<grid, 256, 0, s>>>(part, nblk, inv_rows, grad, loss);
+    const dim3 grid((kMlpParams + 1 + 31) / 32, 2);
+    k_mlp_reduce<<<grid, dim3(32, SUM_SPLIT), 0, s>>>(part, nblk, inv_rows, grad, loss);
     return cudaGetLastError();
 }
 
@@ -875,8 +964,8 @@ cudaError_t launch_mlp_adam(float* theta, float* m, float* v, const float* part,
     a.inv_rows = inv_rows;
     a.nblk = nblk;
     a.step = step;
-    const dim3 grid((kMlpParams + 1 + 255) / 256, 2);
-    k_mlp_adam<<<grid, 256, 0, s>>>(theta, m, v, part, a, losses, steps);
+    const dim3 grid((kMlpParams + 1 + 31) / 32, 2);
+    k_mlp_adam<<<grid, dim3(32, SUM_SPLIT), 0, s>>>(theta, m, v, part, a, losses, steps);
     return cudaGetLastError();
 }
 
