@@ -490,7 +490,8 @@ sdd_status sdd_keypoint_fill(sdd_ctx* ctx, const uint8_t* mask, double* values_x
  * With multigrid, max_iter caps the inner iterations: inside sdd_step's graph
  * the refinement sweeps and inner iterations are graph while-loops that stop
  * once every field has converged (at most 30 inner iterations per sweep and
- * 8 sweeps, within max_iter); a direct sdd_subdomain_solve runs a fixed 5 x 6.
+ * 8 sweeps, within max_iter); a direct sdd_subdomain_solve is a graph of its
+ * own, at most 5 x 6, kept until rtol or max_iter change.
  * sdd_solver_in_use returns the solver the next solve will use (1 Jacobi,
  * 2 multigrid, 3 direct). */
 #define SDD_SOLVER_AUTO 0

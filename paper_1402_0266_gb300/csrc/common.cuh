@@ -277,18 +277,21 @@ struct MgArgs {
     int32_t mx[kMgMaxLevels], my[kMgMaxLevels];
     long long off[kMgMaxLevels];
     int32_t B0;              // blocks per system for level-0 vectors (partial sums)
+    int32_t T0;              // tiles per system of level 0 (partial sums of the V-cycle's last launch)
     // level arrays (all levels, padded boxes with a zero frame)
     float* D;
     float* CX;               // coefficient between a node and its east neighbour
     float* CY;               // ... and its north neighbour
     float* MS;               // mass term 1 / (w Dt)
-    float* U[2];             // V-cycle iterate (level 0: the preconditioned residual z)
+    float* U[2];             // V-cycle iterate
     float* F[2];             // V-cycle right-hand side (level 0: the residual r)
+    float* Z[2];             // V-cycle result of the levels above `tail` (level 0: the preconditioned residual z)
     // level-0 Krylov vectors: search direction, product, correction
     float* Pv[2];
     float* Qv[2];
     float* Cv[2];
-    float* part;             // [nsys][B0][4] single-precision partial sums
+    float* part;             // [nsys][max(B0, T0)][4] single-precision partial sums
+    float* part_rr;          // [nsys][B0][4] those of ||r||^2
     double* part64;          // [nsys][B0][4] double-precision partial sums
     double* stop2;           // [nsys][2]
     float* rz;               // [nsys][2][2] (r, z) by parity
@@ -307,7 +310,6 @@ struct MgArgs {
 bool mg_levels(int mx, int my, MgArgs& a);
 long long mg_layout(MgArgs& a, int nsys);
 cudaError_t launch_mg_setup(const MgArgs& a, cudaStream_t s);
-cudaError_t launch_mg_solve(const MgArgs& a, cudaStream_t s);
 cudaError_t launch_mg_solve_graph(const MgArgs& a, cudaStream_t s, cudaStream_t s2, cudaStream_t s3);
 // the same solve inside one thread-block cluster per subdomain (mgc.cu); mgc_config returns the unknowns
 // per thread (0: subdomains too large) and the cluster shape
