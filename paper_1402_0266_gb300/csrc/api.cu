@@ -137,6 +137,7 @@ struct sdd_ctx {
     DevBuf<uint32_t> d_step;
     bool user_faces = false;
     bool dirty_w = true, dirty_fields = true;
+    bool dirty_faces = true;      // the face data of the current w (a solve builds them without the drift records)
 
     Plan mc_plan;     // sdd_interface_mc
     Plan step_plan;   // the interface nodes of sdd_step
@@ -331,8 +332,17 @@ sdd_status prepare_parts(sdd_ctx* c, cudaStream_t s, bool w_part, bool f_part)
         CU(c, launch_prep_cells(c->w.p, c->fld[c->cur][0].p, c->fld[c->cur][1].p, c->nx, c->ny,
                                 dw ? c->bcoef.p : nullptr, df ? c->fcoef.p : nullptr, c->d_status.p, s, c->zmap.p));
     }
-    if (w_part) c->dirty_w = false;
+    if (w_part) c->dirty_w = c->dirty_faces = false;
     if (f_part) c->dirty_fields = false;
+    return SDD_OK;
+}
+
+// The face data alone: all that a direct solve needs of the tables (its set-up checks w).
+sdd_status prepare_faces(sdd_ctx* c, cudaStream_t s)
+{
+    if (c->dirty_faces && !c->user_faces)
+        CU(c, launch_winslow_faces(c->w.p, c->nx, c->ny, c->faces64.p, c->faces32.p, s));
+    c->dirty_faces = false;
     return SDD_OK;
 }
 
@@ -345,7 +355,7 @@ sdd_status prepare(sdd_ctx* c, cudaStream_t s)
         }
         CU(c, launch_prep_cells(c->w.p, c->fld[c->cur][0].p, c->fld[c->cur][1].p, c->nx, c->ny, c->bcoef.p,
                                 c->fcoef.p, c->d_status.p, s, c->zmap.p));
-        c->dirty_w = c->dirty_fields = false;
+        c->dirty_w = c->dirty_faces = c->dirty_fields = false;
         return SDD_OK;
     }
     return prepare_parts(c, s, true, true);
@@ -1096,7 +1106,7 @@ sdd_status enqueue_solve_dirichlet(sdd_ctx* c, const SolveCall& k, const double*
 sdd_status enqueue_solve_system(sdd_ctx* c, const SolveCall& k, cudaStream_t s)
 {
     CU(c, launch_solve_setup(k.w, k.px, k.pe, c->nx, c->ny, k.Dt, c->cx.p, c->cy.p, c->dg.p, c->rhs0.p, c->cxf.p,
-                             c->cyf.p, c->dgf.p, c->dinvf.p, s));
+                             c->cyf.p, c->dgf.p, c->dinvf.p, c->d_status.p, s));
     if (k.use_mg) CU(c, launch_mg_setup(k.m, s));
     return SDD_OK;
 }
@@ -1550,7 +1560,7 @@ sdd_status sdd_set_w(sdd_ctx* c, const float* w)
 {
     if (!c || !w) return fail(c, SDD_EINVAL, "null argument");
     CU(c, cudaMemcpyAsync(c->w.p, w, (size_t)c->nx * c->ny * sizeof(float), cudaMemcpyDeviceToDevice, c->stream));
-    c->dirty_w = true;
+    c->dirty_w = c->dirty_faces = true;
     return SDD_OK;
 }
 
@@ -1558,7 +1568,7 @@ sdd_status sdd_set_w_host(sdd_ctx* c, const float* w)
 {
     if (!c || !w) return fail(c, SDD_EINVAL, "null argument");
     CU(c, cudaMemcpyAsync(c->w.p, w, (size_t)c->nx * c->ny * sizeof(float), cudaMemcpyHostToDevice, c->stream));
-    c->dirty_w = true;
+    c->dirty_w = c->dirty_faces = true;
     return SDD_OK;
 }
 
@@ -1586,7 +1596,7 @@ sdd_status sdd_set_boundary(sdd_ctx* c, const double* faces)
         c->user_faces = true;
     } else {
         c->user_faces = false;
-        c->dirty_w = true;  // recompute the paper's data from w
+        c->dirty_w = c->dirty_faces = true;  // recompute the paper's data from w
     }
     drop_graphs(c);
     return SDD_OK;
@@ -2000,7 +2010,7 @@ sdd_status sdd_subdomain_solve(sdd_ctx* c, double Dt, const double* iface_xi, co
     }
     if (!c->iface_idx.empty() && (!iface_xi || !iface_eta)) return fail(c, SDD_EINVAL, "null interface values");
     if (!(Dt > 0.0) || !(rtol >= 0.0) || max_iter < 0) return fail(c, SDD_EINVAL, "Dt, rtol or max_iter rejected");
-    sdd_status st = prepare(c, c->stream);
+    sdd_status st = prepare_faces(c, c->stream);
     if (st != SDD_OK) return st;
     if ((st = solve_direct(c, Dt, iface_xi, iface_eta, rtol, max_iter, xi_out, eta_out)) != SDD_OK) return st;
     if (iters_out) {
@@ -2029,7 +2039,7 @@ static sdd_status capture_step(sdd_ctx* c, const sdd_step_params* p, int K, int 
     cudaGraph_t g = nullptr;
     CU(c, cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
     // the graph always recomputes the tables: w and the fields change every step
-    const bool keep_w = c->dirty_w, keep_f = c->dirty_fields;
+    const bool keep_w = c->dirty_w, keep_f = c->dirty_fields, keep_faces = c->dirty_faces;
     c->dirty_w = true;
     c->dirty_fields = true;
     const int saved = c->cur;
@@ -2125,6 +2135,7 @@ static sdd_status capture_step(sdd_ctx* c, const sdd_step_params* p, int K, int 
     c->cur = saved;
     c->dirty_w = keep_w;
     c->dirty_fields = keep_f;
+    c->dirty_faces = keep_faces;
     cudaError_t e = cudaStreamEndCapture(s, &g);
     if (st != SDD_OK) {
         if (g) cudaGraphDestroy(g);
@@ -2229,7 +2240,7 @@ sdd_status sdd_step(sdd_ctx* c, const sdd_step_params* p)
     }
     c->cur = 1 - c->cur;
     c->step_index += 1;
-    c->dirty_w = false;
+    c->dirty_w = c->dirty_faces = false;
     c->dirty_fields = true;  // the new fields need their tables before a direct estimate
     return SDD_OK;
 }
@@ -2383,10 +2394,11 @@ sdd_status capture_batch_step(sdd_batch* b, const sdd_step_params* p, int K, int
     cudaGraph_t g = nullptr;
     CU(&b->err, cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
     sdd_status st = SDD_OK;
-    std::vector<char> keep_w(b->ctxs.size()), keep_f(b->ctxs.size());
+    std::vector<char> keep_w(b->ctxs.size()), keep_f(b->ctxs.size()), keep_faces(b->ctxs.size());
     for (size_t k = 0; k < b->ctxs.size(); ++k) {
         keep_w[k] = b->ctxs[k]->dirty_w;
         keep_f[k] = b->ctxs[k]->dirty_fields;
+        keep_faces[k] = b->ctxs[k]->dirty_faces;
     }
     auto rec_ev = [&](int k) {
         if (st != SDD_OK) return;
@@ -2418,6 +2430,7 @@ sdd_status capture_batch_step(sdd_batch* b, const sdd_step_params* p, int K, int
     for (size_t k = 0; k < b->ctxs.size(); ++k) {
         b->ctxs[k]->dirty_w = keep_w[k];
         b->ctxs[k]->dirty_fields = keep_f[k];
+        b->ctxs[k]->dirty_faces = keep_faces[k];
     }
     cudaError_t e = cudaStreamEndCapture(s, &g);
     if (st != SDD_OK) {
@@ -2613,7 +2626,7 @@ sdd_status sdd_batch_step(sdd_batch* b, const sdd_step_params* p)
     for (sdd_ctx* c : b->ctxs) {
         c->cur = 1 - c->cur;
         c->step_index = b->step_index + 1;
-        c->dirty_w = false;
+        c->dirty_w = c->dirty_faces = false;
         c->dirty_fields = true;
     }
     b->step_index += 1;

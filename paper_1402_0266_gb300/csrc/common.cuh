@@ -120,6 +120,21 @@ constexpr int kZmapBytes = (kZmapTiles * kZmapTiles + 15) / 16 * 16;
 // Largest grid of the single-instance path kernels: cell indices that single precision adds to 2^23 exactly.
 constexpr long long kOneMaxCells = 1LL << 23;
 
+// 1 / v to about an ulp for positive v: a single-precision reciprocal and two Newton steps, four operations of
+// the SM's two double-precision lanes where a division takes about ten. Anything whose reciprocal leaves the
+// normal numbers of single precision is divided.
+__device__ __forceinline__ double reciprocal(double v)
+{
+    const float vf = (float)v;
+    if (!(vf > 1e-37f && vf < 1e37f)) return 1.0 / v;
+    double r = (double)__frcp_rn(vf);
+    r = fma(r, fma(-v, r, 1.0), r);
+    return fma(r, fma(-v, r, 1.0), r);
+}
+
+// A density value that the status word reports: not finite or not positive.
+__device__ __forceinline__ bool bad_w(float v) { return !(v > 0.0f) || !isfinite(v); }
+
 // Start coordinate of a node's paths: the node's in single precision, inside the square when the node is.
 inline float start_coord(double v)
 {
@@ -318,7 +333,7 @@ cudaError_t launch_mgc(const MgArgs& a, int upt, int C, int rows_max, size_t sme
 
 cudaError_t launch_solve_setup(const float* w, const double* prev_xi, const double* prev_eta, int nx, int ny,
                                double Dt, double* cx, double* cy, double* dg, double* rhs0, float* cxf, float* cyf,
-                               float* dgf, float* dinvf, cudaStream_t s);
+                               float* dgf, float* dinvf, int* status, cudaStream_t s);
 int solve_cluster_size(int nsys, int min_rows, int max_mx, int max_my);
 cudaError_t launch_dirichlet(const double* faces64, const double* prev_xi, const double* prev_eta,
                              const double* iface_xi, const double* iface_eta, const int32_t* iface_idx,

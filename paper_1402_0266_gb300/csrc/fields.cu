@@ -20,15 +20,6 @@ namespace sdd {
 
 namespace {
 
-// 1 / v to about an ulp for a positive v that single precision holds: a single-precision reciprocal and two
-// Newton steps, four operations of the SM's two double-precision lanes where a division takes about ten.
-__device__ __forceinline__ double reciprocal(double v)
-{
-    double r = (double)__frcp_rn((float)v);
-    r = fma(r, fma(-v, r, 1.0), r);
-    return fma(r, fma(-v, r, 1.0), r);
-}
-
 __device__ __forceinline__ double2 node_drift(const float* __restrict__ w, int nx, int ny, int i, int j,
                                               double rx, double ry)
 {
@@ -63,8 +54,6 @@ __device__ __forceinline__ void bilinear_coefs2(double u00, double u10, double u
     hi = make_float4((float)(u01 - u00), (float)(v01 - v00), (float)((u11 - u10) - (u01 - u00)),
                      (float)((v11 - v10) - (v01 - v00)));
 }
-
-__device__ __forceinline__ bool bad_w(float v) { return !(v > 0.0f) || !isfinite(v); }
 
 // One block per 32 x TY cells: the drift at the tile's 33 x (TY + 1) nodes once (in
 // shared memory, double precision), then each cell's records. TY is 8, or 2 where blocks of 8 rows

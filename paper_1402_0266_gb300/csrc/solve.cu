@@ -39,10 +39,10 @@ namespace {
 
 
 __global__ void k_solve_setup(const float* __restrict__ w, const double* __restrict__ pxi,
-                              const double* __restrict__ peta, int nx, int ny, double Dt, double* __restrict__ cx,
+                              const double* __restrict__ peta, int nx, int ny, double rDt, double* __restrict__ cx,
                               double* __restrict__ cy, double* __restrict__ dg, double* __restrict__ rhs0,
                               float* __restrict__ cxf, float* __restrict__ cyf, float* __restrict__ dgf,
-                              float* __restrict__ dinvf)
+                              float* __restrict__ dinvf, int* status)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int j = blockIdx.y * blockDim.y + threadIdx.y;
@@ -50,23 +50,25 @@ __global__ void k_solve_setup(const float* __restrict__ w, const double* __restr
     const long long n = (long long)j * nx + i;
     const double ihx2 = (double)(nx - 1) * (double)(nx - 1);
     const double ihy2 = (double)(ny - 1) * (double)(ny - 1);
+    if (bad_w(w[n])) atomicOr(status, STATUS_BAD_W);
     const double wc = (double)w[n];
-    const double e = (i + 1 < nx) ? ihx2 / (0.5 * (wc + (double)w[n + 1])) : 0.0;
-    const double no = (j + 1 < ny) ? ihy2 / (0.5 * (wc + (double)w[n + nx])) : 0.0;
+    // (five divisions a node by the SM's two double-precision lanes took 40 us at 513^2)
+    const double e = (i + 1 < nx) ? ihx2 * reciprocal(0.5 * (wc + (double)w[n + 1])) : 0.0;
+    const double no = (j + 1 < ny) ? ihy2 * reciprocal(0.5 * (wc + (double)w[n + nx])) : 0.0;
     cx[n] = e;
     cy[n] = no;
     cxf[n] = (float)e;
     cyf[n] = (float)no;
-    double d = 1.0 / (wc * Dt);
+    double d = rDt * reciprocal(wc);
     rhs0[n] = pxi[n] * d;
     rhs0[(long long)nx * ny + n] = peta[n] * d;
     if (i > 0 && i + 1 < nx && j > 0 && j + 1 < ny) {
         const double wwest = (double)w[n - 1], wsouth = (double)w[n - nx];
-        d += e + no + ihx2 / (0.5 * (wc + wwest)) + ihy2 / (0.5 * (wc + wsouth));
+        d += e + no + ihx2 * reciprocal(0.5 * (wc + wwest)) + ihy2 * reciprocal(0.5 * (wc + wsouth));
     }
     dg[n] = d;
     dgf[n] = (float)d;
-    dinvf[n] = (float)(1.0 / d);
+    dinvf[n] = (float)reciprocal(d);
 }
 
 // Dirichlet data of the new fields: the face data on the outer boundary, the
@@ -692,11 +694,12 @@ __global__ void k_bump_step(uint32_t* step)
 
 cudaError_t launch_solve_setup(const float* w, const double* prev_xi, const double* prev_eta, int nx, int ny,
                                double Dt, double* cx, double* cy, double* dg, double* rhs0, float* cxf, float* cyf,
-                               float* dgf, float* dinvf, cudaStream_t s)
+                               float* dgf, float* dinvf, int* status, cudaStream_t s)
 {
     const dim3 block(32, 8);
     const dim3 grid((nx + 31) / 32, (ny + 7) / 8);
-    k_solve_setup<<<grid, block, 0, s>>>(w, prev_xi, prev_eta, nx, ny, Dt, cx, cy, dg, rhs0, cxf, cyf, dgf, dinvf);
+    k_solve_setup<<<grid, block, 0, s>>>(w, prev_xi, prev_eta, nx, ny, 1.0 / Dt, cx, cy, dg, rhs0, cxf, cyf, dgf, dinvf,
+                                       status);
     return cudaGetLastError();
 }
 
