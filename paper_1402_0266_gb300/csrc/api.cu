@@ -750,7 +750,7 @@ sdd_status run_plan_on(std::string* err, Plan& P, const InstDev* inst, const Out
         CU(err, launch_score_surv(sa, cv, s));
         return SDD_OK;
     }
-    CU(err, launch_finalize(f, s));
+    CU(err, launch_finalize(f, (long long)P.ntasks, s));
     return SDD_OK;
 }
 

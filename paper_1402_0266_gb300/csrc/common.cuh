@@ -174,7 +174,8 @@ enum : int {
 cudaError_t launch_paths(const PathArgs& a, int exit_mode, bool record, int grid, int block, cudaStream_t s,
                          int cvm = 0);
 // exit_mode 0 with an even number of sub-steps has its own kernel (no odd last pair)
-cudaError_t launch_finalize(const FinalArgs& a, cudaStream_t s);
+// ntasks: the tasks of all nodes
+cudaError_t launch_finalize(const FinalArgs& a, long long ntasks, cudaStream_t s);
 cudaError_t launch_score_surv(const ScoreArgs& a, bool cv, cudaStream_t s);
 int path_kernel_blocks_per_sm(int exit_mode, bool record, int block, int cvm = 0, bool map = false,
                               bool single = false, bool defer = false);

@@ -31,6 +31,7 @@
 #include <cmath>
 #include <cstring>
 
+#include "cluster.cuh"
 #include "common.cuh"
 
 namespace sdd {
@@ -830,38 +831,208 @@ __global__ void __launch_bounds__(512, 2) k_paths_exp(const PathArgs a)
     }
 }
 
+__device__ __forceinline__ double face_value64(const InstDev& I, int field, int face, double s)
+{
+    const int n = (face < 2) ? I.ny : I.nx;
+    long long off = (long long)field * (2LL * I.ny + 2LL * I.nx);
+    if (face >= 1) off += I.ny;
+    if (face >= 2) off += I.ny;
+    if (face >= 3) off += I.nx;
+    const double* v = I.faces64 + off;
+    const double g = s * (double)(n - 1);
+    int k = (int)floor(g);
+    k = max(0, min(k, n - 2));
+    const double f = g - (double)k;
+    return (1.0 - f) * v[k] + f * v[k + 1];
+}
+
+// A node that no path was walked for (left to the interface fill, or on the boundary): its outputs by one warp.
+__device__ bool pathless_node(const FinalArgs& a, int node, const NodeDev& nd, int lane)
+{
+    const bool filled = a.node_mask && !a.node_mask[node];
+    if (!filled && nd.ntasks != 0) return false;
+    const OutDev o = a.out_table ? a.out_table[nd.inst] : a.out0;
+    const int k = nd.local;
+    double vx = 0.0, ve = 0.0;
+    if (!filled) {
+        // a node on the boundary: its Dirichlet value, every path exits at time 0
+        const InstDev I = a.inst[nd.inst];
+        int face;
+        double tg;
+        if (nd.x <= 0.0) { face = 0; tg = nd.y; }
+        else if (nd.x >= 1.0) { face = 1; tg = nd.y; }
+        else if (nd.y <= 0.0) { face = 2; tg = nd.x; }
+        else { face = 3; tg = nd.x; }
+        vx = face_value64(I, 0, face, tg);
+        ve = face_value64(I, 1, face, tg);
+        for (int p = lane; p < nd.n_paths; p += 32) {
+            const long long ri = nd.rec0 + p;
+            if (a.rec.steps) a.rec.steps[ri] = 0;
+            if (a.rec.code) a.rec.code[ri] = face;
+            if (a.rec.score_xi) a.rec.score_xi[ri] = (float)vx;
+            if (a.rec.score_eta) a.rec.score_eta[ri] = (float)ve;
+            if (a.rec.x_end) a.rec.x_end[ri] = nd.xf;
+            if (a.rec.y_end) a.rec.y_end[ri] = nd.yf;
+        }
+    }
+    if (lane == 0) {
+        if (o.mean_xi) o.mean_xi[k] = vx;
+        if (o.mean_eta) o.mean_eta[k] = ve;
+        if (o.se_xi) o.se_xi[k] = 0.0;
+        if (o.se_eta) o.se_eta[k] = 0.0;
+        if (o.n_exit) o.n_exit[k] = filled ? 0 : nd.n_paths;
+        if (o.path_steps) o.path_steps[k] = 0;
+    }
+    return true;
+}
+
+// Thread t of T: compensated sums of the node's task partials t, t + T, ...
+__device__ __forceinline__ void task_sums(const FinalArgs& a, const NodeDev& nd, int t, int T, double (&v)[4],
+                                          long long& ex, long long& st)
+{
+    double c[4] = {0, 0, 0, 0};
+    ex = st = 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v[q] = 0.0;
+    for (int k = t; k < nd.ntasks; k += T) {
+        const Partial p = a.partials[nd.task0 + k];
+        const double in[4] = {p.s_xi, p.q_xi, p.s_eta, p.q_eta};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            if (k == t) {
+                v[q] = in[q];
+                continue;
+            }
+            const double y = in[q] - c[q];
+            const double tt = v[q] + y;
+            c[q] = (tt - v[q]) - y;
+            v[q] = tt;
+        }
+        ex += p.exits;
+        st += p.steps;
+    }
+    if (T < nd.ntasks)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) v[q] -= c[q];
+}
+
+// The node's mean and standard error s / sqrt(N), s^2 = (Q - S^2 / N) / (N - 1) of the shifted scores,
+// by one warp with sum lane & 3 in each lane: lane 0 for xi, lane 2 for eta.
+__device__ __forceinline__ void node_outputs(const FinalArgs& a, const NodeDev& nd, int lane, double tot, long long ex,
+                                             long long st)
+{
+    const OutDev o = a.out_table ? a.out_table[nd.inst] : a.out0;
+    const int k = nd.local;
+    const double sq = __shfl_down_sync(FULL, tot, 1);   // lane 0: Q of xi, lane 2: Q of eta
+    if (lane == 0 || lane == 2) {
+        const double N = (double)nd.n_paths;
+        const double m = tot / N;
+        const double var = nd.n_paths > 1 ? fmax(0.0, (sq - tot * m) * reciprocal(N - 1.0)) : 0.0;
+        double* const mean = lane ? o.mean_eta : o.mean_xi;
+        double* const se = lane ? o.se_eta : o.se_xi;
+        if (mean) mean[k] = (double)(lane ? nd.yf : nd.xf) + m;
+        if (se) se[k] = sqrt(var * reciprocal(N));
+    }
+    if (lane == 0) {
+        if (o.n_exit) o.n_exit[k] = ex;
+        if (o.path_steps) o.path_steps[k] = st;
+    }
+}
+
+// What a warp or a block contributes to a node.
+struct NodeSums {
+    double v[4];
+    long long ex, st;
+};
+
+__device__ __forceinline__ void put_sums(NodeSums* p, int lane, double v, long long ex, long long st)
+{
+    if (lane < 4) p->v[lane] = v;
+    if (lane == 0) {
+        p->ex = ex;
+        p->st = st;
+    }
+}
+
+// Sums of n contributions by one warp, in a fixed order: sum lane & 3 in each lane, the counts in all.
+__device__ __forceinline__ double join_sums(const NodeSums* p, int n, int lane, long long& ex, long long& st)
+{
+    double v = 0.0;
+    ex = st = 0;
+    for (int g = lane >> 2; g < n; g += 8) v += p[g].v[lane & 3];
+    for (int off = 4; off < 32 && off < 4 * n; off <<= 1) v += __shfl_xor_sync(FULL, v, off);
+    for (int g = 0; g < n; ++g) {
+        ex += p[g].ex;
+        st += p[g].st;
+    }
+    return v;
+}
+
+constexpr int FINAL_WARPS = 8;
+
+// One node by `warps` warps (a block; one: a warp of a two-warp block). A node's task partials are a
+// chain of loads and of double-precision additions on lanes that hold two of them an SM cycle: one warp a node took
+// 16 us for 253 nodes of 10,000 paths, four take 9.
+__global__ void __launch_bounds__(FINAL_WARPS * 32) k_finalize(const FinalArgs a, int warps)
+{
+    __shared__ NodeSums part[FINAL_WARPS];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int node = warps == 1 ? blockIdx.x * (int)(blockDim.x >> 5) + warp : blockIdx.x;
+    if (node >= a.nnodes) return;
+    const NodeDev nd = a.nodes[node];
+    if (nd.ntasks == 0 || (a.node_mask && !a.node_mask[node])) {
+        if (warps == 1 || warp == 0) pathless_node(a, node, nd, lane);
+        return;   // uniform over the node's warps
+    }
+    double v[4];
+    long long ex, st;
+    task_sums(a, nd, warps == 1 ? lane : (int)threadIdx.x, 32 * warps, v, ex, st);
+    double tot = warp_sum4(v[0], v[1], v[2], v[3]);
+    ex = warp_sum_ll(ex);
+    st = warp_sum_ll(st);
+    if (warps > 1) {
+        put_sums(part + warp, lane, tot, ex, st);
+        __syncthreads();
+        if (warp != 0) return;
+        tot = join_sums(part, warps, lane, ex, st);
+    }
+    node_outputs(a, nd, lane, tot, ex, st);
+}
+
 // Scores of the paths that survived a mesh step, once the fields of the step's
 // start are final (the estimate of the next mesh step runs beside the
-// subdomain solve that produces them). One block per node: the node's paths
-// end in one neighbourhood, so its gathers share L1; thread k takes paths k,
-// k + T, ... SCORE_BATCH at a time (records, then gathers, in flight
+// subdomain solve that produces them), then the node's reduction. A cluster of blocks per node: the node's paths
+// end in one neighbourhood, so a block's gathers share L1; each block takes a run of the paths, thread k of it paths
+// k, k + T, ... SCORE_BATCH at a time (records, then gathers, in flight
 // together) and sums xi and eta at the end points minus the paths'
-// control-variate sums; the block's sums, in warp order, join the partial
-// sums of the node's first task in the node's reduction, which the block's
-// first warp then runs (the mean and standard error of every node, boundary
-// and masked nodes included). The next batch's records are read while the
-// current batch's gathers are in flight. T = 256 threads at 64 registers puts
-// four blocks on an SM (many nodes: one wave for up to four per SM); with no
-// more nodes than SMs, T = 1024 gives each node's paths four times the threads.
+// control-variate sums; task partials are dealt to the cluster's threads. Each block leaves its sums
+// with block 0, whose first warp writes the outputs. The next batch's records are read while the
+// current batch's gathers are in flight. T = 256 threads at 64 registers puts four blocks on an SM; the cluster is
+// the largest that leaves one wave of such blocks: with one block of 1024 threads per node, the 77 nodes of a
+// 41 x 41 grid left half the SMs idle, and the task partials went through one warp: 26.6 us, now 16.9.
 constexpr int SCORE_BATCH = 2;
+constexpr int SCORE_THREADS = 256;
+constexpr int SCORE_MAX_CLUSTER = 8;
 
-__device__ void finalize_node(const FinalArgs& a, int node, int lane, double more);
-
-template <bool CV, int SCORE_THREADS>
-__global__ void __launch_bounds__(SCORE_THREADS, 1024 / SCORE_THREADS) k_score_surv(const ScoreArgs a)
+template <bool CV>
+__global__ void __launch_bounds__(SCORE_THREADS, 4) k_score_surv(const ScoreArgs a)
 {
-    __shared__ double red[SCORE_THREADS / 32][4];
+    __shared__ double task_v[4][SCORE_THREADS];
+    __shared__ long long task_n[2][SCORE_THREADS];
+    __shared__ NodeSums part[SCORE_THREADS / 32], blocks[SCORE_MAX_CLUSTER];
+    cg::cluster_group cl = cg::this_cluster();
+    const int C = (int)cl.num_blocks(), rank = (int)cl.block_rank();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int node = blockIdx.x;
+    const int node = blockIdx.x / C;
     const NodeDev& nd = a.nodes[node];
     if (nd.ntasks == 0 || (a.fin.node_mask && !a.fin.node_mask[node])) {
         // a boundary node or one left to the interface fill: no paths to score
-        if (warp == 0) finalize_node(a.fin, node, lane, 0.0);
-        return;   // uniform over the block
+        if (warp == 0 && rank == 0) pathless_node(a.fin, node, nd, lane);
+        return;   // uniform over the cluster
     }
     const InstDev I = a.inst[nd.inst];
     const float x0 = nd.xf, y0 = nd.yf;
-    const int end = nd.n_paths;
+    const int first = (int)((long long)nd.n_paths * rank / C), end = (int)((long long)nd.n_paths * (rank + 1) / C);
     Acc ax{0.f, 0.f, 0.f, 0.f}, ae{0.f, 0.f, 0.f, 0.f};
     // the records of the batch that starts at path p0 (past the end: the skip mark)
     auto load_batch = [&](int p0, float2 (&r)[SCORE_BATCH], float2 (&cvs)[SCORE_BATCH]) {
@@ -880,8 +1051,18 @@ __global__ void __launch_bounds__(SCORE_THREADS, 1024 / SCORE_THREADS) k_score_s
     };
     float2 r[SCORE_BATCH];
     float2 cvs[SCORE_BATCH];
-    load_batch(threadIdx.x, r, cvs);
-    for (int p0 = threadIdx.x; p0 < end; p0 += SCORE_BATCH * SCORE_THREADS) {
+    load_batch(first + threadIdx.x, r, cvs);
+    {
+        // this thread's share of the task partials, kept in shared memory over the scoring
+        double v[4];
+        long long ex, st;
+        task_sums(a.fin, nd, rank * SCORE_THREADS + threadIdx.x, C * SCORE_THREADS, v, ex, st);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) task_v[q][threadIdx.x] = v[q];
+        task_n[0][threadIdx.x] = ex;
+        task_n[1][threadIdx.x] = st;
+    }
+    for (int p0 = first + threadIdx.x; p0 < end; p0 += SCORE_BATCH * SCORE_THREADS) {
         // one round of loads for the batch: a survivor gathers the field record at its
         // end point, a plain exit the face data on both sides of its crossing
         // (f0 = xi[k], xi[k + 1], eta[k], eta[k + 1]; st.x the fraction)
@@ -932,130 +1113,18 @@ __global__ void __launch_bounds__(SCORE_THREADS, 1024 / SCORE_THREADS) k_score_s
             cvs[u] = cn[u];
         }
     }
-    const double v = warp_sum4(ax.sum(), ax.sumsq(), ae.sum(), ae.sumsq());
-    if (lane < 4) red[warp][lane] = v;
+    double tot = warp_sum4(ax.sum() + task_v[0][threadIdx.x], ax.sumsq() + task_v[1][threadIdx.x],
+                           ae.sum() + task_v[2][threadIdx.x], ae.sumsq() + task_v[3][threadIdx.x]);
+    long long ex = warp_sum_ll(task_n[0][threadIdx.x]), st = warp_sum_ll(task_n[1][threadIdx.x]);
+    put_sums(part + warp, lane, tot, ex, st);
     __syncthreads();
-    if (warp == 0) {
-        // sum lane & 3 over the block's warps, in a fixed order
-        double tot = 0.0;
-        for (int g = lane >> 2; g < SCORE_THREADS / 32; g += 8) tot += red[g][lane & 3];
-#pragma unroll
-        for (int off = 4; off < 32; off <<= 1) tot += __shfl_xor_sync(FULL, tot, off);
-        finalize_node(a.fin, node, lane, tot);   // the node's mean and standard error
+    if (warp == 0) tot = join_sums(part, SCORE_THREADS / 32, lane, ex, st);
+    if (C > 1) {
+        if (warp == 0) put_sums(cl.map_shared_rank(blocks, 0) + rank, lane, tot, ex, st);
+        cl.sync();
+        if (rank == 0 && warp == 0) tot = join_sums(blocks, C, lane, ex, st);
     }
-}
-
-__device__ __forceinline__ double face_value64(const InstDev& I, int field, int face, double s)
-{
-    const int n = (face < 2) ? I.ny : I.nx;
-    long long off = (long long)field * (2LL * I.ny + 2LL * I.nx);
-    if (face >= 1) off += I.ny;
-    if (face >= 2) off += I.ny;
-    if (face >= 3) off += I.nx;
-    const double* v = I.faces64 + off;
-    const double g = s * (double)(n - 1);
-    int k = (int)floor(g);
-    k = max(0, min(k, n - 2));
-    const double f = g - (double)k;
-    return (1.0 - f) * v[k] + f * v[k + 1];
-}
-
-// One warp per node: compensated sums of the node's task partials (each lane a
-// fixed stride of tasks), a fixed butterfly across the warp that leaves sum
-// lane & 3 in each lane (`more` joins it there), then the mean and the standard error
-// s / sqrt(N), s^2 = (Q - S^2 / N) / (N - 1) of the shifted scores: lane 0 for
-// xi, lane 2 for eta.
-__device__ void finalize_node(const FinalArgs& a, int node, int lane, double more)
-{
-    const NodeDev nd = a.nodes[node];
-    const OutDev o = a.out_table ? a.out_table[nd.inst] : a.out0;
-    const int k = nd.local;
-    if (a.node_mask && !a.node_mask[node]) {
-        // not estimated this step: no paths; the interface fill writes its value
-        if (lane == 0) {
-            if (o.mean_xi) o.mean_xi[k] = 0.0;
-            if (o.mean_eta) o.mean_eta[k] = 0.0;
-            if (o.se_xi) o.se_xi[k] = 0.0;
-            if (o.se_eta) o.se_eta[k] = 0.0;
-            if (o.n_exit) o.n_exit[k] = 0;
-            if (o.path_steps) o.path_steps[k] = 0;
-        }
-        return;
-    }
-    if (nd.ntasks == 0) {
-        // a node on the boundary: its Dirichlet value, every path exits at time 0
-        const InstDev I = a.inst[nd.inst];
-        int face;
-        double tg;
-        if (nd.x <= 0.0) { face = 0; tg = nd.y; }
-        else if (nd.x >= 1.0) { face = 1; tg = nd.y; }
-        else if (nd.y <= 0.0) { face = 2; tg = nd.x; }
-        else { face = 3; tg = nd.x; }
-        const double vx = face_value64(I, 0, face, tg), ve = face_value64(I, 1, face, tg);
-        if (lane == 0) {
-            if (o.mean_xi) o.mean_xi[k] = vx;
-            if (o.mean_eta) o.mean_eta[k] = ve;
-            if (o.se_xi) o.se_xi[k] = 0.0;
-            if (o.se_eta) o.se_eta[k] = 0.0;
-            if (o.n_exit) o.n_exit[k] = nd.n_paths;
-            if (o.path_steps) o.path_steps[k] = 0;
-        }
-        for (int p = lane; p < nd.n_paths; p += 32) {
-            const long long ri = nd.rec0 + p;
-            if (a.rec.steps) a.rec.steps[ri] = 0;
-            if (a.rec.code) a.rec.code[ri] = face;
-            if (a.rec.score_xi) a.rec.score_xi[ri] = (float)vx;
-            if (a.rec.score_eta) a.rec.score_eta[ri] = (float)ve;
-            if (a.rec.x_end) a.rec.x_end[ri] = nd.xf;
-            if (a.rec.y_end) a.rec.y_end[ri] = nd.yf;
-        }
-        return;
-    }
-    double v[4] = {0, 0, 0, 0}, c[4] = {0, 0, 0, 0};
-    long long ex = 0, st = 0;
-    for (int t = nd.task0 + lane; t < nd.task0 + nd.ntasks; t += 32) {
-        const Partial p = a.partials[t];
-        const double in[4] = {p.s_xi, p.q_xi, p.s_eta, p.q_eta};
-        const bool first = t < nd.task0 + 32;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            if (first) {
-                v[q] = in[q];
-                continue;
-            }
-            const double y = in[q] - c[q];
-            const double tt = v[q] + y;
-            c[q] = (tt - v[q]) - y;
-            v[q] = tt;
-        }
-        ex += p.exits;
-        st += p.steps;
-    }
-    const double tot = warp_sum4(v[0] - c[0], v[1] - c[1], v[2] - c[2], v[3] - c[3]) + more;
-    const double sq = __shfl_down_sync(FULL, tot, 1);   // lane 0: Q of xi, lane 2: Q of eta
-    ex = warp_sum_ll(ex);
-    st = warp_sum_ll(st);
-    if (lane == 0 || lane == 2) {
-        const double N = (double)nd.n_paths;
-        const double m = tot / N;
-        const double var = nd.n_paths > 1 ? fmax(0.0, (sq - tot * m) / (N - 1.0)) : 0.0;
-        double* const mean = lane ? o.mean_eta : o.mean_xi;
-        double* const se = lane ? o.se_eta : o.se_xi;
-        if (mean) mean[k] = (double)(lane ? nd.yf : nd.xf) + m;
-        if (se) se[k] = sqrt(var / N);
-    }
-    if (lane == 0) {
-        if (o.n_exit) o.n_exit[k] = ex;
-        if (o.path_steps) o.path_steps[k] = st;
-    }
-}
-
-__global__ void k_finalize(const FinalArgs a)
-{
-    const int node = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5);
-    const int lane = threadIdx.x & 31;
-    if (node >= a.nnodes) return;
-    finalize_node(a, node, lane, 0.0);
+    if (rank == 0 && warp == 0) node_outputs(a.fin, nd, lane, tot, ex, st);
 }
 
 __global__ void k_rng_draw(uint64_t seed, const uint32_t* __restrict__ ctrs, long long count,
@@ -1150,22 +1219,31 @@ cudaError_t launch_score_surv(const ScoreArgs& a, bool cv, cudaStream_t s)
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (a.nnodes <= sms) {
-        if (cv) k_score_surv<true, 1024><<<a.nnodes, 1024, 0, s>>>(a);
-        else k_score_surv<false, 1024><<<a.nnodes, 1024, 0, s>>>(a);
-    } else {
-        if (cv) k_score_surv<true, 256><<<a.nnodes, 256, 0, s>>>(a);
-        else k_score_surv<false, 256><<<a.nnodes, 256, 0, s>>>(a);
-    }
-    return cudaGetLastError();
+    int C = SCORE_MAX_CLUSTER;
+    while (C > 1 && (long long)a.nnodes * C > 4LL * sms) C >>= 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(a.nnodes * C));
+    cfg.blockDim = dim3(SCORE_THREADS);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)C;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cv ? cudaLaunchKernelEx(&cfg, k_score_surv<true>, a) : cudaLaunchKernelEx(&cfg, k_score_surv<false>, a);
 }
 
-cudaError_t launch_finalize(const FinalArgs& a, cudaStream_t s)
+cudaError_t launch_finalize(const FinalArgs& a, long long ntasks, cudaStream_t s)
 {
-    const int block = 64;   // few nodes per block: their double-precision sums spread over the SMs
-    const long long threads = (long long)a.nnodes * 32;
-    const int grid = (int)((threads + block - 1) / block);
-    if (grid > 0) k_finalize<<<grid, block, 0, s>>>(a);
+    if (a.nnodes <= 0) return cudaSuccess;
+    // two of a node's task partials per thread on average
+    int warps = 1;
+    while (warps < FINAL_WARPS && 64LL * warps * a.nnodes < ntasks) warps *= 2;
+    // blocks of a few warps: their double-precision sums spread over the SMs
+    const int per_block = warps == 1 ? 2 : 1;
+    k_finalize<<<(unsigned)((a.nnodes + per_block - 1) / per_block), 32 * std::max(2, warps), 0, s>>>(a, warps);
     return cudaGetLastError();
 }
 

@@ -255,7 +255,7 @@ sdd_status sdd_interface_mc_static(const sdd_fields* f, const sdd_nodes* nodes, 
         fa.out0.n_exit = (long long*)out->n_exit;
         fa.out0.path_steps = (long long*)out->path_steps;
         fa.nnodes = (int32_t)count;
-        STATIC_CU(launch_finalize(fa, s));
+        STATIC_CU(launch_finalize(fa, (long long)t, s));
     }
     // the call's device status: into the caller's word, or read here after the stream's work
     if (status_out) {
