@@ -319,21 +319,25 @@ sdd_status upload_inst(sdd_ctx* c)
 
 int64_t faces_len(const sdd_ctx* c) { return 2LL * (2LL * c->nx + 2LL * c->ny); }
 
-// Field tables for the current w, fields and face data (enqueued on s).
-// The tables of the current w (faces, drift records) and fields (field
-// records) on stream s, where they changed since they were last built.
-sdd_status prepare_parts(sdd_ctx* c, cudaStream_t s, bool w_part, bool f_part)
+// What building the tables of the current w (faces, drift records) and fields (field records) takes, where they
+// changed since they were last built; they count as built.
+PrepItem take_dirty(sdd_ctx* c, bool w_part, bool f_part)
 {
-    const bool dw = w_part && c->dirty_w, df = f_part && c->dirty_fields;
-    if (dw && !c->user_faces) {
-        CU(c, launch_winslow_faces(c->w.p, c->nx, c->ny, c->faces64.p, c->faces32.p, s));
-    }
-    if (dw || df) {
-        CU(c, launch_prep_cells(c->w.p, c->fld[c->cur][0].p, c->fld[c->cur][1].p, c->nx, c->ny,
-                                dw ? c->bcoef.p : nullptr, df ? c->fcoef.p : nullptr, c->d_status.p, s, c->zmap.p));
-    }
+    const bool dw = w_part && c->dirty_w, df = f_part && c->dirty_fields, faces = dw && !c->user_faces;
     if (w_part) c->dirty_w = c->dirty_faces = false;
     if (f_part) c->dirty_fields = false;
+    return PrepItem{c->w.p, c->fld[c->cur][0].p, c->fld[c->cur][1].p, dw ? c->bcoef.p : nullptr,
+                    df ? c->fcoef.p : nullptr, faces ? c->faces64.p : nullptr, c->faces32.p, c->zmap.p, c->d_status.p,
+                    c->nx, c->ny};
+}
+
+sdd_status prepare_parts(sdd_ctx* c, cudaStream_t s, bool w_part, bool f_part)
+{
+    const PrepItem it = take_dirty(c, w_part, f_part);
+    if (!it.bcoef && !it.fcoef) return SDD_OK;
+    const cudaError_t e = launch_prep(&it, 1, s);
+    if (e != cudaSuccess) c->dirty_w = c->dirty_faces = c->dirty_fields = true;
+    CU(c, e);
     return SDD_OK;
 }
 
@@ -346,19 +350,21 @@ sdd_status prepare_faces(sdd_ctx* c, cudaStream_t s)
     return SDD_OK;
 }
 
-sdd_status prepare(sdd_ctx* c, cudaStream_t s)
+sdd_status prepare(sdd_ctx* c, cudaStream_t s) { return prepare_parts(c, s, true, true); }
+
+// The tables of several instances.
+sdd_status prepare_all(std::string* err, const std::vector<sdd_ctx*>& ctxs, cudaStream_t s)
 {
-    if (c->dirty_w && c->dirty_fields) {
-        // both record sets in one pass
-        if (!c->user_faces) {
-            CU(c, launch_winslow_faces(c->w.p, c->nx, c->ny, c->faces64.p, c->faces32.p, s));
-        }
-        CU(c, launch_prep_cells(c->w.p, c->fld[c->cur][0].p, c->fld[c->cur][1].p, c->nx, c->ny, c->bcoef.p,
-                                c->fcoef.p, c->d_status.p, s, c->zmap.p));
-        c->dirty_w = c->dirty_faces = c->dirty_fields = false;
-        return SDD_OK;
+    std::vector<PrepItem> items;
+    for (sdd_ctx* c : ctxs) {
+        const PrepItem it = take_dirty(c, true, true);
+        if (it.bcoef || it.fcoef) items.push_back(it);
     }
-    return prepare_parts(c, s, true, true);
+    const cudaError_t e = launch_prep(items.data(), (int)items.size(), s);
+    if (e != cudaSuccess)
+        for (sdd_ctx* c : ctxs) c->dirty_w = c->dirty_faces = c->dirty_fields = true;
+    CU(err, e);
+    return SDD_OK;
 }
 
 bool valid_params(sdd_ctx* c, double dt, double Dt, int exit_mode, int* K)
@@ -2091,8 +2097,9 @@ static sdd_status capture_step(sdd_ctx* c, const sdd_step_params* p, int K, int 
     }
     if (st == SDD_OK && c->pipe) {
         // the drift records; the face data come from the third branch forked above
-        cu(launch_prep_cells(c->w.p, nullptr, nullptr, c->nx, c->ny, c->bcoef.p, nullptr, c->d_status.p, s,
-                             c->zmap.p));
+        PrepItem it = take_dirty(c, true, false);
+        it.faces64 = nullptr;
+        cu(launch_prep(&it, 1, s));
         if (!c->user_faces && p->exit_mode != 0) cu(cudaStreamWaitEvent(s, c->fev[1], 0));
         c->dirty_w = false;
     } else if (st == SDD_OK) {
@@ -2406,12 +2413,8 @@ sdd_status capture_batch_step(sdd_batch* b, const sdd_step_params* p, int K, int
         if (e != cudaSuccess) st = fail(&b->err, SDD_ECUDA, "event: %s", cudaGetErrorString(e));
     };
     rec_ev(0);
-    for (sdd_ctx* c : b->ctxs) {
-        if (st != SDD_OK) break;
-        c->dirty_w = c->dirty_fields = true;
-        st = prepare(c, s);
-        if (st != SDD_OK) b->err = c->err;
-    }
+    for (sdd_ctx* c : b->ctxs) c->dirty_w = c->dirty_fields = true;
+    if (st == SDD_OK) st = prepare_all(&b->err, b->ctxs, s);
     if (st == SDD_OK)
         st = run_plan_on(&b->err, b->step_plan, b->d_inst.p, b->d_step_out.p, OutDev{}, p->dt, K, p->seed, 0,
                          b->d_step.p, p->exit_mode, nullptr, s, b->ev[1], b->ev[2]);
@@ -2556,8 +2559,7 @@ sdd_status sdd_batch_interface_mc(sdd_batch* b, const sdd_nodes* nodes, const sd
     pick_shape(b->tuned, segs, K, p->exit_mode, &ppt, &block);
     sdd_status st = build_plan_segs(&b->err, b->sm_count, b->mc_plan, segs, ppt, block, p->exit_mode, false);
     if (st != SDD_OK) return st;
-    for (sdd_ctx* c : b->ctxs)
-        if ((st = prepare(c, b->stream)) != SDD_OK) return fail(&b->err, st, "%s", c->err.c_str());
+    if ((st = prepare_all(&b->err, b->ctxs, b->stream)) != SDD_OK) return st;
     std::vector<OutDev> outs(n);
     for (int32_t k = 0; k < n; ++k) outs[k] = out_from(&out[k]);
     CU(&b->err, cudaMemcpyAsync(b->d_out.p, outs.data(), n * sizeof(OutDev), cudaMemcpyHostToDevice, b->stream));
@@ -2647,12 +2649,10 @@ sdd_status sdd_batch_autotune(sdd_batch* b, const sdd_nodes* nodes, const sdd_mc
         segs[k] = NodeSeg{nodes[k].x, nodes[k].y, nodes[k].n_paths, nodes[k].count, k, ctr};
         ctr += (uint32_t)nodes[k].count;
     }
-    for (sdd_ctx* c : b->ctxs) {
-        sdd_status st = prepare(c, b->stream);
-        if (st != SDD_OK) return fail(&b->err, st, "%s", c->err.c_str());
-    }
+    sdd_status st = prepare_all(&b->err, b->ctxs, b->stream);
+    if (st != SDD_OK) return st;
     TunedShape best{};
-    sdd_status st = autotune_plan(&b->err, b->sm_count, segs, b->d_inst.p, n, K, p->dt, p->exit_mode, b->stream,
+    st = autotune_plan(&b->err, b->sm_count, segs, b->d_inst.p, n, K, p->dt, p->exit_mode, b->stream,
                                   b->tuned, &best);
     if (st != SDD_OK) return st;
     if (out) {

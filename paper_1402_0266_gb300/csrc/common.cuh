@@ -182,11 +182,20 @@ int path_kernel_blocks_per_sm(int exit_mode, bool record, int block, int cvm = 0
 // the largest block the path kernel of this exit mode is compiled for (single: one instance)
 int path_kernel_max_block(int exit_mode, int cvm = 0, bool single = false);
 
-// Cell records of the drift (from w; bcoef null: skipped) and of the fields
-// (from xi, eta; fcoef null: skipped); with the drift records, if zmap is
-// non-null, their zero map (kZmapBytes bytes).
-cudaError_t launch_prep_cells(const float* w, const double* xi, const double* eta, int nx, int ny, float4* bcoef,
-                              float4* fcoef, int* status, cudaStream_t s, uint8_t* zmap = nullptr);
+// The tables of a grid to build: cell records of the drift (from w; bcoef null: skipped) and of the fields
+// (from xi, eta; fcoef null: skipped), the paper's boundary data (faces64 and its single-precision copy;
+// faces64 null: skipped); with the drift records, if zmap is non-null, their zero map (kZmapBytes bytes).
+struct PrepItem {
+    const float* w;
+    const double *xi, *eta;
+    float4 *bcoef, *fcoef;
+    double* faces64;
+    float* faces32;
+    uint8_t* zmap;
+    int* status;
+    int32_t nx, ny;
+};
+cudaError_t launch_prep(const PrepItem* items, int n, cudaStream_t s);
 // The paper's boundary data from w (faces64) and, if faces32 is non-null, its single-precision copy.
 cudaError_t launch_winslow_faces(const float* w, int nx, int ny, double* faces64, float* faces32, cudaStream_t s);
 cudaError_t launch_cv_cells(const double* grad, int slices, int nx, int ny, uint4* cvcoef, cudaStream_t s);

@@ -14,6 +14,8 @@
 //    int_0^s w / int_0^1 w (cumulative trapezoid, double precision).
 #include <cuda_fp16.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace sdd {
@@ -55,21 +57,129 @@ __device__ __forceinline__ void bilinear_coefs2(double u00, double u10, double u
                      (float)((v11 - v10) - (v01 - v00)));
 }
 
-// One block per 32 x TY cells: the drift at the tile's 33 x (TY + 1) nodes once (in
+// Face data of one line of w: the cumulative trapezoid over its total, by one block: each thread sums a
+// contiguous run of intervals, the run totals are scanned over the block, then each thread writes its run.
+// (By one warp per line a 2049^2 grid's faces took 280 us, 64 dependent loads a thread.)
+constexpr int FACE_THREADS = 256;
+constexpr int FACE_BLOCKS = 5;   // blocks a grid's faces take
+
+template <int T>
+__device__ void block_cumtrapz(const float* __restrict__ v, long long stride, int n, double* __restrict__ out,
+                               float* __restrict__ out32)
+{
+    __shared__ double part[T / 32];
+    const int t = threadIdx.y * blockDim.x + threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int run = (n - 1 + T - 1) / T;
+    const int k0 = min(1 + t * run, n), k1 = min(k0 + run, n);
+    double mine = 0.0;
+    for (int k = k0; k < k1; ++k) mine += 0.5 * ((double)v[(k - 1) * stride] + (double)v[k * stride]);
+    double incl = mine;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const double o = __shfl_up_sync(0xffffffffu, incl, off);
+        if (lane >= off) incl += o;
+    }
+    if (lane == 31) part[warp] = incl;
+    __syncthreads();
+    double acc = incl - mine, total = 0.0;
+    for (int q = 0; q < T / 32; ++q) {
+        if (q < warp) acc += part[q];
+        total += part[q];
+    }
+    if (t == 0) {
+        out[0] = 0.0;
+        if (out32) out32[0] = 0.f;
+    }
+    for (int k = k0; k < k1; ++k) {
+        acc += 0.5 * ((double)v[(k - 1) * stride] + (double)v[k * stride]);
+        const double f = acc / total;
+        out[k] = f;
+        if (out32) out32[k] = (float)f;
+    }
+}
+
+// Part b of a grid's faces by a block of T threads. 0, 1: xi on y = 0, 1; 2, 3: eta on x = 0, 1; 4: xi on x = 0, 1
+// and eta on y = 0, 1 (0 and 1).
+template <int T>
+__device__ void face_block(int b, const float* __restrict__ w, int nx, int ny, double* __restrict__ faces,
+                           float* __restrict__ faces32)
+{
+    const long long per_field = 2LL * ny + 2LL * nx;
+    // line q of a field: left, right (ny), bottom, top (nx)
+    auto line = [&](int field, int q) { return field * per_field + (q < 2 ? q * (long long)ny : 2LL * ny + (q - 2) * (long long)nx); };
+    if (b < 4) {
+        const long long at = b < 2 ? line(0, 2 + b) : line(1, b - 2);
+        const float* v = b == 0 ? w : b == 1 ? w + (long long)(ny - 1) * nx : b == 2 ? w : w + (nx - 1);
+        block_cumtrapz<T>(v, b < 2 ? 1 : nx, b < 2 ? nx : ny, faces + at, faces32 ? faces32 + at : nullptr);
+        return;
+    }
+    for (int q = 0; q < 4; ++q) {
+        const long long at = q < 2 ? line(0, q) : line(1, q);
+        const int n = q < 2 ? ny : nx;
+        const double f = q & 1 ? 1.0 : 0.0;
+        for (int k = threadIdx.y * blockDim.x + threadIdx.x; k < n; k += T) {
+            faces[at + k] = f;
+            if (faces32) faces32[at + k] = (float)f;
+        }
+    }
+}
+
+__global__ void __launch_bounds__(FACE_THREADS) k_winslow_faces(const float* __restrict__ w, int nx, int ny,
+                                                                double* __restrict__ faces,
+                                                                float* __restrict__ faces32)
+{
+    face_block<FACE_THREADS>(blockIdx.x, w, nx, ny, faces, faces32);
+}
+
+// The tables of one to N grids in one launch. Per grid five blocks for its faces where they are wanted, then
+// one block per 32 x TY cells: the drift at the tile's 33 x (TY + 1) nodes once (in
 // shared memory, double precision), then each cell's records. TY is 8, or 2 where blocks of 8 rows
 // would not give every SM four of them: the kernel is bound by the double-precision lanes of the SMs in use.
+// A small grid's faces and cells take 5 and 7 us by themselves, latency for the most part: with a launch for
+// each, 16 grids of 65^2 to 513^2 spent 250 of the 1650 us of a batch's estimate on them; now it takes 1444.
 constexpr int PREP_TX = 32;
+constexpr int PREP_MANY = 16;
 
-template <int PREP_TY>
-__global__ void __launch_bounds__(PREP_TX * PREP_TY) k_prep_cells(const float* __restrict__ w,
-                                                                  const double* __restrict__ xi,
-                                                                  const double* __restrict__ eta, int nx, int ny,
-                                                                  float4* __restrict__ bcoef,
-                                                                  float4* __restrict__ fcoef, int* status,
-                                                                  uint8_t* __restrict__ zmap)
+template <int N>
+struct PrepArgs {
+    PrepItem it[N];
+    int32_t block0[N];   // first block of each
+    int32_t n;
+};
+
+// The zero maps of several grids, cleared before their cells mark them.
+__global__ void k_clear_zmaps(const __grid_constant__ PrepArgs<PREP_MANY> a)
+{
+    uint8_t* z = a.it[blockIdx.x].zmap;
+    if (!z || !a.it[blockIdx.x].bcoef) return;
+    for (int k = threadIdx.x; k < kZmapBytes / 4; k += blockDim.x) reinterpret_cast<uint32_t*>(z)[k] = 0u;
+}
+
+template <int PREP_TY, int N>
+__global__ void __launch_bounds__(PREP_TX * PREP_TY) k_prep_cells(const __grid_constant__ PrepArgs<N> a)
 {
     __shared__ double2 bn[PREP_TY + 1][PREP_TX + 1];
-    const int ix0 = blockIdx.x * PREP_TX, iy0 = blockIdx.y * PREP_TY;
+    int g = 0;
+    while (N > 1 && g + 1 < a.n && (int)blockIdx.x >= a.block0[g + 1]) ++g;
+    const PrepItem& I = a.it[g];
+    const float* __restrict__ w = I.w;
+    const double* __restrict__ xi = I.xi;
+    const double* __restrict__ eta = I.eta;
+    float4* __restrict__ bcoef = I.bcoef;
+    float4* __restrict__ fcoef = I.fcoef;
+    uint8_t* __restrict__ zmap = I.zmap;
+    int* status = I.status;
+    const int nx = I.nx, ny = I.ny;
+    int b = (int)blockIdx.x - a.block0[g];
+    if (I.faces64) {
+        if (b < FACE_BLOCKS) {
+            face_block<PREP_TX * PREP_TY>(b, w, nx, ny, I.faces64, I.faces32);
+            return;
+        }
+        b -= FACE_BLOCKS;
+    }
+    const int tiles = (nx - 1 + PREP_TX - 1) / PREP_TX;
+    const int ix0 = b % tiles * PREP_TX, iy0 = b / tiles * PREP_TY;
     const int ix = ix0 + threadIdx.x, iy = iy0 + threadIdx.y;
     const bool cell_in = ix < nx - 1 && iy < ny - 1;
     if (bcoef) {
@@ -151,71 +261,6 @@ __global__ void k_cv_cells(const double* __restrict__ g, int slices, int nx, int
     cv[2 * cell + 1] = make_uint4(w[4], w[5], w[6], w[7]);
 }
 
-// Face data of one line of w: the cumulative trapezoid over its total, by one block: each thread sums a
-// contiguous run of intervals, the run totals are scanned over the block, then each thread writes its run.
-// (By one warp per line a 2049^2 grid's faces took 280 us, 64 dependent loads a thread.)
-constexpr int FACE_THREADS = 256;
-
-__device__ void block_cumtrapz(const float* __restrict__ v, long long stride, int n, double* __restrict__ out,
-                               float* __restrict__ out32)
-{
-    __shared__ double part[FACE_THREADS / 32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int run = (n - 1 + FACE_THREADS - 1) / FACE_THREADS;
-    const int k0 = min(1 + (int)threadIdx.x * run, n), k1 = min(k0 + run, n);
-    double mine = 0.0;
-    for (int k = k0; k < k1; ++k) mine += 0.5 * ((double)v[(k - 1) * stride] + (double)v[k * stride]);
-    double incl = mine;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        const double o = __shfl_up_sync(0xffffffffu, incl, off);
-        if (lane >= off) incl += o;
-    }
-    if (lane == 31) part[warp] = incl;
-    __syncthreads();
-    double acc = incl - mine, total = 0.0;
-    for (int q = 0; q < FACE_THREADS / 32; ++q) {
-        if (q < warp) acc += part[q];
-        total += part[q];
-    }
-    if (threadIdx.x == 0) {
-        out[0] = 0.0;
-        if (out32) out32[0] = 0.f;
-    }
-    for (int k = k0; k < k1; ++k) {
-        acc += 0.5 * ((double)v[(k - 1) * stride] + (double)v[k * stride]);
-        const double f = acc / total;
-        out[k] = f;
-        if (out32) out32[k] = (float)f;
-    }
-}
-
-// Block 0, 1: xi on y = 0, 1; 2, 3: eta on x = 0, 1; 4: xi on x = 0, 1 and eta on y = 0, 1 (0 and 1).
-__global__ void __launch_bounds__(FACE_THREADS) k_winslow_faces(const float* __restrict__ w, int nx, int ny,
-                                                                double* __restrict__ faces,
-                                                                float* __restrict__ faces32)
-{
-    const long long per_field = 2LL * ny + 2LL * nx;
-    // line q of a field: left, right (ny), bottom, top (nx)
-    auto line = [&](int field, int q) { return field * per_field + (q < 2 ? q * (long long)ny : 2LL * ny + (q - 2) * (long long)nx); };
-    const int b = blockIdx.x;
-    if (b < 4) {
-        const long long at = b < 2 ? line(0, 2 + b) : line(1, b - 2);
-        const float* v = b == 0 ? w : b == 1 ? w + (long long)(ny - 1) * nx : b == 2 ? w : w + (nx - 1);
-        block_cumtrapz(v, b < 2 ? 1 : nx, b < 2 ? nx : ny, faces + at, faces32 ? faces32 + at : nullptr);
-        return;
-    }
-    for (int q = 0; q < 4; ++q) {
-        const long long at = q < 2 ? line(0, q) : line(1, q);
-        const int n = q < 2 ? ny : nx;
-        const double f = q & 1 ? 1.0 : 0.0;
-        for (int k = threadIdx.x; k < n; k += blockDim.x) {
-            faces[at + k] = f;
-            if (faces32) faces32[at + k] = (float)f;
-        }
-    }
-}
-
 __global__ void k_faces32(const double* __restrict__ f64, float* __restrict__ f32, int n)
 {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
@@ -224,19 +269,45 @@ __global__ void k_faces32(const double* __restrict__ f64, float* __restrict__ f3
 
 }  // namespace
 
-cudaError_t launch_prep_cells(const float* w, const double* xi, const double* eta, int nx, int ny, float4* bcoef,
-                              float4* fcoef, int* status, cudaStream_t s, uint8_t* zmap)
+template <int TY, int N>
+static cudaError_t launch_prep_n(const PrepItem* items, int n, cudaStream_t s)
 {
-    const unsigned tiles = (unsigned)(nx - 1 + PREP_TX - 1) / PREP_TX;
-    if (bcoef && zmap) {
-        const cudaError_t e = cudaMemsetAsync(zmap, 0, kZmapBytes, s);
+    PrepArgs<N> a;
+    a.n = n;
+    long long blocks = 0;
+    for (int k = 0; k < n; ++k) {
+        a.it[k] = items[k];
+        a.block0[k] = (int32_t)blocks;
+        blocks += (items[k].faces64 ? FACE_BLOCKS : 0);
+        if (items[k].bcoef || items[k].fcoef)
+            blocks += (long long)((items[k].nx - 1 + PREP_TX - 1) / PREP_TX) * ((items[k].ny - 1 + TY - 1) / TY);
+    }
+    if constexpr (N == 1) {
+        if (items[0].bcoef && items[0].zmap) {
+            const cudaError_t e = cudaMemsetAsync(items[0].zmap, 0, kZmapBytes, s);
+            if (e != cudaSuccess) return e;
+        }
+    } else {
+        k_clear_zmaps<<<n, 256, 0, s>>>(a);
+    }
+    if (blocks > 0) k_prep_cells<TY, N><<<(unsigned)blocks, dim3(PREP_TX, TY), 0, s>>>(a);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_prep(const PrepItem* items, int n, cudaStream_t s)
+{
+    for (int k0 = 0; k0 < n; k0 += PREP_MANY) {
+        const int m = std::min(n - k0, PREP_MANY);
+        long long blocks8 = 0;
+        for (int k = k0; k < k0 + m; ++k)
+            blocks8 += (long long)((items[k].nx - 1 + PREP_TX - 1) / PREP_TX) * ((items[k].ny - 1 + 7) / 8);
+        const bool tall = blocks8 >= 4 * 152;
+        const PrepItem* q = items + k0;
+        const cudaError_t e = m == 1 ? (tall ? launch_prep_n<8, 1>(q, m, s) : launch_prep_n<2, 1>(q, m, s))
+                                     : (tall ? launch_prep_n<8, PREP_MANY>(q, m, s) : launch_prep_n<2, PREP_MANY>(q, m, s));
         if (e != cudaSuccess) return e;
     }
-    if ((long long)tiles * ((ny - 1 + 7) / 8) >= 4 * 152)
-        k_prep_cells<8><<<dim3(tiles, (ny - 1 + 7) / 8), dim3(PREP_TX, 8), 0, s>>>(w, xi, eta, nx, ny, bcoef, fcoef, status, zmap);
-    else
-        k_prep_cells<2><<<dim3(tiles, (ny - 1 + 1) / 2), dim3(PREP_TX, 2), 0, s>>>(w, xi, eta, nx, ny, bcoef, fcoef, status, zmap);
-    return cudaGetLastError();
+    return cudaSuccess;
 }
 
 cudaError_t launch_cv_cells(const double* grad, int slices, int nx, int ny, uint4* cvcoef, cudaStream_t s)
@@ -249,7 +320,7 @@ cudaError_t launch_cv_cells(const double* grad, int slices, int nx, int ny, uint
 
 cudaError_t launch_winslow_faces(const float* w, int nx, int ny, double* faces64, float* faces32, cudaStream_t s)
 {
-    k_winslow_faces<<<5, FACE_THREADS, 0, s>>>(w, nx, ny, faces64, faces32);
+    k_winslow_faces<<<FACE_BLOCKS, FACE_THREADS, 0, s>>>(w, nx, ny, faces64, faces32);
     return cudaGetLastError();
 }
 
