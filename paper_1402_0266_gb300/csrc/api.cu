@@ -697,6 +697,7 @@ sdd_status run_plan_on(std::string* err, Plan& P, const InstDev* inst, const Out
         a.dt = (float)dt;
         a.bm_scale = (float)(-4.0 * dt * std::log(2.0));
         a.bridge_cut = (float)(18.0 * dt);
+        a.inv_dt = 1.0f / a.dt;
         a.horizon = (float)((double)K * dt);
         a.keys = philox_keys(seed);
         a.step_index = step_index;

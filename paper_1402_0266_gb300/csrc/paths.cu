@@ -166,28 +166,14 @@ __device__ __forceinline__ void exit_crossing(float x, float y, float xn, float 
     face = f;
 }
 
-// Exit through the boundary between X_j and X_{j+1}: the boundary data at the crossing.
-__device__ __forceinline__ void plain_exit(const InstDev& I, float x, float y, float xn, float yn, int& face,
-                                        float& yxi, float& yeta, float& xe, float& ye)
-{
-    float t;
-    exit_crossing(x, y, xn, yn, face, t);
-    yxi = face_value(I, 0, face, t);
-    yeta = face_value(I, 1, face, t);
-    xe = (face == 0) ? 0.0f : (face == 1) ? 1.0f : t;
-    ye = (face == 2) ? 0.0f : (face == 3) ? 1.0f : t;
-}
-
 // Brownian-bridge test between two inside points: the half plane behind face
 // k is touched with probability exp(-d0 d1 / dt) (sigma^2 = 2); the faces
 // combine as 1 - prod (1 - p_k). On exit: the face of largest p_k, at the
-// projection of the sub-step midpoint.
-__device__ __forceinline__ bool bridge_exit(const InstDev& I, float x, float y, float xn, float yn, float dt, float u,
-                                         int& face, float& yxi, float& yeta, float& xe, float& ye)
+// projection t of the sub-step midpoint. inv: 1 / dt.
+__device__ __forceinline__ bool bridge_test(float x, float y, float xn, float yn, float inv, float u, int& face, float& t)
 {
     const float d0[4] = {x, 1.0f - x, y, 1.0f - y};
     const float d1[4] = {xn, 1.0f - xn, yn, 1.0f - yn};
-    const float inv = 1.0f / dt;
     float stay = 1.0f, pmax = -1.0f;
     int f = 0;
 #pragma unroll
@@ -197,14 +183,35 @@ __device__ __forceinline__ bool bridge_exit(const InstDev& I, float x, float y, 
         if (p > pmax) { pmax = p; f = k; }
     }
     if (!(u < 1.0f - stay)) return false;
-    float t = (f < 2) ? 0.5f * (y + yn) : 0.5f * (x + xn);
+    t = (f < 2) ? 0.5f * (y + yn) : 0.5f * (x + xn);
     t = fminf(fmaxf(t, 0.0f), 1.0f);
     face = f;
-    yxi = face_value(I, 0, f, t);
-    yeta = face_value(I, 1, f, t);
-    xe = (f == 0) ? 0.0f : (f == 1) ? 1.0f : t;
-    ye = (f == 2) ? 0.0f : (f == 3) ? 1.0f : t;
     return true;
+}
+
+// Distance of a point inside the square to the nearest face.
+__device__ __forceinline__ float face_distance(float2 p)
+{
+    return fminf(fminf(p.x, 1.0f - p.x), fminf(p.y, 1.0f - p.y));
+}
+
+// The boundary data at tangential coordinate t of a face, and the point.
+__device__ __forceinline__ void face_point(const InstDev& I, int face, float t, float& yxi, float& yeta, float& xe,
+                                           float& ye)
+{
+    yxi = face_value(I, 0, face, t);
+    yeta = face_value(I, 1, face, t);
+    xe = (face == 0) ? 0.0f : (face == 1) ? 1.0f : t;
+    ye = (face == 2) ? 0.0f : (face == 3) ? 1.0f : t;
+}
+
+// Exit through the boundary between X_j and X_{j+1}: the boundary data at the crossing.
+__device__ __forceinline__ void plain_exit(const InstDev& I, float x, float y, float xn, float yn, int& face,
+                                        float& yxi, float& yeta, float& xe, float& ye)
+{
+    float t;
+    exit_crossing(x, y, xn, yn, face, t);
+    face_point(I, face, t, yxi, yeta, xe, ye);
 }
 
 // 32 bytes through the non-coherent path as eight words.
@@ -439,6 +446,36 @@ struct LaneSums {
     }
 };
 
+// How a lane's path left, until the warp scores it: the sub-step's two ends (a bridge exit: the second holds
+// the tangential coordinate), sub-steps taken and face, the control-variate sums.
+template <int BLOCK, bool CV>
+struct LaneExits {
+    float2 p0[BLOCK], p1[BLOCK];
+    int info[BLOCK];
+    float cv[CV ? 2 : 1][CV ? BLOCK : 1];
+
+    __device__ __forceinline__ void put(float2 a, float2 b, int i, float cxi, float ceta)
+    {
+        p0[threadIdx.x] = a;
+        p1[threadIdx.x] = b;
+        info[threadIdx.x] = i;
+        if (CV) {
+            cv[0][threadIdx.x] = cxi;
+            cv[CV ? 1 : 0][threadIdx.x] = ceta;
+        }
+    }
+    __device__ __forceinline__ void get(float2& a, float2& b, int& i, float& cxi, float& ceta) const
+    {
+        a = p0[threadIdx.x];
+        b = p1[threadIdx.x];
+        i = info[threadIdx.x];
+        if (CV) {
+            cxi = cv[0][threadIdx.x];
+            ceta = cv[CV ? 1 : 0][threadIdx.x];
+        }
+    }
+};
+
 // Node data read again where a path starts or ends rather than held in registers
 // (volatile: the compiler would otherwise keep the first read).
 __device__ __forceinline__ float2 node_start(const NodeDev* nd)
@@ -478,8 +515,10 @@ __device__ __forceinline__ unsigned lanes_below()
 // and redirected gathers without skipping them, 92 instructions per path-step.
 template <int MODE, bool RECORD, int CVM, int VAR, bool DEFER, bool MAP>
 __device__ __forceinline__ void walk_tasks(const PathArgs& a, const uint8_t* zsm,
-                                           LaneSums<paths_max_block(CVM, VAR), !DEFER || MODE == 1>& sums)
+                                           LaneSums<paths_max_block(CVM, VAR), !DEFER || MODE == 1>& sums,
+                                           LaneExits<paths_max_block(CVM, VAR), CVM != 0>& left)
 {
+    constexpr int LEFT = 7;   // a path that left by the plain test; otherwise the face of a bridge exit
     constexpr bool CV = CVM != 0;
     constexpr bool CVT = CVM == 1;   // node values in time slices
     constexpr bool ONE = VAR != VAR_MULTI;
@@ -511,10 +550,11 @@ __device__ __forceinline__ void walk_tasks(const PathArgs& a, const uint8_t* zsm
         const uint32_t nodek = nd->ctr ^ a.keys.rk[0];
         const uint32_t end = (uint32_t)task.path0 + (uint32_t)task.npaths;
         uint32_t next = (uint32_t)task.path0, path = 0;
-        bool alive = false;
+        bool alive = false, ended = false;   // ended: a path that left, to be scored
         PathWords pw{};
         float2 pos = f2(0.5f, 0.5f);
         int m = 0;        // the path's pass: its draw
+        float dm = 0.f;   // bridge test: the position's distance to the boundary
         float2 cvx = f2(0.f, 0.f), cve = f2(0.f, 0.f);  // control-variate sums of the path
         int cvq = 0, cvn = CVT ? a.cv_bound[1] : 0;      // slice of the current sub-step, start of the next
         sums.clear();
@@ -560,6 +600,7 @@ __device__ __forceinline__ void walk_tasks(const PathArgs& a, const uint8_t* zsm
                         path = cand;
                         pw = path_words(path, step, a.keys);
                         pos = node_start(nd);
+                        if (!PAIRS) dm = face_distance(pos);
                         m = 0;
                         if (CV) cvx = cve = f2(0.f, 0.f);
                         if (CVT) {
@@ -582,8 +623,8 @@ __device__ __forceinline__ void walk_tasks(const PathArgs& a, const uint8_t* zsm
             const bool inA = inside2(pa);
             float2 pn = pa;   // where the pass ends
             bool out;
-            int code = 0;
-            float yxi = 0.f, yeta = 0.f, xe = 0.f, ye = 0.f;
+            int face = LEFT;
+            float tb = 0.f;
             if (PAIRS) {
                 // an odd K: the last pair has no sub-step B
                 const bool haveB = MODE == 2 || 2 * m + 1 < K;
@@ -592,71 +633,84 @@ __device__ __forceinline__ void walk_tasks(const PathArgs& a, const uint8_t* zsm
                 out = alive && !(inA && (!haveB || inside2(pb)));
             } else {
                 out = alive && !inA;
-                const float dm0 = fminf(fminf(pos.x, 1.0f - pos.x), fminf(pos.y, 1.0f - pos.y));
-                const float dm1 = fminf(fminf(pa.x, 1.0f - pa.x), fminf(pa.y, 1.0f - pa.y));
-                if (alive && inA && dm0 * dm1 < a.bridge_cut &&
-                    bridge_exit(I, pos.x, pos.y, pa.x, pa.y, a.dt, uniform_pos(r.z), code, yxi, yeta, xe, ye)) {
-                    code += 4;
+                const float dm1 = face_distance(pa);
+                if (alive && inA && dm * dm1 < a.bridge_cut &&
+                    bridge_test(pos.x, pos.y, pa.x, pa.y, a.inv_dt, uniform_pos(r.z), face, tb))
                     out = true;
-                }
+                dm = dm1;
             }
             --k;
-            if (k == 0 || __any_sync(FULL, out)) {
-                if (out || (alive && m == P - 1)) {
-                    const long long ri = DEFER || RECORD ? node_records(nd) + (long long)path : 0;
-                    int taken = K;
-                    bool later = DEFER;   // scored by k_score_surv once the fields are final
-                    if (out) {
-                        ++sums.exits[threadIdx.x];
-                        taken = !PAIRS ? m + 1 : inA ? 2 * m + 2 : 2 * m + 1;
-                        const float2 p0 = PAIRS && inA ? pa : pos, p1 = PAIRS && inA ? pn : pa;
-                        if (MODE == 1 && code >= 4) {
-                            // a bridge exit is scored here; its record holds the skip mark
-                            later = false;
-                            if (DEFER) put_record<CV>(a.surv, ri, f2(REC_SKIP, 0.f), cvx.x + cvx.y, cve.x + cve.y);
-                        } else if (DEFER) {
-                            put_record<CV>(a.surv, ri, exit_record(p0.x, p0.y, p1.x, p1.y), cvx.x + cvx.y,
-                                           cve.x + cve.y);
-                        } else {
-                            plain_exit(I, p0.x, p0.y, p1.x, p1.y, code, yxi, yeta, xe, ye);
-                        }
-                    } else if (DEFER) {
-                        put_record<CV>(a.surv, ri, pn, cvx.x + cvx.y, cve.x + cve.y);
-                    } else {
-                        // survived the mesh step: xi, eta of its start at the end point
-                        const Cell c = locate<ONE>(I, pn);
-                        float4 f0, f1;
-                        load_cell(rec2<ONE>(I.fcoef, c.idx), f0, f1);
-                        const float2 v = eval2(f0, f1, c.st);
-                        yxi = v.x;
-                        yeta = v.y;
-                        xe = pn.x;
-                        ye = pn.y;
-                        code = -1;
-                    }
-                    sums.steps[threadIdx.x] += taken;
-                    if (ACC && !later) {
-                        if (CV) {
-                            yxi -= cvx.x + cvx.y;
-                            yeta -= cve.x + cve.y;
-                        }
-                        const float2 c = node_start(nd);
-                        sums.add(0, yxi - c.x);
-                        sums.add(1, yeta - c.y);
-                    }
-                    if (RECORD) {
-                        if (a.rec.steps) a.rec.steps[ri] = taken;
-                        if (a.rec.code) a.rec.code[ri] = code;
-                        if (a.rec.score_xi) a.rec.score_xi[ri] = yxi;
-                        if (a.rec.score_eta) a.rec.score_eta[ri] = yeta;
-                        if (a.rec.x_end) a.rec.x_end[ri] = xe;
-                        if (a.rec.y_end) a.rec.y_end[ri] = ye;
-                    }
+            if (__any_sync(FULL, out)) {
+                // the paths that left wait for the next refill: now if enough lanes are idle, or all
+                if (out) {
+                    const float2 p0 = PAIRS && inA ? pa : pos, p1 = PAIRS && inA ? pn : pa;
+                    const int taken = !PAIRS ? m + 1 : inA ? 2 * m + 2 : 2 * m + 1;
+                    left.put(p0, !PAIRS && face != LEFT ? f2(tb, 0.f) : p1, taken | face << 28, cvx.x + cvx.y, cve.x + cve.y);
                     alive = false;
+                    ended = true;
                 }
-                // take new paths now if enough lanes are idle, or all
                 const int idle = 32 - __popc(__ballot_sync(FULL, alive));
                 if (idle == 32 || (idle >= REFILL_MIN && next < end)) k = 0;
+            }
+            if (k == 0 && (ended || (alive && m == P - 1))) {
+                const long long ri = DEFER || RECORD ? node_records(nd) + (long long)path : 0;
+                int taken = K, code = -1;
+                bool later = DEFER;   // scored by k_score_surv once the fields are final
+                float yxi = 0.f, yeta = 0.f, xe = 0.f, ye = 0.f, cxi = 0.f, ceta = 0.f;
+                if (CV) {
+                    cxi = cvx.x + cvx.y;
+                    ceta = cve.x + cve.y;
+                }
+                if (ended) {
+                    ++sums.exits[threadIdx.x];
+                    float2 p0, p1;
+                    int info;
+                    left.get(p0, p1, info, cxi, ceta);
+                    taken = info & 0x0fffffff;
+                    face = info >> 28;
+                    if (MODE == 1 && face != LEFT) {
+                        // a bridge exit is scored here; its record holds the skip mark
+                        face_point(I, face, p1.x, yxi, yeta, xe, ye);
+                        code = face + 4;
+                        later = false;
+                        if (DEFER) put_record<CV>(a.surv, ri, f2(REC_SKIP, 0.f), cxi, ceta);
+                    } else if (DEFER) {
+                        put_record<CV>(a.surv, ri, exit_record(p0.x, p0.y, p1.x, p1.y), cxi, ceta);
+                    } else {
+                        plain_exit(I, p0.x, p0.y, p1.x, p1.y, code, yxi, yeta, xe, ye);
+                    }
+                } else if (DEFER) {
+                    put_record<CV>(a.surv, ri, pn, cxi, ceta);
+                } else {
+                    // survived the mesh step: xi, eta of its start at the end point
+                    const Cell c = locate<ONE>(I, pn);
+                    float4 f0, f1;
+                    load_cell(rec2<ONE>(I.fcoef, c.idx), f0, f1);
+                    const float2 v = eval2(f0, f1, c.st);
+                    yxi = v.x;
+                    yeta = v.y;
+                    xe = pn.x;
+                    ye = pn.y;
+                }
+                sums.steps[threadIdx.x] += taken;
+                if (ACC && !later) {
+                    if (CV) {
+                        yxi -= cxi;
+                        yeta -= ceta;
+                    }
+                    const float2 c = node_start(nd);
+                    sums.add(0, yxi - c.x);
+                    sums.add(1, yeta - c.y);
+                }
+                if (RECORD) {
+                    if (a.rec.steps) a.rec.steps[ri] = taken;
+                    if (a.rec.code) a.rec.code[ri] = code;
+                    if (a.rec.score_xi) a.rec.score_xi[ri] = yxi;
+                    if (a.rec.score_eta) a.rec.score_eta[ri] = yeta;
+                    if (a.rec.x_end) a.rec.x_end[ri] = xe;
+                    if (a.rec.y_end) a.rec.y_end[ri] = ye;
+                }
+                alive = ended = false;
             }
             pos = pn;
             ++m;
@@ -676,6 +730,7 @@ __global__ void __launch_bounds__(paths_max_block(CVM, VAR), paths_min_blocks(CV
     k_paths(const PathArgs a)
 {
     __shared__ LaneSums<paths_max_block(CVM, VAR), !DEFER || MODE == 1> sums;
+    __shared__ LaneExits<paths_max_block(CVM, VAR), CVM != 0> left;
     if (VAR == VAR_ONE && a.zmap) {
         // stage the zero map, and leave it unused where nearly every tile is marked
         extern __shared__ __align__(16) uint8_t zsm[];
@@ -691,11 +746,11 @@ __global__ void __launch_bounds__(paths_max_block(CVM, VAR), paths_min_blocks(CV
         atomicAdd(&marked, mine);
         __syncthreads();
         if (marked < kZmapTiles * kZmapTiles * 7 / 8) {
-            walk_tasks<MODE, RECORD, CVM, VAR, DEFER, true>(a, zsm, sums);
+            walk_tasks<MODE, RECORD, CVM, VAR, DEFER, true>(a, zsm, sums, left);
             return;
         }
     }
-    walk_tasks<MODE, RECORD, CVM, VAR, DEFER, false>(a, nullptr, sums);
+    walk_tasks<MODE, RECORD, CVM, VAR, DEFER, false>(a, nullptr, sums, left);
 }
 
 // Exponential time-stepping (exit_mode 2), the alternative integrator Sec. 4
@@ -703,17 +758,23 @@ __global__ void __launch_bounds__(paths_max_block(CVM, VAR), paths_min_blocks(CV
 // 2^-23 from word 3 of the block (path, node, j, step), cut at the end of the
 // mesh step (and after 4K + 16 sub-steps); normals from words 0, 1 scaled by
 // sqrt(2 tau_j); the plain test, then the Brownian-bridge test over tau_j with
-// the uniform of word 2. No software pipelining: one block per sub-step.
+// the uniform of word 2.
+//
+// The paths of a warp end at different sub-steps, one or two of them in nearly every pass: a lane whose
+// path is done waits, so that the scores, the sums and the new paths (as many instructions as a
+// pass) are made for EXP_REFILL lanes at a time. Bound by issue slots. 253 nodes x 8000 paths at K = 20:
+// 406 us with a path's end handled in its pass and ten rounds a draw, now EXPNOW.
+constexpr int EXP_REFILL = 6;
+
 template <bool RECORD>
 __global__ void __launch_bounds__(512, 2) k_paths_exp(const PathArgs a)
 {
-    const int lane = threadIdx.x & 31;
-    const unsigned below = (1u << lane) - 1u;
+    __shared__ LaneSums<512, true> sums;
     const uint32_t step = a.step_ptr ? *a.step_ptr : a.step_index;
-    const int K = a.K;
-    const int cap = 4 * K + 16;
+    const int cap = 4 * a.K + 16;
     const float T = a.horizon;
     const float ln2dt = a.dt * 0.69314718055994530942f;
+    constexpr int SURVIVED = -1, LEFT = -2;   // otherwise 4 + the face of a bridge exit
     for (;;) {
         int tq = 0;
         if (lanes_below() == 0) tq = atomicAdd(a.queue, 1);
@@ -721,23 +782,80 @@ __global__ void __launch_bounds__(512, 2) k_paths_exp(const PathArgs a)
         if (t >= a.ntasks) return;
         const Task task = a.tasks[t];
         if (a.node_mask && !a.node_mask[task.node]) continue;
-        const NodeDev& nd = a.nodes[task.node];
-        const InstDev I = a.inst[nd.inst];
-        const float x0 = nd.xf, y0 = nd.yf;
-        const uint32_t nctr = nd.ctr;
-        const int end = task.path0 + task.npaths;
-        int next = task.path0 + 32;
-        int path = task.path0 + lane;
-        bool alive = path < end;
-        float2 pos = f2(x0, y0);
-        int j = 0;
-        float tm = 0.f;
-        Acc ax{0.f, 0.f, 0.f, 0.f}, ae{0.f, 0.f, 0.f, 0.f};
-        int exits = 0, steps = 0;
-        while (__any_sync(FULL, alive)) {
+        const NodeDev* const nd = a.nodes + task.node;
+        const InstDev I = a.inst[nd->inst];
+        const uint32_t nodek = nd->ctr ^ a.keys.rk[0];
+        const uint32_t end = (uint32_t)task.path0 + (uint32_t)task.npaths;
+        uint32_t next = (uint32_t)task.path0, path = 0;
+        bool alive = false, ended = false;
+        PathWords pw{};
+        float2 pos = f2(0.5f, 0.5f), pe = f2(0.f, 0.f);   // pe: the point past an exit, or (t, -) of a bridge exit
+        int j = 0, code = SURVIVED;
+        float tm = 0.f, dm = 0.f;   // time, distance to the boundary
+        sums.clear();
+        bool refill = true;
+        for (;;) {
+            if (refill) {
+                if (ended) {
+                    ended = false;
+                    const long long ri = a.surv || RECORD ? node_records(nd) + (long long)path : 0;
+                    float yxi = 0.f, yeta = 0.f, xe = 0.f, ye = 0.f;
+                    bool later = a.surv != nullptr;   // scored by k_score_surv once the fields are final
+                    if (code != SURVIVED) ++sums.exits[threadIdx.x];
+                    if (code >= 4) {
+                        face_point(I, code - 4, pe.x, yxi, yeta, xe, ye);
+                        if (a.surv) put_record<false>(a.surv, ri, f2(REC_SKIP, 0.f), 0.f, 0.f);
+                        later = false;
+                    } else if (a.surv) {
+                        put_record<false>(a.surv, ri, code == LEFT ? exit_record(pos.x, pos.y, pe.x, pe.y) : pos, 0.f, 0.f);
+                    } else if (code == LEFT) {
+                        plain_exit(I, pos.x, pos.y, pe.x, pe.y, code, yxi, yeta, xe, ye);
+                    } else {
+                        const Cell cf = locate<false>(I, pos);
+                        float4 f0, f1;
+                        load_cell(rec2<false>(I.fcoef, cf.idx), f0, f1);
+                        const float2 v = eval2(f0, f1, cf.st);
+                        yxi = v.x;
+                        yeta = v.y;
+                        xe = pos.x;
+                        ye = pos.y;
+                    }
+                    sums.steps[threadIdx.x] += j;
+                    if (!later) {
+                        const float2 c = node_start(nd);
+                        sums.add(0, yxi - c.x);
+                        sums.add(1, yeta - c.y);
+                    }
+                    if (RECORD) {
+                        if (a.rec.steps) a.rec.steps[ri] = j;
+                        if (a.rec.code) a.rec.code[ri] = code;
+                        if (a.rec.score_xi) a.rec.score_xi[ri] = yxi;
+                        if (a.rec.score_eta) a.rec.score_eta[ri] = yeta;
+                        if (a.rec.x_end) a.rec.x_end[ri] = xe;
+                        if (a.rec.y_end) a.rec.y_end[ri] = ye;
+                    }
+                }
+                // the lanes without a path take the task's next ones, in lane order
+                const unsigned idle = __ballot_sync(FULL, !alive);
+                if (next < end) {
+                    const uint32_t cand = next + __popc(idle & lanes_below());
+                    next += __popc(idle);
+                    if (!alive && cand < end) {
+                        alive = true;
+                        path = cand;
+                        pw = path_words(path, step, a.keys);
+                        pos = node_start(nd);
+                        dm = face_distance(pos);
+                        j = 0;
+                        tm = 0.f;
+                    }
+                } else if (idle == FULL) {
+                    break;
+                }
+            }
             if (alive) {
-                uint4 r = make_uint4((uint32_t)path, nctr, (uint32_t)j, step);
-                philox_rounds_rk<0, 10>(r, a.keys);
+                uint4 r = draw_begin(pw, nodek, (uint32_t)j);
+                philox_rounds_rk<2, 10>(r, a.keys);
                 const float u3 = 2.0f - __uint_as_float(0x3F800000u | (r.w & 0x7FFFFFu));
                 float tau = -ln2dt * __log2f(u3);
                 bool last = false;
@@ -747,87 +865,37 @@ __global__ void __launch_bounds__(512, 2) k_paths_exp(const PathArgs a)
                 }
                 float2 z;
                 box_muller(r.x, r.y, -2.77258872223978123767f * tau, z.x, z.y);   // -4 ln 2 tau: sqrt(2 tau) N(0,1)
-                const float ub = uniform_pos(r.z);
                 const Cell c = locate<false>(I, pos);
                 float4 g0, g1;
                 load_cell(rec2<false>(I.bcoef, c.idx), g0, g1);
                 const float2 pn = em(g0, g1, c.st, pos, f2(tau, tau), z);
-                bool done = false;
-                int code = -1;
-                float yxi = 0.f, yeta = 0.f, xe = 0.f, ye = 0.f;
-                float2 seg = f2(REC_SKIP, 0.f);
+                ++j;
                 if (!inside2(pn)) {
-                    if (a.surv) seg = exit_record(pos.x, pos.y, pn.x, pn.y), code = 0;
-                    else plain_exit(I, pos.x, pos.y, pn.x, pn.y, code, yxi, yeta, xe, ye);
-                    done = true;
+                    code = LEFT;
+                    ended = true;
+                    pe = pn;
                 } else {
-                    const float dm0 = fminf(fminf(pos.x, 1.0f - pos.x), fminf(pos.y, 1.0f - pos.y));
-                    const float dm1 = fminf(fminf(pn.x, 1.0f - pn.x), fminf(pn.y, 1.0f - pn.y));
-                    if (dm0 * dm1 < 18.0f * tau && bridge_exit(I, pos.x, pos.y, pn.x, pn.y, tau, ub, code, yxi, yeta, xe, ye)) {
+                    const float dm1 = face_distance(pn);
+                    if (dm * dm1 < 18.0f * tau &&
+                        bridge_test(pos.x, pos.y, pn.x, pn.y, 1.0f / tau, uniform_pos(r.z), code, pe.x)) {
                         code += 4;
-                        done = true;
+                        ended = true;
                     } else {
                         pos = pn;
+                        dm = dm1;
                         tm += tau;
-                        if (last) done = true;
+                        code = SURVIVED;
+                        ended = last;
                     }
                 }
-                ++j;
-                if (done) {
-                    bool later = false;
-                    if (code < 0) {
-                        if (a.surv) {
-                            later = true;
-                            put_record<false>(a.surv, nd.rec0 + path, pos, 0.f, 0.f);
-                        } else {
-                            const Cell cf = locate<false>(I, pos);
-                            float4 f0, f1;
-                            load_cell(rec2<false>(I.fcoef, cf.idx), f0, f1);
-                            const float2 v = eval2(f0, f1, cf.st);
-                            yxi = v.x;
-                            yeta = v.y;
-                            xe = pos.x;
-                            ye = pos.y;
-                        }
-                    } else {
-                        ++exits;
-                        if (a.surv) {
-                            later = seg.x != REC_SKIP;
-                            put_record<false>(a.surv, nd.rec0 + path, seg, 0.f, 0.f);
-                        }
-                    }
-                    if (!later) {
-                        ax.add(yxi - x0);
-                        ae.add(yeta - y0);
-                    }
-                    steps += j;
-                    if (RECORD) {
-                        const long long ri = nd.rec0 + path;
-                        if (a.rec.steps) a.rec.steps[ri] = j;
-                        if (a.rec.code) a.rec.code[ri] = code;
-                        if (a.rec.score_xi) a.rec.score_xi[ri] = yxi;
-                        if (a.rec.score_eta) a.rec.score_eta[ri] = yeta;
-                        if (a.rec.x_end) a.rec.x_end[ri] = xe;
-                        if (a.rec.y_end) a.rec.y_end[ri] = ye;
-                    }
-                    alive = false;
-                }
+                alive = !ended;
             }
-            const unsigned need = __ballot_sync(FULL, !alive);
-            if (need != 0u && next < end) {
-                const int cand = next + __popc(need & below);
-                if (!alive && cand < end) {
-                    path = cand;
-                    alive = true;
-                    pos = f2(x0, y0);
-                    j = 0;
-                    tm = 0.f;
-                }
-                next += __popc(need);
-            }
+            const int idle = 32 - __popc(__ballot_sync(FULL, alive));
+            refill = idle == 32 || (idle >= EXP_REFILL && next < end);
         }
+        const Acc ax = sums.get(0), ae = sums.get(1);
         const double tot = warp_sum4(ax.sum(), ax.sumsq(), ae.sum(), ae.sumsq());
-        put_partial(a.partials + t, tot, warp_sum_int(exits), warp_sum_int(steps));
+        put_partial(a.partials + t, tot, warp_sum_int(sums.exits[threadIdx.x]), warp_sum_int(sums.steps[threadIdx.x]));
     }
 }
 

@@ -233,6 +233,7 @@ sdd_status sdd_interface_mc_static(const sdd_fields* f, const sdd_nodes* nodes, 
         a.dt = (float)p->dt;
         a.bm_scale = (float)(-4.0 * p->dt * std::log(2.0));
         a.bridge_cut = (float)(18.0 * p->dt);
+        a.inv_dt = 1.0f / a.dt;
         a.horizon = (float)((double)a.K * p->dt);
         a.keys = philox_keys(p->seed);
         a.step_index = p->step_index;
