@@ -357,9 +357,10 @@ __device__ __forceinline__ float2 exit_record(float x, float y, float xn, float 
     return f2(-1.0f - (float)face, t);
 }
 
-// Idle lanes that call for a refill. A lane whose path left the domain stays
-// idle until this many do, or until some path of the warp reaches the end of
-// the step: a refill costs its warp about one pass's worth of bookkeeping.
+// Idle lanes that call for a refill. A lane whose path left the domain waits until this many have, or until some
+// path of the warp reaches the end of the step; then all that ended are scored and replaced together (the crossing,
+// the boundary data and the sums take more instructions than a pass). 601 nodes of a 194 x 131 grid, 45 sub-steps:
+// 297 us with each exit scored in its pass, now 277; 4 lanes or 18 instead of 8 are up to 1 % slower.
 constexpr int REFILL_MIN = 8;
 
 // The draws of one path: Philox block d of path p, its first two rounds reduced
@@ -763,7 +764,7 @@ __global__ void __launch_bounds__(paths_max_block(CVM, VAR), paths_min_blocks(CV
 // The paths of a warp end at different sub-steps, one or two of them in nearly every pass: a lane whose
 // path is done waits, so that the scores, the sums and the new paths (as many instructions as a
 // pass) are made for EXP_REFILL lanes at a time. Bound by issue slots. 253 nodes x 8000 paths at K = 20:
-// 406 us with a path's end handled in its pass and ten rounds a draw, now EXPNOW.
+// 406 us with a path's end handled in its pass and ten rounds a draw, now 372.
 constexpr int EXP_REFILL = 6;
 
 template <bool RECORD>
@@ -1069,18 +1070,19 @@ __global__ void __launch_bounds__(FINAL_WARPS * 32) k_finalize(const FinalArgs a
 
 // Scores of the paths that survived a mesh step, once the fields of the step's
 // start are final (the estimate of the next mesh step runs beside the
-// subdomain solve that produces them), then the node's reduction. A cluster of blocks per node: the node's paths
-// end in one neighbourhood, so a block's gathers share L1; each block takes a run of the paths, thread k of it paths
-// k, k + T, ... SCORE_BATCH at a time (records, then gathers, in flight
+// subdomain solve that produces them), then the node's reduction. A cluster of C blocks of T threads per node: the
+// node's paths end in one neighbourhood, so a block's gathers share L1; thread k of the cluster's C T takes paths
+// k, k + C T, ... SCORE_BATCH at a time (records, then gathers, in flight
 // together) and sums xi and eta at the end points minus the paths'
-// control-variate sums; task partials are dealt to the cluster's threads. Each block leaves its sums
+// control-variate sums; task partials are dealt to the cluster's threads as well. Each block leaves its sums
 // with block 0, whose first warp writes the outputs. The next batch's records are read while the
-// current batch's gathers are in flight. T = 256 threads at 64 registers puts four blocks on an SM; the cluster is
-// the largest that leaves one wave of such blocks: with one block of 1024 threads per node, the 77 nodes of a
-// 41 x 41 grid left half the SMs idle, and the task partials went through one warp: 26.6 us, now 16.9.
+// current batch's gathers are in flight. T = 256 threads at 64 registers puts four blocks on an SM (many nodes: one
+// wave for up to four per SM); with no more nodes than SMs, four blocks per node make one wave of them. (One block
+// of 1024 threads per node left half the SMs idle on a 41 x 41 grid's 77 nodes, and the task partials went
+// through one warp: 26.6 us, now 16.9.)
 constexpr int SCORE_BATCH = 2;
 constexpr int SCORE_THREADS = 256;
-constexpr int SCORE_MAX_CLUSTER = 8;
+constexpr int SCORE_MAX_CLUSTER = 4;
 
 template <bool CV>
 __global__ void __launch_bounds__(SCORE_THREADS, 4) k_score_surv(const ScoreArgs a)
@@ -1100,13 +1102,13 @@ __global__ void __launch_bounds__(SCORE_THREADS, 4) k_score_surv(const ScoreArgs
     }
     const InstDev I = a.inst[nd.inst];
     const float x0 = nd.xf, y0 = nd.yf;
-    const int first = (int)((long long)nd.n_paths * rank / C), end = (int)((long long)nd.n_paths * (rank + 1) / C);
+    const int first = rank * SCORE_THREADS + threadIdx.x, threads = C * SCORE_THREADS, end = nd.n_paths;
     Acc ax{0.f, 0.f, 0.f, 0.f}, ae{0.f, 0.f, 0.f, 0.f};
     // the records of the batch that starts at path p0 (past the end: the skip mark)
     auto load_batch = [&](int p0, float2 (&r)[SCORE_BATCH], float2 (&cvs)[SCORE_BATCH]) {
 #pragma unroll
         for (int u = 0; u < SCORE_BATCH; ++u) {
-            const int p = p0 + u * SCORE_THREADS;
+            const int p = p0 + u * threads;
             r[u] = f2(REC_SKIP, 0.f);
             cvs[u] = f2(0.f, 0.f);
             if (p < end) {
@@ -1119,18 +1121,18 @@ __global__ void __launch_bounds__(SCORE_THREADS, 4) k_score_surv(const ScoreArgs
     };
     float2 r[SCORE_BATCH];
     float2 cvs[SCORE_BATCH];
-    load_batch(first + threadIdx.x, r, cvs);
+    load_batch(first, r, cvs);
     {
         // this thread's share of the task partials, kept in shared memory over the scoring
         double v[4];
         long long ex, st;
-        task_sums(a.fin, nd, rank * SCORE_THREADS + threadIdx.x, C * SCORE_THREADS, v, ex, st);
+        task_sums(a.fin, nd, first, threads, v, ex, st);
 #pragma unroll
         for (int q = 0; q < 4; ++q) task_v[q][threadIdx.x] = v[q];
         task_n[0][threadIdx.x] = ex;
         task_n[1][threadIdx.x] = st;
     }
-    for (int p0 = first + threadIdx.x; p0 < end; p0 += SCORE_BATCH * SCORE_THREADS) {
+    for (int p0 = first; p0 < end; p0 += SCORE_BATCH * threads) {
         // one round of loads for the batch: a survivor gathers the field record at its
         // end point, a plain exit the face data on both sides of its crossing
         // (f0 = xi[k], xi[k + 1], eta[k], eta[k + 1]; st.x the fraction)
@@ -1157,7 +1159,7 @@ __global__ void __launch_bounds__(SCORE_THREADS, 4) k_score_surv(const ScoreArgs
         // the next batch's records while this batch's gathers are in flight
         float2 rn[SCORE_BATCH];
         float2 cn[SCORE_BATCH];
-        load_batch(p0 + SCORE_BATCH * SCORE_THREADS, rn, cn);
+        load_batch(p0 + SCORE_BATCH * threads, rn, cn);
 #pragma unroll
         for (int u = 0; u < SCORE_BATCH; ++u) {
             if (r[u].x == REC_SKIP) continue;   // scored in the path kernel, or past the end
@@ -1287,8 +1289,7 @@ cudaError_t launch_score_surv(const ScoreArgs& a, bool cv, cudaStream_t s)
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    int C = SCORE_MAX_CLUSTER;
-    while (C > 1 && (long long)a.nnodes * C > 4LL * sms) C >>= 1;
+    const int C = a.nnodes <= sms ? SCORE_MAX_CLUSTER : 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(a.nnodes * C));
     cfg.blockDim = dim3(SCORE_THREADS);

@@ -1,4 +1,4 @@
-"""A node's sums over its tasks and paths: one to eight warps per node in an estimate, one to eight blocks per node in
+"""A node's sums over its tasks and paths: one to eight warps per node in an estimate, one or four blocks per node in
 the deferred scoring of a mesh step, with fewer paths than threads, ragged shares and nodes without paths."""
 import numpy as np
 import pytest
@@ -44,13 +44,13 @@ def test_estimate_is_the_mean_of_its_paths(sdd, nodes, paths):
             d = (g["score_" + f][one] - np.float32(start)).astype(np.float32)
             S, Q = d.astype(np.float64).sum(), (d * d).astype(np.float64).sum()
             N = counts[k]
-            # compensated single-precision sums of at most 260 scores: 260 x 4 x 2^-48 of the largest, below 1e-11
+            # each lane sums its few scores in compensated single precision, off by a rounding of some scores
             assert abs(g["mean_" + f][k] - (np.float64(np.float32(start)) + S / N)) <= 1e-11
             var = max(0.0, (Q - S * S / N) / (N - 1)) if N > 1 else 0.0
             assert abs(g["se_" + f][k] ** 2 * N - var) <= 1e-10 * Q / max(N - 1, 1)
 
 
-# 1, 77, 253 and 509 interface nodes: clusters of eight, four, two and one
+# 5, 77, 253 and 509 interface nodes: clusters of four blocks, single blocks
 @pytest.mark.parametrize("n,sub", [(5, 2), (41, 2), (129, 2), (257, 2)])
 @pytest.mark.parametrize("paths", [1, 7, 300, 2049])
 def test_deferred_scores_match_the_step_without_deferral(sdd, n, sub, paths):
