@@ -273,14 +273,15 @@ __global__ void k_norm(const double* __restrict__ part, int nblk, long long n, d
 // ---------------------------------------------------------------- training
 
 struct GradSmem {
-    float th[kMlpStride];      // the network's parameters
-    float w2t[H * H];          // W2 transposed: [k][j]
+    float th[kMlpStride];      // the network's parameters; W2 in pairs of units: [j / 2][k] (W2[j][k], W2[j + 1][k])
+    float2 w2t[H / 2 * H];     // W2 in pairs of inputs: [k / 2][j] (W2[j][k], W2[j][k + 1])
     float h1[TILE * LD];       // tanh(a1), later dL/da1
     float h2[TILE * LD];       // tanh(a2), later dL/da2
     float z[TILE * ZS];
     float y[TILE];
     float d[TILE];
     float quarter[4][H];       // sums over a quarter of the tile's rows
+    float quarter2[4][H];
     float red[GRAD_THREADS / 32];
 };
 
@@ -298,26 +299,29 @@ struct TileSum {
     __device__ __forceinline__ float value() const { return s + c; }
 };
 
-// dst[r][c] += sum_q a[row(r)][q] b[q][4 tx + c] over q < 64: a row-major with stride LD, read four q at a
-// time (a warp reads two rows of a and 64 columns of b), b with stride H.
+// acc[r][c] += sum_q a[row(r)][q] b[q][col(c)] over q < 64, even and odd q apart, columns 2 tx, 2 tx + 1 and 32 more
+// (a warp's reads of b then touch every bank once): a row-major with stride LD,
+// read four q at a time (a warp reads two rows of a and 64 columns of b), b in pairs of q, [q / 2][column].
 template <int RPT>
-__device__ __forceinline__ void tile_product(float (&acc)[RPT][4], const float* a, const float* b, int tx, int ty)
+__device__ __forceinline__ void tile_product(float2 (&acc)[RPT][4], const float* a, const float2* b, int tx, int ty)
 {
 #pragma unroll 4
     for (int q = 0; q < H; q += 4) {
-        float4 bv[4];
+        float4 bv[2][2];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) bv[e] = *reinterpret_cast<const float4*>(&b[(q + e) * H + 4 * tx]);
+        for (int e = 0; e < 2; ++e)
+#pragma unroll
+            for (int c = 0; c < 2; ++c) bv[e][c] = *reinterpret_cast<const float4*>(&b[(q / 2 + e) * H + 2 * tx + 32 * c]);
 #pragma unroll
         for (int r = 0; r < RPT; ++r) {
             const float4 av = *reinterpret_cast<const float4*>(&a[(ty + 16 * r) * LD + q]);
-            const float ae[4] = {av.x, av.y, av.z, av.w};
+            const float2 ae[2] = {make_float2(av.x, av.y), make_float2(av.z, av.w)};
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                acc[r][0] = fmaf(ae[e], bv[e].x, acc[r][0]);
-                acc[r][1] = fmaf(ae[e], bv[e].y, acc[r][1]);
-                acc[r][2] = fmaf(ae[e], bv[e].z, acc[r][2]);
-                acc[r][3] = fmaf(ae[e], bv[e].w, acc[r][3]);
+            for (int e = 0; e < 2; ++e) {
+                acc[r][0] = __ffma2_rn(ae[e], make_float2(bv[e][0].x, bv[e][0].y), acc[r][0]);
+                acc[r][1] = __ffma2_rn(ae[e], make_float2(bv[e][0].z, bv[e][0].w), acc[r][1]);
+                acc[r][2] = __ffma2_rn(ae[e], make_float2(bv[e][1].x, bv[e][1].y), acc[r][2]);
+                acc[r][3] = __ffma2_rn(ae[e], make_float2(bv[e][1].z, bv[e][1].w), acc[r][3]);
             }
         }
     }
@@ -327,11 +331,12 @@ __device__ __forceinline__ void tile_product(float (&acc)[RPT][4], const float* 
 // gradient of the batch loss (1 / batch) sum (g - y)^2, written to part[(f nblk + block) stride + p];
 // part[.. + kMlpParams] = its sum of squared errors.
 //
-// Three 64 x 64 products and 128 tanhf per row: 4-by-4 register tiles, operands read four deep (12
-// shared-memory wavefronts per 64 FMAs a thread; read one by one they were 6 per 16), W2's gradient kept in
-// registers over the tiles. A tile's partial gradient is 18 KB, so blocks take several tiles and write one.
-// 65,536 rows: 126 us (147 us for a block and a partial per tile, whose sum took 163 us more; now 9), issue slots
-// 60 % busy, the shared-memory loads the next bound; tiles of 128 rows were within 3 %.
+// Three 64 x 64 products and 128 tanhf per row: 4-by-4 register tiles, operands read four deep, W2's gradient kept in
+// registers over the tiles. A tile's partial gradient is 18 KB, so blocks take several tiles and write one, and
+// a tile's inputs are read while the one before is at work. Bound by the shared-memory loads (a 16-byte
+// load of a warp takes four cycles, 81 % busy): the multiply-adds are in pairs, which halves their issue
+// slots. 65,536 rows: 111 us (127 with single multiply-adds; 147 for a block and a partial per tile, whose sum took
+// 163 us more, now 9). Blocks of 128 threads with 8-by-4 tiles load a third less, but hold 12 warps an SM: 121 us.
 __global__ void __launch_bounds__(GRAD_THREADS, 2) k_mlp_grad(const float* __restrict__ theta,
                                                               const float* __restrict__ norm,
                                                               const float* __restrict__ feats,
@@ -346,22 +351,43 @@ __global__ void __launch_bounds__(GRAD_THREADS, 2) k_mlp_grad(const float* __res
     const int lane = t & 31, wid = t >> 5, tx = t & 15, ty = t >> 4;
     const int j = t & 63, quarter = t >> 6;
     const float* th = theta + (long long)f * kMlpStride;
-    for (int p = t; p < kMlpParams; p += GRAD_THREADS) S.th[p] = th[p];
-    for (int p = t; p < H * H; p += GRAD_THREADS) S.w2t[(p & 63) * H + (p >> 6)] = th[OW2 + p];
+    for (int p = t; p < kMlpParams; p += GRAD_THREADS)
+        if (p < OW2 || p >= OW2 + H * H) S.th[p] = th[p];
+    float2* const w2 = reinterpret_cast<float2*>(&S.th[OW2]);
+    for (int p = t; p < H * H / 2; p += GRAD_THREADS) {
+        const int q = p / H, c = p % H;
+        S.w2t[p] = make_float2(th[OW2 + c * H + 2 * q], th[OW2 + c * H + 2 * q + 1]);
+        w2[p] = make_float2(th[OW2 + 2 * q * H + c], th[OW2 + (2 * q + 1) * H + c]);
+    }
 
-    TileSum gw2[4][4], gb2[4], small[2], loss;   // small: thread t's outputs of W1, b1 (t, t + 256) or w3 (loss: b3 too)
-    TileSum gw3, gb3;
+    TileSum gw2[4][4], small[2], loss;   // small: thread t's outputs of W1, b1 (t, t + 256)
+    TileSum gw3, gb2, gb3;
     const int ntiles = (int)((rows + ROWS - 1) / ROWS);
-    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    // a tile's inputs, read while the tile before is at work
+    constexpr int NIN = (ROWS * D + GRAD_THREADS - 1) / GRAD_THREADS;
+    float in[NIN], target = 0.f;
+    auto load_inputs = [&](int tile) {
         const long long r0 = row0 + (long long)tile * ROWS;
-        const int have = (int)min((long long)ROWS, row0 + rows - r0);
-        __syncthreads();   // the tile before is done (and the parameters are in place)
-        for (int p = t; p < ROWS * D; p += GRAD_THREADS) {
-            const int c = p % D;
-            S.z[p / D * ZS + c] = p < have * D ? (feats[r0 * D + p] - norm[c]) * norm[D + c] : 0.f;
+        const int have = tile < ntiles ? (int)min((long long)ROWS, row0 + rows - r0) : 0;
+#pragma unroll
+        for (int q = 0; q < NIN; ++q) {
+            const int p = t + q * GRAD_THREADS;
+            in[q] = p < have * D ? feats[r0 * D + p] : 0.f;
         }
-        for (int i = t; i < ROWS; i += GRAD_THREADS) S.y[i] = i < have ? targets[2 * (r0 + i) + f] : 0.f;
+        target = t < have ? targets[2 * (r0 + t) + f] : 0.f;
+    };
+    load_inputs(blockIdx.x);
+    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+        const int have = (int)min((long long)ROWS, rows - (long long)tile * ROWS);
+        __syncthreads();   // the tile before is done (and the parameters are in place)
+#pragma unroll
+        for (int q = 0; q < NIN; ++q) {
+            const int p = t + q * GRAD_THREADS, c = p % D;
+            if (p < ROWS * D) S.z[p / D * ZS + c] = p < have * D ? (in[q] - norm[c]) * norm[D + c] : 0.f;
+        }
+        if (t < ROWS) S.y[t] = target;
         __syncthreads();
+        load_inputs(tile + (int)gridDim.x);
 
         // layer 1: thread owns unit j and rows quarter + 4 m
         {
@@ -384,16 +410,18 @@ __global__ void __launch_bounds__(GRAD_THREADS, 2) k_mlp_grad(const float* __res
 
         // layer 2: a2[i][j] = b2[j] + sum_k h1[i][k] W2[j][k], rows ty + 16 r, units 4 tx..
         {
-            float acc[RPT][4];
+            float2 acc[RPT][4];
 #pragma unroll
             for (int r = 0; r < RPT; ++r)
 #pragma unroll
-                for (int c = 0; c < 4; ++c) acc[r][c] = S.th[OB2 + 4 * tx + c];
+                for (int c = 0; c < 4; ++c) acc[r][c] = make_float2(S.th[OB2 + 2 * tx + (c & 1) + 16 * (c & 2)], 0.f);
             tile_product<RPT>(acc, S.h1, S.w2t, tx, ty);
 #pragma unroll
             for (int r = 0; r < RPT; ++r)
-                *reinterpret_cast<float4*>(&S.h2[(ty + 16 * r) * LD + 4 * tx]) =
-                    make_float4(tanhf(acc[r][0]), tanhf(acc[r][1]), tanhf(acc[r][2]), tanhf(acc[r][3]));
+#pragma unroll
+                for (int c = 0; c < 4; c += 2)
+                    *reinterpret_cast<float2*>(&S.h2[(ty + 16 * r) * LD + 2 * tx + 16 * c]) =
+                        make_float2(tanhf(acc[r][c].x + acc[r][c].y), tanhf(acc[r][c + 1].x + acc[r][c + 1].y));
         }
         __syncthreads();
 
@@ -418,21 +446,27 @@ __global__ void __launch_bounds__(GRAD_THREADS, 2) k_mlp_grad(const float* __res
         }
         __syncthreads();
         // dL/dw3[j] = sum_i d_i h2[i][j] by quarters of the rows, dL/db3 = sum_i d_i, the loss;
-        // then dL/da2 = d_i w3_j (1 - h2^2) in place, rows by the same threads
+        // then dL/da2 = d_i w3_j (1 - h2^2) in place, rows by the same threads, dL/db2 its sum
         {
             const float w3 = S.th[OW3 + j];
-            float a = 0.f;
+            float a = 0.f, b = 0.f;
 #pragma unroll 8
             for (int i = quarter * QROWS; i < (quarter + 1) * QROWS; ++i) {
                 const float h = S.h2[i * LD + j], d = S.d[i];
                 a = fmaf(d, h, a);
-                S.h2[i * LD + j] = d * w3 * (1.f - h * h);
+                const float g = d * w3 * (1.f - h * h);
+                b += g;
+                S.h2[i * LD + j] = g;
             }
             S.quarter[quarter][j] = a;
+            S.quarter2[quarter][j] = b;
         }
         __syncthreads();
         if (t < H) {
             gw3.add((S.quarter[0][t] + S.quarter[1][t]) + (S.quarter[2][t] + S.quarter[3][t]));
+        } else if (t >= 128 && t < 128 + H) {
+            const int o = t - 128;
+            gb2.add((S.quarter2[0][o] + S.quarter2[1][o]) + (S.quarter2[2][o] + S.quarter2[3][o]));
         } else if (wid == 2) {
             float a = 0.f;
             for (int i = lane; i < ROWS; i += 32) a += S.d[i];
@@ -443,44 +477,44 @@ __global__ void __launch_bounds__(GRAD_THREADS, 2) k_mlp_grad(const float* __res
             for (int q = 0; q < GRAD_THREADS / 32; ++q) a += S.red[q];
             loss.add(a);
         }
-        // dL/dW2[j][k] = sum_i g2[i][j] h1[i][k] (units 4 ty.., inputs 4 tx..), dL/db2
+        // dL/dW2[j][k] = sum_i g2[i][j] h1[i][k] (units 4 ty.., inputs 4 tx..)
         {
-            float acc[4][4] = {};
-            float db[4] = {0.f, 0.f, 0.f, 0.f};
+            float2 acc[4][2] = {};
 #pragma unroll 4
             for (int i = 0; i < ROWS; ++i) {
                 const float4 g = *reinterpret_cast<const float4*>(&S.h2[i * LD + 4 * ty]);
                 const float4 h = *reinterpret_cast<const float4*>(&S.h1[i * LD + 4 * tx]);
-                const float gv[4] = {g.x, g.y, g.z, g.w};
+                const float2 gv[4] = {make_float2(g.x, g.x), make_float2(g.y, g.y), make_float2(g.z, g.z),
+                                      make_float2(g.w, g.w)};
 #pragma unroll
                 for (int r = 0; r < 4; ++r) {
-                    acc[r][0] = fmaf(gv[r], h.x, acc[r][0]);
-                    acc[r][1] = fmaf(gv[r], h.y, acc[r][1]);
-                    acc[r][2] = fmaf(gv[r], h.z, acc[r][2]);
-                    acc[r][3] = fmaf(gv[r], h.w, acc[r][3]);
-                    db[r] += gv[r];
+                    acc[r][0] = __ffma2_rn(gv[r], make_float2(h.x, h.y), acc[r][0]);
+                    acc[r][1] = __ffma2_rn(gv[r], make_float2(h.z, h.w), acc[r][1]);
                 }
             }
 #pragma unroll
-            for (int r = 0; r < 4; ++r) {
+            for (int r = 0; r < 4; ++r)
 #pragma unroll
-                for (int c = 0; c < 4; ++c) gw2[r][c].add(acc[r][c]);
-                gb2[r].add(db[r]);
-            }
+                for (int c = 0; c < 2; ++c) {
+                    gw2[r][2 * c].add(acc[r][c].x);
+                    gw2[r][2 * c + 1].add(acc[r][c].y);
+                }
         }
         __syncthreads();   // h1 is overwritten next
         // dL/da1[i][k] = (sum_j g2[i][j] W2[j][k]) (1 - h1[i][k]^2), rows ty + 16 r, inputs 4 tx..;
         // each thread overwrites only its own h1 entries, which no other thread reads in this phase
         {
-            float acc[RPT][4] = {};
-            tile_product<RPT>(acc, S.h2, S.th + OW2, tx, ty);
+            float2 acc[RPT][4] = {};
+            tile_product<RPT>(acc, S.h2, w2, tx, ty);
 #pragma unroll
-            for (int r = 0; r < RPT; ++r) {
-                float4* const h = reinterpret_cast<float4*>(&S.h1[(ty + 16 * r) * LD + 4 * tx]);
-                const float4 v = *h;
-                *h = make_float4(acc[r][0] * (1.f - v.x * v.x), acc[r][1] * (1.f - v.y * v.y),
-                                 acc[r][2] * (1.f - v.z * v.z), acc[r][3] * (1.f - v.w * v.w));
-            }
+            for (int r = 0; r < RPT; ++r)
+#pragma unroll
+                for (int c = 0; c < 4; c += 2) {
+                    float2* const h = reinterpret_cast<float2*>(&S.h1[(ty + 16 * r) * LD + 2 * tx + 16 * c]);
+                    const float2 v = *h;
+                    *h = make_float2((acc[r][c].x + acc[r][c].y) * (1.f - v.x * v.x),
+                                     (acc[r][c + 1].x + acc[r][c + 1].y) * (1.f - v.y * v.y));
+                }
         }
         __syncthreads();
         // dL/dW1[j][c] = sum_i g1[i][j] z[i][c], dL/db1[j] = sum_i g1[i][j], by quarters of the rows
@@ -521,11 +555,11 @@ __global__ void __launch_bounds__(GRAD_THREADS, 2) k_mlp_grad(const float* __res
     for (int r = 0; r < 4; ++r) {
         *reinterpret_cast<float4*>(&out[OW2 + (4 * ty + r) * H + 4 * tx]) =
             make_float4(gw2[r][0].value(), gw2[r][1].value(), gw2[r][2].value(), gw2[r][3].value());
-        if (tx == 0) out[OB2 + 4 * ty + r] = gb2[r].value();
     }
     if (t < H) out[OW3 + t] = gw3.value();
     else if (t == 64) out[OB3] = gb3.value();
     else if (t == 96) out[kMlpParams] = loss.value();
+    else if (t >= 128 && t < 128 + H) out[OB2 + t - 128] = gb2.value();
 }
 
 // Sum over the blocks' partials of parameter p (kMlpParams: the loss) in double precision: SUM_SPLIT threads
