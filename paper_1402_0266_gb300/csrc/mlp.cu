@@ -655,15 +655,18 @@ struct TabArgs {
 // ---- the 64 x 64 layer on the fifth-generation tensor cores
 //
 // A CTA of 256 threads takes tiles of 128 points (point p = slice * nodes +
-// node). Threads t and t + 128 share point t % 128, each with half of the 64
-// units: they compute layer 1 and write three BF16 rows into shared memory: h1 = tanh(a1), u1 = (1 - h1^2) W1 dz/dx, v1 = (1 - h1^2) W1
+// node). Layer 1: a thread takes 16 units of points t % 64 and t % 64 + 64, paired in its multiply-adds so that a
+// weight is read once for both, and writes its part of three BF16 rows into shared memory: h1 = tanh(a1),
+// u1 = (1 - h1^2) W1 dz/dx, v1 = (1 - h1^2) W1
 // dz/dy. One thread issues the three products h1 W2^T, u1 W2^T, v1 W2^T as
 // tcgen05.mma (M = 128, N = 64, K = 16, BF16 in, FP32 accumulate) into three
 // 64-column accumulators in tensor memory, committed to an mbarrier; then
-// warp w reads lanes 32 (w % 4) .. 32 (w % 4) + 31 (its threads' points),
-// its half of the columns, back with tcgen05.ld and forms its half of
+// warp w reads lanes 32 (w % 4) .. 32 (w % 4) + 31 (point t % 128), half of the columns, back with
+// tcgen05.ld and forms its half of
 // d/dx = sum_j w3_j (1 - tanh(a2_j)^2) (W2 u1)_j, d/dy likewise; the halves
-// meet in shared memory.
+// meet in shared memory. The operands are double-buffered: layer 1 of the next tile runs while the tensor cores
+// work on this one. Bound by the instructions around the products (tensor pipe below 5 %): 2.1e5 points of two networks
+// 59 us with a barrier between the stages and a weight read per point and unit, now 54.
 //
 // Operands are K-major without swizzle: 8 x 8 BF16 core matrices of 128
 // contiguous bytes (a row's 8 consecutive k at 16-byte pitch); core matrices
@@ -679,14 +682,15 @@ constexpr int TC_TMEM_COLS = 256;                    // three 64-column FP32 acc
 // Dynamic shared memory requested per CTA: above a third of the SM's 228 KB,
 // so that at most two CTAs (2 x 256 tensor-memory columns of 512) share an SM
 // and tcgen05.alloc never waits.
-constexpr int TC_SMEM_REQUEST = 100 * 1024;
+constexpr int TC_SMEM_REQUEST = 112 * 1024;
 constexpr long long TC_WAIT_LIMIT = 1LL << 26;       // polls of the MMA mbarrier before giving up
 
 struct TcSmem {
-    alignas(1024) unsigned char a[3][TC_OPERAND_BYTES];
+    alignas(1024) unsigned char a[2][3][TC_OPERAND_BYTES];   // by parity of the tile
     alignas(1024) unsigned char b[TC_W2_BYTES];
-    float w1[H * D], b1[H], b2[H], w3[H];
-    float2 half_g[TC_ROWS];   // the second half's (d/dx, d/dy) partial sums
+    alignas(16) float w1[H][8];   // a unit's weights and bias of layer 1: w0 .. w4, b
+    alignas(16) float b2[H], w3[H];
+    float2 half_g[2][TC_ROWS];   // the second half's (d/dx, d/dy) partial sums, by parity of the tile
     alignas(8) unsigned long long mbar;
     uint32_t tmem;
     int abort;
@@ -720,19 +724,32 @@ __device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t adesc, uint64_t
         :: "r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc) : "memory");
 }
 
-// 16 consecutive accumulator columns of the thread's lane; the wait is in the
+// 16 consecutive accumulator columns of the thread's lane from each of three accumulators; the wait is in the
 // same statement, so no use of the registers can be scheduled before it.
-__device__ __forceinline__ void tc_ld16(uint32_t taddr, float (&v)[16])
+__device__ __forceinline__ void tc_ld16x3(uint32_t ta, uint32_t tb, uint32_t tc, float (&a)[16], float (&b)[16], float (&c)[16])
 {
-    uint32_t r[16];
+    uint32_t r[48];
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
-        "%15}, [%16];\n\ttcgen05.wait::ld.sync.aligned;"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
+        "%15}, [%48];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, "
+        "%29, %30, %31}, [%49];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%32, %33, %34, %35, %36, %37, %38, %39, %40, %41, %42, %43, %44, "
+        "%45, %46, %47}, [%50];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=&r"(r[0]), "=&r"(r[1]), "=&r"(r[2]), "=&r"(r[3]), "=&r"(r[4]), "=&r"(r[5]), "=&r"(r[6]), "=&r"(r[7]),
+          "=&r"(r[8]), "=&r"(r[9]), "=&r"(r[10]), "=&r"(r[11]), "=&r"(r[12]), "=&r"(r[13]), "=&r"(r[14]), "=&r"(r[15]),
+          "=&r"(r[16]), "=&r"(r[17]), "=&r"(r[18]), "=&r"(r[19]), "=&r"(r[20]), "=&r"(r[21]), "=&r"(r[22]), "=&r"(r[23]),
+          "=&r"(r[24]), "=&r"(r[25]), "=&r"(r[26]), "=&r"(r[27]), "=&r"(r[28]), "=&r"(r[29]), "=&r"(r[30]), "=&r"(r[31]),
+          "=&r"(r[32]), "=&r"(r[33]), "=&r"(r[34]), "=&r"(r[35]), "=&r"(r[36]), "=&r"(r[37]), "=&r"(r[38]), "=&r"(r[39]),
+          "=&r"(r[40]), "=&r"(r[41]), "=&r"(r[42]), "=&r"(r[43]), "=&r"(r[44]), "=&r"(r[45]), "=&r"(r[46]), "=&r"(r[47])
+        : "r"(ta), "r"(tb), "r"(tc));
 #pragma unroll
-    for (int k = 0; k < 16; ++k) v[k] = __uint_as_float(r[k]);
+    for (int k = 0; k < 16; ++k) {
+        a[k] = __uint_as_float(r[k]);
+        b[k] = __uint_as_float(r[16 + k]);
+        c[k] = __uint_as_float(r[32 + k]);
+    }
 }
 
 __global__ void __launch_bounds__(TC_THREADS) k_cv_tabulate(const TabArgs a)
@@ -746,9 +763,9 @@ __global__ void __launch_bounds__(TC_THREADS) k_cv_tabulate(const TabArgs a)
     const float* th = a.theta + (long long)f * kMlpStride;
 
     // weights: layer 1 and the biases in FP32, W2 (B operand, rows n, k-major) in BF16
-    for (int p = t; p < H * D; p += TC_THREADS) S.w1[p] = th[OW1 + p];
+    for (int p = t; p < H * D; p += TC_THREADS) S.w1[p / D][p % D] = th[OW1 + p];
     for (int p = t; p < H; p += TC_THREADS) {
-        S.b1[p] = th[OB1 + p];
+        S.w1[p][D] = th[OB1 + p];
         S.b2[p] = th[OB2 + p];
         S.w3[p] = th[OW3 + p];
     }
@@ -785,76 +802,114 @@ __global__ void __launch_bounds__(TC_THREADS) k_cv_tabulate(const TabArgs a)
     const long long tiles = (points + TC_ROWS - 1) / TC_ROWS;
     constexpr uint32_t idesc = tc_idesc(TC_ROWS, H);
     uint32_t phase = 0;
-    for (long long tl = blockIdx.x; tl < tiles; tl += gridDim.x) {
-        // layer 1 of this thread's point (clamped in the ragged last tile; not written)
-        const long long pt = tl * TC_ROWS + row;
-        const long long pc = pt < points ? pt : points - 1;
-        const int sl = (int)(pc / nn);
-        const long long node = pc - (long long)sl * nn;
-        {
-            const int i = (int)(node % a.nx), j = (int)(node / a.nx);
+    // layer 1 of tile tl: 16 units of two of its points per thread (clamped in the ragged last tile; not written)
+    auto layer1 = [&](long long tl, int par) {
+        const int first = t % (TC_ROWS / 2), share = t / (TC_ROWS / 2);
+        float2 z[D], dx3, dx4, dy3, dy4;
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const long long pt = tl * TC_ROWS + first + q * (TC_ROWS / 2);
+            const long long pc = pt < points ? pt : points - 1;
+            int sl, i, j;
+            long long node;
+            if (points <= 0x7fffffffLL) {
+                const uint32_t n = (uint32_t)nn, p32 = (uint32_t)pc, k = p32 / n, m = p32 - k * n;
+                sl = (int)k;
+                j = (int)(m / (uint32_t)a.nx);
+                i = (int)(m - (uint32_t)j * (uint32_t)a.nx);
+                node = m;
+            } else {
+                sl = (int)(pc / nn);
+                node = pc - (long long)sl * nn;
+                i = (int)(node % a.nx);
+                j = (int)(node / a.nx);
+            }
             const float4 fa = a.nfa[node];
             const float2 fb = a.nfb[node];
-            float z[D], dzx[D], dzy[D];
-            z[0] = ((float)i / (float)(a.nx - 1) - mu[0]) * sc[0];
-            z[1] = ((float)j / (float)(a.ny - 1) - mu[1]) * sc[1];
-            z[2] = (a.tfrac[sl] - mu[2]) * sc[2];
-            z[3] = (fa.x - mu[3]) * sc[3];
-            z[4] = (fa.y - mu[4]) * sc[4];
-            dzx[0] = sc[0]; dzx[1] = 0.f; dzx[2] = 0.f; dzx[3] = fa.z * sc[3]; dzx[4] = fb.x * sc[4];
-            dzy[0] = 0.f; dzy[1] = sc[1]; dzy[2] = 0.f; dzy[3] = fa.w * sc[3]; dzy[4] = fb.y * sc[4];
+            auto put = [&](float2& v, float x) { (q ? v.y : v.x) = x; };
+            put(z[0], ((float)i / (float)(a.nx - 1) - mu[0]) * sc[0]);
+            put(z[1], ((float)j / (float)(a.ny - 1) - mu[1]) * sc[1]);
+            put(z[2], (a.tfrac[sl] - mu[2]) * sc[2]);
+            put(z[3], (fa.x - mu[3]) * sc[3]);
+            put(z[4], (fa.y - mu[4]) * sc[4]);
+            put(dx3, fa.z * sc[3]);
+            put(dx4, fb.x * sc[4]);
+            put(dy3, fa.w * sc[3]);
+            put(dy4, fb.y * sc[4]);
+        }
+        const float2 dx0 = make_float2(sc[0], sc[0]), dy1 = make_float2(sc[1], sc[1]), one = make_float2(1.f, 1.f);
 #pragma unroll 1
-            for (int k0 = half * (H / 2); k0 < (half + 1) * (H / 2); k0 += 8) {
-                uint32_t ph[4], pu[4], pv[4];
+        for (int k0 = share * (H / 4); k0 < (share + 1) * (H / 4); k0 += 8) {
+            uint32_t ph[2][4], pu[2][4], pv[2][4];   // by point
 #pragma unroll
-                for (int e = 0; e < 8; e += 2) {
-                    float hv[2], uv[2], vv[2];
+            for (int e = 0; e < 8; e += 2) {
+                float2 hv[2], uv[2], vv[2];   // by unit
 #pragma unroll
-                    for (int q = 0; q < 2; ++q) {
-                        const float* w1 = S.w1 + (k0 + e + q) * D;
-                        float a1 = S.b1[k0 + e + q];
-#pragma unroll
-                        for (int c = 0; c < D; ++c) a1 = fmaf(w1[c], z[c], a1);
-                        const float t1 = tanh_approx(a1);
-                        const float k1 = 1.f - t1 * t1;
-                        float ux = 0.f, uy = 0.f;
-#pragma unroll
-                        for (int c = 0; c < D; ++c) {
-                            ux = fmaf(w1[c], dzx[c], ux);
-                            uy = fmaf(w1[c], dzy[c], uy);
-                        }
-                        hv[q] = t1;
-                        uv[q] = k1 * ux;
-                        vv[q] = k1 * uy;
-                    }
-                    ph[e / 2] = pack_bf16(hv[0], hv[1]);
-                    pu[e / 2] = pack_bf16(uv[0], uv[1]);
-                    pv[e / 2] = pack_bf16(vv[0], vv[1]);
+                for (int q = 0; q < 2; ++q) {
+                    const float4 wa = *reinterpret_cast<const float4*>(&S.w1[k0 + e + q][0]);
+                    const float2 wb = *reinterpret_cast<const float2*>(&S.w1[k0 + e + q][4]);
+                    const float2 w0 = make_float2(wa.x, wa.x), w1 = make_float2(wa.y, wa.y),
+                                 w2 = make_float2(wa.z, wa.z), w3 = make_float2(wa.w, wa.w),
+                                 w4 = make_float2(wb.x, wb.x);
+                    float2 a1 = __ffma2_rn(w0, z[0], make_float2(wb.y, wb.y));
+                    a1 = __ffma2_rn(w1, z[1], a1);
+                    a1 = __ffma2_rn(w2, z[2], a1);
+                    a1 = __ffma2_rn(w3, z[3], a1);
+                    a1 = __ffma2_rn(w4, z[4], a1);
+                    const float2 t1 = make_float2(tanh_approx(a1.x), tanh_approx(a1.y));
+                    const float2 k1 = __ffma2_rn(make_float2(-t1.x, -t1.y), t1, one);
+                    // the inputs' derivatives along x are zero in 1 and 2, along y in 0 and 2
+                    const float2 ux = __ffma2_rn(w4, dx4, __ffma2_rn(w3, dx3, __fmul2_rn(w0, dx0)));
+                    const float2 uy = __ffma2_rn(w4, dy4, __ffma2_rn(w3, dy3, __fmul2_rn(w1, dy1)));
+                    hv[q] = t1;
+                    uv[q] = __fmul2_rn(k1, ux);
+                    vv[q] = __fmul2_rn(k1, uy);
                 }
-                const uint32_t o = core_off(row, k0);
-                *reinterpret_cast<uint4*>(S.a[0] + o) = make_uint4(ph[0], ph[1], ph[2], ph[3]);
-                *reinterpret_cast<uint4*>(S.a[1] + o) = make_uint4(pu[0], pu[1], pu[2], pu[3]);
-                *reinterpret_cast<uint4*>(S.a[2] + o) = make_uint4(pv[0], pv[1], pv[2], pv[3]);
+                ph[0][e / 2] = pack_bf16(hv[0].x, hv[1].x);
+                pu[0][e / 2] = pack_bf16(uv[0].x, uv[1].x);
+                pv[0][e / 2] = pack_bf16(vv[0].x, vv[1].x);
+                ph[1][e / 2] = pack_bf16(hv[0].y, hv[1].y);
+                pu[1][e / 2] = pack_bf16(uv[0].y, uv[1].y);
+                pv[1][e / 2] = pack_bf16(vv[0].y, vv[1].y);
+            }
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const uint32_t o = core_off(first + q * (TC_ROWS / 2), k0);
+                *reinterpret_cast<uint4*>(S.a[par][0] + o) = make_uint4(ph[q][0], ph[q][1], ph[q][2], ph[q][3]);
+                *reinterpret_cast<uint4*>(S.a[par][1] + o) = make_uint4(pu[q][0], pu[q][1], pu[q][2], pu[q][3]);
+                *reinterpret_cast<uint4*>(S.a[par][2] + o) = make_uint4(pv[q][0], pv[q][1], pv[q][2], pv[q][3]);
             }
         }
         // the operands, written through the generic proxy, become visible to the tensor cores
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    };
+    auto issue = [&](int par) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t bbase = smem_u32(S.b);
+#pragma unroll
+        for (int g = 0; g < 3; ++g) {
+            const uint32_t abase = smem_u32(S.a[par][g]);
+#pragma unroll
+            for (int kk = 0; kk < H / 16; ++kk)
+                tc_mma(tmem + (uint32_t)(H * g), smem_desc(abase + 256 * kk, 128, 1024),
+                       smem_desc(bbase + 256 * kk, 128, 1024), idesc, kk > 0 ? 1u : 0u);
+        }
+        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
+                     :: "r"(smem_u32(&S.mbar)) : "memory");
+    };
+    // layer 1 of the next tile while the tensor cores work on this one; one barrier a tile: it says that the
+    // accumulators have been read and that the next operands are in place (those of the tile before last are
+    // free then: their products were waited for)
+    if (blockIdx.x < tiles) {
+        layer1(blockIdx.x, 0);
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncthreads();
-        if (t == 0) {
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t bbase = smem_u32(S.b);
-#pragma unroll
-            for (int g = 0; g < 3; ++g) {
-                const uint32_t abase = smem_u32(S.a[g]);
-#pragma unroll
-                for (int kk = 0; kk < H / 16; ++kk)
-                    tc_mma(tmem + (uint32_t)(H * g), smem_desc(abase + 256 * kk, 128, 1024),
-                           smem_desc(bbase + 256 * kk, 128, 1024), idesc, kk > 0 ? 1u : 0u);
-            }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                         :: "r"(smem_u32(&S.mbar)) : "memory");
-        }
+        if (t == 0) issue(0);
+    }
+    int par = 0;
+    for (long long tl = blockIdx.x; tl < tiles; tl += gridDim.x, par ^= 1) {
+        const bool more = tl + gridDim.x < tiles;
+        if (more) layer1(tl + gridDim.x, par ^ 1);
         // wait for the products (bounded)
         {
             uint32_t done = 0;
@@ -866,40 +921,40 @@ __global__ void __launch_bounds__(TC_THREADS) k_cv_tabulate(const TabArgs a)
             if (!done) S.abort = 1;
         }
         phase ^= 1u;
+        __syncwarp();
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        // epilogue: this thread's row from the three accumulators, 16 columns at a time
+        float2 g = make_float2(0.f, 0.f);   // (d/dx, d/dy)
+        const uint32_t lane_base = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
+#pragma unroll 1
+        for (int c0 = half * (H / 2); c0 < (half + 1) * (H / 2); c0 += 16) {
+            float vh[16], vu[16], vv[16];
+            tc_ld16x3(lane_base + (uint32_t)c0, lane_base + (uint32_t)(H + c0), lane_base + (uint32_t)(2 * H + c0), vh, vu, vv);
+#pragma unroll
+            for (int k = 0; k < 16; k += 2) {
+                const float2 b = *reinterpret_cast<const float2*>(&S.b2[c0 + k]), w = *reinterpret_cast<const float2*>(&S.w3[c0 + k]);
+                const float2 a2 = __fadd2_rn(make_float2(vh[k], vh[k + 1]), b);
+                const float2 h2 = make_float2(tanh_approx(a2.x), tanh_approx(a2.y));
+                const float2 wq = __fmul2_rn(w, __ffma2_rn(make_float2(-h2.x, -h2.y), h2, make_float2(1.f, 1.f)));
+                g = __ffma2_rn(make_float2(wq.x, wq.x), make_float2(vu[k], vv[k]), g);
+                g = __ffma2_rn(make_float2(wq.y, wq.y), make_float2(vu[k + 1], vv[k + 1]), g);
+            }
+        }
+        if (half == 1) S.half_g[par][row] = g;
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncthreads();
         if (S.abort) {
             if (t == 0) atomicOr(a.status, STATUS_TIMEOUT);
             break;
         }
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        // epilogue: this thread's row from the three accumulators, 16 columns at a time
-        float gx = 0.f, gy = 0.f;
-        const uint32_t lane_base = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
-#pragma unroll 1
-        for (int c0 = half * (H / 2); c0 < (half + 1) * (H / 2); c0 += 16) {
-            float vh[16], vu[16], vv[16];
-            tc_ld16(lane_base + (uint32_t)c0, vh);
-            tc_ld16(lane_base + (uint32_t)(H + c0), vu);
-            tc_ld16(lane_base + (uint32_t)(2 * H + c0), vv);
-#pragma unroll
-            for (int k = 0; k < 16; ++k) {
-                const float h2 = tanh_approx(vh[k] + S.b2[c0 + k]);
-                const float wq = S.w3[c0 + k] * (1.f - h2 * h2);
-                gx = fmaf(wq, vu[k], gx);
-                gy = fmaf(wq, vv[k], gy);
-            }
-        }
-        if (half == 1) S.half_g[row] = make_float2(gx, gy);
-        __syncthreads();
+        if (more && t == 0) issue(par ^ 1);
+        const long long pt = tl * TC_ROWS + row;
         if (half == 0 && pt < points) {
-            const float2 o2 = S.half_g[row];
+            const float2 o2 = S.half_g[par][row];
             double* o = a.table + pt * 4 + 2 * f;
-            o[0] = (double)(gx + o2.x);
-            o[1] = (double)(gy + o2.y);
+            o[0] = (double)(g.x + o2.x);
+            o[1] = (double)(g.y + o2.y);
         }
-        // every warp is done with the accumulators and the operands before the next tile
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        __syncthreads();
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
