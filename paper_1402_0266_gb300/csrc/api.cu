@@ -864,7 +864,7 @@ sdd_status setup_solver(sdd_ctx* c)
     if (!c->systems.empty())
         CU(c, cudaMemcpy(c->d_systems.p, c->systems.data(), c->systems.size() * sizeof(SolveSys),
                          cudaMemcpyHostToDevice));
-    CU(c, c->d_iters.alloc(2 * std::max<size_t>(std::max(c->systems.size(), subs.size()), 1)));
+    CU(c, c->d_iters.alloc(std::max<size_t>(std::max(c->systems.size(), subs.size()), 1)));
 
     // multigrid: every subdomain the same odd sizes, coarsening down to a small box
     c->mg_ok = false;

@@ -109,7 +109,6 @@ __global__ void __launch_bounds__(SOLVE_THREADS) k_pcg_cluster(const SolveArgs a
     cg::cluster_group cl = cg::this_cluster();
     const int C = (int)cl.num_blocks();
     const int rank = (int)cl.block_rank();
-    if (a.iters[a.nsys + blockIdx.x / C]) return;   // solved by k_cheb
     const SolveSys S = a.sys[blockIdx.x / C];
     const int nx = a.nx;
     const int mx = S.i1 - S.i0, my = S.j1 - S.j0;
@@ -221,14 +220,23 @@ __global__ void __launch_bounds__(SOLVE_THREADS) k_pcg_cluster(const SolveArgs a
     cl.sync();  // no block leaves while others may still read its shared memory
 }
 
-// Chebyshev iterations for subdomains whose bands fit the blocks of a cluster, both fields together. Solves with
-// their set-up, before and after: 4 x 19^2 unknowns 157 -> 71 us, 4 x 63^2 520 -> 156, 9 x 65^2 1358 -> 288,
-// 9 x 119^2 2918 -> 875, 16 x 95^2 2548 -> 1272. The method:
+// log2 of a positive normal double, off the double-precision lanes (the library's logarithm and a division
+// were 2 us of latency a sweep).
+__device__ __forceinline__ float log2_of(double v)
+{
+    const int hi = __double2hiint(v);
+    return (float)((hi >> 20) - 1023) + log2f(__int_as_float(0x3F800000 | ((hi & 0xFFFFF) << 3)));
+}
+
+// Chebyshev iterations for subdomains whose bands fit the blocks of a cluster, both fields together, and
+// conjugate gradients (cg_solve) in the same launch for what they leave. Solves with their set-up, conjugate gradients
+// alone and now: 4 x 19^2 unknowns 157 -> 54 us, 4 x 63^2 520 -> 136, 9 x 65^2 1358 -> 256, 9 x 119^2 2918 -> 819,
+// 16 x 95^2 2548 -> 1283 (a launch of its own for cg_solve and the library's logarithm cost 17 us more). The method:
 // A d = r with the diagonal as preconditioner over the interval [lo, 1 + rho] of the eigenvalues of
 // D^-1 A, in single precision, inside the double-precision refinement of the other kernels.
 // rho is Gershgorin's bound, the largest row sum of D^-1 (D - A) (below 1: the mass term), so the upper
 // end holds; lo adds to 1 - rho most of what the Dirichlet frame contributes with uniform coefficients.
-// Where that is too much, the modes below lo fall more slowly than the rest, never grow, and k_pcg_cg2,
+// Where that is too much, the modes below lo fall more slowly than the rest, never grow, and cg_solve,
 // which closes every solve, takes them over.
 //
 // Why not conjugate gradients alone: an iteration of theirs is a product, two barriers and a reduction of
@@ -240,10 +248,11 @@ __global__ void __launch_bounds__(SOLVE_THREADS) k_pcg_cluster(const SolveArgs a
 // correction e) in registers; the steps d live in shared memory as pairs (both fields), a zero frame around
 // the band and halo rows that the neighbouring blocks store into before the barrier. Planes alternate with the
 // iteration's parity: a plane is rewritten only after the next iteration's barrier, which every reader has passed.
+//
+// planes: [parity] (rows_max + 2) x (mx + 2). True if the systems are solved; total: the iterations.
 template <int UPT, bool ONE>
-__global__ void __launch_bounds__(SOLVE_THREADS) k_cheb(const SolveArgs a, int rows_max)
+__device__ __forceinline__ bool cheb_solve(const SolveArgs& a, int rows_max, float2* planes, int& total)
 {
-    extern __shared__ float2 planes[];   // [parity]: (rows_max + 2) x (mx + 2)
     __shared__ ClusterSlots<double> red64[2];
     __shared__ float warp_max[SOLVE_WARPS], block_max;
     cg::cluster_group cl = cg::this_cluster();
@@ -322,7 +331,8 @@ __global__ void __launch_bounds__(SOLVE_THREADS) k_cheb(const SolveArgs a, int r
     const float theta = 0.5f * (hi + lo), delta = 0.5f * (hi - lo), sigma = theta / delta;
     const float per_iter = logf(sigma + sqrtf((sigma - 1.f) * (sigma + 1.f)));
 
-    int total = 0, b = 0;
+    int b = 0;
+    total = 0;
     bool converged = false;
     for (int sweep = 0; sweep < 6; ++sweep) {
         // the residual, double precision
@@ -350,7 +360,7 @@ __global__ void __launch_bounds__(SOLVE_THREADS) k_cheb(const SolveArgs a, int r
 #pragma unroll
         for (int f = 0; f < 2; ++f) {
             active[f] = rr[f] > stop2[f];
-            if (active[f]) left = fmaxf(left, stop2[f] > 0.0 ? 0.5f * (float)log(rr[f] / stop2[f]) : 100.f);
+            if (active[f]) left = fmaxf(left, stop2[f] > 0.0 ? 0.34657359f * (log2_of(rr[f]) - log2_of(stop2[f])) : 100.f);
             else
 #pragma unroll
                 for (int k = 0; k < UPT; ++k) z[f][k] = 0.f;
@@ -362,6 +372,7 @@ __global__ void __launch_bounds__(SOLVE_THREADS) k_cheb(const SolveArgs a, int r
         if (total >= min(a.max_iter, 4000)) break;
         total += its;
         float r_old = 1.f / sigma, ca = 0.f, cb = 1.f / theta;
+        const float two_delta = 2.f / delta;
         for (int it = 0; it < its; ++it, b ^= 1) {
             float2* mine = planes + b * plane;
 #pragma unroll
@@ -380,9 +391,9 @@ __global__ void __launch_bounds__(SOLVE_THREADS) k_cheb(const SolveArgs a, int r
                     if (lr == rows - 1 && nb_hi) nb_hi[b * plane + sidx[k] - rows * W] = v;
                 }
             }
-            const float r_new = 1.f / (2.f * sigma - r_old);
+            const float r_new = __frcp_rn(2.f * sigma - r_old);
             ca = r_new * r_old;
-            cb = 2.f * r_new / delta;
+            cb = r_new * two_delta;
             r_old = r_new;
             sync();
 #pragma unroll
@@ -402,15 +413,11 @@ __global__ void __launch_bounds__(SOLVE_THREADS) k_cheb(const SolveArgs a, int r
             }
         sync();   // the next residual reads the neighbours' x
     }
-    if (threadIdx.x == 0 && rank == 0) {
-        a.iters[blockIdx.x / C] = total;
-        a.iters[a.nsys + blockIdx.x / C] = converged ? 1 : 0;
-    }
-    if (!ONE) cl.sync();   // no block leaves while others may still write into its shared memory
+    return converged;   // the sum before has a barrier: no block writes into another's planes any more
 }
 
-// Register-resident conjugate gradients for subdomains whose band fits in the block, run after k_cheb on
-// the systems that it left short of rtol (little mass, strong contrasts: the modes below its interval):
+// Register-resident conjugate gradients for subdomains whose band fits in the block, for
+// the systems that cheb_solve left short of rtol (little mass, strong contrasts: the modes below its interval):
 // one cluster solves both fields of a subdomain (same matrix, two right-hand
 // sides), so the cluster barriers are shared by the two solves. Each thread
 // keeps UPT unknowns (coefficients and, per field, the CG vectors) in
@@ -425,10 +432,11 @@ __global__ void __launch_bounds__(SOLVE_THREADS) k_cheb(const SolveArgs a, int r
 // double-buffered by the iteration's parity; a buffer is rewritten only two
 // barriers after it was read. A field that has converged stops changing
 // while the other one finishes.
+//
+// m_s: u, [parity][field] planes of (rows_max + 2) x (mx + 2), zero frame. before: iterations already made.
 template <int UPT, bool ONE>
-__global__ void __launch_bounds__(SOLVE_THREADS) k_pcg_cg2(const SolveArgs a, int rows_max)
+__device__ __forceinline__ void cg_solve(const SolveArgs& a, int rows_max, float* m_s, int before)
 {
-    extern __shared__ float m_s[];  // u: [parity][field] planes of (rows_max + 2) x (mx + 2), zero frame
     __shared__ float slots[2][16][8];   // [parity][block]: (gamma, delta, rr) of field 0, then field 1
     __shared__ float warp_part[2][SOLVE_WARPS][8];
     cg::cluster_group cl = cg::this_cluster();
@@ -439,7 +447,6 @@ __global__ void __launch_bounds__(SOLVE_THREADS) k_pcg_cg2(const SolveArgs a, in
         if (ONE) __syncthreads();
         else cl.sync();
     };
-    if (a.iters[a.nsys + blockIdx.x / C]) return;   // solved by k_cheb
     const SolveSys S = a.sys[blockIdx.x / C];
     const int nx = a.nx;
     const int mx = S.i1 - S.i0, my = S.j1 - S.j0;
@@ -679,10 +686,26 @@ __global__ void __launch_bounds__(SOLVE_THREADS) k_pcg_cg2(const SolveArgs a, in
         sync();
     }
     if (threadIdx.x == 0 && rank == 0) {
-        a.iters[blockIdx.x / C] = converged ? total + a.iters[blockIdx.x / C] : a.max_iter + 1;
+        a.iters[blockIdx.x / C] = converged ? total + before : a.max_iter + 1;
         if (!converged) atomicOr(a.status, STATUS_NOCONV);
     }
     if (!ONE) cl.sync();  // no block leaves while others may still write into its shared memory
+}
+
+template <int UPT, bool ONE>
+__global__ void __launch_bounds__(SOLVE_THREADS) k_solve(const SolveArgs a, int rows_max)
+{
+    extern __shared__ __align__(16) unsigned char solve_smem[];
+    int total;
+    const bool solved = cheb_solve<UPT, ONE>(a, rows_max, reinterpret_cast<float2*>(solve_smem), total);
+    if (!solved) {
+        cg_solve<UPT, ONE>(a, rows_max, reinterpret_cast<float*>(solve_smem), total);
+        return;
+    }
+    cg::cluster_group cl = cg::this_cluster();
+    const int C = ONE ? 1 : (int)cl.num_blocks();
+    if (threadIdx.x == 0 && (ONE || cl.block_rank() == 0)) a.iters[blockIdx.x / C] = total;
+    if (!ONE) cl.sync();   // no block leaves while others may still read its shared memory
 }
 
 __global__ void k_bump_step(uint32_t* step)
@@ -739,7 +762,7 @@ static int clusters_at_once(int k)
 {
     static int at_once[5] = {-1, -1, -1, -1, -1};
     if (at_once[k] < 0) {
-        const auto fn = k_cheb<4, false>;
+        const auto fn = k_solve<4, false>;
         cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(1u << k);
@@ -759,7 +782,7 @@ static int clusters_at_once(int k)
 }
 
 // Blocks per system (a power of two up to 16, no more than the smallest system's rows) for systems of at
-// most max_mx columns and max_my rows: the least time by what k_cheb measured, rounds of clusters that run
+// most max_mx columns and max_my rows: the least time by what the Chebyshev iterations measured, rounds of clusters that run
 // at once x (0.4 us + 0.25 us per unknown of a thread) an iteration. One block (no cluster barrier) pays for
 // up to 256 unknowns; above, its SM's few double-precision units make the residuals longer than the barrier.
 // Bands that need more than 4 unknowns per thread leave the register-resident kernels and are the last choice.
@@ -801,7 +824,7 @@ template <int UPT>
 static cudaError_t launch_reg(const SolveArgs& a, int rows_max, int max_mx, cudaStream_t s)
 {
     const size_t smem = 4 * (size_t)(rows_max + 2) * (size_t)(max_mx + 2) * sizeof(float);
-    const auto fn = a.cluster == 1 ? k_pcg_cg2<UPT, true> : k_pcg_cg2<UPT, false>;
+    const auto fn = a.cluster == 1 ? k_solve<UPT, true> : k_solve<UPT, false>;
     if (a.cluster > 8) cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -810,23 +833,6 @@ static cudaError_t launch_reg(const SolveArgs& a, int rows_max, int max_mx, cuda
     cudaLaunchAttribute at[1];
     cudaLaunchConfig_t cfg = cluster_config(a, smem, s, at);
     // no more warps than the largest band needs (their sums cost exchanges)
-    const int band = rows_max * max_mx;
-    cfg.blockDim = dim3((unsigned)std::min(SOLVE_THREADS, ((band + UPT - 1) / UPT + 31) / 32 * 32));
-    return cudaLaunchKernelEx(&cfg, fn, a, rows_max);
-}
-
-template <int UPT>
-static cudaError_t launch_cheb(const SolveArgs& a, int rows_max, int max_mx, cudaStream_t s)
-{
-    const size_t smem = 2 * (size_t)(rows_max + 2) * (size_t)(max_mx + 2) * sizeof(float2);
-    const auto fn = a.cluster == 1 ? k_cheb<UPT, true> : k_cheb<UPT, false>;
-    if (a.cluster > 8) cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
-    cudaLaunchAttribute at[1];
-    cudaLaunchConfig_t cfg = cluster_config(a, smem, s, at);
     const int band = rows_max * max_mx;
     cfg.blockDim = dim3((unsigned)std::min(SOLVE_THREADS, ((band + UPT - 1) / UPT + 31) / 32 * 32));
     return cudaLaunchKernelEx(&cfg, fn, a, rows_max);
@@ -846,11 +852,10 @@ int solve_reg_upt(int max_band_unknowns)
 cudaError_t launch_pcg(const SolveArgs& a, int upt, int rows_max, int max_mx, cudaStream_t s)
 {
     if (a.nsys <= 0) return cudaSuccess;
-    cudaError_t e;
     switch (upt) {
-    case 1: return (e = launch_cheb<1>(a, rows_max, max_mx, s)) != cudaSuccess ? e : launch_reg<1>(a, rows_max, max_mx, s);
-    case 2: return (e = launch_cheb<2>(a, rows_max, max_mx, s)) != cudaSuccess ? e : launch_reg<2>(a, rows_max, max_mx, s);
-    case 4: return (e = launch_cheb<4>(a, rows_max, max_mx, s)) != cudaSuccess ? e : launch_reg<4>(a, rows_max, max_mx, s);
+    case 1: return launch_reg<1>(a, rows_max, max_mx, s);
+    case 2: return launch_reg<2>(a, rows_max, max_mx, s);
+    case 4: return launch_reg<4>(a, rows_max, max_mx, s);
     default: {
         if (a.cluster > 8) cudaFuncSetAttribute(k_pcg_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         cudaLaunchAttribute at[1];
