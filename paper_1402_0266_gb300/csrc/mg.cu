@@ -26,6 +26,7 @@
 // CUDA graph whose while-nodes stop once every field has converged; systems
 // (and fields) that have converged before stop changing.
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
 
@@ -380,18 +381,82 @@ __global__ void __launch_bounds__(TAIL_THREADS) k_mg_tail(const MgArgs a)
     __syncthreads();
     for (int l = lt; l < L; ++l) {
         const Lv v = level(a, l, s);
-        for (int k = threadIdx.x; k < v.W * v.H; k += TAIL_THREADS) {
-            const long long e = v.off + k;
-            const float d = a.D[e];
-            T.id[l][k] = d > 0.f ? 1.f / d : 0.f;
-            T.cx[l][k] = a.CX[e];
-            T.cy[l][k] = a.CY[e];
-            T.u[l][k] = make_float2(0.f, 0.f);
-            T.f[l][k] = l == lt ? make_float2(a.F[0][e], a.F[1][e]) : make_float2(0.f, 0.f);
+        const int n = v.W * v.H;
+        // five nodes a thread in flight (a 65^2 box in one round)
+        constexpr int BATCH = 5;
+        for (int k0 = threadIdx.x; k0 < n; k0 += BATCH * TAIL_THREADS) {
+            float d[BATCH], cx[BATCH], cy[BATCH];
+            float2 f[BATCH];
+#pragma unroll
+            for (int q = 0; q < BATCH; ++q) {
+                const int k = k0 + q * TAIL_THREADS;
+                d[q] = 0.f;
+                f[q] = make_float2(0.f, 0.f);
+                if (k >= n) continue;
+                const long long e = v.off + k;
+                d[q] = a.D[e];
+                cx[q] = a.CX[e];
+                cy[q] = a.CY[e];
+                if (l == lt) f[q] = make_float2(a.F[0][e], a.F[1][e]);
+            }
+#pragma unroll
+            for (int q = 0; q < BATCH; ++q) {
+                const int k = k0 + q * TAIL_THREADS;
+                if (k >= n) continue;
+                T.id[l][k] = d[q] > 0.f ? 1.f / d[q] : 0.f;
+                T.cx[l][k] = cx[q];
+                T.cy[l][k] = cy[q];
+                T.u[l][k] = make_float2(0.f, 0.f);
+                T.f[l][k] = f[q];
+            }
         }
     }
     __syncthreads();
+    // the first level's coefficients in registers where a thread has two nodes of each colour at most
+    const int W0 = a.mx[lt] + 2;
+    const bool held = a.mx[lt] <= 64 && a.my[lt] <= 2 * WARPS;
+    float hw[2][2], he[2][2], hs[2][2], hn[2][2], hd[2][2];   // [colour][row]
+    float2 hf[2][2];
+    auto held_at = [&](int color, int r, int& e) {
+        const int j = 1 + warp + r * WARPS, i = 1 + 2 * lane + ((j + 1 + color) & 1);
+        e = j * W0 + i;
+        return j <= a.my[lt] && i <= a.mx[lt];
+    };
+#pragma unroll
+    for (int color = 0; color < 2; ++color)
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            int e;
+            hw[color][r] = he[color][r] = hs[color][r] = hn[color][r] = hd[color][r] = 0.f;
+            hf[color][r] = make_float2(0.f, 0.f);
+            if (!held || !held_at(color, r, e)) continue;
+            hw[color][r] = T.cx[lt][e - 1];
+            he[color][r] = T.cx[lt][e];
+            hs[color][r] = T.cy[lt][e - W0];
+            hn[color][r] = T.cy[lt][e];
+            hd[color][r] = T.id[lt][e];
+            hf[color][r] = T.f[lt][e];
+        }
+    auto held_sweep = [&](auto colour) {
+        constexpr int color = decltype(colour)::value;
+        float2* const u = T.u[lt];
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            int e;
+            if (!held_at(color, r, e)) continue;
+            const float2 w = u[e - 1], o = u[e + 1], t = u[e - W0], n = u[e + W0], b = hf[color][r];
+            const float cw = hw[color][r], ce = he[color][r], cs = hs[color][r], cn = hn[color][r], d = hd[color][r];
+            u[e] = make_float2((b.x + cw * w.x + ce * o.x + cs * t.x + cn * n.x) * d,
+                               (b.y + cw * w.y + ce * o.y + cs * t.y + cn * n.y) * d);
+        }
+        __syncthreads();
+    };
     auto sweep = [&](int l, int color) {
+        if (held && l == lt) {
+            if (color == 0) held_sweep(std::integral_constant<int, 0>());
+            else held_sweep(std::integral_constant<int, 1>());
+            return;
+        }
         const int mx = a.mx[l], my = a.my[l], W = mx + 2;
         float2* const u = T.u[l];
         for (int j = 1 + warp; j <= my; j += WARPS)
