@@ -335,7 +335,7 @@ __global__ void __launch_bounds__(MG_THREADS) k_mg_up(const MgArgs a, int l, int
 
 // The levels from `tail` down in shared memory, one block per system: a row of a level per warp and step, so
 // that no index is divided. The 50 phases of the levels from 63^2 down are a chain of block barriers, the
-// bound here: 51 us, 61 us with the levels in global memory. A level of at most 4096
+// bound here: 29 us (51 from a cold cache, where the levels in global memory took 61). A level of at most 4096
 // unknowns and all below it fill at most 214,200 bytes (31 x 543) over every shape that mg_levels admits.
 struct TailSmem {
     float2* u[kMgMaxLevels];
