@@ -411,9 +411,9 @@ __device__ __forceinline__ uint32_t zmap_offset(float2 p)
 constexpr int VAR_MULTI = 0, VAR_ONE = 1;
 constexpr int kOneMaxBlock = 256;
 constexpr int paths_max_block(int cvm, int var) { return cvm ? kCvMaxBlock : var != VAR_MULTI ? kOneMaxBlock : 512; }
-constexpr int paths_min_blocks(int cvm, int var, bool defer)
+constexpr int paths_min_blocks(int mode, int cvm, int var)
 {
-    return cvm ? (var != VAR_MULTI ? 4 : 3) : var != VAR_MULTI ? 5 : 2;
+    return cvm ? (var != VAR_MULTI ? 4 : 3) : var == VAR_MULTI ? 2 : mode == 1 ? 4 : 5;
 }
 
 // A lane's sums over a task, in shared memory: they change once per path, and the
@@ -512,8 +512,8 @@ __device__ __forceinline__ unsigned lanes_below()
 // in shared memory and 48 registers (40 warps per SM; 32 and 48 warps are within 2 %), a draw made
 // where it is used rather than a pass ahead (fewer registers and moves; the other warps cover the
 // gathers), and bookkeeping only when a path ends. On a 2049^2 ring (28,609 nodes x 2e4 paths x 100
-// sub-steps): 145 ms per launch against 179 ms for the kernel that tested every path in every pass
-// and redirected gathers without skipping them, 92 instructions per path-step.
+// sub-steps): 145 ms per launch and 73 instructions per path-step, against 179 ms and 92 for the kernel that tested
+// every path in every pass and redirected gathers without skipping them.
 template <int MODE, bool RECORD, int CVM, int VAR, bool DEFER, bool MAP>
 __device__ __forceinline__ void walk_tasks(const PathArgs& a, const uint8_t* zsm,
                                            LaneSums<paths_max_block(CVM, VAR), !DEFER || MODE == 1>& sums,
@@ -529,8 +529,10 @@ __device__ __forceinline__ void walk_tasks(const PathArgs& a, const uint8_t* zsm
     const int K = a.K;
     const int P = PAIRS ? (K + 1) >> 1 : K;   // passes of a path: sub-step pairs, or sub-steps
     const float2 dt2 = f2(a.dt, a.dt);
-    // records that lanes without a cell read: the all-zero one (batches: any), the first cell's
-    const uint32_t zcell = (ONE ? kCellBits : 0u) + a.zcell, cell0 = ONE ? kCellBits : 0u;
+    // records that lanes without a cell read: the all-zero one, the first cell's
+    constexpr bool READ_ZERO = MODE == 1 || CVT;
+    [[maybe_unused]] const uint32_t zcell = (ONE ? kCellBits : 0u) + a.zcell;
+    const uint32_t cell0 = ONE ? kCellBits : 0u;
 
     // Each warp takes the next task as soon as its last one is done (no wait
     // for the block's other warps); tasks go node by node, so warps started
@@ -560,6 +562,7 @@ __device__ __forceinline__ void walk_tasks(const PathArgs& a, const uint8_t* zsm
         int cvq = 0, cvn = CVT ? a.cv_bound[1] : 0;      // slice of the current sub-step, start of the next
         sums.clear();
 
+        float4 lo = make_float4(0.f, 0.f, 0.f, 0.f), hi = lo;   // the cell record read last
         // One sub-step from p with increment z, for lanes with ok (the others' results are not used,
         // and their p may lie anywhere): p + b(p) dt + z.
         auto advance = [&](float2 p, float2 z, bool ok, bool count, int j) -> float2 {
@@ -569,8 +572,16 @@ __device__ __forceinline__ void walk_tasks(const PathArgs& a, const uint8_t* zsm
             if (CV || !MAP || __any_sync(FULL, g)) {
                 Cell c = locate<ONE>(I, p);
                 if (CV) c.idx = ok ? c.idx : cell0;
-                float4 lo, hi;
-                load_cell(rec2<ONE>(I.bcoef, g ? c.idx : zcell), lo, hi);
+                // lanes without drift or path do not read: beside lanes that miss L1 their hit on the zero record costs
+                // the warp three cycles, and unread it saves one each (257^2 steps 8053 -> 7853 us, a batch of 16
+                // grids 1441 -> 1360, 1025^2 with field cells 2864 -> 2717). Bound by instructions, the bridge test and
+                // the time slices read the zero record instead of clearing eight registers (732 against 744 us, 133 against 136).
+                if (MAP && READ_ZERO) {
+                    load_cell(rec2<ONE>(I.bcoef, g ? c.idx : zcell), lo, hi);
+                } else {
+                    if (MAP && !g) lo = hi = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (g) load_cell(rec2<ONE>(I.bcoef, c.idx), lo, hi);
+                }
                 if (CV) {
                     // the model at X_j; the sub-step counts only when the path takes it
                     const float2 zt = count ? z : f2(0.f, 0.f);
@@ -727,7 +738,7 @@ __device__ __forceinline__ void walk_tasks(const PathArgs& a, const uint8_t* zsm
 }
 
 template <int MODE, bool RECORD, int CVM, int VAR, bool DEFER>
-__global__ void __launch_bounds__(paths_max_block(CVM, VAR), paths_min_blocks(CVM, VAR, DEFER))
+__global__ void __launch_bounds__(paths_max_block(CVM, VAR), paths_min_blocks(MODE, CVM, VAR))
     k_paths(const PathArgs a)
 {
     __shared__ LaneSums<paths_max_block(CVM, VAR), !DEFER || MODE == 1> sums;
