@@ -423,8 +423,8 @@ sdd_status sdd_interface_nodes(sdd_ctx* ctx, double* x, double* y, int64_t* coun
  * wbar the average of w over the two nodes, with Dirichlet data from the face
  * data on the outer boundary and from iface_xi / iface_eta (DEVICE, one
  * double per interface node in the order of sdd_interface_nodes) on the
- * interfaces. Solved in double precision by Jacobi-preconditioned conjugate
- * gradients to ||r|| <= rtol ||b|| or max_iter iterations.
+ * interfaces. Solved by the context's solver (SDD_SOLVER_*) until the double-
+ * precision residual is ||r|| <= rtol ||b||, or for max_iter iterations.
  * Outputs xi_out, eta_out: DEVICE nx*ny doubles (full fields). iters_out
  * (HOST, may be NULL): the largest iteration count over the systems; asking
  * for it waits for the solve. The context's fields are not changed.

@@ -512,7 +512,7 @@ __device__ __forceinline__ unsigned lanes_below()
 // in shared memory and 48 registers (40 warps per SM; 32 and 48 warps are within 2 %), a draw made
 // where it is used rather than a pass ahead (fewer registers and moves; the other warps cover the
 // gathers), and bookkeeping only when a path ends. On a 2049^2 ring (28,609 nodes x 2e4 paths x 100
-// sub-steps): 145 ms per launch and 73 instructions per path-step, against 179 ms and 92 for the kernel that tested
+// sub-steps): 144 ms per launch and 75 instructions per path-step, against 179 ms and 92 for the kernel that tested
 // every path in every pass and redirected gathers without skipping them.
 template <int MODE, bool RECORD, int CVM, int VAR, bool DEFER, bool MAP>
 __device__ __forceinline__ void walk_tasks(const PathArgs& a, const uint8_t* zsm,
