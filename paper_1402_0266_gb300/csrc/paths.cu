@@ -1111,6 +1111,9 @@ __global__ void __launch_bounds__(SCORE_THREADS, 4) k_score_surv(const ScoreArgs
         if (warp == 0 && rank == 0) pathless_node(a.fin, node, nd, lane);
         return;   // uniform over the cluster
     }
+    // a block's shared memory may be written by the others of its cluster once it has started: every block arrives
+    // here, and waits for all before the first remote store (the scoring lies between, so the wait is short)
+    if (C > 1) cl.barrier_arrive();
     const InstDev I = a.inst[nd.inst];
     const float x0 = nd.xf, y0 = nd.yf;
     const int first = rank * SCORE_THREADS + threadIdx.x, threads = C * SCORE_THREADS, end = nd.n_paths;
@@ -1201,6 +1204,7 @@ __global__ void __launch_bounds__(SCORE_THREADS, 4) k_score_surv(const ScoreArgs
     __syncthreads();
     if (warp == 0) tot = join_sums(part, SCORE_THREADS / 32, lane, ex, st);
     if (C > 1) {
+        cl.barrier_wait();
         if (warp == 0) put_sums(cl.map_shared_rank(blocks, 0) + rank, lane, tot, ex, st);
         cl.sync();
         if (rank == 0 && warp == 0) tot = join_sums(blocks, C, lane, ex, st);
