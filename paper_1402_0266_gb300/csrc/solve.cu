@@ -356,17 +356,18 @@ __device__ __forceinline__ bool cheb_solve(const SolveArgs& a, int rows_max, flo
         cluster_sum2(cl, red64, seq, rr[0], rr[1]);
         // iterations for what is left of the reduction, at most 1e-5 per sweep
         float left = 0.f;
-        bool active[2];
+        bool active[2], number = true;
 #pragma unroll
         for (int f = 0; f < 2; ++f) {
-            active[f] = rr[f] > stop2[f];
+            active[f] = !(rr[f] <= stop2[f]);   // so that what is not a number never counts as solved
+            number = number && (!active[f] || rr[f] > stop2[f]);
             if (active[f]) left = fmaxf(left, stop2[f] > 0.0 ? 0.34657359f * (log2_of(rr[f]) - log2_of(stop2[f])) : 100.f);
             else
 #pragma unroll
                 for (int k = 0; k < UPT; ++k) z[f][k] = 0.f;
         }
         converged = !active[0] && !active[1];
-        if (converged) break;
+        if (converged || !number) break;   // no number: cg_solve reports it
         int its = (int)ceilf((fminf(left, 11.5f) + 2.f) / per_iter);
         its = max(1, min(its, min(a.max_iter, 4000) - total));
         if (total >= min(a.max_iter, 4000)) break;
