@@ -424,7 +424,8 @@ sdd_status sdd_interface_nodes(sdd_ctx* ctx, double* x, double* y, int64_t* coun
  * data on the outer boundary and from iface_xi / iface_eta (DEVICE, one
  * double per interface node in the order of sdd_interface_nodes) on the
  * interfaces. Solved by the context's solver (SDD_SOLVER_*) until the double-
- * precision residual is ||r|| <= rtol ||b||, or for max_iter iterations.
+ * precision residual is ||r|| <= rtol ||b||, or for max_iter iterations (of
+ * both methods together where SDD_SOLVER_JACOBI uses two).
  * Outputs xi_out, eta_out: DEVICE nx*ny doubles (full fields). iters_out
  * (HOST, may be NULL): the largest iteration count over the systems; asking
  * for it waits for the solve. The context's fields are not changed.
@@ -478,8 +479,9 @@ sdd_status sdd_keypoint_fill(sdd_ctx* ctx, const uint8_t* mask, double* values_x
  *                      Jacobi-PCG on these sizes, so never chosen automatically;
  *   SDD_SOLVER_JACOBI  Jacobi preconditioner; one thread-block cluster per
  *                      subdomain; when the subdomain fits its registers,
- *                      Chebyshev iterations first (at most max_iter of
- *                      them) and conjugate gradients for what they leave;
+ *                      Chebyshev iterations first (where those that they
+ *                      need fit half of max_iter) and conjugate gradients
+ *                      for what they leave;
  *   SDD_SOLVER_MG      a geometric multigrid V-cycle as preconditioner
  *                      (available when every subdomain has the same odd
  *                      sizes that halve, (m - 1) / 2, down to a box of at

@@ -249,7 +249,8 @@ __device__ __forceinline__ float log2_of(double v)
 // the band and halo rows that the neighbouring blocks store into before the barrier. Planes alternate with the
 // iteration's parity: a plane is rewritten only after the next iteration's barrier, which every reader has passed.
 //
-// planes: [parity] (rows_max + 2) x (mx + 2). True if the systems are solved; total: the iterations.
+// planes: [parity] (rows_max + 2) x (mx + 2). True if the systems are solved; total: the iterations, at most half of
+// max_iter.
 template <int UPT, bool ONE>
 __device__ __forceinline__ bool cheb_solve(const SolveArgs& a, int rows_max, float2* planes, int& total)
 {
@@ -368,9 +369,11 @@ __device__ __forceinline__ bool cheb_solve(const SolveArgs& a, int rows_max, flo
         }
         converged = !active[0] && !active[1];
         if (converged || !number) break;   // no number: cg_solve reports it
-        int its = (int)ceilf((fminf(left, 11.5f) + 2.f) / per_iter);
-        its = max(1, min(its, min(a.max_iter, 4000) - total));
-        if (total >= min(a.max_iter, 4000)) break;
+        // max_iter bounds both methods together: what is left has to fit the half of it that is not kept for
+        // conjugate gradients, which otherwise take the system as it is
+        const float sweeps = ceilf(left / 11.5f);
+        if ((float)total + (left + 2.f * sweeps) / per_iter + sweeps > 0.5f * (float)a.max_iter) break;
+        const int its = (int)ceilf((fminf(left, 11.5f) + 2.f) / per_iter);
         total += its;
         float r_old = 1.f / sigma, ca = 0.f, cb = 1.f / theta;
         const float two_delta = 2.f / delta;
@@ -434,7 +437,7 @@ __device__ __forceinline__ bool cheb_solve(const SolveArgs& a, int rows_max, flo
 // barriers after it was read. A field that has converged stops changing
 // while the other one finishes.
 //
-// m_s: u, [parity][field] planes of (rows_max + 2) x (mx + 2), zero frame. before: iterations already made.
+// m_s: u, [parity][field] planes of (rows_max + 2) x (mx + 2), zero frame. before: iterations already made (they count towards max_iter).
 template <int UPT, bool ONE>
 __device__ __forceinline__ void cg_solve(const SolveArgs& a, int rows_max, float* m_s, int before)
 {
@@ -579,7 +582,7 @@ __device__ __forceinline__ void cg_solve(const SolveArgs& a, int rows_max, float
     cluster_sum2(cl, red64, seq, bb[0], bb[1]);
     const double stop2[2] = {a.rtol * a.rtol * bb[0], a.rtol * a.rtol * bb[1]};
 
-    int total = 0, it = 0;
+    int total = before, it = 0;
     bool converged = false;
     for (int outer = 0; outer < a.max_outer; ++outer) {
         double rr64[2] = {0.0, 0.0};
@@ -687,7 +690,7 @@ __device__ __forceinline__ void cg_solve(const SolveArgs& a, int rows_max, float
         sync();
     }
     if (threadIdx.x == 0 && rank == 0) {
-        a.iters[blockIdx.x / C] = converged ? total + before : a.max_iter + 1;
+        a.iters[blockIdx.x / C] = converged ? total : a.max_iter + 1;
         if (!converged) atomicOr(a.status, STATUS_NOCONV);
     }
     if (!ONE) cl.sync();  // no block leaves while others may still write into its shared memory
