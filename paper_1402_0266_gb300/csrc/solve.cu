@@ -242,7 +242,14 @@ __device__ __forceinline__ float log2_of(double v)
 // Why not conjugate gradients alone: an iteration of theirs is a product, two barriers and a reduction of
 // six sums, a latency chain of about 2.3 us whatever the cluster size; here it is one barrier (one block:
 // a block barrier) and a product whose operands are in registers and shared memory, with no scalar to wait
-// for. The iteration count is the same to 1.4 times theirs in this range of mass terms.
+// for: 0.5 us with one unknown a thread, 1.3 with four. The iteration count is 0.9 to 1.3 times theirs where the mass term
+// counts (4 x 119^2 unknowns: up to Dt = 1e-2) and twice theirs without it, faster still (Dt = 1: 1.24 against 2.07 ms).
+//
+// What they lose: blocks of very different density (a 50 : 1 checkerboard at Dt >= 3e-2) have modes far below lo, and
+// sweep after sweep falls short. A sweep that brings the residual down by less than a third of its factor
+// (in the logarithm) is the last: 16 x 65^2 unknowns at Dt = 0.3 take 2.15 ms with one such sweep, 3.10 with six, 2.40 in the
+// kernel that ran conjugate gradients alone before; over Dt = 1e-4 to 1e3, 9^2 to 119^2 unknowns and five densities no
+// solve takes longer than in that kernel (0.993 times at most).
 //
 // Layout: each thread keeps UPT unknowns (scaled coefficients and, per field, scaled residual z, step d,
 // correction e) in registers; the steps d live in shared memory as pairs (both fields), a zero frame around
@@ -335,6 +342,7 @@ __device__ __forceinline__ bool cheb_solve(const SolveArgs& a, int rows_max, flo
     int b = 0;
     total = 0;
     bool converged = false;
+    float goal = 1e30f;   // what a sweep has to leave at most for another (the logarithm of the reduction to come)
     for (int sweep = 0; sweep < 6; ++sweep) {
         // the residual, double precision
         double rr[2] = {0.0, 0.0};
@@ -369,6 +377,8 @@ __device__ __forceinline__ bool cheb_solve(const SolveArgs& a, int rows_max, flo
         }
         converged = !active[0] && !active[1];
         if (converged || !number) break;   // no number: cg_solve reports it
+        if (left > goal) break;            // the sweep before fell short
+        goal = left - 0.35f * fminf(left, 11.5f);
         // max_iter bounds both methods together: what is left has to fit the half of it that is not kept for
         // conjugate gradients, which otherwise take the system as it is
         const float sweeps = ceilf(left / 11.5f);
