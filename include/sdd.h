@@ -480,7 +480,7 @@ sdd_status sdd_keypoint_fill(sdd_ctx* ctx, const uint8_t* mask, double* values_x
  *   SDD_SOLVER_JACOBI  Jacobi preconditioner; one thread-block cluster per
  *                      subdomain; when the subdomain fits its registers,
  *                      Chebyshev iterations first (where those that they
- *                      need fit half of max_iter) and conjugate gradients
+ *                      need fit a quarter of max_iter) and conjugate gradients
  *                      for what they leave;
  *   SDD_SOLVER_MG      a geometric multigrid V-cycle as preconditioner
  *                      (available when every subdomain has the same odd
