@@ -126,13 +126,14 @@ typedef struct {
  *               node's results are then those of the whole list, bit for
  *               bit. A batch numbers its nodes from node_word0 on.
  *   zero_map    0: automatic (the autotuner's choice for the node set, else
- *               on; always on with a control variate); 1 on; 2 off. With it
+ *               on, but for exit_mode 1 on grids of more than 2^23 cells;
+ *               always on with a control variate); 1 on; 2 off. With it
  *               on, the path kernel of a context skips the drift where the
  *               records of a tile's cells are all zero (w constant there): the
  *               same values, so the same results bit for bit, with fewer
  *               gathers and a few more instructions per sub-step. The kernel
  *               leaves the map aside when nearly every tile has drift. Batches
- *               and grids of more than 2^23 cells ignore it. */
+ *               ignore it. */
 typedef struct {
     double dt;
     double Dt;

@@ -118,7 +118,7 @@ struct PathArgs {
 constexpr int kZmapTiles = 47;
 constexpr int kZmapBytes = (kZmapTiles * kZmapTiles + 15) / 16 * 16;
 
-// Largest grid of the single-instance path kernels: cell indices that single precision adds to 2^23 exactly.
+// Largest grid whose cell indices single precision adds to 2^23 exactly (larger ones: an integer index).
 constexpr long long kOneMaxCells = 1LL << 23;
 
 // 1 / v to about an ulp for positive v: a single-precision reciprocal and two Newton steps, four operations of
@@ -178,8 +178,8 @@ cudaError_t launch_paths(const PathArgs& a, int exit_mode, bool record, int grid
 // ntasks: the tasks of all nodes
 cudaError_t launch_finalize(const FinalArgs& a, long long ntasks, cudaStream_t s);
 cudaError_t launch_score_surv(const ScoreArgs& a, bool cv, cudaStream_t s);
-int path_kernel_blocks_per_sm(int exit_mode, bool record, int block, int cvm = 0, bool map = false,
-                              bool single = false, bool defer = false);
+// a: the launch (null: a batch's, without deferred scoring)
+int path_kernel_blocks_per_sm(int exit_mode, bool record, int block, int cvm = 0, const PathArgs* a = nullptr);
 // the largest block the path kernel of this exit mode is compiled for (single: one instance)
 int path_kernel_max_block(int exit_mode, int cvm = 0, bool single = false);
 

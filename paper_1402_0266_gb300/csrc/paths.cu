@@ -47,7 +47,7 @@ __device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b
 
 struct Cell {
     float2 st;        // local coordinates (s, t) in [0, 1)
-    uint32_t idx;     // row-major cell index (plus kCellBits in single-instance kernels)
+    uint32_t idx;     // row-major cell index (plus kCellBits in the kernels of one instance of at most kOneMaxCells cells)
 };
 
 // Cell of pos, strictly inside the unit square, and local coordinates. g = pos (n - 1) stays below n - 1: the
@@ -406,14 +406,23 @@ __device__ __forceinline__ uint32_t zmap_offset(float2 p)
 // from both scores, G from node values interpolated bilinearly in time slices
 // (1, cv_eval) or one value per cell (2, cv_cell).
 // VAR_MULTI: each task's instance from the instance table (batches); VAR_ONE: a
-// single instance whose tables are kernel parameters, with its zero map if it has one.
+// single instance whose tables are kernel parameters, with its zero map if it has one; VAR_BIG: the same for
+// grids of more than kOneMaxCells cells, with an integer cell index. Its blocks stay at paths_min_blocks an SM (32 warps, 24
+// with a control variate): where L2 does not hold the records, more warps spread the gathers over more of them. 4,774
+// nodes x 8,000 paths x 100 sub-steps at 4097^2: drift everywhere 17.3 ms (19.6 with 40 warps, 17.3 in the batch
+// kernel), with cell gradients 39.2 (45.7 with 32 warps, 39.1); the ring 11.7 (10.9 with 40, 17.0 in the batch kernel, which has
+// no map) and 22.3 with cell gradients (38.2).
 // DEFER: survivors and plain exits leave records for k_score_surv.
-constexpr int VAR_MULTI = 0, VAR_ONE = 1;
+constexpr int VAR_MULTI = 0, VAR_ONE = 1, VAR_BIG = 2;
+int variant(const PathArgs& a)
+{
+    return !a.single ? VAR_MULTI : (long long)(a.one.nx - 1) * (a.one.ny - 1) > kOneMaxCells ? VAR_BIG : VAR_ONE;
+}
 constexpr int kOneMaxBlock = 256;
 constexpr int paths_max_block(int cvm, int var) { return cvm ? kCvMaxBlock : var != VAR_MULTI ? kOneMaxBlock : 512; }
 constexpr int paths_min_blocks(int mode, int cvm, int var)
 {
-    return cvm ? (var != VAR_MULTI ? 4 : 3) : var == VAR_MULTI ? 2 : mode == 1 ? 4 : 5;
+    return cvm ? (var == VAR_ONE ? 4 : 3) : var == VAR_MULTI ? 2 : var == VAR_BIG || mode == 1 ? 4 : 5;
 }
 
 // A lane's sums over a task, in shared memory: they change once per path, and the
@@ -522,7 +531,7 @@ __device__ __forceinline__ void walk_tasks(const PathArgs& a, const uint8_t* zsm
     constexpr int LEFT = 7;   // a path that left by the plain test; otherwise the face of a bridge exit
     constexpr bool CV = CVM != 0;
     constexpr bool CVT = CVM == 1;   // node values in time slices
-    constexpr bool ONE = VAR != VAR_MULTI;
+    constexpr bool ONE = VAR == VAR_ONE;
     constexpr bool PAIRS = MODE != 1;
     constexpr bool ACC = !DEFER || MODE == 1;   // some scores are summed here
     const uint32_t step = a.step_ptr ? *a.step_ptr : a.step_index;
@@ -743,7 +752,7 @@ __global__ void __launch_bounds__(paths_max_block(CVM, VAR), paths_min_blocks(MO
 {
     __shared__ LaneSums<paths_max_block(CVM, VAR), !DEFER || MODE == 1> sums;
     __shared__ LaneExits<paths_max_block(CVM, VAR), CVM != 0> left;
-    if (VAR == VAR_ONE && a.zmap) {
+    if (VAR != VAR_MULTI && a.zmap) {
         // stage the zero map, and leave it unused where nearly every tile is marked
         extern __shared__ __align__(16) uint8_t zsm[];
         __shared__ int marked;
@@ -1258,10 +1267,12 @@ const void* pick_var(int mode, bool record, int cvm, bool defer)
 }
 
 // cvm: 0 no control variate, 1 node values in time slices, 2 one value per cell
-const void* pick(int mode, bool record, int cvm, bool single, bool defer)
+const void* pick(int mode, bool record, int cvm, int var, bool defer)
 {
     if (mode == 3) return record ? (const void*)k_paths_exp<true> : (const void*)k_paths_exp<false>;
-    return single ? pick_var<VAR_ONE>(mode, record, cvm, defer) : pick_var<VAR_MULTI>(mode, record, cvm, defer);
+    if (var == VAR_ONE) return pick_var<VAR_ONE>(mode, record, cvm, defer);
+    if (var == VAR_BIG) return pick_var<VAR_BIG>(mode, record, cvm, defer);
+    return pick_var<VAR_MULTI>(mode, record, cvm, defer);
 }
 
 int kernel_mode(int exit_mode, int K)
@@ -1277,15 +1288,16 @@ int path_kernel_max_block(int exit_mode, int cvm, bool single)
     return exit_mode == 2 ? 512 : paths_max_block(cvm, single ? VAR_ONE : VAR_MULTI);
 }
 
-int path_kernel_blocks_per_sm(int exit_mode, bool record, int block, int cvm, bool map, bool single, bool defer)
+int path_kernel_blocks_per_sm(int exit_mode, bool record, int block, int cvm, const PathArgs* a)
 {
     int n = 0;
     // the even-K kernel has the same footprint class; size the grid for the larger of the two
     const int mode = exit_mode == 2 ? 3 : exit_mode == 1 ? 1 : 0;
-    const size_t smem = map && mode != 3 ? kZmapBytes : 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, pick(mode, record, cvm, single, defer), block, smem) !=
-        cudaSuccess)
+    const size_t smem = a && a->zmap && mode != 3 ? kZmapBytes : 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+            &n, pick(mode, record, cvm, a ? variant(*a) : VAR_MULTI, a && a->surv), block, smem) != cudaSuccess)
         return 1;
+    if (a && variant(*a) == VAR_BIG) n = std::min(n, paths_min_blocks(mode, cvm, VAR_BIG));
     return n > 0 ? n : 1;
 }
 
@@ -1294,7 +1306,7 @@ cudaError_t launch_paths(const PathArgs& a, int exit_mode, bool record, int grid
     const int mode = kernel_mode(exit_mode, a.K);
     const size_t smem = a.zmap && mode != 3 ? kZmapBytes : 0;
     void* args[] = {(void*)&a};
-    return cudaLaunchKernel(pick(mode, record, cvm, a.single != 0, a.surv != nullptr), dim3((unsigned)grid),
+    return cudaLaunchKernel(pick(mode, record, cvm, variant(a), a.surv != nullptr), dim3((unsigned)grid),
                             dim3((unsigned)block), args, smem, s);
 }
 
