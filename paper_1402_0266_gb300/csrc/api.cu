@@ -333,7 +333,7 @@ sdd_status prepare_parts(sdd_ctx* c, cudaStream_t s, bool w_part, bool f_part)
 {
     const PrepItem it = take_dirty(c, w_part, f_part);
     if (!it.bcoef && !it.fcoef) return SDD_OK;
-    const cudaError_t e = launch_prep(&it, 1, s);
+    const cudaError_t e = launch_prep(&it, 1, c->sm_count, s);
     if (e != cudaSuccess) c->dirty_w = c->dirty_faces = c->dirty_fields = true;
     CU(c, e);
     return SDD_OK;
@@ -358,7 +358,7 @@ sdd_status prepare_all(std::string* err, const std::vector<sdd_ctx*>& ctxs, cuda
         const PrepItem it = take_dirty(c, true, true);
         if (it.bcoef || it.fcoef) items.push_back(it);
     }
-    const cudaError_t e = launch_prep(items.data(), (int)items.size(), s);
+    const cudaError_t e = launch_prep(items.data(), (int)items.size(), ctxs[0]->sm_count, s);
     if (e != cudaSuccess)
         for (sdd_ctx* c : ctxs) c->dirty_w = c->dirty_faces = c->dirty_fields = true;
     CU(err, e);
@@ -845,7 +845,7 @@ sdd_status setup_solver(sdd_ctx* c)
             mx_max = std::max(mx_max, mx);
         }
         c->solve_upt = solve_reg_upt(band_max);
-        if (4 * (size_t)(rows_max + 2) * (mx_max + 2) * sizeof(float) > 200 * 1024 || C > 16) c->solve_upt = 0;
+        if (4 * (size_t)(rows_max + 2) * (mx_max + 2) * sizeof(float) > kSolveMaxSmem || C > 16) c->solve_upt = 0;
         if (c->solve_upt) {
             c->systems = subs;
             c->solve_cluster = C;
@@ -1309,7 +1309,7 @@ sdd_status train_loop(sdd_ctx* c, float* theta, const float* norm, const float* 
     if (nb < 1) return fail(c, SDD_EINVAL, "fewer rows than one batch");
     int64_t total = (int64_t)p->epochs * nb;
     const int64_t run = p->max_steps > 0 ? std::min<int64_t>(p->max_steps, total) : total;
-    const int nblk = mlp_grad_blocks(p->batch);
+    const int nblk = mlp_grad_blocks(p->batch, c->sm_count);
     CU(c, c->cv_m.alloc(2 * (size_t)kMlpStride));
     CU(c, c->cv_v.alloc(2 * (size_t)kMlpStride));
     CU(c, c->cv_part.alloc(2 * (size_t)nblk * kMlpStride));
@@ -1319,7 +1319,8 @@ sdd_status train_loop(sdd_ctx* c, float* theta, const float* norm, const float* 
     for (int64_t t = 0; t < run; ++t) {
         const int64_t b = t % nb;
         const double lr = p->lr * 0.5 * (1.0 + std::cos(M_PI * (double)t / (double)total));
-        CU(c, launch_mlp_grad(theta, norm, feats, targets, b * p->batch, p->batch, inv, c->cv_part.p, c->stream));
+        CU(c, launch_mlp_grad(theta, norm, feats, targets, b * p->batch, p->batch, inv, c->cv_part.p, c->sm_count,
+                              c->stream));
         CU(c, launch_mlp_adam(theta, c->cv_m.p, c->cv_v.p, c->cv_part.p, nblk, lr, t + 1, inv, losses, run, t,
                               c->stream));
     }
@@ -1838,10 +1839,10 @@ sdd_status sdd_mlp_grad(sdd_ctx* c, const float* theta, const float* norm, const
     const int tile = mlp_tile_rows();
     if (rows < tile || rows % tile != 0 || rows > (1LL << 28))
         return fail(c, SDD_EINVAL, "rows must be a positive multiple of %d", tile);
-    const int nblk = mlp_grad_blocks(rows);
+    const int nblk = mlp_grad_blocks(rows, c->sm_count);
     CU(c, c->cv_grad_part.alloc(2 * (size_t)nblk * kMlpStride));
     const float inv = (float)(1.0 / (double)rows);
-    CU(c, launch_mlp_grad(theta, norm, feats, targets, 0, rows, inv, c->cv_grad_part.p, c->stream));
+    CU(c, launch_mlp_grad(theta, norm, feats, targets, 0, rows, inv, c->cv_grad_part.p, c->sm_count, c->stream));
     CU(c, launch_mlp_reduce(c->cv_grad_part.p, nblk, inv, grad, loss, c->stream));
     return SDD_OK;
 }
@@ -2104,7 +2105,7 @@ static sdd_status capture_step(sdd_ctx* c, const sdd_step_params* p, int K, int 
         // the drift records; the face data come from the third branch forked above
         PrepItem it = take_dirty(c, true, false);
         it.faces64 = nullptr;
-        cu(launch_prep(&it, 1, s));
+        cu(launch_prep(&it, 1, c->sm_count, s));
         if (!c->user_faces && p->exit_mode != 0) cu(cudaStreamWaitEvent(s, c->fev[1], 0));
         c->dirty_w = false;
     } else if (st == SDD_OK) {

@@ -196,7 +196,7 @@ struct PrepItem {
     int* status;
     int32_t nx, ny;
 };
-cudaError_t launch_prep(const PrepItem* items, int n, cudaStream_t s);
+cudaError_t launch_prep(const PrepItem* items, int n, int sm_count, cudaStream_t s);
 // The paper's boundary data from w (faces64) and, if faces32 is non-null, its single-precision copy.
 cudaError_t launch_winslow_faces(const float* w, int nx, int ny, double* faces64, float* faces32, cudaStream_t s);
 cudaError_t launch_cv_cells(const double* grad, int slices, int nx, int ny, uint4* cvcoef, cudaStream_t s);
@@ -234,9 +234,9 @@ cudaError_t launch_cv_scatter(const double* xs, const double* ys, const double* 
 size_t mlp_norm_scratch_doubles();
 cudaError_t launch_mlp_norm(const float* feats, long long n, double* scratch, float* norm, cudaStream_t s);
 int mlp_tile_rows();                      // batches are multiples of this
-int mlp_grad_blocks(long long rows);      // partial gradients per network that a batch of `rows` writes
+int mlp_grad_blocks(long long rows, int sm_count);   // partial gradients per network that a batch of `rows` writes
 cudaError_t launch_mlp_grad(const float* theta, const float* norm, const float* feats, const float* targets,
-                            long long row0, long long rows, float inv_batch, float* part, cudaStream_t s);
+                            long long row0, long long rows, float inv_batch, float* part, int sm_count, cudaStream_t s);
 cudaError_t launch_mlp_reduce(const float* part, int nblk, float inv_rows, float* grad, float* loss, cudaStream_t s);
 cudaError_t launch_mlp_adam(float* theta, float* m, float* v, const float* part, int nblk, double lr, long long t,
                             float inv_rows, float* losses, long long steps, long long step, cudaStream_t s);
@@ -346,6 +346,7 @@ cudaError_t launch_solve_setup(const float* w, const double* prev_xi, const doub
                                double Dt, double* cx, double* cy, double* dg, double* rhs0, float* cxf, float* cyf,
                                float* dgf, float* dinvf, int* status, cudaStream_t s);
 int solve_cluster_size(int nsys, int min_rows, int max_mx, int max_my);
+constexpr int kSolveMaxSmem = 200 * 1024;   // shared memory of the register-resident kernel, at most
 cudaError_t launch_dirichlet(const double* faces64, const double* prev_xi, const double* prev_eta,
                              const double* iface_xi, const double* iface_eta, const int32_t* iface_idx,
                              int n_iface, int nx, int ny, double* xi_out, double* eta_out, cudaStream_t s);

@@ -294,14 +294,14 @@ static cudaError_t launch_prep_n(const PrepItem* items, int n, cudaStream_t s)
     return cudaGetLastError();
 }
 
-cudaError_t launch_prep(const PrepItem* items, int n, cudaStream_t s)
+cudaError_t launch_prep(const PrepItem* items, int n, int sm_count, cudaStream_t s)
 {
     for (int k0 = 0; k0 < n; k0 += PREP_MANY) {
         const int m = std::min(n - k0, PREP_MANY);
         long long blocks8 = 0;
         for (int k = k0; k < k0 + m; ++k)
             blocks8 += (long long)((items[k].nx - 1 + PREP_TX - 1) / PREP_TX) * ((items[k].ny - 1 + 7) / 8);
-        const bool tall = blocks8 >= 4 * 152;
+        const bool tall = blocks8 >= 4LL * sm_count;
         const PrepItem* q = items + k0;
         const cudaError_t e = m == 1 ? (tall ? launch_prep_n<8, 1>(q, m, s) : launch_prep_n<2, 1>(q, m, s))
                                      : (tall ? launch_prep_n<8, PREP_MANY>(q, m, s) : launch_prep_n<2, PREP_MANY>(q, m, s));

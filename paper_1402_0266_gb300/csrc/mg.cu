@@ -35,6 +35,7 @@ namespace {
 
 constexpr int MG_THREADS = 256;
 constexpr int TAIL_THREADS = 1024;
+constexpr int TAIL_MAX_SMEM = 214200;   // of k_mg_tail, over every shape that mg_levels admits
 
 // padded index -> (i, j) of level l
 struct Lv {
@@ -864,8 +865,9 @@ static cudaError_t vcycle(const MgArgs& a, cudaStream_t s)
         return e;
     auto grid = [&](int l) { return dim3((unsigned)(tiles(a.mx[l]) * tiles(a.my[l])), (unsigned)a.nsys); };
     for (int l = 0; l < a.tail; ++l) k_mg_down<<<grid(l), MG_THREADS, sizeof(PreSmem), s>>>(a, l, tiles(a.mx[l]));
+    // the limit is that of every shape, so that another thread's launch keeps it
     const size_t smem = tail_smem_bytes(a);
-    if ((e = cudaFuncSetAttribute(k_mg_tail, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+    if ((e = cudaFuncSetAttribute(k_mg_tail, cudaFuncAttributeMaxDynamicSharedMemorySize, TAIL_MAX_SMEM)) != cudaSuccess)
         return e;
     k_mg_tail<<<a.nsys, TAIL_THREADS, smem, s>>>(a);
     for (int l = a.tail - 1; l >= 0; --l)

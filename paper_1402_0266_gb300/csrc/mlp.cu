@@ -1032,15 +1032,19 @@ cudaError_t launch_mlp_norm(const float* feats, long long n, double* scratch, fl
 int mlp_tile_rows() { return TILE; }
 
 // Two blocks per SM, one for each network (three, at 80 registers, took as long).
-int mlp_grad_blocks(long long rows) { return (int)std::min<long long>(152, (rows + TILE - 1) / TILE); }
+int mlp_grad_blocks(long long rows, int sm_count)
+{
+    return (int)std::min<long long>(sm_count, (rows + TILE - 1) / TILE);
+}
 
 cudaError_t launch_mlp_grad(const float* theta, const float* norm, const float* feats, const float* targets,
-                            long long row0, long long rows, float inv_batch, float* part, cudaStream_t s)
+                            long long row0, long long rows, float inv_batch, float* part, int sm_count,
+                            cudaStream_t s)
 {
     const size_t smem = sizeof(GradSmem);
     cudaError_t e = cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    const dim3 grid((unsigned)mlp_grad_blocks(rows), 2);
+    const dim3 grid((unsigned)mlp_grad_blocks(rows, sm_count), 2);
     k_mlp_grad<<<grid, GRAD_THREADS, smem, s>>>(theta, norm, feats, targets, row0, rows, inv_batch, part);
     return cudaGetLastError();
 }

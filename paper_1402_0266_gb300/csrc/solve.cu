@@ -771,29 +771,26 @@ cudaError_t launch_scatter_iface(const double* iface_xi, const double* iface_eta
     return cudaGetLastError();
 }
 
-// Clusters of 2^k blocks that run at once, a block per SM (nine clusters of 16 do not, although 144 SMs
+// Clusters of 2^k blocks that run at once on the current device, a block per SM (nine clusters of 16 do not, although 144 SMs
 // would hold them: clusters stay inside the GPU's groups of SMs).
 static int clusters_at_once(int k)
 {
-    static int at_once[5] = {-1, -1, -1, -1, -1};
-    if (at_once[k] < 0) {
-        const auto fn = k_solve<4, false>;
-        cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(1u << k);
-        cfg.blockDim = dim3(SOLVE_THREADS);
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = 1u << k;
-        at[0].val.clusterDim.y = 1;
-        at[0].val.clusterDim.z = 1;
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
-        int n = 0;
-        at_once[k] = cudaOccupancyMaxActiveClusters(&n, fn, &cfg) == cudaSuccess ? n : 0;
-        cudaGetLastError();
-    }
-    return at_once[k];
+    const auto fn = k_solve<4, false>;
+    cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(1u << k);
+    cfg.blockDim = dim3(SOLVE_THREADS);
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 1u << k;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, fn, &cfg) != cudaSuccess) n = 0;
+    cudaGetLastError();
+    return n;
 }
 
 // Blocks per system (a power of two up to 16, no more than the smallest system's rows) for systems of at
@@ -801,6 +798,7 @@ static int clusters_at_once(int k)
 // at once x (0.4 us + 0.25 us per unknown of a thread) an iteration. One block (no cluster barrier) pays for
 // up to 256 unknowns; above, its SM's few double-precision units make the residuals longer than the barrier.
 // Bands that need more than 4 unknowns per thread leave the register-resident kernels and are the last choice.
+// Asked for once per context, of the context's device.
 int solve_cluster_size(int nsys, int min_rows, int max_mx, int max_my)
 {
     if (max_mx * max_my <= 256) return 1;
@@ -842,7 +840,8 @@ static cudaError_t launch_reg(const SolveArgs& a, int rows_max, int max_mx, cuda
     const auto fn = a.cluster == 1 ? k_solve<UPT, true> : k_solve<UPT, false>;
     if (a.cluster > 8) cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        // the largest that any context asks for: another thread's launch keeps its limit
+        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSolveMaxSmem);
         if (e != cudaSuccess) return e;
     }
     cudaLaunchAttribute at[1];

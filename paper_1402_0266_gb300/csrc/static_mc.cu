@@ -219,7 +219,7 @@ sdd_status sdd_interface_mc_static(const sdd_fields* f, const sdd_nodes* nodes, 
     else STATIC_CU(launch_winslow_faces(f->w, nx, ny, faces64, nullptr, s));
     STATIC_CU(launch_faces32(faces64, faces32, nfaces, s));
     const PrepItem tables{f->w, f->xi, f->eta, bcoef, fcoef, nullptr, nullptr, nullptr, status, nx, ny};
-    STATIC_CU(launch_prep(&tables, 1, s));
+    STATIC_CU(launch_prep(&tables, 1, sm_count, s));
     // the paths, then the per-node means
     if (t > 0) {
         PathArgs a{};
