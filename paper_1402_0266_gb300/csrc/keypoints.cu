@@ -39,6 +39,13 @@ __device__ __forceinline__ double larger(double a, double b)
     return __longlong_as_double(max(__double_as_longlong(a), __double_as_longlong(b)));
 }
 
+// |d|, 0 where d is not a number: beside a density that is none the other differences keep their maximum.
+__device__ __forceinline__ double magnitude(double d)
+{
+    const double m = fabs(d);
+    return __double_as_longlong(m) > 0x7ff0000000000000LL ? 0.0 : m;
+}
+
 // One block per line: the profiles in shared memory, their largest sizes, then
 // the extremum test at every position the line owns. Two 41-position lines: 27 us with every
 // thread of 1,024 comparing 32 warps' maxima in double precision, 7 us now.
@@ -61,8 +68,8 @@ __global__ void __launch_bounds__(KP_THREADS) k_keypoints(const float* __restric
         const double d2 = (rp - r0) - (r0 - rm);
         prof[t] = d1;
         prof[n + t] = d2;
-        m1 = larger(m1, fabs(d1));
-        m2 = larger(m2, fabs(d2));
+        m1 = larger(m1, magnitude(d1));
+        m2 = larger(m2, magnitude(d2));
     }
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     for (int o = 16; o; o >>= 1) {
