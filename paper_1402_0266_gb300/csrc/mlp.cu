@@ -296,7 +296,8 @@ struct TileSum {
         c += (s - (t - b)) + (v - b);
         s = t;
     }
-    __device__ __forceinline__ float value() const { return s + c; }
+    // the error of a sum that is infinite is not a number
+    __device__ __forceinline__ float value() const { return isfinite(c) ? s + c : s; }
 };
 
 // acc[r][c] += sum_q a[row(r)][q] b[q][col(c)] over q < 64, even and odd q apart, columns 2 tx, 2 tx + 1 and 32 more
