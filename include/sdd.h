@@ -477,7 +477,7 @@ sdd_status sdd_keypoint_fill(sdd_ctx* ctx, const uint8_t* mask, double* values_x
  *                      SDD_EINVAL; status bit when rtol is missed, and
  *                      after a pivot that is not positive the subdomain's
  *                      fields keep their previous values); slower than
- *                      Jacobi-PCG on these sizes, so never chosen automatically;
+ *                      Jacobi on these sizes, so never chosen automatically;
  *   SDD_SOLVER_JACOBI  Jacobi preconditioner; one thread-block cluster per
  *                      subdomain; when the subdomain fits its registers,
  *                      Chebyshev iterations first (where those that they
@@ -512,7 +512,7 @@ int32_t sdd_solver_in_use(const sdd_ctx* ctx);
  * statistics of the step can be read with sdd_last_interface_stats.
  *
  * Pipelining: where the subdomain solve's iterations are one kernel launch
- * (the cluster multigrid or Jacobi-PCG kernels) and the paths do not read the
+ * (the cluster multigrid or Jacobi kernels) and the paths do not read the
  * fields (no SDD_CV_FIELDS), the iterations of step n's solve run inside step
  * n + 1's graph, beside its paths; the paths that survive step n + 1 are
  * scored once they are done. Every call that reads or writes the fields

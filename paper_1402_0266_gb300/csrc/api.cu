@@ -169,7 +169,7 @@ struct sdd_ctx {
     // multigrid-preconditioned solver (every subdomain the same size)
     bool mg_ok = false;
     MgArgs mg{};
-    int solver = 0;                 // 0 automatic, 1 Jacobi-PCG, 2 multigrid-PCG, 3 direct
+    int solver = 0;                 // 0 automatic, 1 Jacobi, 2 multigrid-PCG, 3 direct
     size_t solve_nsys_used = 0;     // systems of the last enqueued solve (entries of d_iters)
     DevBuf<SolveSys> mg_sys;
     DevBuf<float> mg_lv[10], mg_kv[6], mg_part, mg_rz, mg_rr0;
@@ -984,17 +984,19 @@ sdd_status enqueue_keypoints(sdd_ctx* c, uint8_t* mask, cudaStream_t s)
 }
 
 // Automatic solver choice: multigrid where the register-resident Jacobi kernel
-// does not fit, and from 10,000 unknowns per subdomain (127^2: 1.32 against
-// 1.56 ms per step at 257^2 with 2 x 2 subdomains; 19^2: Jacobi is faster).
+// does not fit, and from 10,000 unknowns per subdomain, where its time hardly depends on Dt: a direct solve of 4 x 127^2
+// unknowns takes 0.60 ms at Dt = 1e-4 and 1e-3, 0.66 to 0.85 at 1e-2 and 0.1; Jacobi takes 0.15, 0.33, 0.79 and 1.2
+// (the line was drawn when conjugate gradients alone took 1.56 ms of a step at Dt = 1e-2 against 1.32). Below,
+// Jacobi is faster up to Dt = 0.1 (63^2: 0.07 to 0.37 ms against 0.32 to 0.54).
 bool mg_auto(const sdd_ctx* c)
 {
     return c->solve_upt == 0 || (long long)c->mg.mx[0] * c->mg.my[0] >= 10000;
 }
 
-// The solver the next solve uses: 3 direct, 2 multigrid-PCG, 1 Jacobi-PCG. The
+// The solver the next solve uses: 3 direct, 2 multigrid-PCG, 1 Jacobi. The
 // direct solve is taken only on request: its column and substitution chains
-// are sequential, and Jacobi-PCG is faster on every subdomain it fits (19^2:
-// 159 against 176 us per solve with the set-up, 31^2: 222 against 605 us).
+// are sequential, and Jacobi is faster on every subdomain it fits (four of 19^2 with the set-up:
+// 46 to 127 us at Dt = 1e-4 to 0.1 against 181, of 31^2 50 to 183 against 495 to 607).
 int solver_choice(const sdd_ctx* c)
 {
     if (c->solver == 3 && c->chol_ok) return 3;
@@ -1098,7 +1100,7 @@ SolveCall make_solve_call(sdd_ctx* c, double Dt, double rtol, int max_iter, doub
 }
 
 // The iterations are one kernel launch (the cluster multigrid solve or the
-// Jacobi-PCG kernels), so they can run beside other work.
+// Jacobi kernels), so they can run beside other work.
 bool solve_single_launch(const SolveCall& k) { return k.use_chol || !k.use_mg || k.mgc_upt > 0; }
 
 // The Dirichlet data of an implicit subdomain step on stream s: the faces and

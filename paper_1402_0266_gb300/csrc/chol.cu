@@ -17,9 +17,9 @@
 // digits); a field that does not get there sets the status bit.
 //
 // Speed: the factorisation is m sequential column steps (one block barrier
-// each) and every substitution 2 m sequential steps; on 19 x 19 subdomains a
-// solve with its set-up takes 176 us against 159 us for Jacobi-PCG (51
-// iterations), on 31 x 31 605 against 222 us. It is the exact solve the
+// each) and every substitution 2 m sequential steps; on four 19 x 19 subdomains a
+// solve with its set-up takes 181 us against 46 to 127 us with the Jacobi preconditioner
+// (Dt = 1e-4 to 0.1), on 31 x 31 495 to 607 against 50 to 183 us. It is the exact solve the
 // paper uses, offered on request, not the automatic choice.
 //
 // Layout in shared memory: row k of the band holds, at d = 0 .. mx, the

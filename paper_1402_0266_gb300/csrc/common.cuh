@@ -276,7 +276,7 @@ struct SolveArgs {
     int32_t max_outer;       // refinement sweeps allowed
     double rtol;             // on the double-precision residual, relative to ||b||
     float inner_tol;         // inner reduction of ||r|| per refinement sweep
-    int32_t* iters;          // per system: total inner iterations (max_iter + 1 when not converged); then, per system, 1 when the first kernel solved it
+    int32_t* iters;          // per system: total inner iterations (max_iter + 1 when not converged)
     int* status;
 };
 

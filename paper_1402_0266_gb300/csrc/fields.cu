@@ -136,7 +136,8 @@ __global__ void __launch_bounds__(FACE_THREADS) k_winslow_faces(const float* __r
 // shared memory, double precision), then each cell's records. TY is 8, or 2 where blocks of 8 rows
 // would not give every SM four of them: the kernel is bound by the double-precision lanes of the SMs in use.
 // A small grid's faces and cells take 5 and 7 us by themselves, latency for the most part: with a launch for
-// each, 16 grids of 65^2 to 513^2 spent 250 of the 1650 us of a batch's estimate on them; now it takes 1444.
+// each, 16 grids of 65^2 to 513^2 spent 250 of the 1650 us of a batch's estimate on them; with one launch it took
+// 1444 (1371 with the path kernel's gathers left out where there is no drift).
 constexpr int PREP_TX = 32;
 constexpr int PREP_MANY = 16;
 

@@ -2,7 +2,7 @@
 //
 // The subdomain systems of Sec. 4 (the implicit step of Eq. (3) in the
 // symmetric form xi / (w Dt) + sum_nb c_nb (xi - xi_nb) = rhs, an SPD
-// M-matrix) become ill-conditioned as the grid is refined: Jacobi-PCG needs
+// M-matrix) become ill-conditioned as the grid is refined: the Jacobi preconditioner needs
 // O(sqrt(Dt) / h) iterations, about 1,800 at 2049^2 with Dt = 1e-3. A
 // geometric multigrid V-cycle as preconditioner brings that to a few tens.
 //
@@ -19,7 +19,7 @@
 // of at most 4096 unknowns run inside one block per system; a larger level is
 // one launch down and one up.
 //
-// Precision, as in the Jacobi-PCG kernels: the residual b - A x and the
+// Precision, as in the Jacobi kernels: the residual b - A x and the
 // update x += d are double precision; the inner conjugate gradients on A d = r
 // and the V-cycle are single precision (iterative refinement). Every dot
 // product is reduced per block, then in block order. The solve runs inside a

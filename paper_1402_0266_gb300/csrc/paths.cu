@@ -510,12 +510,12 @@ __device__ __forceinline__ unsigned lanes_below()
 }
 
 // The tasks of one warp. MAP: the drift is read through the zero map zsm: a lane in
-// an unmarked tile has zero drift (it reads the all-zero record when other lanes of
-// its warp need theirs), and a warp without a lane in a marked tile only adds the increment.
+// an unmarked tile has zero drift (it reads nothing; with the bridge test or time slices the all-zero
+// record), and a warp without a lane in a marked tile only adds the increment.
 //
 // What bounds it (GB300, two sub-steps of a warp's 32 paths = one pass): a gather of 32 records that
 // miss L1 takes 34 cycles of the SM whatever its width (32 bytes per cycle from L2), so a pass with
-// drift everywhere costs 64 or more (2.7e11 path-steps/s at 2049^2, L1 data pipe 87 % busy); a pass
+// drift everywhere costs 64 or more (2.7e11 path-steps/s at 2049^2, L1 data pipe 80 % busy); a pass
 // without drift is 119 instructions, 45 cycles, bound by issue slots and the FMA pipe's wide
 // multiplies (4.5e11). Hence the branch around the gather, the draws' shared first rounds, the sums
 // in shared memory and 48 registers (40 warps per SM; 32 and 48 warps are within 2 %), a draw made
@@ -1061,7 +1061,7 @@ constexpr int FINAL_WARPS = 8;
 
 // One node by `warps` warps (a block; one: a warp of a two-warp block). A node's task partials are a
 // chain of loads and of double-precision additions on lanes that hold two of them an SM cycle: one warp a node took
-// 16 us for 253 nodes of 10,000 paths, four take 9.
+// 16 us for 253 nodes of 8,000 paths, four take 9.
 __global__ void __launch_bounds__(FINAL_WARPS * 32) k_finalize(const FinalArgs a, int warps)
 {
     __shared__ NodeSums part[FINAL_WARPS];

@@ -432,7 +432,7 @@ __device__ __forceinline__ bool cheb_solve(const SolveArgs& a, int rows_max, flo
 }
 
 // Register-resident conjugate gradients for subdomains whose band fits in the block, for
-// the systems that cheb_solve left short of rtol (little mass, strong contrasts: the modes below its interval):
+// the systems that cheb_solve left short of rtol (strong contrasts: the modes below its interval) or alone (max_iter):
 // one cluster solves both fields of a subdomain (same matrix, two right-hand
 // sides), so the cluster barriers are shared by the two solves. Each thread
 // keeps UPT unknowns (coefficients and, per field, the CG vectors) in
