@@ -985,9 +985,9 @@ sdd_status enqueue_keypoints(sdd_ctx* c, uint8_t* mask, cudaStream_t s)
 
 // Automatic solver choice: multigrid where the register-resident Jacobi kernel
 // does not fit, and from 10,000 unknowns per subdomain, where its time hardly depends on Dt: a direct solve of 4 x 127^2
-// unknowns takes 0.60 ms at Dt = 1e-4 and 1e-3, 0.66 to 0.85 at 1e-2 and 0.1; Jacobi takes 0.15, 0.33, 0.79 and 1.2
+// unknowns takes 0.60 ms at Dt = 1e-4 and 1e-3, 0.66 to 0.85 at 1e-2 and 0.1; Jacobi takes 0.13, 0.28, 0.62 and 0.95
 // (the line was drawn when conjugate gradients alone took 1.56 ms of a step at Dt = 1e-2 against 1.32). Below,
-// Jacobi is faster up to Dt = 0.1 (63^2: 0.07 to 0.37 ms against 0.32 to 0.54).
+// Jacobi is faster up to Dt = 0.1 (63^2: 0.06 to 0.32 ms against 0.32 to 0.54).
 bool mg_auto(const sdd_ctx* c)
 {
     return c->solve_upt == 0 || (long long)c->mg.mx[0] * c->mg.my[0] >= 10000;
@@ -996,7 +996,7 @@ bool mg_auto(const sdd_ctx* c)
 // The solver the next solve uses: 3 direct, 2 multigrid-PCG, 1 Jacobi. The
 // direct solve is taken only on request: its column and substitution chains
 // are sequential, and Jacobi is faster on every subdomain it fits (four of 19^2 with the set-up:
-// 46 to 127 us at Dt = 1e-4 to 0.1 against 181, of 31^2 50 to 183 against 495 to 607).
+// 45 to 111 us at Dt = 1e-4 to 0.1 against 181, of 31^2 49 to 156 against 495 to 608).
 int solver_choice(const sdd_ctx* c)
 {
     if (c->solver == 3 && c->chol_ok) return 3;

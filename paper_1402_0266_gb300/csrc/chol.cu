@@ -18,8 +18,8 @@
 //
 // Speed: the factorisation is m sequential column steps (one block barrier
 // each) and every substitution 2 m sequential steps; on four 19 x 19 subdomains a
-// solve with its set-up takes 181 us against 46 to 127 us with the Jacobi preconditioner
-// (Dt = 1e-4 to 0.1), on 31 x 31 495 to 607 against 50 to 183 us. It is the exact solve the
+// solve with its set-up takes 181 us against 45 to 111 us with the Jacobi preconditioner
+// (Dt = 1e-4 to 0.1), on 31 x 31 495 to 608 against 49 to 156 us. It is the exact solve the
 // paper uses, offered on request, not the automatic choice.
 //
 // Layout in shared memory: row k of the band holds, at d = 0 .. mx, the

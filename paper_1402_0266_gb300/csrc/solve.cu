@@ -229,9 +229,9 @@ __device__ __forceinline__ float log2_of(double v)
 }
 
 // Chebyshev iterations for subdomains whose bands fit the blocks of a cluster, both fields together, and
-// conjugate gradients (cg_solve) in the same launch for what they leave. Solves with their set-up, conjugate gradients
-// alone and now: 4 x 19^2 unknowns 157 -> 54 us, 4 x 63^2 520 -> 136, 9 x 65^2 1358 -> 256, 9 x 119^2 2918 -> 819,
-// 16 x 95^2 2548 -> 1283 (a launch of its own for cg_solve and the library's logarithm cost 17 us more). The method:
+// conjugate gradients (cg_solve) in the same launch for what they leave. Solves with their set-up, each waited for, ring
+// density, Dt = 1e-3, in the kernel that ran conjugate gradients alone before and now: 4 x 19^2 unknowns 186 -> 72 us,
+// 4 x 63^2 439 -> 120, 4 x 119^2 835 -> 252, 16 x 65^2 1307 -> 294, 9 x 119^2 2085 -> 446. The method:
 // A d = r with the diagonal as preconditioner over the interval [lo, 1 + rho] of the eigenvalues of
 // D^-1 A, in single precision, inside the double-precision refinement of the other kernels.
 // rho is Gershgorin's bound, the largest row sum of D^-1 (D - A) (below 1: the mass term), so the upper
@@ -242,14 +242,16 @@ __device__ __forceinline__ float log2_of(double v)
 // Why not conjugate gradients alone: an iteration of theirs is a product, two barriers and a reduction of
 // six sums, a latency chain of about 2.3 us whatever the cluster size; here it is one barrier (one block:
 // a block barrier) and a product whose operands are in registers and shared memory, with no scalar to wait
-// for: 0.5 us with one unknown a thread, 1.3 with four. The iteration count is 0.9 to 1.3 times theirs where the mass term
-// counts (4 x 119^2 unknowns: up to Dt = 1e-2) and twice theirs without it, faster still (Dt = 1: 1.24 against 2.07 ms).
+// for: 0.39 us with one unknown a thread, 0.87 with four. (Which unknowns neighbour another block is found once: by a
+// division per unknown and iteration, where the compiler left it in the loop, 9 x 100^2 took 808 us instead of 545.) The
+// iteration count is 0.9 to 1.3 times theirs where the mass term counts (4 x 119^2 unknowns: up to Dt = 1e-2) and
+// twice theirs without it, faster still (Dt = 1: 0.96 against 2.07 ms).
 //
 // What they lose: blocks of very different density (a 50 : 1 checkerboard at Dt >= 3e-2) have modes far below lo, and
 // sweep after sweep falls short. A sweep that brings the residual down by less than a third of its factor
-// (in the logarithm) is the last: 16 x 65^2 unknowns at Dt = 0.3 take 2.15 ms with one such sweep, 3.10 with six, 2.40 in the
-// kernel that ran conjugate gradients alone before; over Dt = 1e-4 to 1e3, 9^2 to 119^2 unknowns and five densities no
-// solve takes longer than in that kernel (0.993 times at most).
+// (in the logarithm) is the last: with six of them 16 x 65^2 unknowns took 3.10 ms at Dt = 0.3, 2.40 in the kernel that ran
+// conjugate gradients alone before, now 1.91; over Dt = 1e-4 to 1e3, 9^2 to 119^2 unknowns and five densities no
+// solve takes longer than in that kernel (0.93 times at most).
 //
 // Layout: each thread keeps UPT unknowns (scaled coefficients and, per field, scaled residual z, step d,
 // correction e) in registers; the steps d live in shared memory as pairs (both fields), a zero frame around
@@ -290,6 +292,7 @@ __device__ __forceinline__ bool cheb_solve(const SolveArgs& a, int rows_max, flo
     int n_[UPT], sidx[UPT];   // grid index (-1: no unknown), place in a plane
     float cw[UPT], ce[UPT], cs[UPT], cn[UPT];   // couplings to unknowns over the diagonal (0 to Dirichlet nodes)
     float z[2][UPT], d[2][UPT], e[2][UPT];
+    unsigned edge = 0;   // bit 2 k: unknown k is in the band's lowest row, another block below; 2 k + 1: highest, above
     float rho = 0.f;
     double bb[2] = {0.0, 0.0};
 #pragma unroll
@@ -305,6 +308,8 @@ __device__ __forceinline__ bool cheb_solve(const SolveArgs& a, int rows_max, flo
         const int i = S.i0 + lc, j = row0 + lr, n = j * nx + i;
         n_[k] = n;
         sidx[k] = (lr + 1) * W + lc + 1;
+        if (lr == 0 && nb_lo) edge |= 1u << 2 * k;
+        if (lr == rows - 1 && nb_hi) edge |= 2u << 2 * k;
         const float di = a.dinvf[n];
         double b0 = rhs0[n], b1 = rhs1[n];
         if (i > S.i0) cw[k] = a.cxf[n - 1] * di;
@@ -376,14 +381,15 @@ __device__ __forceinline__ bool cheb_solve(const SolveArgs& a, int rows_max, flo
                 for (int k = 0; k < UPT; ++k) z[f][k] = 0.f;
         }
         converged = !active[0] && !active[1];
-        if (converged || !number) break;   // no number: cg_solve reports it
-        if (left > goal) break;            // the sweep before fell short
+        // Left to conjugate gradients: what is not a number (they report it), what the sweep before brought too
+        // little of, and what does not fit a quarter of max_iter, which bounds both methods together. (With half of
+        // it, checkerboards of 10^4 : 1 at Dt = 1e3 that conjugate gradients solve in 885 iterations were not solved
+        // within 970: of those a sweep that fell short had used 182.)
+        const float sweeps = ceilf(left * (1.f / 11.5f));
+        const bool leave = converged || !number || left > goal ||
+                           left + 2.f * sweeps > per_iter * (0.25f * (float)a.max_iter - (float)total - sweeps);
+        if (leave) break;
         goal = left - 0.35f * fminf(left, 11.5f);
-        // max_iter bounds both methods together: what is left has to fit a quarter of it, or conjugate gradients take the
-        // system as it is. (With half, checkerboards of 10^4 : 1 at Dt = 1e3 that they solve in 885 iterations were
-        // not solved within 970: of those a sweep that fell short had used 182.)
-        const float sweeps = ceilf(left / 11.5f);
-        if ((float)total + (left + 2.f * sweeps) / per_iter + sweeps > 0.25f * (float)a.max_iter) break;
         const int its = (int)ceilf((fminf(left, 11.5f) + 2.f) / per_iter);
         total += its;
         float r_old = 1.f / sigma, ca = 0.f, cb = 1.f / theta;
@@ -401,9 +407,8 @@ __device__ __forceinline__ bool cheb_solve(const SolveArgs& a, int rows_max, flo
                 const float2 v = make_float2(d[0][k], d[1][k]);
                 mine[sidx[k]] = v;
                 if (!ONE) {
-                    const int lr = sidx[k] / W - 1;
-                    if (lr == 0 && nb_lo) nb_lo[b * plane + sidx[k] + rows_below * W] = v;
-                    if (lr == rows - 1 && nb_hi) nb_hi[b * plane + sidx[k] - rows * W] = v;
+                    if (edge & 1u << 2 * k) nb_lo[b * plane + sidx[k] + rows_below * W] = v;
+                    if (edge & 2u << 2 * k) nb_hi[b * plane + sidx[k] - rows * W] = v;
                 }
             }
             const float r_new = __frcp_rn(2.f * sigma - r_old);
@@ -795,7 +800,7 @@ static int clusters_at_once(int k)
 
 // Blocks per system (a power of two up to 16, no more than the smallest system's rows) for systems of at
 // most max_mx columns and max_my rows: the least time by what the Chebyshev iterations measured, rounds of clusters that run
-// at once x (0.4 us + 0.25 us per unknown of a thread) an iteration. One block (no cluster barrier) pays for
+// at once x (0.4 us + 0.25 us per unknown of a thread) an iteration (0.3 + 0.16 since, the same proportion). One block (no cluster barrier) pays for
 // up to 256 unknowns; above, its SM's few double-precision units make the residuals longer than the barrier.
 // Bands that need more than 4 unknowns per thread leave the register-resident kernels and are the last choice.
 // Asked for once per context, of the context's device.
