@@ -99,3 +99,27 @@ def test_the_tuner_finds_the_zero_map(sdd):
     xs, ys = np.random.default_rng(0).uniform(0.2, 0.8, (2, 400))
     shape = sdd.sdd_autotune(ctx, xs, ys, np.full(400, 8000), dt=1e-5, Dt=1e-3)
     assert shape["zero_map"] == 1
+
+
+def test_deferred_scores_match_the_step_without_deferral(sdd):
+    import torch
+    n, sub = 2945, 23   # 529 subdomains of 127^2 unknowns: one launch solves them, so the step can defer its scores
+    X, Y = W.identity_fields(n)
+    got = []
+    for pipeline in (True, False):
+        ctx = sdd.sdd_init(n, n, sub, sub, w=torch.from_numpy(W.w_ring(n, 0.0)).cuda(), xi0=torch.from_numpy(X).cuda(),
+                           eta0=torch.from_numpy(Y).cuda())
+        sdd.sdd_set_pipeline(ctx, pipeline)
+        for k in range(2):
+            sdd.sdd_set_w(ctx, torch.from_numpy(W.w_ring(n, 1e-3 * k)).cuda())
+            sdd.sdd_step(ctx, dt=2e-6, Dt=1e-5, seed=3, paths_per_node=7)
+            assert sdd.sdd_pipeline_in_use(ctx) == pipeline
+        sdd.sdd_sync(ctx)
+        got.append(_np(sdd.sdd_last_interface_stats(ctx)))
+        del ctx
+    a, b = got
+    for k in ("n_exit", "path_steps"):
+        np.testing.assert_array_equal(a[k], b[k], err_msg=k)
+    for k in ("mean_xi", "mean_eta", "se_xi", "se_eta"):
+        # scores agree to a few units of single-precision rounding, in differently grouped sums
+        assert np.abs(a[k] - b[k]).max() <= 2e-6, k
